@@ -137,9 +137,10 @@ static void drop_graph(cpm_ctx* c) {
 static void free_geometry(cpm_ctx* c) {
     drop_graph(c);
     free_ktable(c);
+    free_rows(c);
     void* ptrs[] = {c->sx, c->group, c->s32, c->site64.X, c->site64.Y, c->site64.Z, c->site32.X, c->site32.Y,
                     c->site32.Z, c->A, c->W, c->S, c->S32, c->SG, c->u, c->dvec, c->sxyz, c->zmap, c->zuniq, c->Sb, c->SZ, c->rtab, c->rtab_id,
-                    c->sperm, c->schunks, c->rqueue, c->tcz, c->tcxy, c->c0e, c->ccm_buf, c->ccm_scr, c->SGx,
+                    c->sperm, c->schunks, c->rqueue, c->tcz, c->tcxy, c->c0e, c->c0tab, c->ccm_buf, c->ccm_scr, c->SGx,
                     c->h2d_idx, c->h2d_norm, c->rsite, c->rsite_tab, c->rrun_cell, c->rrun_sh,
                     c->rchunk, c->rsite_idx, c->rbox};
     for (void* p : ptrs) dev_free(c, p);
@@ -148,7 +149,7 @@ static void free_geometry(cpm_ctx* c) {
     c->Sb = nullptr; c->SZ = nullptr;
     c->rtab = nullptr; c->rtab_id = nullptr; c->nrtab = 0;
     c->sperm = nullptr; c->schunks = nullptr; c->rqueue = nullptr; c->nschunk = 0;
-    c->tcz = nullptr; c->tcxy = nullptr; c->c0e = nullptr;
+    c->tcz = nullptr; c->tcxy = nullptr; c->c0e = nullptr; c->c0tab = nullptr;
     c->ccm_buf = nullptr; c->ccm_scr = nullptr; c->SGx = nullptr; c->ccm_scr_bytes = 0; c->ccm_ready = false;
     c->h2d_idx = nullptr; c->h2d_norm = nullptr; c->nh2d = 0;
     c->rsite = nullptr; c->rsite_tab = nullptr; c->rpoly = cpm::RealPoly{}; c->rpoly_blocks = 0;
@@ -446,8 +447,11 @@ static cpm_status assemble_impl(cpm_ctx* c, int64_t n, const double* xyz, const 
     CPM_TRY(launch_phases<double>(st, c->g, k, c->sxyz, n, c->site64.X, c->site64.Y, c->site64.Z));
     CPM_TRY(launch_phases<float>(st, c->g, k, c->sxyz, n, c->site32.X, c->site32.Y, c->site32.Z));
     CPM_LAUNCH(c, "k_phases(sites)");
-    if (c->p.k_prec == CPM_PREC_F16X2) CPM_TRY(tc_recip_prepare(c));
     CPM_TRY(build_col0_sites(c));
+    if (c->p.kspace != CPM_KSPACE_P3M) {
+        CPM_TRY(build_rows(c));
+        if (c->rows.tcitems && !c->rows.layered) CPM_TRY(tc_recip_prepare(c));
+    }
     if (c->p.kspace == CPM_KSPACE_P3M) CPM_TRY(p3m_prepare(c));
     const size_t nn = (size_t)n * n;
     if (with_A) {

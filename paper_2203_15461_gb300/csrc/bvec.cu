@@ -5,12 +5,10 @@
 //             + sum_k w_k Re[exp(-i k.R_i) rho(k)]                      reciprocal space
 //             - pi Q_tot / (V alpha^2) + B_i ]                          background, Sec. II.E
 //
-// Reciprocal space in two contractions over the column layout of the k set
-// (column c = (nx, ny), harmonic nz):
-//   structure factor  rho[c][nz] = sum_j (Q_j X_j[nx_c] Y_j[ny_c]) Z_j[nz]
-//   site potential    b_i      += sum_c Re[ conj(X_i[nx_c] Y_i[ny_c]) sum_nz w[c][nz] rho[c][nz] conj(Z_i[nz]) ]
-// register-tiled on the CUDA cores here (k_prec FP64 and FP32), or as tensor-core products
-// (k_prec F16X2, tc_recip.cu).
+// Reciprocal space: the structure factor and the potential per distinct site height in recip_rows.cu (k_prec
+// FP64 and FP32) or tc_recip.cu (F16X2); for electrodes whose sites hardly share heights the potential of
+// every site by itself, over the column layout of the k set (column c = (nx, ny), harmonic nz):
+//   b_i += sum_c Re[ conj(X_i[nx_c] Y_i[ny_c]) sum_nz w[c][nz] rho[c][nz] conj(Z_i[nz]) ]
 #include <algorithm>
 
 #include "common.cuh"
@@ -631,7 +629,7 @@ cpm_status build_pair_tables(cpm_ctx* c, const std::vector<double>& etas) {
 }
 
 // ----------------------------------------------------------------------------- reciprocal space
-constexpr int SF_BM = 64, SF_BN = 64, SF_BK = 16;
+constexpr int SF_BM = 64, SF_BN = 64, SF_BK = 16;   // site stage: columns x sites x harmonics per step
 
 template <typename T>
 __device__ __forceinline__ int tile_maxext(const int* colext, int c0, int ncols) {
@@ -641,186 +639,6 @@ __device__ __forceinline__ int tile_maxext(const int* colext, int c0, int ncols)
     if (threadIdx.x < SF_BM && c0 + (int)threadIdx.x < ncols) atomicMax(&mx, colext[c0 + threadIdx.x]);
     __syncthreads();
     return mx;
-}
-
-// rho_part[s][r][c][nz] = sum over the s-th particle chunk of replica r of Q_j X_j Y_j Z_j.
-template <typename T>
-__global__ void __launch_bounds__(256) k_sf(const int2* __restrict__ cols, const int* __restrict__ colext, int ncols,
-                                            int NY, int NZ, int nzw, const c2<T>* __restrict__ EX,
-                                            const c2<T>* __restrict__ EY, const c2<T>* __restrict__ EZ,
-                                            const T* __restrict__ Qv, int64_t ptot, int64_t ne, int splits,
-                                            int64_t chunk, int m, c2<T>* __restrict__ rho_part) {
-    __shared__ c2<T> Ps[SF_BK][SF_BM + 1];
-    __shared__ c2<T> Zs[SF_BK][SF_BN + 1];
-    // z tiles are centred on nz = 0: tile t covers grid indices zbase + t*BN ... + BN - 1
-    const int zbase = NZ - SF_BN / 2 - SF_BN * ((int)gridDim.y / 2);
-    const int c0 = blockIdx.x * SF_BM, z0 = zbase + blockIdx.y * SF_BN;
-    const int r = blockIdx.z / splits, s = blockIdx.z % splits;
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    c2<T>* outp = rho_part + ((int64_t)s * m + r) * ncols * nzw;
-    const int mx = tile_maxext<T>(colext, c0, ncols);
-    const bool skip = (z0 - NZ > mx) || (z0 + SF_BN - 1 - NZ < -mx);
-    typedef c2<T> V;
-    V acc[4][4];
-#pragma unroll
-    for (int p = 0; p < 4; ++p)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) acc[p][q] = cmake<T>(0, 0);
-    const int64_t jb = (int64_t)r * ne + (int64_t)s * chunk;
-    const int64_t je = min((int64_t)r * ne + ne, jb + chunk);
-    if (!skip) {
-        for (int64_t j0 = jb; j0 < je; j0 += SF_BK) {
-            for (int e = threadIdx.x; e < SF_BK * SF_BM; e += 256) {
-                int kk = e % SF_BK, mm = e / SF_BK;
-                int64_t j = j0 + kk;
-                int c = c0 + mm;
-                V v = cmake<T>(0, 0);
-                if (j < je && c < ncols) {
-                    int2 cn = cols[c];
-                    V xy = cmul(EX[(int64_t)cn.x * ptot + j], EY[(int64_t)(cn.y + NY) * ptot + j]);
-                    T qj = Qv[j];
-                    v.x = qj * xy.x; v.y = qj * xy.y;
-                }
-                Ps[kk][mm] = v;
-                int z = z0 + mm;
-                V zv = cmake<T>(0, 0);
-                if (j < je && z >= 0 && z < nzw) zv = EZ[(int64_t)z * ptot + j];
-                Zs[kk][mm] = zv;
-            }
-            __syncthreads();
-#pragma unroll 4
-            for (int kk = 0; kk < SF_BK; ++kk) {
-                V av[4], bv[4];
-#pragma unroll
-                for (int p = 0; p < 4; ++p) av[p] = Ps[kk][ty + 16 * p];
-#pragma unroll
-                for (int q = 0; q < 4; ++q) bv[q] = Zs[kk][tx + 16 * q];
-#pragma unroll
-                for (int p = 0; p < 4; ++p)
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        acc[p][q].x += av[p].x * bv[q].x - av[p].y * bv[q].y;
-                        acc[p][q].y += av[p].x * bv[q].y + av[p].y * bv[q].x;
-                    }
-            }
-            __syncthreads();
-        }
-    }
-#pragma unroll
-    for (int p = 0; p < 4; ++p) {
-        int c = c0 + ty + 16 * p;
-        if (c >= ncols) continue;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            int z = z0 + tx + 16 * q;
-            if (z >= 0 && z < nzw) outp[(int64_t)c * nzw + z] = acc[p][q];
-        }
-    }
-}
-
-// Single-precision structure factor with a 64-column x 128-harmonic accumulator tile per block:
-// warp w owns harmonics [16w, 16w + 16) of the tile's z range and skips the contraction when that
-// slab lies outside the largest |nz| of the tile's columns (columns are sorted by k_perp, so the
-// slab test removes most of the padding of the dense grid); the charge operand Q_j X_j Y_j of the
-// tile's columns is formed once per chunk of charges and shared by all 128 harmonics.
-constexpr int S2_BM = 64, S2_BZ = 128, S2_BK = 16;
-
-__global__ void __launch_bounds__(256, 2) k_sf32(const int2* __restrict__ cols, const int* __restrict__ colext,
-                                                 int ncols, int NY, int NZ, int nzw, const float2* __restrict__ EX,
-                                                 const float2* __restrict__ EY, const float2* __restrict__ EZ,
-                                                 const float* __restrict__ Qv, int64_t ptot, int64_t ne, int splits,
-                                                 int64_t chunk, int m, int nsup, float2* __restrict__ rho_part) {
-    __shared__ float2 Ps[S2_BK][S2_BM + 1];
-    __shared__ float2 Zs[S2_BK][S2_BZ + 1];
-    const int c0 = blockIdx.x * S2_BM;
-    const int zbase = NZ - S2_BZ / 2 - S2_BZ * (nsup / 2) + S2_BZ * (int)blockIdx.y;   // grid index of row 0
-    const int r = blockIdx.z / splits, s = blockIdx.z % splits;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int cg = lane & 15, zh = lane >> 4;
-    float2* outp = rho_part + ((int64_t)s * m + r) * ncols * nzw;
-    const int mx = tile_maxext<float>(colext, c0, ncols);
-    // harmonics of this warp: zbase + 16 warp + zh + 2 q, q = 0..7  (nz = index - NZ)
-    const int wz0 = zbase + 16 * warp - NZ, wz1 = wz0 + 15;
-    const bool active = mx >= 0 && !(wz0 > mx || wz1 < -mx);
-    const bool block_any = mx >= 0 && !(zbase - NZ > mx || zbase + S2_BZ - 1 - NZ < -mx);
-    float2 acc[4][8];
-#pragma unroll
-    for (int p = 0; p < 4; ++p)
-#pragma unroll
-        for (int q = 0; q < 8; ++q) acc[p][q] = make_float2(0.f, 0.f);
-    const int64_t jb = (int64_t)r * ne + (int64_t)s * chunk;
-    const int64_t je = min((int64_t)r * ne + ne, jb + chunk);
-    if (block_any) {
-        for (int64_t j0 = jb; j0 < je; j0 += S2_BK) {
-            for (int e = threadIdx.x; e < S2_BK * S2_BM; e += 256) {
-                const int kk = e % S2_BK, mm = e / S2_BK;
-                const int64_t j = j0 + kk;
-                const int c = c0 + mm;
-                float2 v = make_float2(0.f, 0.f);
-                if (j < je && c < ncols) {
-                    const int2 cn = cols[c];
-                    const float2 xy = cmul(EX[(int64_t)cn.x * ptot + j], EY[(int64_t)(cn.y + NY) * ptot + j]);
-                    const float qj = Qv[j];
-                    v = make_float2(qj * xy.x, qj * xy.y);
-                }
-                Ps[kk][mm] = v;
-            }
-            for (int e = threadIdx.x; e < S2_BK * S2_BZ; e += 256) {
-                const int kk = e % S2_BK, zz = e / S2_BK;
-                const int64_t j = j0 + kk;
-                const int z = zbase + zz;
-                Zs[kk][zz] = (j < je && z >= 0 && z < nzw) ? EZ[(int64_t)z * ptot + j] : make_float2(0.f, 0.f);
-            }
-            __syncthreads();
-            if (active) {
-#pragma unroll 2
-                for (int kk = 0; kk < S2_BK; ++kk) {
-                    float2 av[4], bv[8];
-#pragma unroll
-                    for (int p = 0; p < 4; ++p) av[p] = Ps[kk][cg + 16 * p];
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) bv[q] = Zs[kk][16 * warp + zh + 2 * q];
-#pragma unroll
-                    for (int p = 0; p < 4; ++p)
-#pragma unroll
-                        for (int q = 0; q < 8; ++q) {
-                            acc[p][q].x += av[p].x * bv[q].x - av[p].y * bv[q].y;
-                            acc[p][q].y += av[p].x * bv[q].y + av[p].y * bv[q].x;
-                        }
-                }
-            }
-            __syncthreads();
-        }
-    }
-#pragma unroll
-    for (int p = 0; p < 4; ++p) {
-        const int c = c0 + cg + 16 * p;
-        if (c >= ncols) continue;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const int z = zbase + 16 * warp + zh + 2 * q;
-            if (z >= 0 && z < nzw) outp[(int64_t)c * nzw + z] = acc[p][q];
-        }
-    }
-}
-
-// wrho[r][c][nz] = w[c][nz] * sum_s rho_part[s][r][c][nz]  (Neumaier-compensated over the splits)
-template <typename T>
-__global__ void k_sf_reduce(const c2<T>* rho_part, const T* w, int64_t per_rep, int m, int splits, c2<T>* wrho) {
-    int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= per_rep * m) return;
-    T sx = 0, sy = 0, cx = 0, cy = 0;
-    for (int s = 0; s < splits; ++s) {
-        c2<T> v = rho_part[(int64_t)s * per_rep * m + t];
-        T tx = sx + v.x;
-        cx += fabs(sx) >= fabs(v.x) ? (sx - tx) + v.x : (v.x - tx) + sx;
-        sx = tx;
-        T ty = sy + v.y;
-        cy += fabs(sy) >= fabs(v.y) ? (sy - ty) + v.y : (v.y - ty) + sy;
-        sy = ty;
-    }
-    T wt = w[t % per_rep];
-    wrho[t] = cmake<T>(wt * (sx + cx), wt * (sy + cy));
 }
 
 // partial[r][tile][i] = sum over the tile's columns c of Re[conj(X_i Y_i) sum_nz wrho[c][nz] conj(Z_i[nz])]
@@ -909,17 +727,18 @@ __global__ void __launch_bounds__(256) k_site(const int2* __restrict__ cols, con
 // in double-float: their weights are the largest of the whole set (they carry the laterally
 // averaged charge profile), so their terms would dominate the rounding of a single-precision sum.
 // Phases by a double-float recurrence in nz from an exactly reduced first harmonic.
-__device__ __forceinline__ double2 z_phase_n(double z, double invLz, int nz) {
+__device__ __forceinline__ uint64_t z_fraction(double z, double invLz) {
     double s = z * invLz;
     s -= floor(s);
     double t = s * 18446744073709551616.0;
-    uint64_t u = t >= 18446744073709551616.0 ? 0ull : (uint64_t)t;
-    u *= (uint64_t)nz;   // fraction of nz z / Lz, reduced exactly (mod 2^64)
+    return t >= 18446744073709551616.0 ? 0ull : (uint64_t)t;
+}
+__device__ __forceinline__ double2 z_phase_n(double z, double invLz, int nz) {
+    const uint64_t u = z_fraction(z, invLz) * (uint64_t)nz;   // fraction of nz z / Lz, reduced exactly (mod 2^64)
     double sn, cs;
     sincospi((double)(int64_t)u * 0x1p-63, &sn, &cs);
     return make_double2(cs, sn);
 }
-__device__ __forceinline__ double2 z_phase1(double z, double invLz) { return z_phase_n(z, invLz, 1); }
 
 // Double-float arithmetic (pairs of floats, about 48 significant bits; Dekker 1971, Knuth TAOCP
 // vol. 2): the k_perp = 0 column needs better than FP32 accuracy, and FP32 pairs run far faster
@@ -957,98 +776,121 @@ __device__ __forceinline__ dcx dcx_mul(dcx a, dcx b) {
     return {df_add(df_mul(a.re, b.re), df_neg(df_mul(a.im, b.im))), df_add(df_mul(a.re, b.im), df_mul(a.im, b.re))};
 }
 
-// part[r][chunk][nz - 1] for nz in one block of C0_NB harmonics: each thread takes 2 charges of the
-// chunk (256 charges per block), raises exp(i theta) of both to the block's first harmonic and steps
-// through the block by a double-float recurrence (the two charges' chains interleaved); the block
-// sums its threads in a fixed order.
-constexpr int C0_THREADS = 128, C0_PER_THREAD = 2, C0_NB = 6;
-
-__device__ __forceinline__ dcx dcx_pow(dcx e1, int pw) {   // e1^pw by binary powering, pw >= 1
-    dcx e = {{1.f, 0.f}, {0.f, 0.f}}, base = e1;
-    for (; pw > 0; pw >>= 1) {
-        if (pw & 1) e = dcx_mul(e, base);
-        base = dcx_mul(base, base);
-    }
-    return e;
+// exp(2 pi i f) in double-float from the 64-bit fixed-point fraction f: the nearest of 256 tabulated angles, then
+// the rest (at most pi / 256) by its Taylor series, the terms that matter in double-float (error about 2^-47).
+// One FP64 sincospi costs as much of this GPU as 4,000 FP32 operations; this takes about 150.
+constexpr int C0_TAB = 256;
+__device__ __forceinline__ dcx c0_phase(uint64_t u, const float4* __restrict__ tab) {
+    const uint64_t ur = u + (1ull << 55);
+    const int64_t d = (int64_t)(u - (ur & 0xFF00000000000000ull));   // in [-2^55, 2^55)
+    const dfl t = df_fast((float)(int32_t)(d >> 32), (float)(uint32_t)d * 0x1p-32f);
+    constexpr float c_hi = (float)(2.0 * PI * 0x1p-32), c_lo = (float)(2.0 * PI * 0x1p-32 - (double)c_hi);
+    const dfl x = df_mul(t, {c_hi, c_lo});
+    const dfl x2 = df_mul(x, x);
+    // cos x - 1 = x^2 (-1/2 + x^2 / 24 - x^4 / 720), sin x = x + x x^2 (-1/6 + x^2 / 120)
+    const dfl ca = df_two_sum(-0.5f, x2.hi * fmaf(x2.hi, -1.f / 720.f, 1.f / 24.f));
+    const dfl cm1 = df_mul(x2, ca);
+    constexpr float s6 = (float)(-1.0 / 6.0), s6l = (float)(-1.0 / 6.0 - (double)s6);
+    dfl sa = df_two_sum(s6, x2.hi * (1.f / 120.f));
+    sa.lo += s6l;
+    const dfl sn = df_add(x, df_mul(x, df_mul(x2, sa)));
+    const float4 e = tab[ur >> 56];
+    const dfl C = {e.x, e.y}, S = {e.z, e.w};
+    // (C + i S)(1 + cm1 + i sn)
+    return {df_add(C, df_add(df_mul(C, cm1), df_neg(df_mul(S, sn)))), df_add(S, df_add(df_mul(S, cm1), df_mul(C, sn)))};
 }
 
-__global__ void __launch_bounds__(C0_THREADS) k_col0_rho(const float4* __restrict__ e1s, const float2* __restrict__ Qd,
-                                                       int64_t ne, int nz0, double2* __restrict__ part) {
-    __shared__ double2 red[C0_THREADS / 32][C0_NB];
-    const int chunk = blockIdx.x, nb = blockIdx.y, r = blockIdx.z;
-    const int nzs = nb * C0_NB + 1;   // first harmonic of this block
+__global__ void k_col0_tab(float4* __restrict__ tab) {
+    const int t = threadIdx.x;
+    if (t >= C0_TAB) return;
+    double s, c;
+    sincospi(2.0 * t / C0_TAB, &s, &c);
+    const dfl C = df_of(c), S = df_of(s);
+    tab[t] = make_float4(C.hi, C.lo, S.hi, S.lo);
+}
+
+// part[r][chunk][nz - 1]: each thread takes one charge of the chunk, steps through the harmonics by a double-float
+// recurrence, and the block sums its threads in a fixed order.
+constexpr int C0_THREADS = 128;
+
+// grid (charge chunks, m).  The replica's last block (ticket) then adds the chunks (lanes over the
+// chunks, a fixed tree), weights them and leaves b0[r][u] = sum_nz Re[conj(e0[u][nz]) w_nz rho_nz] for every
+// distinct site height: one launch where input, sum, reduction and evaluation were four dependent ones
+// (26 us of a 512-site step's side stream, most of it the gaps between them).
+__global__ void __launch_bounds__(C0_THREADS) k_col0(const double* __restrict__ xyz, const double* __restrict__ Q,
+                                                     int64_t ne, double invLz, int nz0, const double* __restrict__ w,
+                                                     int NZ, const double2* __restrict__ e0, int nzu,
+                                                     const float4* __restrict__ tab, double2* __restrict__ part,
+                                                     int* __restrict__ tickets, double* __restrict__ b0) {
+    __shared__ double2 red[C0_THREADS / 32][COL0_NZ];
+    __shared__ double2 sw[COL0_NZ];
+    const int chunk = blockIdx.x, r = blockIdx.y;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    dcx acc[C0_NB];
-#pragma unroll
-    for (int k = 0; k < C0_NB; ++k) acc[k] = {{0.f, 0.f}, {0.f, 0.f}};
-    // the thread's two charges (a zero charge, also past the end, contributes exact zeros)
-    dfl q[C0_PER_THREAD];
-    dcx e1[C0_PER_THREAD], e[C0_PER_THREAD];
-#pragma unroll
-    for (int t = 0; t < C0_PER_THREAD; ++t) {
-        const int64_t j = (int64_t)chunk * C0_THREADS * C0_PER_THREAD + (int64_t)t * C0_THREADS + threadIdx.x;
-        float2 qf = make_float2(0.f, 0.f);
-        float4 f = make_float4(1.f, 0.f, 0.f, 0.f);
-        if (j < ne) {
-            const int64_t p = (int64_t)r * ne + j;
-            qf = Qd[p];
-            f = e1s[p];
-        }
-        q[t] = {qf.x, qf.y};
-        e1[t] = {{f.x, f.y}, {f.z, f.w}};
-        e[t] = dcx_pow(e1[t], nzs);
-    }
-#pragma unroll
-    for (int k = 0; k < C0_NB; ++k) {
-#pragma unroll
-        for (int t = 0; t < C0_PER_THREAD; ++t) {
-            acc[k].re = df_add(acc[k].re, df_mul(q[t], e[t].re));
-            acc[k].im = df_add(acc[k].im, df_mul(q[t], e[t].im));
-            e[t] = dcx_mul(e[t], e1[t]);
+    // a zero charge, also past the end, contributes exact zeros
+    dfl q = {0.f, 0.f};
+    dcx e1 = {{1.f, 0.f}, {0.f, 0.f}};
+    const int64_t j = (int64_t)chunk * C0_THREADS + threadIdx.x;
+    if (j < ne) {
+        const int64_t p = (int64_t)r * ne + j;
+        const double qd = Q[p];
+        if (qd != 0.0) {
+            q = df_of(qd);
+            e1 = c0_phase(z_fraction(xyz[3 * p + 2], invLz), tab);
         }
     }
+    dcx e = {df_mul(q, e1.re), df_mul(q, e1.im)};
+    for (int k = 0; k < nz0; ++k) {   // warp sums in double-float, one FP64 value per warp
+        dfl re = e.re, im = e.im;
 #pragma unroll
-    for (int k = 0; k < C0_NB; ++k) {   // warp sums in double-float, one FP64 value per warp
-        dfl re = acc[k].re, im = acc[k].im;
         for (int o = 16; o > 0; o >>= 1) {
-            const dfl ore = {__shfl_down_sync(0xffffffffu, re.hi, o), __shfl_down_sync(0xffffffffu, re.lo, o)};
-            const dfl oim = {__shfl_down_sync(0xffffffffu, im.hi, o), __shfl_down_sync(0xffffffffu, im.lo, o)};
+            const dfl ore = {__shfl_xor_sync(0xffffffffu, re.hi, o), __shfl_xor_sync(0xffffffffu, re.lo, o)};
+            const dfl oim = {__shfl_xor_sync(0xffffffffu, im.hi, o), __shfl_xor_sync(0xffffffffu, im.lo, o)};
             re = df_add(re, ore);
             im = df_add(im, oim);
         }
-        if (lane == 0) red[warp][k] = make_double2((double)re.hi + (double)re.lo, (double)im.hi + (double)im.lo);
+        if (lane == k) red[warp][k] = make_double2((double)re.hi + (double)re.lo, (double)im.hi + (double)im.lo);
+        e = dcx_mul(e, e1);
     }
     __syncthreads();
-    if (threadIdx.x < C0_NB) {
-        const int k = threadIdx.x, nz = nzs + k;
-        if (nz <= nz0) {
-            double2 tt = red[0][k];
-            for (int w = 1; w < C0_THREADS / 32; ++w) { tt.x += red[w][k].x; tt.y += red[w][k].y; }
-            part[((int64_t)r * gridDim.x + chunk) * nz0 + nz - 1] = tt;
+    if ((int)threadIdx.x < nz0) {
+        const int k = threadIdx.x;
+        double2 tt = red[0][k];
+        for (int v = 1; v < C0_THREADS / 32; ++v) { tt.x += red[v][k].x; tt.y += red[v][k].y; }
+        part[((int64_t)r * gridDim.x + chunk) * nz0 + k] = tt;
+    }
+    if (!last_block_of(&tickets[r], gridDim.x)) return;
+    // ten groups of threads over the chunks, one thread per harmonic, the group sums added in group order
+    constexpr int G = C0_THREADS / COL0_NZ;
+    __shared__ double2 sp[G][COL0_NZ];
+    const int gk = threadIdx.x % COL0_NZ, gg = threadIdx.x / COL0_NZ;
+    if (gg < G && gk < nz0) {
+        double2 a = make_double2(0.0, 0.0);
+#pragma unroll 4
+        for (int ch = gg; ch < (int)gridDim.x; ch += G) {
+            const double2 v = __ldcg(&part[((int64_t)r * gridDim.x + ch) * nz0 + gk]);
+            a.x += v.x;
+            a.y += v.y;
         }
+        sp[gg][gk] = a;
     }
-}
-
-// wrho0[r][nz - 1] = w(0, 0, nz) * sum over chunks of part: one warp per (r, nz), lanes over the
-// chunks, combined in a fixed order
-__global__ void k_col0_reduce(const double2* __restrict__ part, int nchunks, int nz0, const double* __restrict__ w,
-                              int NZ, int m, double2* __restrict__ wrho0) {
-    const int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (t >= m * nz0) return;
-    const int r = t / nz0, k = t % nz0;
-    double2 a = make_double2(0.0, 0.0);
-    for (int ch = lane; ch < nchunks; ch += 32) {
-        const double2 v = part[((int64_t)r * nchunks + ch) * nz0 + k];
-        a.x += v.x;
-        a.y += v.y;
+    __syncthreads();
+    if ((int)threadIdx.x < nz0) {
+        double2 a = sp[0][threadIdx.x];
+        for (int g = 1; g < G; ++g) { a.x += sp[g][threadIdx.x].x; a.y += sp[g][threadIdx.x].y; }
+        const double wt = w[NZ + threadIdx.x + 1];   // column 0 occupies the first row of the dense grid
+        sw[threadIdx.x] = make_double2(wt * a.x, wt * a.y);
     }
-    for (int o = 16; o > 0; o >>= 1) {
-        a.x += __shfl_down_sync(0xffffffffu, a.x, o);
-        a.y += __shfl_down_sync(0xffffffffu, a.y, o);
-    }
-    if (lane == 0) {
-        const double wt = w[NZ + k + 1];   // column 0 occupies the first row of the dense grid
-        wrho0[t] = make_double2(wt * a.x, wt * a.y);
+    __syncthreads();
+    for (int u = threadIdx.x; u < nzu; u += C0_THREADS) {
+        double s = 0.0;
+#pragma unroll
+        for (int k = 0; k < COL0_NZ; ++k) {
+            if (k < nz0) {
+                const double2 e = e0[(int64_t)u * nz0 + k];
+                s += e.x * sw[k].x + e.y * sw[k].y;
+            }
+        }
+        b0[(int64_t)r * nzu + u] = s;
     }
 }
 
@@ -1059,21 +901,6 @@ __global__ void k_col0_e0(const double* __restrict__ zu, int nzu, double invLz, 
     if (t >= nzu * nz0) return;
     const int iu = t / nz0, nz = t % nz0 + 1;
     e0[t] = z_phase_n(zu[iu], invLz, nz);
-}
-
-// b0[r][u] = sum_nz Re[conj(e0[u][nz]) wrho0[r][nz]]: one warp per (r, u), lanes over nz
-__global__ void k_col0_site(const double2* __restrict__ e0, int nzu, int m, int nz0, const double2* __restrict__ wrho0,
-                            double* __restrict__ b0) {
-    const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (w >= m * nzu) return;
-    const int r = w / nzu, iu = w % nzu;
-    double acc = 0.0;
-    for (int k = lane; k < nz0; k += 32) {
-        const double2 e = e0[(int64_t)iu * nz0 + k], v = wrho0[(int64_t)r * nz0 + k];
-        acc += e.x * v.x + e.y * v.y;
-    }
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-    if (lane == 0) b0[w] = acc;
 }
 
 // Single-precision site potential with a 64-column x 128-site tile per block (4 columns x 8 sites
@@ -1209,58 +1036,58 @@ static size_t al(size_t b) { return (b + 255) & ~(size_t)255; }
 template <typename T>
 struct BvecPlan {
     CellGrid cg;
-    int splits, nctiles, ctiles, ztiles;
-    int64_t chunk;
-    size_t off_EX, off_EY, off_EZ, off_Q, off_rp, off_wr, off_part, off_real, off_stats, off_key, off_cnt, off_cur,
-        off_nzc, off_start, off_wpos, off_sorted, off_order, off_c0part, off_c0w, off_b0, off_u, off_c0e1, off_ew,
+    int nctiles, ctiles;
+    int cw, splits;                     // stored functions per row and charge ranges of the structure factor
+    bool rows;                          // reciprocal sums in the product basis: on the CUDA cores (rd, recip_rows.cu)
+    RowDims rd;                         // or the tensor cores (tc, td, tc_recip.cu)
+    TcRecipDims td;
+    size_t off_EX, off_EY, off_EZ, off_rp, off_wr, off_part, off_real, off_stats, off_key, off_cnt, off_cur,
+        off_nzc, off_start, off_wpos, off_sorted, off_order, off_c0part, off_b0, off_T, off_w16, off_ew,
         off_ewT, off_pm, off_p3m, total;
     int c0chunks;
     bool p3m;                           // reciprocal part of b by P3M (p3m.cu)
-    bool tc;                            // reciprocal sums on the tensor cores (tc_recip.cu)
-    size_t off_qabs, off_tcpart, off_w16, off_spart, off_qpart, off_c0q;
+    bool tc;
+    size_t off_qmax, off_spart;
 };
 
 template <typename T>
 static BvecPlan<T> plan_bvec(const cpm_ctx* c, int m, int64_t ne) {
-    BvecPlan<T> p;
+    BvecPlan<T> p{};
     const KTable& k = c->kt;
     p.cg = make_grid(c->g);
     p.ctiles = (k.ncols + SF_BM - 1) / SF_BM;
-    // odd number 2h + 1 of BN-wide z tiles centred on nz = 0, covering -NZ..NZ
-    const int zh = k.NZ + 1 - SF_BN / 2 > 0 ? (k.NZ + 1 - SF_BN / 2 + SF_BN - 1) / SF_BN : 0;
-    p.ztiles = 2 * zh + 1;
     p.p3m = c->p.kspace == CPM_KSPACE_P3M;
     p.nctiles = p.p3m ? 0 : p.ctiles;
-    p.tc = !p.p3m && std::is_same<T, float>::value && c->p.k_prec == CPM_PREC_F16X2 && tc_recip_supported(k);
-    TcRecipDims td{};
+    p.tc = !p.p3m && std::is_same<T, float>::value && c->p.k_prec == CPM_PREC_F16X2 && c->rows.tcitems > 0;
+    p.rows = !p.p3m && k.nk > 0;
     if (p.tc) {
-        td = tc_recip_dims(c, m, ne);
-        p.nctiles = td.ncb;
+        p.td = tc_recip_dims(c, m, ne);
+        p.cw = p.td.cw;
+        p.splits = p.td.splits;
+        p.nctiles = p.td.ncb;
+    } else if (p.rows) {
+        p.rd = row_dims<T>(c, m, ne);
+        p.cw = p.rd.cw;
+        p.splits = p.rd.splits;
     }
-    // the single-precision structure factor uses 128-harmonic super-tiles (k_sf32)
-    const int zh2 = k.NZ + 1 - S2_BZ / 2 > 0 ? (k.NZ + 1 - S2_BZ / 2 + S2_BZ - 1) / S2_BZ : 0;
-    const int yt = std::is_same<T, float>::value ? 2 * zh2 + 1 : p.ztiles;
-    const int64_t base = (int64_t)p.ctiles * yt * m;
-    int64_t want = (4 * 152 + base - 1) / std::max<int64_t>(base, 1);
-    int64_t maxs = std::max<int64_t>(1, (ne + 127) / 128);
-    p.splits = (int)std::max<int64_t>(1, std::min<int64_t>(want, std::min<int64_t>(maxs, 64)));
-    p.chunk = (ne + p.splits - 1) / p.splits;
-    p.chunk = ((p.chunk + SF_BK - 1) / SF_BK) * SF_BK;
+    if (p.rows && c->rows.layered) p.nctiles = c->rows.nchunk;
     const int64_t ptot = (int64_t)m * ne;
     const int64_t pph = p.p3m ? 0 : ptot;   // points with electrolyte phase tables (none with P3M)
-    const size_t pe = phase_elems(k, pph);
     const size_t grid = (size_t)k.ncols * k.nzw;
     size_t o = 0;
-    const int64_t tabX = (int64_t)(k.NX + 1) * pph, tabY = (int64_t)(2 * k.NY + 1) * pph;
-    p.off_EX = o; o += al(sizeof(c2<T>) * tabX);
-    p.off_EY = o; o += al(sizeof(c2<T>) * tabY);
-    p.off_EZ = o; o += al(sizeof(c2<T>) * (pe - tabX - tabY));
-    p.off_Q = o; o += al(sizeof(T) * ptot);
-    if (p.tc || p.p3m) {   // the CUDA-core structure-factor buffers are not used
-        p.off_rp = p.off_wr = o;
+    if (p.tc) {
+        p.off_EX = p.off_EY = p.off_EZ = o; o += al(sizeof(float2) * charge_slots(k) * m * p.td.nep);
     } else {
-        p.off_rp = o; o += al(sizeof(c2<T>) * grid * m * p.splits);
-        p.off_wr = o; o += al(sizeof(c2<T>) * grid * m);
+        p.off_EX = o; o += al(sizeof(c2<T>) * (k.NX + 1) * pph);
+        p.off_EY = o; o += al(sizeof(c2<T>) * (k.NY + 1) * pph);
+        p.off_EZ = o; o += al(sizeof(c2<T>) * (k.NZ + 1) * pph);
+    }
+    p.off_rp = p.off_wr = p.off_T = p.off_w16 = o;
+    if (p.rows) {
+        p.off_rp = o; o += al(sizeof(T) * (size_t)p.splits * m * 4 * c->rows.np * p.cw);
+        p.off_wr = o; o += c->rows.layered ? 0 : al(sizeof(c2<T>) * grid * m);
+        p.off_T = o; o += c->rows.layered ? al(sizeof(T) * rows_T_elems<T>(c, m)) : 0;
+        p.off_w16 = o; o += p.tc && !c->rows.layered ? al(tc_recip_w16_bytes(p.td)) : 0;
     }
     p.off_part = o; o += al(sizeof(T) * (size_t)m * p.nctiles * c->n);
     p.off_real = o; o += al(sizeof(double) * (size_t)m * c->n);
@@ -1269,21 +1096,16 @@ static BvecPlan<T> plan_bvec(const cpm_ctx* c, int m, int64_t ne) {
     p.off_cnt = o; o += al(sizeof(int) * ((size_t)m * p.cg.ncells + 1));
     p.off_cur = o; o += al(sizeof(int) * ((size_t)m * p.cg.ncells + 1));
     p.off_nzc = o; o += al(sizeof(int) * (size_t)m);
+    p.off_qmax = o; o += al(3 * sizeof(float) * (size_t)m);
     p.off_start = o; o += al(sizeof(int) * ((size_t)m * p.cg.ncells + 1));
     p.off_wpos = o; o += al(sizeof(typename V4<T>::t) * ptot);
     p.off_sorted = o; o += al(sizeof(typename V4<T>::t) * ptot);
     p.off_order = o; o += al(sizeof(int) * ptot);
-    p.c0chunks = (int)std::max<int64_t>(1, (ne + C0_THREADS * C0_PER_THREAD - 1) / (C0_THREADS * C0_PER_THREAD));
+    p.c0chunks = (int)std::max<int64_t>(1, (ne + C0_THREADS - 1) / C0_THREADS);
     const int nz0 = std::max(std::min(k.ext0, COL0_NZ), 1);
     p.off_c0part = o; o += al(sizeof(double2) * (size_t)m * p.c0chunks * nz0);
-    p.off_c0w = o; o += al(sizeof(double2) * (size_t)m * nz0);
     p.off_b0 = o; o += al(sizeof(double) * (size_t)m * std::max(c->nzu, 1));
-    p.off_u = o; o += al(sizeof(uint64_t) * 3 * pph);
-    p.off_c0e1 = o; o += al(sizeof(float4) * pph);
-    p.off_c0q = o; o += al(sizeof(float2) * pph);
-    p.off_qabs = o; o += al(sizeof(float2) * m);
     p.off_spart = o; o += al(sizeof(double) * ST_Q * (size_t)std::max<int64_t>(1, (ne + ST_THREADS - 1) / ST_THREADS) * m);
-    p.off_qpart = o; o += al(sizeof(double) * 2 * (size_t)std::max<int64_t>(1, (ne + FR_THREADS - 1) / FR_THREADS) * m);
     p.off_ew = p.off_ewT = o;
     if (c->g.bc == CPM_BC_EW2D) {
         p.off_ew = o; o += al(sizeof(double) * (size_t)m * c->n);
@@ -1293,11 +1115,6 @@ static BvecPlan<T> plan_bvec(const cpm_ctx* c, int m, int64_t ne) {
     if (p.p3m) {
         p.off_pm = o; o += al(sizeof(double) * (size_t)m * c->n);
         p.off_p3m = o; o += al(p3m_scratch_bytes<T>(c, m, ne));
-    }
-    p.off_tcpart = p.off_w16 = o;
-    if (p.tc) {
-        p.off_tcpart = o; o += al(tc_recip_part_bytes(td, m, k.nzw));
-        p.off_w16 = o; o += al(tc_recip_w16_bytes(td));
     }
     p.total = o;
     return p;
@@ -1320,8 +1137,7 @@ cpm_status bvec_run(cpm_ctx* c, int m, int64_t ne, const double* xyz, const doub
     c2<T>* EX = (c2<T>*)(scr + p.off_EX);
     c2<T>* EY = (c2<T>*)(scr + p.off_EY);
     c2<T>* EZ = (c2<T>*)(scr + p.off_EZ);
-    T* Qv = (T*)(scr + p.off_Q);
-    c2<T>* rp = (c2<T>*)(scr + p.off_rp);
+    T* rp = (T*)(scr + p.off_rp);
     c2<T>* wr = (c2<T>*)(scr + p.off_wr);
     T* part = (T*)(scr + p.off_part);
     double* real = (double*)(scr + p.off_real);
@@ -1334,17 +1150,20 @@ cpm_status bvec_run(cpm_ctx* c, int m, int64_t ne, const double* xyz, const doub
     V4T* wpos = (V4T*)(scr + p.off_wpos);
     V4T* sorted = (V4T*)(scr + p.off_sorted);
     int* order = (int*)(scr + p.off_order);
+    float* qmax = (float*)(scr + p.off_qmax);     // per replica: max |Q|, index past the last nonzero charge, sum |Q|
+    int* qlast = (int*)(qmax + m);
+    float* qsum = (float*)(qlast + m);
     const int nc = m * p.cg.ncells;
-    c->launches += 4 + (ptot > 0 ? 2 : 0) + ((k.nk > 0 && ptot > 0 && !p.p3m) ? 5 : 0);
+    c->launches += 4 + (ptot > 0 ? 2 : 0) + ((k.nk > 0 && ptot > 0 && !p.p3m) ? 4 + (c->rows.layered || !p.tc ? 0 : 2) : 0);
 
     // Three chains: the origin stream bins the charges (per-replica totals) and runs the cell list and
-    // the real-space sum; side stream 1 takes the fractions, the charges in the working precision and
-    // their scales in one pass, then the phase tables and the reciprocal sums; side stream 2 sums the
-    // k_perp = 0 column once the fractions are written.  k_combine joins them.  With per-kernel
-    // profiling on, everything runs on the origin stream in the same order.
+    // the real-space sum; side stream 1 takes the phase tables and the reciprocal sums; side stream 2 sums the
+    // k_perp = 0 column.  k_combine joins them.  With per-kernel profiling on, everything runs on the
+    // origin stream in the same order.
     const bool recip = k.nk > 0 && ptot > 0 && !p.p3m;
     const bool fork = !c->prof_on;
     cudaStream_t s0 = st, s1 = st, s2 = st;
+    CPM_CUDA(c, cudaMemsetAsync(cnt, 0, p.off_start - p.off_cnt, st));   // counts, cursors, nonzero counts, charge scales
     if (fork) {
         CPM_TRY(ensure_aux(c));
         s1 = c->aux[0];
@@ -1354,41 +1173,32 @@ cpm_status bvec_run(cpm_ctx* c, int m, int64_t ne, const double* xyz, const doub
     }
     if (recip) {
         prof_begin(c, CPM_K_PHASES);
-        // the k_perp = 0 chain needs only the fractions: it starts after k_fracs
-        CPM_TRY(launch_phases_u<T>(s1, c->g, k, xyz, Q, ne, m, (uint64_t*)(scr + p.off_u), Qv,
-                                   (double*)(scr + p.off_qpart), c->tickets + m,
-                                   p.tc ? (float2*)(scr + p.off_qabs) : nullptr, EX, EY, EZ,
-                                   fork ? c->fev[1] : nullptr, p.tc ? TC_ZSCALE : 1.f));
+        if (p.tc) {
+            CPM_TRY(launch_charge_slots(c, s1, m, ne, p.td.nep, xyz, Q, (float2*)EX, qmax, qlast));
+            if (!c->rows.layered) CPM_TRY(tc_recip_scales(c, s1, m, ne, Q, qsum));
+        } else {
+            CPM_TRY(launch_charge_phases<T>(c, s1, ptot, xyz, Q, EX, EY, EZ));
+        }
         prof_end(c, CPM_K_PHASES);
-    } else if (fork) {
-        CPM_CUDA(c, cudaEventRecord(c->fev[1], s1));
     }
-    if (fork) CPM_CUDA(c, cudaStreamWaitEvent(s2, c->fev[1], 0));
+    if (fork) {   // the short k_perp = 0 chain starts behind the phases: beside them it delays the long one
+        CPM_CUDA(c, cudaEventRecord(c->fev[1], s1));
+        CPM_CUDA(c, cudaStreamWaitEvent(s2, c->fev[1], 0));
+    }
     double* b0 = nullptr;
     if (std::is_same<T, float>::value && k.ext0 > 0 && ptot > 0 && !p.p3m) {
-        // the k_perp = 0 column in FP64 (its single-precision weights are zero)
-        double2* c0part = (double2*)(scr + p.off_c0part);
-        double2* c0w = (double2*)(scr + p.off_c0w);
+        // the k_perp = 0 column in double-float (its single-precision weights are zero)
         b0 = (double*)(scr + p.off_b0);
         prof_begin(c, CPM_K_COL0);
         const int nz0 = std::min(k.ext0, COL0_NZ);
-        const int nblk = (nz0 + C0_NB - 1) / C0_NB;
-        float4* e1s = (float4*)(scr + p.off_c0e1);
-        float2* q0 = (float2*)(scr + p.off_c0q);
-        CPM_TRY(launch_col0_inputs(s2, (const uint64_t*)(scr + p.off_u), Q, ptot, e1s, q0));
-        k_col0_rho<<<dim3(p.c0chunks, nblk, m), C0_THREADS, 0, s2>>>(e1s, q0, ne, nz0, c0part);
-        CPM_LAUNCH(c, "k_col0_rho");
-        k_col0_reduce<<<(m * nz0 * 32 + 255) / 256, 256, 0, s2>>>(c0part, p.c0chunks, nz0, k.w, k.NZ, m, c0w);
-        CPM_LAUNCH(c, "k_col0_reduce");
-        k_col0_site<<<(m * c->nzu * 32 + 255) / 256, 256, 0, s2>>>(c->c0e, c->nzu, m, nz0, c0w, b0);
-        CPM_LAUNCH(c, "k_col0_site");
+        k_col0<<<dim3(p.c0chunks, m), C0_THREADS, 0, s2>>>(xyz, Q, ne, c->g.inv[2], nz0, k.w, k.NZ, c->c0e, c->nzu, c->c0tab,
+                                                           (double2*)(scr + p.off_c0part), c->tickets + m, b0);
+        CPM_LAUNCH(c, "k_col0");
         prof_end(c, CPM_K_COL0);
-        c->launches += 4;
+        c->launches += 1;
     }
     // binning and the per-replica totals (one pass over the charges)
     prof_begin(c, CPM_K_CELLS);
-    float2* qabs = (float2*)(scr + p.off_qabs);
-    CPM_CUDA(c, cudaMemsetAsync(cnt, 0, p.off_start - p.off_cnt, st));   // counts, cursors, nonzero counts
     int* nzc = (int*)(scr + p.off_nzc);
     {
         const float3 inv_h = make_float3((float)(1.0 / p.cg.h[0]), (float)(1.0 / p.cg.h[1]), (float)(1.0 / p.cg.h[2]));
@@ -1399,38 +1209,22 @@ cpm_status bvec_run(cpm_ctx* c, int m, int64_t ne, const double* xyz, const doub
     }
     prof_end(c, CPM_K_CELLS);
     if (recip) {
-        if (p.tc) {
-            c->stream = s1;   // tc_recip_run launches on the context stream
-            const cpm_status rs = tc_recip_run(c, m, ne, (const float2*)EX, (const float2*)EY, (const float2*)EZ,
-                                               (const float*)Qv, qabs, scr + p.off_tcpart, scr + p.off_w16,
-                                               (float*)part);
-            c->stream = s0;
-            CPM_TRY(rs);
-        } else {
+        const float* qs = p.tc ? qmax : nullptr;
         prof_begin(c, CPM_K_SF);
-        if (std::is_same<T, float>::value) {
-            const int zh2 = k.NZ + 1 - S2_BZ / 2 > 0 ? (k.NZ + 1 - S2_BZ / 2 + S2_BZ - 1) / S2_BZ : 0;
-            const int nsup = 2 * zh2 + 1;
-            dim3 gsf(p.ctiles, nsup, m * p.splits);
-            k_sf32<<<gsf, 256, 0, s1>>>(k.cols, k.colext, k.ncols, k.NY, k.NZ, k.nzw, (const float2*)EX,
-                                        (const float2*)EY, (const float2*)EZ, (const float*)Qv, ptot, ne, p.splits,
-                                        p.chunk, m, nsup, (float2*)rp);
-        } else {
-            dim3 gsf(p.ctiles, p.ztiles, m * p.splits);
-            k_sf<T><<<gsf, 256, 0, s1>>>(k.cols, k.colext, k.ncols, k.NY, k.NZ, k.nzw, EX, EY, EZ, Qv, ptot, ne,
-                                         p.splits, p.chunk, m, rp);
-        }
+        if (p.tc) CPM_TRY(tc_recip_sf(c, s1, p.td, m, (const float2*)EX, qmax, qlast, (float*)rp));
+        else CPM_TRY(rows_sf<T>(c, s1, p.rd, m, ne, EX, EY, EZ, rp));
         prof_end(c, CPM_K_SF);
-        CPM_LAUNCH(c, "k_sf");
-        prof_begin(c, CPM_K_SFRED);
-        const int64_t per_rep = (int64_t)k.ncols * k.nzw;
-        const T* w = std::is_same<T, float>::value ? (const T*)k.w32 : (const T*)k.w;
-        k_sf_reduce<T><<<(unsigned)((per_rep * m + 255) / 256), 256, 0, s1>>>(rp, w, per_rep, m, p.splits, wr);
-        prof_end(c, CPM_K_SFRED);
-        CPM_LAUNCH(c, "k_sf_reduce");
-        prof_begin(c, CPM_K_SITE);
         const Phases<T>& sp = site_tables<T>(c);
-        if (std::is_same<T, float>::value) {
+        prof_begin(c, CPM_K_SFRED);
+        if (c->rows.layered) CPM_TRY(rows_layers<T>(c, s1, p.cw, p.splits, m, rp, qs, (T*)(scr + p.off_T)));
+        else CPM_TRY(rows_to_cols<T>(c, s1, p.cw, p.splits, m, rp, qs, wr));
+        prof_end(c, CPM_K_SFRED);
+        prof_begin(c, CPM_K_SITE);
+        if (c->rows.layered) {
+            CPM_TRY(rows_sites<T>(c, s1, m, (const T*)(scr + p.off_T), part));
+        } else if (p.tc) {
+            CPM_TRY(tc_recip_sites(c, s1, p.td, m, (const float2*)wr, qsum, scr + p.off_w16, (float*)part));
+        } else if (std::is_same<T, float>::value) {
             dim3 gs((unsigned)((n + T2_BS - 1) / T2_BS), p.ctiles, m);
             k_site32<<<gs, 256, 0, s1>>>(k.cols, k.colext, k.ncols, k.NY, k.NZ, k.nzw, (const float2*)wr,
                                          (const float2*)sp.X, (const float2*)sp.Y, (const float2*)sp.Z, n, p.nctiles,
@@ -1442,7 +1236,6 @@ cpm_status bvec_run(cpm_ctx* c, int m, int64_t ne, const double* xyz, const doub
         }
         prof_end(c, CPM_K_SITE);
         CPM_LAUNCH(c, "k_site");
-        }
     } else if (p.nctiles > 0) {
         CPM_CUDA(c, cudaMemsetAsync(part, 0, sizeof(T) * (size_t)m * p.nctiles * n, s1));
     }
@@ -1520,6 +1313,11 @@ cpm_status build_col0_sites(cpm_ctx* c) {
     CPM_TRY(dev_alloc(c, (void**)&c->c0e, sizeof(double2) * (size_t)c->nzu * nz0));
     k_col0_e0<<<(c->nzu * nz0 + 255) / 256, 256, 0, c->stream>>>(c->zuniq, c->nzu, c->g.inv[2], nz0, c->c0e);
     CPM_LAUNCH(c, "k_col0_e0");
+    dev_free(c, c->c0tab);
+    c->c0tab = nullptr;
+    CPM_TRY(dev_alloc(c, (void**)&c->c0tab, sizeof(float4) * C0_TAB));
+    k_col0_tab<<<1, C0_TAB, 0, c->stream>>>(c->c0tab);
+    CPM_LAUNCH(c, "k_col0_tab");
     return CPM_OK;
 }
 
@@ -1534,7 +1332,7 @@ cpm_status ensure_aux(cpm_ctx* c) {
 cpm_status reserve_bvec(cpm_ctx* c, int m, int64_t ne) {
     const bool f32 = c->p.k_prec != CPM_PREC_FP64;
     CPM_TRY(ensure_aux(c));
-    CPM_TRY(ensure_tickets(c, 2 * m));   // k_bin takes [0, m), k_fracs [m, 2m)
+    CPM_TRY(ensure_tickets(c, 2 * m));   // k_bin takes [0, m), k_col0 [m, 2m)
     return ensure_scratch(c, f32 ? bvec_scratch_bytes<float>(c, m, ne) : bvec_scratch_bytes<double>(c, m, ne));
 }
 
@@ -1542,7 +1340,7 @@ cpm_status bvec(cpm_ctx* c, int m, int64_t ne, const double* xyz, const double* 
     const bool f32 = c->p.k_prec != CPM_PREC_FP64;
     const size_t need = f32 ? bvec_scratch_bytes<float>(c, m, ne) : bvec_scratch_bytes<double>(c, m, ne);
     CPM_TRY(ensure_scratch(c, need));
-    CPM_TRY(ensure_tickets(c, 2 * m));   // k_bin takes [0, m), k_fracs [m, 2m)
+    CPM_TRY(ensure_tickets(c, 2 * m));   // k_bin takes [0, m), k_col0 [m, 2m)
     char* scr = (char*)c->scratch;
     return f32 ? bvec_run<float>(c, m, ne, xyz, Q, b_out, bhl, scr) : bvec_run<double>(c, m, ne, xyz, Q, b_out, bhl, scr);
 }

@@ -104,6 +104,14 @@ enum : unsigned { ST_NOT_SPD = 1u, ST_NONFINITE = 2u, ST_TIMEOUT = 4u };
 constexpr float TC_ZSCALE = 16384.f;
 constexpr int COL0_NZ = 12;
 
+// 2^e with bound * 2^e < 2^top; 1 for a zero or non-finite bound
+__device__ __forceinline__ float pow2_below(float bound, int top) {
+    if (!(bound > 0.f) || !isfinite(bound)) return 1.f;
+    int e;
+    frexpf(bound, &e);   // bound = f 2^e, f in [0.5, 1)
+    return ldexpf(1.f, top - e);
+}
+
 struct KTable {
     int NX = 0, NY = 0, NZ = 0;
     int ncols = 0, nzw = 0;
@@ -116,6 +124,39 @@ struct KTable {
     float* w32 = nullptr;
     int4* klist = nullptr;          // [nk] compact list: (column, nz, nx, ny)
     double* kw = nullptr;           // [nk] weight of each compact entry
+};
+
+// The k set in the real product basis (recip_rows.cu): pairs (nx, ny) with nx, ny >= 0 in the order of
+// |k_perp|, four rows (cos / sin of x times cos / sin of y) each.
+constexpr int ROW_TILE = 128;          // sites per block of the height-wise site stage
+constexpr int LAYER_MIN_SITES = 8;     // sites per distinct height from which that stage is taken
+constexpr int ROW_TC_PAIRS = 64;       // pairs, charges per step and staged x and y harmonics of a CTA of the
+constexpr int ROW_TC_STEP = 64;        // tensor-core structure factor (tc_recip.cu)
+constexpr int ROW_TC_SLOTS = 50;
+struct RowTable {
+    int np = 0, nrows = 0, nslots = 0;   // pairs, rows that are not identically zero, (nx, ny) slots
+    int nchunk = 0, ntiles = 0;          // nx ranges and site tiles of the site stage
+    int chunkmax = 0;                    // most slots of one range
+    bool layered = false;                // the sites share few heights
+    int4* pairs = nullptr;               // [np] (nx, ny, largest nz, slot)
+    int* list = nullptr;                 // [nrows] 4 pair + part
+    int* colpair = nullptr;              // [ncols] pair of each signed column
+    int* nxoff = nullptr;                // [NX + 2] first slot of each nx (slot = nxoff[nx] + ny)
+    int* chunkb = nullptr;               // [nchunk + 1] first nx of each range
+    double* W = nullptr;                 // [np][NZ + 1] weights of the octant vectors
+    float* W32 = nullptr;
+    double2* zu64 = nullptr;             // [NZ + 1][nzu] (cos, sin) of the harmonics at the site heights
+    float2* zu32 = nullptr;
+    int* lperm = nullptr;                // [n] sites by height
+    int4* ltiles = nullptr;              // [ntiles] (height, first, count, 0)
+    int tcitems = 0;                     // work items of the tensor-core structure factor, 0: it does not fit
+    int4* tcitem = nullptr;              // (first pair, pairs, harmonic tile, harmonics of the tile)
+    int4* tcrange = nullptr;             // (first nx, count, first ny, count) of the item's pairs
+    std::vector<int> hext, hlist;        // host copies: extents of the pairs, the row list
+};
+struct RowDims {
+    int cw, xt, yt, splits;              // stored harmonic functions per row, tiles, charge ranges
+    int64_t chunk;                       // charges per range
 };
 
 // Phase tables of a point set: X[h][p] = exp(2 pi i h x_p / Lx) for h = 0..NX,
@@ -208,6 +249,7 @@ struct cpm_ctx {
     cpm::RealPoly rpoly{};       // fitted pair function of the gathered real-space kernel
     int rpoly_blocks = 0;        // its persistent grid (resident blocks per SM x SMs)
     cpm::KTable kt;
+    cpm::RowTable rows;
     int2* h2d_idx = nullptr;     // EW2D: half-plane 2D vectors (nx, ny), 0 < |h| <= kcut
     double* h2d_norm = nullptr;  // their |h|
     int nh2d = 0;
@@ -227,6 +269,7 @@ struct cpm_ctx {
     unsigned* status = nullptr;  // device status word
     int* tickets = nullptr;      // [tickets_n] per-replica arrival counters, zero between launches
     int tickets_n = 0;
+    float4* c0tab = nullptr;     // double-float cos and sin of 256 angles (k_perp = 0 column)
     double2* c0e = nullptr;      // [nzu][min(ext0, COL0_NZ)] exp(i kz z_u) of the k_perp = 0 column at the sites
     double* nbuf = nullptr;      // neutrality fix: per-block partial sums of q
     size_t nbuf_bytes = 0;
@@ -282,8 +325,6 @@ struct cpm_ctx {
     void* tcz = nullptr;         // tensor-core reciprocal space: site phase planes [2][npad][KZ] (fp16)
     float2* tcxy = nullptr;      // [ncols][n] column factors X_i Y_i of the sites
     float tc_wmax = 0.f;         // bound on the k-space weights
-    int tc_mx[32] = {};          // largest harmonic extent of each 128-column structure-factor tile
-    int tc_nmx = 0;              // tiles in tc_mx (0: the kernel finds them)
     void* p3m_G = nullptr;       // P3M (kspace = CPM_KSPACE_P3M): influence function / V on the mesh (k_prec's T)
     void* p3m_tw = nullptr;      // its FFT twiddles exp(-2 pi i j / K), j < K / 2, for K = Kx, Ky, Kz
     void* p3m_G64 = nullptr;     // the same in FP64 for the P3M elastance when k_prec is single precision
@@ -337,16 +378,6 @@ template <typename T>
 cpm_status launch_phases(cudaStream_t st, const Geometry& g, const KTable& k, const double* xyz, int64_t P,
                          c2<T>* X, c2<T>* Y, c2<T>* Z);
 size_t phase_elems(const KTable& k, int64_t P);
-constexpr int FR_THREADS = 256;   // threads per block of the fractions kernel (k_fracs)
-// fractions u, charges Qv in T and (qabs non-null) the per-replica max |Q|, sum |Q| (qpart: m x blocks
-// x 2 doubles, tickets: m counters), then the phase tables; after_fracs is recorded after the first kernel
-template <typename T>
-cpm_status launch_phases_u(cudaStream_t st, const Geometry& g, const KTable& k, const double* xyz, const double* Q,
-                           int64_t ne, int m, uint64_t* u, T* Qv, double* qpart, int* tickets, float2* qabs,
-                           c2<T>* X, c2<T>* Y, c2<T>* Z, cudaEvent_t after_fracs = nullptr, float zscale = 1.f);
-// inputs of the double-float k_perp = 0 column from the z fractions (u as written by the phase kernels)
-cpm_status launch_col0_inputs(cudaStream_t st, const uint64_t* u, const double* Q, int64_t P, float4* e1,
-                              float2* q2);
 
 // api.cu
 cpm_status ensure_scratch(cpm_ctx* c, size_t bytes);
@@ -370,6 +401,31 @@ __device__ __forceinline__ bool last_block_of(int* ticket, int nblocks) {
 
 // assemble.cu
 cpm_status assemble_A(cpm_ctx* c);
+
+// recip_rows.cu: the reciprocal sums in the real product basis
+cpm_status build_rows(cpm_ctx* c);
+void free_rows(cpm_ctx* c);
+template <typename T> RowDims row_dims(const cpm_ctx* c, int m, int64_t ne);
+template <typename T>
+cpm_status launch_charge_phases(cpm_ctx* c, cudaStream_t st, int64_t P, const double* xyz, const double* Q, c2<T>* X,
+                                c2<T>* Y, c2<T>* Z);
+template <typename T>
+cpm_status rows_sf(cpm_ctx* c, cudaStream_t st, const RowDims& d, int m, int64_t ne, const c2<T>* X, const c2<T>* Y,
+                   const c2<T>* Z, T* part);
+// the same phases as one table [slot][m nep] for the tensor-core stage: x (times Q), y, then z as 8 + NZ / 8 + 1
+// factors; every replica padded to nep charges; max |Q| and the index past the last nonzero charge of every
+// replica into qmax, qlast (zero before)
+int64_t charge_slots(const KTable& k);
+cpm_status launch_charge_slots(cpm_ctx* c, cudaStream_t st, int m, int64_t ne, int64_t nep, const double* xyz,
+                               const double* Q, float2* tab, float* qmax, int* qlast);
+// qmax (tensor-core stage 1): part is scaled by 2^14 pow2_below(max |Q|, 14)
+template <typename T>
+cpm_status rows_layers(cpm_ctx* c, cudaStream_t st, int cw, int splits, int m, const T* part, const float* qmax, T* Tbuf);
+template <typename T> int64_t rows_T_elems(const cpm_ctx* c, int m);   // room for the height-wise coefficients
+template <typename T>
+cpm_status rows_sites(cpm_ctx* c, cudaStream_t st, int m, const T* Tbuf, T* partial);
+template <typename T>
+cpm_status rows_to_cols(cpm_ctx* c, cudaStream_t st, int cw, int splits, int m, const T* part, const float* qmax, c2<T>* wrho);
 
 // ew2d.cu: the exact 2D-periodic slab sum
 cpm_status build_ew2d(cpm_ctx* c);
@@ -440,19 +496,22 @@ cpm_status gemv_tma(cpm_ctx* c, int m, const float2* bhl, float2* part, int64_t 
 
 // tc_recip.cu: reciprocal-space sums of b on the tensor cores (k_prec = CPM_PREC_F16X2)
 struct TcRecipDims {
-    int mtiles, ntiles, cpad, splits;   // stage 1: column tiles, harmonic tiles, padded columns, charge splits
-    int64_t chunk;                      // charges per split
+    int64_t nep;                        // charges per replica, padded to whole K steps
+    int cw, splits, spc;                // stage 1: stored functions per row, charge ranges, K steps per range
     int mr, nrb, CT, ncb, NB, ngroups;  // stage 2: replicas per block, blocks, columns per group, ...
     int KZ;                             // padded K extent (2 x harmonics)
     int64_t npad;                       // padded site count
 };
-bool tc_recip_supported(const KTable& k);   // phase-table rows fit the staging buffer
 TcRecipDims tc_recip_dims(const cpm_ctx* c, int m, int64_t ne);
-size_t tc_recip_part_bytes(const TcRecipDims& d, int m, int nzw);
 size_t tc_recip_w16_bytes(const TcRecipDims& d);
 cpm_status tc_recip_prepare(cpm_ctx* c);
-cpm_status tc_recip_run(cpm_ctx* c, int m, int64_t ne, const float2* EX, const float2* EY, const float2* EZ,
-                        const float* Qv, const float2* qabs, void* part, void* w16, float* site_partial);
+cpm_status tc_recip_scales(cpm_ctx* c, cudaStream_t st, int m, int64_t ne, const double* Q, float* qsum);
+// tab: the charge phases of launch_charge_slots; part as rows_sf, times 2^14 pow2_below(max |Q|, 14)
+cpm_status tc_recip_sf(cpm_ctx* c, cudaStream_t st, const TcRecipDims& d, int m, const float2* tab, const float* qmax,
+                       const int* qlast, float* part);
+// the site stage of electrodes whose sites hardly share heights, from w rho of the signed columns
+cpm_status tc_recip_sites(cpm_ctx* c, cudaStream_t st, const TcRecipDims& d, int m, const float2* wrho,
+                          const float* qsum, void* w16, float* site_partial);
 
 // p3m.cu: the reciprocal part of b by P3M (cpm_params.kspace = CPM_KSPACE_P3M)
 constexpr int P3M_MAX_MESH = 512;                 // mesh points per axis (powers of two, at least 8)

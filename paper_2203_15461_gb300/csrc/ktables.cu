@@ -236,171 +236,6 @@ __global__ void k_phases(const double* __restrict__ xyz, int64_t P, double ix, d
     }
 }
 
-// The fixed-point fractions of each point once per axis (u[d][p]), then the tables from them:
-// the table kernel then needs no FP64 arithmetic at all.  The same pass writes the charges in the
-// working precision (Qv) and, when qabs is given, max |Q| and sum |Q| of each replica (the scales
-// of the tensor-core reciprocal sums), so that the reciprocal chain needs nothing from the binning
-// of the real-space chain: each block reduces its charges into part[r][b][2] (lane l takes threads
-// l, l + 32, ..., then a shuffle tree) and the replica's last block adds the block values in block
-// order.  grid (charge blocks, m); point p = r ne + j.
-template <typename T>
-__global__ void __launch_bounds__(FR_THREADS) k_fracs(const double* __restrict__ xyz, const double* __restrict__ Q,
-                                                    int64_t ne, double ix, double iy, double iz,
-                                                    uint64_t* __restrict__ u, T* __restrict__ Qv,
-                                                    double* __restrict__ part, int* __restrict__ tickets,
-                                                    float2* __restrict__ qabs) {
-    const int b = blockIdx.x, nb = gridDim.x, r = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t j = (int64_t)b * FR_THREADS + threadIdx.x;
-    const int64_t P = (int64_t)gridDim.y * ne;
-    double aq = 0.0;
-    if (j < ne) {
-        const int64_t p = (int64_t)r * ne + j;
-        u[p] = frac_fixed(xyz[3 * p + 0], ix);
-        u[P + p] = frac_fixed(xyz[3 * p + 1], iy);
-        u[2 * P + p] = frac_fixed(xyz[3 * p + 2], iz);
-        const double q = Q[p];
-        Qv[p] = (T)q;
-        aq = fabs(q);
-    }
-    if (!qabs) return;   // uniform
-    __shared__ double sv[FR_THREADS];
-    sv[threadIdx.x] = aq;
-    __syncthreads();
-    if (warp < 2) {   // warp 0: max |Q|, warp 1: sum |Q|
-        double v = sv[lane];
-        for (int k = 1; k < FR_THREADS / 32; ++k) v = warp == 0 ? fmax(v, sv[lane + 32 * k]) : v + sv[lane + 32 * k];
-        for (int o = 16; o > 0; o >>= 1) {
-            const double w = __shfl_down_sync(0xffffffffu, v, o);
-            v = warp == 0 ? fmax(v, w) : v + w;
-        }
-        if (lane == 0) part[((int64_t)r * nb + b) * 2 + warp] = v;
-    }
-    if (!last_block_of(&tickets[r], nb)) return;
-    __shared__ double buf[2][FR_THREADS];
-    const volatile double* pv = part + (int64_t)r * nb * 2;
-    double v = 0.0;
-    for (int k0 = 0; k0 < nb; k0 += FR_THREADS) {
-        const int k = k0 + threadIdx.x;
-        if (k < nb) {
-            buf[0][threadIdx.x] = pv[2 * k];
-            buf[1][threadIdx.x] = pv[2 * k + 1];
-        }
-        __syncthreads();
-        if (threadIdx.x < 2) {
-            const int t = threadIdx.x, cnt = min(FR_THREADS, nb - k0);
-            for (int kk = 0; kk < cnt; ++kk) {
-                const double x = buf[t][kk];
-                v = (k0 == 0 && kk == 0) ? x : (t == 0 ? fmax(v, x) : v + x);
-            }
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) qabs[r].x = (float)v;
-    if (threadIdx.x == 1) qabs[r].y = (float)v;
-}
-
-// For the double-float k_perp = 0 column of the single-precision paths: the first z harmonic
-// exp(2 pi i z / Lz) as a double-float pair (from the exactly reduced fraction, one FP64 sincospi)
-// and the charge as a double-float pair.
-__global__ void k_col0_inputs(const uint64_t* __restrict__ uz, const double* __restrict__ Q, int64_t P,
-                              float4* __restrict__ e1, float2* __restrict__ q2) {
-    int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= P) return;
-    const double2 e = phase_of<double>(uz[p], 1);
-    const float rh = (float)e.x, ih = (float)e.y;
-    e1[p] = make_float4(rh, (float)(e.x - (double)rh), ih, (float)(e.y - (double)ih));
-    const double qd = Q[p];
-    const float qh = (float)qd;
-    q2[p] = make_float2(qh, (float)(qd - (double)qh));
-}
-
-// grid (points / 256, slots): no index division per entry
-template <typename T>
-__global__ void k_phases_u(const uint64_t* __restrict__ u, int64_t P, int NX, int NY, int NZ, c2<T>* X, c2<T>* Y,
-                           c2<T>* Z) {
-    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= P) return;
-    const int slot = blockIdx.y;
-    if (slot <= NX) {
-        X[(int64_t)slot * P + p] = phase_of<T>(u[p], slot);
-    } else if (slot <= NX + 2 * NY + 1) {
-        int r = slot - (NX + 1);
-        Y[(int64_t)r * P + p] = phase_of<T>(u[P + p], r - NY);
-    } else {
-        int r = slot - (NX + 1) - (2 * NY + 1);
-        Z[(int64_t)r * P + p] = phase_of<T>(u[2 * P + p], r - NZ);
-    }
-}
-
-// Single precision, one thread per (point, axis): the harmonics h = 8a + k >= 0 of the axis are
-// products e^{2 pi i 8a f} e^{2 pi i k f} of sixteen exactly reduced phases at most (k = 0..7 and the
-// multiples of 8, each from the fixed-point fraction f), one rounding more than a direct evaluation
-// (below the precision the single-precision sums keep); h < 0 is the conjugate of -h.  The z table
-// is multiplied by zscale (a power of two: exact).
-// grid (points / 128, 3 axes)
-__global__ void __launch_bounds__(128) k_phases_rows(const uint64_t* __restrict__ u, int64_t P, int NX, int NY,
-                                                     int NZ, float2* __restrict__ X, float2* __restrict__ Y,
-                                                     float2* __restrict__ Z, float zscale) {
-    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= P) return;
-    const int axis = blockIdx.y;
-    const int H = axis == 0 ? NX : axis == 1 ? NY : NZ;   // largest |h|
-    float2* T = axis == 0 ? X : axis == 1 ? Y : Z;
-    const int64_t h0row = axis == 0 ? 0 : H;              // row of h = 0
-    const uint64_t f = u[(int64_t)axis * P + p];
-    const float sc = axis == 2 ? zscale : 1.f;
-    float2 base[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) base[k] = k <= H ? phase_of<float>(f, k) : make_float2(1.f, 0.f);
-    for (int a = 0; 8 * a <= H; ++a) {
-        const float2 g = a == 0 ? make_float2(1.f, 0.f) : phase_of<float>(f, 8 * a);
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const int h = 8 * a + k;
-            if (h > H) break;
-            const float2 b = base[k];
-            float2 v = a == 0 ? b : make_float2(g.x * b.x - g.y * b.y, g.x * b.y + g.y * b.x);
-            v.x *= sc;
-            v.y *= sc;
-            T[(h0row + h) * P + p] = v;
-            if (axis != 0 && h > 0) T[(h0row - h) * P + p] = make_float2(v.x, -v.y);
-        }
-    }
-}
-
-cpm_status launch_col0_inputs(cudaStream_t st, const uint64_t* u, const double* Q, int64_t P, float4* e1,
-                              float2* q2) {
-    if (P == 0) return CPM_OK;
-    k_col0_inputs<<<(unsigned)((P + 255) / 256), 256, 0, st>>>(u + 2 * P, Q, P, e1, q2);
-    return cudaGetLastError() == cudaSuccess ? CPM_OK : CPM_E_CUDA;
-}
-
-template <typename T>
-cpm_status launch_phases_u(cudaStream_t st, const Geometry& g, const KTable& k, const double* xyz, const double* Q,
-                           int64_t ne, int m, uint64_t* u, T* Qv, double* qpart, int* tickets, float2* qabs,
-                           c2<T>* X, c2<T>* Y, c2<T>* Z, cudaEvent_t after_fracs, float zscale) {
-    const int64_t P = (int64_t)m * ne;
-    if (P == 0) return CPM_OK;
-    k_fracs<T><<<dim3((unsigned)((ne + FR_THREADS - 1) / FR_THREADS), (unsigned)m), FR_THREADS, 0, st>>>(
-        xyz, Q, ne, g.inv[0], g.inv[1], g.inv[2], u, Qv, qpart, tickets, qabs);
-    if (after_fracs && cudaEventRecord(after_fracs, st) != cudaSuccess) return CPM_E_CUDA;
-    if (std::is_same<T, float>::value) {
-        k_phases_rows<<<dim3((unsigned)((P + 127) / 128), 3), 128, 0, st>>>(u, P, k.NX, k.NY, k.NZ, (float2*)X,
-                                                                            (float2*)Y, (float2*)Z, zscale);
-    } else {
-        const int nslot = (k.NX + 1) + (2 * k.NY + 1) + (2 * k.NZ + 1);
-        k_phases_u<T><<<dim3((unsigned)((P + 255) / 256), (unsigned)nslot), 256, 0, st>>>(u, P, k.NX, k.NY, k.NZ, X,
-                                                                                          Y, Z);
-    }
-    return cudaGetLastError() == cudaSuccess ? CPM_OK : CPM_E_CUDA;
-}
-template cpm_status launch_phases_u<float>(cudaStream_t, const Geometry&, const KTable&, const double*, const double*,
-                                           int64_t, int, uint64_t*, float*, double*, int*, float2*, float2*, float2*,
-                                           float2*, cudaEvent_t, float);
-template cpm_status launch_phases_u<double>(cudaStream_t, const Geometry&, const KTable&, const double*,
-                                            const double*, int64_t, int, uint64_t*, double*, double*, int*, float2*,
-                                            double2*, double2*, double2*, cudaEvent_t, float);
-
 template <typename T>
 cpm_status launch_phases(cudaStream_t st, const Geometry& g, const KTable& k, const double* xyz, int64_t P,
                          c2<T>* X, c2<T>* Y, c2<T>* Z) {

@@ -1,33 +1,25 @@
 // Reciprocal-space part of the electrolyte vector b on the 5th-generation tensor cores.
 //
-// The Ewald sum of b over the half-space k set (Sec. II.E, Gaussian electrode charges of
-// Sec. III.B) factorises over the column layout of the k grid (column c = (nx, ny), harmonic
-// nz, phase tables X, Y, Z of the Cartesian components):
-//
-//   stage 1  rho_r[c][nz] = sum_j P_r[c][j] Z_j[nz],        P_r[c][j] = Q_j X_j[nx_c] Y_j[ny_c]
-//   stage 2  T_r[c][i]    = sum_nz conj(Z_i[nz]) W_r[c][nz],  W_r = w rho_r
-//            b_r[i]      += sum_c Re[ conj(X_i[nx_c] Y_i[ny_c]) T_r[c][i] ]
-//
-// Both stages are dense complex contractions (over the charges j, then over the harmonics nz),
-// so they run as real matrix products with (re, im) interleaved along K and N:
-//   stage 1: A = P (rows c, K = (j, re/im)), B rows (nz, re) = (Zr, -Zi), (nz, im) = (Zi, Zr)
-//   stage 2: A = site phases (rows i, K = (nz, re/im)), B rows (c, r, re) = (Wr, Wi),
-//            (c, r, im) = (Wi, -Wr); the epilogue contracts over c with conj(X_i Y_i).
+// Stage 1 (every geometry) is the structure factor in the real product basis of recip_rows.cu,
+//   R_r[p][t][c] = sum_j Q_j f_t(x_j, y_j) h_c(z_j),
+// a real matrix product over the charges: A = Q f_t (rows 4 pair + part, K = charges), B = h_c (rows c, K =
+// charges).  Heights shared by many sites then take the height-wise stages of recip_rows.cu.  For electrodes
+// whose sites hardly share heights stage 2 here is a complex product over the harmonics,
+//   T_r[c][i] = sum_nz conj(Z_i[nz]) W_r[c][nz],  W_r = w rho_r,
+//   b_r[i]   += sum_c Re[ conj(X_i[nx_c] Y_i[ny_c]) T_r[c][i] ]
+// over the signed columns c = (nx, ny), with (re, im) interleaved along K and N: A = site phases (rows i, K =
+// (nz, re/im)), B rows (c, r, re) = (Wr, Wi), (c, r, im) = (Wi, -Wr); the epilogue contracts over c.
 //
 // Operand precision: every operand x is scaled by a power of two s (|s x| < 2^14) and split as
 // x0 = fp16(s x), x1 = fp16(s x - x0) (22 significant bits); the products x0 y0 + x0 y1 + x1 y0
 // are accumulated in FP32 in tensor memory and the scales are removed exactly afterwards.  The
 // k_perp = 0 column keeps its double-float treatment (its single-precision weight is zero here).
 //
-// Stage 1 builds both operand tiles in shared memory from the phase tables (128 columns x 32
-// charges of P, 2 x 128 harmonic rows x 32 charges of Z per K step, 128-byte swizzle); stage 2
-// streams its operands with TMA.  One thread issues the tcgen05.mma instructions; every
-// mbarrier wait is bounded by wall time and on expiry the CTA records ST_TIMEOUT, frees its
-// tensor memory and returns.
+// One thread issues the tcgen05.mma instructions; every mbarrier wait is bounded by wall time and on expiry
+// the CTA records ST_TIMEOUT, frees its tensor memory and returns.
 #include <cuda_fp16.h>
 
 #include <algorithm>
-#include <vector>
 
 #include "common.cuh"
 #include "tc_common.cuh"
@@ -37,24 +29,18 @@ namespace cpm {
 constexpr uint64_t RT_WAIT_NS = 2000000000ull;   // bound on any single mbarrier wait: 2 s
 
 // stage 1 (structure factor)
-constexpr int RF_BM = 128;                     // columns per tile (MMA M)
-constexpr int RF_ZT = 128;                     // harmonics per tile (MMA N = 2 x 128)
-constexpr int RF_KC = 32;                      // charges per K step (64 fp16 = 128 bytes per row)
+constexpr int RF_PAIRS = ROW_TC_PAIRS;         // pairs per CTA: two row tiles (MMA M = 128) of 32 pairs x 4 parts
+constexpr int RF_KC = ROW_TC_STEP;             // charges per K step (64 fp16 = 128 bytes per operand row)
 constexpr int RF_GEN = 512;                    // operand-building threads (warps 0-15)
 constexpr int RF_THREADS = RF_GEN + 32;        // + the MMA warp
-constexpr int RF_ROWSTEP = RF_GEN / 8;         // tile rows covered by one pass of the builders
-constexpr int RF_PK = RF_BM / RF_ROWSTEP;      // P rows per builder
-constexpr int RF_ZK = RF_ZT / RF_ROWSTEP;      // Z row pairs per builder
-constexpr int RF_A = RF_BM * 128;              // one fp16 term of the P tile (16 KB)
-constexpr int RF_B = 2 * RF_ZT * 128;          // one fp16 term of the Z tile (32 KB)
-constexpr int RF_STAGE = 2 * RF_A + 2 * RF_B;  // 96 KB
+constexpr int RF_TERM = 128 * 128;             // one fp16 term of a 128-row operand tile (16 KB)
+constexpr int RF_STAGE = 6 * RF_TERM;          // A: two tiles x two terms, B: two terms (96 KB)
 constexpr int RF_STAGES = 2;
-constexpr int RF_XYROWS = 60;                 // staged phase-table rows: (NX + 1) + (2 NY + 1) at most
-constexpr int RF_STAGE_XY = (RF_XYROWS + 1) * RF_KC * 8;   // X, Y rows and Q of one K step
-constexpr int RF_PX = ((RF_XYROWS + 1) * RF_KC + RF_GEN - 1) / RF_GEN;   // staging entries per builder
-constexpr int RF_QSLOT = 1 << 16;              // staging slots at or above this are charges
-constexpr int RF_SMEM = 1024 + RF_STAGES * RF_STAGE + 2048 + RF_STAGE_XY;
-constexpr float RF_ZSCALE = TC_ZSCALE;         // charge phases scaled by 2^14 (in the table)
+constexpr int RF_RANGE = 16;                   // K steps of one accumulation at most
+constexpr int RF_SLOTS = ROW_TC_SLOTS + 16;    // staged table rows of a step: x and y harmonics, 8 + 8 z phases
+constexpr int RF_PX = (RF_SLOTS + 15) / 16;    // staging entries (16 bytes) per builder
+constexpr int RF_SMEM = 1024 + RF_STAGES * RF_STAGE + 1024 + RF_SLOTS * RF_KC * 8;
+static_assert(RF_SMEM <= 232448, "shared memory of one CTA");
 
 // stage 2 (site potentials)
 constexpr int RS_BM = 128;                     // sites per tile (MMA M)
@@ -70,19 +56,21 @@ constexpr int RS_ZEXP = 14;                    // site phases scaled by 2^14
 constexpr int RS_CT = 16;                      // columns per group (N = 2 x 16 x replicas of the group)
 constexpr int RS_MR = 8;                       // replicas per group
 
-// 2^e with bound * 2^e < 2^top; 1 for a zero or non-finite bound
-__device__ __forceinline__ float pow2_below(float bound, int top) {
-    if (!(bound > 0.f) || !isfinite(bound)) return 1.f;
-    int e;
-    frexpf(bound, &e);   // bound = f 2^e, f in [0.5, 1)
-    return ldexpf(1.f, top - e);
-}
-
 // (re, im) -> two packed fp16 pairs: hi = fp16(v), lo = fp16(v - hi); low half = re
 __device__ __forceinline__ void split2(float2 v, uint32_t& hi, uint32_t& lo) {
     const __half2 h = __floats2half2_rn(v.x, v.y);
     const float2 f = __half22float2(h);
     const __half2 l = __floats2half2_rn(v.x - f.x, v.y - f.y);
+    hi = *reinterpret_cast<const uint32_t*>(&h);
+    lo = *reinterpret_cast<const uint32_t*>(&l);
+}
+// the same for a packed pair of FP32 values (the pair of charges of one operand word)
+__device__ __forceinline__ void split2p(uint64_t v, uint32_t& hi, uint32_t& lo) {
+    const float2 x = up2(v);
+    const __half2 h = __floats2half2_rn(x.x, x.y);
+    const float2 f = __half22float2(h);
+    const float2 d = up2(sub2(v, pk2(f.x, f.y)));
+    const __half2 l = __floats2half2_rn(d.x, d.y);
     hi = *reinterpret_cast<const uint32_t*>(&h);
     lo = *reinterpret_cast<const uint32_t*>(&l);
 }
@@ -107,24 +95,30 @@ __device__ __forceinline__ void gen_bar() { asm volatile("bar.sync 1, %0;" ::"n"
 __device__ __forceinline__ void sts128(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
     asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
+__device__ __forceinline__ void sts32(uint32_t addr, uint32_t a) {
+    asm volatile("st.shared.b32 [%0], %1;" ::"r"(addr), "r"(a) : "memory");
+}
 // byte offset of 16-byte chunk ch of row r in a K-major tile of 128-byte rows, 128-byte swizzle
 __device__ __forceinline__ uint32_t sw128(int r, int ch) { return (uint32_t)(r * 128 + ((ch ^ (r & 7)) << 4)); }
 
 // ----------------------------------------------------------------------------- stage 1
-// part[s][r][zi][c] = 2^14 sA_r sum over the charges of split s of P_r[c][j] Z_j[zi]   (zi = nz + NZ)
-// grid (column tiles, harmonic tiles, m * splits); sA_r = 2^e with |Q| sA_r < 2^14.
-// largest harmonic extent of each 128-column tile, known on the host (fixed with the k set)
-struct TileMx {
-    int n;          // number of tiles given; 0: the kernel finds the extents itself
-    int mx[32];
-};
-
+// part[s][r][4 p + t][c] = 2^14 sA_r sum over the K steps of range s of replica r; sA_r = 2^e, |Q| sA_r < 2^14.
+// grid items x (m splits), items fastest; an item is (first pair, pairs, harmonic tile, harmonics) and its range of staged
+// harmonics (x0, nx, y0, ny).  Per K step of 64 charges the 512 builders stage the x and y harmonics and the z
+// phases of the step in shared memory (loads issued one step ahead), then each forms the four rows
+// (cos, sin) x (cos, sin) of one pair for eight charges, and eight z functions for two charges (h = 8 a + k as
+// a product of two phases), both split into two fp16 terms in 128-byte-swizzled operand tiles.
+// The leading products have an accumulator of their own, the cross products another: the tensor core truncates
+// the sum at each of its additions, so the error of a long range grows with their number (one accumulator for
+// all three and 86 steps: b of a 16-replica 8,192-site batch 9.7e-6 off; RF_RANGE bounds the steps).
+// What bounds it: shared memory.  A step moves about 64 KB of operand reads and 96 KB of operand writes by
+// the builders and 160 KB of operand reads by the 16 MMAs, at 128 B per clock; real products of pairs need
+// half the MMAs and a quarter of the z operand of complex columns over both signs of nz.
 __global__ void __launch_bounds__(RF_THREADS, 1)
-    k_tc_sf(const int2* __restrict__ cols, const int* __restrict__ colext, int ncols, int NX, int NY, int NZ, int nzw,
-            const float2* __restrict__ EX, const float2* __restrict__ EY, const float2* __restrict__ EZ,
-            const float* __restrict__ Qv, const float2* __restrict__ qabs, int64_t ptot, int64_t ne, int splits,
-            int64_t chunk, int m, int cpad, const __grid_constant__ TileMx tmx, float2* __restrict__ part,
-            unsigned* __restrict__ status, uint64_t wait_ns) {
+    k_tc_rows(const int4* __restrict__ items, const int4* __restrict__ ranges, const int4* __restrict__ pairs,
+              const float2* __restrict__ tab, int64_t P, int64_t nep, int NX, int NY, int NZ,
+              const float* __restrict__ qmax, const int* __restrict__ qlast, int nitems, int splits, int spc, int m, int np,
+              int cw, float* __restrict__ part, unsigned* __restrict__ status, uint64_t wait_ns) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = align1024(smem_raw);
     uint8_t* aux = smem + RF_STAGES * RF_STAGE;
@@ -133,109 +127,48 @@ __global__ void __launch_bounds__(RF_THREADS, 1)
     uint64_t* done = empty + RF_STAGES;
     uint32_t* tmem_slot = (uint32_t*)(done + 1);
     volatile int* abort = (volatile int*)(tmem_slot + 1);
-    int* s_mx = (int*)(tmem_slot + 2);
-    int2* s_cols = (int2*)(aux + 64);
+    float4* stg = (float4*)(aux + 1024);           // [slot][32 units of two charges]
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int c0 = blockIdx.x * RF_BM;
-    const int r = blockIdx.z / splits, sp = blockIdx.z % splits;
+    const int bi = blockIdx.x % nitems, br = blockIdx.x / nitems;
+    const int4 it = items[bi];                     // (first pair, pairs, harmonic tile, harmonics)
+    const int4 rg = ranges[bi];                    // (x0, nx, y0, ny)
+    const int r = br / splits, sp = br % splits;
+    const int ntile = it.y > RF_PAIRS / 2 ? 2 : 1;
+    const int nused = ((2 * it.w + 15) / 16) * 16;
+    const int s0 = sp * spc, nsteps = max(0, min((qlast[r] + RF_KC - 1) / RF_KC, s0 + spc) - s0);
 
-    int mx;
-    if ((int)blockIdx.x < tmx.n) {
-        mx = tmx.mx[blockIdx.x];
-    } else {
-        if (warp == 0) {
-            int v = -1;
-            for (int t = lane; t < RF_BM; t += 32)
-                if (c0 + t < ncols) v = max(v, colext[c0 + t]);
-            for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
-            if (lane == 0) *s_mx = v;
-        }
-        __syncthreads();
-        mx = *s_mx;
-    }
-    const int zoff = blockIdx.y * RF_ZT;
-    const int zcount = min(RF_ZT, 2 * mx + 1 - zoff);
-    if (mx < 0 || zcount <= 0) return;   // block-uniform; nothing allocated yet
-    const int z_lo = NZ - mx + zoff;     // grid index of the tile's first harmonic
-    const int nused = ((2 * zcount + 15) / 16) * 16;
-    const int64_t jb = (int64_t)r * ne + (int64_t)sp * chunk;
-    const int64_t je = min((int64_t)r * ne + ne, jb + chunk);
-    const int nsteps = je > jb ? (int)((je - jb + RF_KC - 1) / RF_KC) : 0;
-    const int rem0 = (int)max((int64_t)0, je - jb);   // charges of this split
-
-    // Operand builders.  Thread g owns 16-byte chunk ch = g % 8 (charges 4 ch .. 4 ch + 3 of the step)
-    // of P rows g / 8 + 64 k and of Z row pairs g / 8 + 64 k.  The X and Y table rows and the charges
-    // of a step are staged in shared memory; the loads of step t + 1 (staging entries and Z values)
-    // are issued before the tiles of step t are built.  Within a staged table row, charge 4 ch + u sits
-    // at 16 (u / 2) + 2 ch + u % 2, so that the eight threads of a quarter warp (one P row) read two
-    // 128-byte runs with two 16-byte loads each; the charges are a row of 32 floats in natural order.
-    // Every source address and staging slot of a thread is fixed for the split and advances by one
-    // step (32 charges) at a time, so it is computed once here.
-    const int g = threadIdx.x, ch = g & 7, rbase = g >> 3;
-    const int xyrows = (NX + 1) + (2 * NY + 1);
-    const int nst = (xyrows + 1) * RF_KC;
-    float2* sxy = (float2*)(aux + 2048);
-    float* sqf = (float*)(sxy + xyrows * RF_KC);
-    const bool vec = (ne & 1) == 0;   // then every Z run of a thread starts on a 16-byte boundary
-    // entry k of this thread is charge jj = g % 32 of staged row (g + RF_GEN k) / 32; xdst: its slot
-    // in the staged table rows, or RF_QSLOT + jj for the charge row, or -1 past the last row
-    const int xjj = g & 31;
-    const float2* xsrc[RF_PX];
-    int xdst[RF_PX];
-    const float2* zsrc[RF_ZK];
-    bool zlive[RF_ZK];
+    const int g = threadIdx.x, nxy = rg.y + rg.w;
+    // staging: 16-byte unit uu of slots g / 32 + 16 k; sources advance by one step (64 charges) at a time
+    const int uu = g & 31;
+    const float4* src[RF_PX];
+    int dst[RF_PX];
+    float4 px[RF_PX];
     float sA = 1.f;
-    float2 px[RF_PX], pz[RF_ZK][4];
     auto prefetch = [&](int t) {
-        const int o = t * RF_KC;
 #pragma unroll
-        for (int k = 0; k < RF_PX; ++k) {
-            float2 v = make_float2(0.f, 0.f);
-            if (xdst[k] >= 0 && xjj + o < rem0)
-                v = xdst[k] < RF_QSLOT ? xsrc[k][o] : make_float2(reinterpret_cast<const float*>(xsrc[k])[o] * sA, 0.f);
-            px[k] = v;
-        }
-        const int jt = o + 4 * ch;   // first charge of this thread's run, relative to the split
-#pragma unroll
-        for (int k = 0; k < RF_ZK; ++k) {
-            if (!zlive[k]) {
-#pragma unroll
-                for (int u = 0; u < 4; ++u) pz[k][u] = make_float2(0.f, 0.f);
-            } else if (vec && jt + 3 < rem0) {
-                const float4 a01 = *reinterpret_cast<const float4*>(zsrc[k] + o);
-                const float4 a23 = *reinterpret_cast<const float4*>(zsrc[k] + o + 2);
-                pz[k][0] = make_float2(a01.x, a01.y);
-                pz[k][1] = make_float2(a01.z, a01.w);
-                pz[k][2] = make_float2(a23.x, a23.y);
-                pz[k][3] = make_float2(a23.z, a23.w);
-            } else {
-#pragma unroll
-                for (int u = 0; u < 4; ++u) pz[k][u] = jt + u < rem0 ? zsrc[k][o + u] : make_float2(0.f, 0.f);
-            }
-        }
+        for (int k = 0; k < RF_PX; ++k)
+            if (dst[k] >= 0) px[k] = src[k][t * (RF_KC / 2)];
     };
     if (warp < RF_GEN / 32) {
-        sA = pow2_below(qabs[r].x, 14);
+        sA = pow2_below(qmax[r], 14);
+        const int64_t p0 = (int64_t)r * nep + (int64_t)s0 * RF_KC + 2 * uu;
 #pragma unroll
         for (int k = 0; k < RF_PX; ++k) {
-            const int e = g + RF_GEN * k, row = e >> 5, jj = xjj;
-            xdst[k] = e >= nst ? -1
-                    : row < xyrows ? row * RF_KC + (((jj & 2) << 3) | ((jj >> 2) << 1) | (jj & 1)) : RF_QSLOT + jj;
-            xsrc[k] = row <= NX ? EX + (int64_t)row * ptot + jb + jj
-                    : row < xyrows ? EY + (int64_t)(row - NX - 1) * ptot + jb + jj
-                                   : reinterpret_cast<const float2*>(Qv + jb + jj);
-        }
-#pragma unroll
-        for (int k = 0; k < RF_ZK; ++k) {
-            const int zr = rbase + RF_ROWSTEP * k;
-            zlive[k] = zr < zcount;
-            zsrc[k] = EZ + (int64_t)(z_lo + min(zr, zcount - 1)) * ptot + jb + 4 * ch;
+            const int slot = (g >> 5) + 16 * k;
+            int row = 0;
+            dst[k] = -1;
+            if (slot < rg.y) row = rg.x + slot;
+            else if (slot < nxy) row = NX + 1 + rg.z + (slot - rg.y);
+            else if (slot < nxy + 8) row = NX + NY + 2 + (slot - nxy);
+            else row = NX + NY + 10 + min(8 * it.z + (slot - nxy - 8), NZ / 8);
+            // x and y units are permuted so that eight threads of eight charges each read 128 contiguous bytes
+            if (slot < nxy) dst[k] = slot * 32 + (uu & 3) * 8 + (uu >> 2);
+            else if (slot < nxy + 16) dst[k] = slot * 32 + uu;
+            src[k] = reinterpret_cast<const float4*>(tab + (int64_t)row * P + p0);
         }
         if (nsteps > 0) prefetch(0);   // in flight during the set-up below
     }
-
-    if (threadIdx.x < RF_BM) s_cols[threadIdx.x] = c0 + (int)threadIdx.x < ncols ? cols[c0 + threadIdx.x] : make_int2(0, 0);
     if (threadIdx.x == 0) {
         for (int s = 0; s < RF_STAGES; ++s) { mbar_init(&full[s], RF_GEN); mbar_init(&empty[s], 1); }
         mbar_init(done, 1);
@@ -244,7 +177,7 @@ __global__ void __launch_bounds__(RF_THREADS, 1)
     }
     if (warp == RF_GEN / 32) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tmem_slot)),
-                     "r"(256u)
+                     "r"(512u)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -254,6 +187,14 @@ __global__ void __launch_bounds__(RF_THREADS, 1)
     const uint32_t tmem = *tmem_slot;
 
     if (warp < RF_GEN / 32) {
+        const int ch = g & 7, pl = g >> 3;             // A: charges 8 ch .. 8 ch + 7 of pair pl
+        const bool live = pl < it.y;                   // rows past the last pair are never read back
+        const int4 pr = live ? pairs[it.x + pl] : make_int4(rg.x, rg.z, 0, 0);
+        const float4* xr = stg + (pr.x - rg.x) * 32 + ch;
+        const float4* yr = stg + (rg.y + pr.y - rg.z) * 32 + ch;
+        const int hq = g >> 5, h0 = 4 * hq;            // B: harmonics h0 .. h0 + 3 of the tile, charges 2 uu, 2 uu + 1
+        const float4* zb = stg + (nxy + (h0 & 4)) * 32 + uu;
+        const float4* zg = stg + (nxy + 8 + (h0 >> 3)) * 32 + uu;
         for (int t = 0; t < nsteps; ++t) {
             const int s = t % RF_STAGES;
             bool ok = true;
@@ -261,164 +202,157 @@ __global__ void __launch_bounds__(RF_THREADS, 1)
             if (!gen_bar_and(ok)) break;   // uniform; also: everyone is done reading the staged step t - 1
 #pragma unroll
             for (int k = 0; k < RF_PX; ++k) {
-                if (xdst[k] >= RF_QSLOT) sqf[xdst[k] - RF_QSLOT] = px[k].x;
-                else if (xdst[k] >= 0) sxy[xdst[k]] = px[k];
-            }
-            const uint32_t sa = su32(smem + s * RF_STAGE);
-            const uint32_t sb = sa + 2 * RF_A;
-            // the Z tile needs nothing staged: built from registers before they take the next step
-#pragma unroll
-            for (int k = 0; k < RF_ZK; ++k) {
-                const int zr = rbase + RF_ROWSTEP * k;
-                if (zr >= zcount) continue;
-                uint32_t h[4], l[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-                    split2(pz[k][u], h[u], l[u]);   // the table holds 2^14 Z
-                const uint32_t o0 = sw128(2 * zr, ch), o1 = sw128(2 * zr + 1, ch);
-                sts128(sb + o0, neg_hi(h[0]), neg_hi(h[1]), neg_hi(h[2]), neg_hi(h[3]));
-                sts128(sb + o1, swap_h(h[0]), swap_h(h[1]), swap_h(h[2]), swap_h(h[3]));
-                sts128(sb + RF_B + o0, neg_hi(l[0]), neg_hi(l[1]), neg_hi(l[2]), neg_hi(l[3]));
-                sts128(sb + RF_B + o1, swap_h(l[0]), swap_h(l[1]), swap_h(l[2]), swap_h(l[3]));
+                if (dst[k] < 0) continue;
+                // (cos, cos, sin, sin) of the two charges: operands of packed arithmetic
+                const float f = (g >> 5) + 16 * k < rg.y ? sA : 1.f;
+                stg[dst[k]] = make_float4(px[k].x * f, px[k].z * f, px[k].y * f, px[k].w * f);
             }
             gen_bar();   // the staged rows of step t are complete
             if (t + 1 < nsteps) prefetch(t + 1);
-            const float4 q4 = reinterpret_cast<const float4*>(sqf)[ch];
-            const float qv[4] = {q4.x, q4.y, q4.z, q4.w};
+            const uint32_t sa = su32(smem + s * RF_STAGE);
+            if (h0 < it.w) {
+                const uint32_t sb = sa + 4 * RF_TERM + 4 * (uu & 3), sl = sb + nused * 128;
+                const float4 gz = *zg;
+                const uint64_t gc = pk2(gz.x, gz.y), gs = pk2(gz.z, gz.w), ngs = pk2(-gz.z, -gz.w);
 #pragma unroll
-            for (int k = 0; k < RF_PK; ++k) {
-                const int row = rbase + RF_ROWSTEP * k;
-                const int2 cn = s_cols[row];
-                const bool live = c0 + row < ncols;
-                float2 x[4], y[4];
-                if (live) {
-                    const float4* xr = reinterpret_cast<const float4*>(sxy + cn.x * RF_KC);
-                    const float4* yr = reinterpret_cast<const float4*>(sxy + (NX + 1 + cn.y + NY) * RF_KC);
-                    const float4 x01 = xr[ch], x23 = xr[8 + ch], y01 = yr[ch], y23 = yr[8 + ch];
-                    x[0] = make_float2(x01.x, x01.y); x[1] = make_float2(x01.z, x01.w);
-                    x[2] = make_float2(x23.x, x23.y); x[3] = make_float2(x23.z, x23.w);
-                    y[0] = make_float2(y01.x, y01.y); y[1] = make_float2(y01.z, y01.w);
-                    y[2] = make_float2(y23.x, y23.y); y[3] = make_float2(y23.z, y23.w);
+                for (int k = 0; k < 4; ++k) {
+                    const float4 bz = zb[k * 32];
+                    const uint64_t bc = pk2(bz.x, bz.y), bs = pk2(bz.z, bz.w);
+                    uint32_t h, l;
+                    const int row = 2 * (h0 + k);
+                    if (row >= nused) break;   // the rows above belong to the second term
+                    split2p(fma2(ngs, bs, mul2(gc, bc)), h, l);
+                    const uint32_t o0 = sw128(row, uu >> 2);
+                    sts32(sb + o0, h);
+                    sts32(sl + o0, l);
+                    split2p(fma2(gs, bc, mul2(gc, bs)), h, l);
+                    const uint32_t o1 = sw128(row + 1, uu >> 2);
+                    sts32(sb + o1, h);
+                    sts32(sl + o1, l);
                 }
-                uint32_t h[4], l[4];
+            }
+            if (live) {
+                const uint32_t at = sa + (pl >> 5) * 2 * RF_TERM;
+                const int row = (pl & 31) * 4;
+                uint32_t h[4][4], l[4][4];   // [part][unit of two charges]
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
-                    float2 p = make_float2(0.f, 0.f);
-                    if (live)
-                        p = make_float2((x[u].x * y[u].x - x[u].y * y[u].y) * qv[u],
-                                        (x[u].x * y[u].y + x[u].y * y[u].x) * qv[u]);
-                    split2(p, h[u], l[u]);
+                    const float4 x = xr[u * 8], y = yr[u * 8];
+                    const uint64_t xc = pk2(x.x, x.y), xs = pk2(x.z, x.w), yc = pk2(y.x, y.y), ys = pk2(y.z, y.w);
+                    split2p(mul2(xc, yc), h[0][u], l[0][u]);
+                    split2p(mul2(xs, yc), h[1][u], l[1][u]);
+                    split2p(mul2(xc, ys), h[2][u], l[2][u]);
+                    split2p(mul2(xs, ys), h[3][u], l[3][u]);
                 }
-                const uint32_t off = sw128(row, ch);
-                sts128(sa + off, h[0], h[1], h[2], h[3]);
-                sts128(sa + RF_A + off, l[0], l[1], l[2], l[3]);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const uint32_t o = sw128(row + q, ch);
+                    sts128(at + o, h[q][0], h[q][1], h[q][2], h[q][3]);
+                    sts128(at + RF_TERM + o, l[q][0], l[q][1], l[q][2], l[q][3]);
+                }
             }
             fence_async_smem();
             mbar_arrive(&full[s]);
         }
     } else if (lane == 0) {
-        // MMA issuer: per 16-wide K slice the products P0 Z0 + P0 Z1 + P1 Z0
-        const uint32_t idesc = idesc_f16(RF_BM, nused);
+        // MMA issuer: per 16-wide K slice and row tile A0 [B0 B1] (the terms of B one after the other: columns
+        // 0 .. nused - 1 the leading products, nused .. 2 nused - 1 the cross ones) and A1 B0 on the latter
+        const uint32_t id1 = idesc_f16(128, nused), id2 = idesc_f16(128, 2 * nused);
         for (int t = 0; t < nsteps; ++t) {
             const int s = t % RF_STAGES;
             if (!mbar_wait(&full[s], (t / RF_STAGES) & 1, abort, wait_ns)) break;
             tc_fence_after();
-            const uint32_t sa = su32(smem + s * RF_STAGE), sb = sa + 2 * RF_A;
+            const uint32_t sa = su32(smem + s * RF_STAGE), sb = sa + 4 * RF_TERM;
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk) {
-                const uint64_t a0 = sdesc_sw128(sa + kk * 32), a1 = sdesc_sw128(sa + RF_A + kk * 32);
-                const uint64_t b0 = sdesc_sw128(sb + kk * 32), b1 = sdesc_sw128(sb + RF_B + kk * 32);
-                umma_f16(tmem, a0, b0, idesc, (t > 0 || kk > 0) ? 1u : 0u);
-                umma_f16(tmem, a0, b1, idesc, 1u);
-                umma_f16(tmem, a1, b0, idesc, 1u);
+                const uint64_t b0 = sdesc_sw128(sb + kk * 32);
+                for (int q = 0; q < ntile; ++q) {
+                    const uint32_t at = sa + q * 2 * RF_TERM + kk * 32, acc = tmem + 256 * q;
+                    umma_f16(acc, sdesc_sw128(at), b0, id2, (t > 0 || kk > 0) ? 1u : 0u);
+                    umma_f16(acc + nused, sdesc_sw128(at + RF_TERM), b0, id1, 1u);
+                }
             }
             umma_commit(&empty[s]);
         }
         umma_commit(done);   // also after an abort: the epilogue then waits for the MMAs in flight
     }
     if (warp < RF_GEN / 32) {
-        // epilogue on all builder warps: warp w reads accumulator lanes 32 (w % 4) .. + 31 (its columns)
-        // and accumulator columns 16 (w / 4) + 64 i (eight harmonics each)
+        // epilogue: warp w reads accumulator lanes 32 (w % 4) .. + 31 of row tile (w / 4) % 2, columns
+        // 16 (w / 8) + 32 i: sixteen harmonic functions of one row per thread
         const bool ok = mbar_wait(done, 0, abort, wait_ns);
         tc_fence_after();
         const bool good = __all_sync(0xffffffffu, ok && !*abort) != 0;
-        if (good) {
-            const int lq = warp & 3, cg = warp >> 2;
-            const int c = c0 + lq * 32 + lane;
-            float2* out = part + ((int64_t)sp * m + r) * nzw * cpad + c;
-            const uint32_t trow = tmem + ((uint32_t)(lq * 32) << 16);
-            for (int q0 = 16 * cg; q0 < nused; q0 += 64) {
+        const int lq = warp & 3, tile = (warp >> 2) & 1;
+        if (!good) {
+            if (lane == 0) atomicOr(status, ST_TIMEOUT);
+        } else if (tile < ntile) {
+            const int row = tile * 128 + lq * 32 + lane;
+            const uint32_t trow = tmem + 256 * tile + ((uint32_t)(lq * 32) << 16);
+            float* out = part + (((int64_t)sp * m + r) * np + it.x) * 4 * cw + (int64_t)row * cw + it.z * 128;
+            for (int q0 = 16 * (warp >> 3); q0 < nused; q0 += 32) {
                 float v[16];
                 if (nsteps > 0) {
+                    float lo[16];
                     tmem_ld16(trow + q0, v);
+                    tmem_ld16(trow + nused + q0, lo);
+#pragma unroll
+                    for (int k = 0; k < 16; ++k) v[k] += lo[k];
                 } else {
 #pragma unroll
                     for (int k = 0; k < 16; ++k) v[k] = 0.f;
                 }
+                if ((row >> 2) < it.y) {
 #pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const int zz = q0 / 2 + u;
-                    if (zz < zcount) out[(int64_t)(z_lo + zz) * cpad] = make_float2(v[2 * u], v[2 * u + 1]);
+                    for (int k = 0; k < 4; ++k)
+                        *reinterpret_cast<float4*>(out + q0 + 4 * k) = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
                 }
             }
-        } else if (lane == 0) {
-            atomicOr(status, ST_TIMEOUT);
         }
     }
     tc_fence_before();
     __syncthreads();
     if (warp == RF_GEN / 32) {
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(256u) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
+    }
+}
+
+// qsum[r] = sum |Q| of replica r, the scale of the site stage: one block each, a fixed order
+__global__ void __launch_bounds__(1024) k_qsum_abs(const double* __restrict__ Q, int64_t ne, float* __restrict__ qsum) {
+    __shared__ float ss[32];
+    const int r = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float sum = 0.f;
+    for (int64_t j = threadIdx.x; j < ne; j += 1024) sum += fabsf((float)Q[(int64_t)r * ne + j]);
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (lane == 0) ss[warp] = sum;
+    __syncthreads();
+    if (warp == 0) {
+        sum = ss[lane];
+        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        if (lane == 0) qsum[r] = sum;
     }
 }
 
 // ----------------------------------------------------------------------------- between the stages
-// W planes (two fp16 terms) of the site stage from the split structure factors:
-//   W_r[c][zi] = sW_r w[c][zi] (sum_s part[s][r][zi][c]) / (2^14 sA_r)   (zero outside the k set)
-// row (group g, pair p, re) = (Wr, Wi) and row (.., im) = (Wi, -Wr) at K = 2 zi, 2 zi + 1.
+// W planes (two fp16 terms) of the site stage from the weighted structure factor w rho of the signed columns:
+// row (group g, pair p, re) = (Wr, Wi) and row (.., im) = (Wi, -Wr) at K = 2 zi, 2 zi + 1, scaled by
+// sW_r = 2^e with wmax (sum |Q|) sW_r < 2^14.
 // Groups hold CT columns x mr replicas: g = (r / mr) ncb + c / CT, p = (r % mr) CT + c % CT.
 // One block transposes a 32-harmonic x 32-column tile of one replica slot.
 __global__ void __launch_bounds__(1024)
-    k_tc_wsplit(const float2* __restrict__ part, int splits, int m, int cpad, int nzw, int NZ,
-                const int* __restrict__ colext, const float* __restrict__ w32, int ncols,
-                const float2* __restrict__ qabs, float wmax, int CT, int mr, int ncb, int NB, int KZ,
-                uint32_t* __restrict__ w16, int64_t plane_words) {
+    k_tc_wsplit(const float2* __restrict__ wrho, int m, int nzw, int ncols, const float* __restrict__ qsum, float wmax,
+                int CT, int mr, int ncb, int NB, int KZ, uint32_t* __restrict__ w16, int64_t plane_words) {
     __shared__ float2 tile[32][33];
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int zb = blockIdx.x * 32, cb0 = blockIdx.y * 32, rp = blockIdx.z;
-    const bool rlive = rp < m;
     {
-        const int zi = zb + ty, c = cb0 + tx;
+        const int zi = zb + tx, c = cb0 + ty;
         float2 W = make_float2(0.f, 0.f);
-        if (rlive && c < ncols && zi < nzw) {
-            const int ext = colext[c], nz = zi - NZ;
-            const float wt = w32[(int64_t)c * nzw + zi];
-            if (nz >= -ext && nz <= ext && wt != 0.f) {
-                const float2 qa = qabs[rp];
-                const float f = pow2_below(wmax * qa.y, 14) / (pow2_below(qa.x, 14) * RF_ZSCALE);
-                float sx = 0.f, sy = 0.f;
-                const float2* pp = part + ((int64_t)rp * nzw + zi) * cpad + c;
-                const int64_t sstride = (int64_t)m * nzw * cpad;
-                int s = 0;
-                for (; s + 8 <= splits; s += 8) {   // eight loads in flight, added in split order
-                    float2 v[8];
-#pragma unroll
-                    for (int k = 0; k < 8; ++k) v[k] = pp[(s + k) * sstride];
-#pragma unroll
-                    for (int k = 0; k < 8; ++k) {
-                        sx += v[k].x;
-                        sy += v[k].y;
-                    }
-                }
-                for (; s < splits; ++s) {
-                    const float2 v = pp[s * sstride];
-                    sx += v.x;
-                    sy += v.y;
-                }
-                W = make_float2(sx * wt * f, sy * wt * f);
-            }
+        if (rp < m && c < ncols && zi < nzw) {
+            const float f = pow2_below(wmax * qsum[rp], 14);
+            const float2 v = wrho[((int64_t)rp * ncols + c) * nzw + zi];
+            W = make_float2(v.x * f, v.y * f);
         }
-        tile[ty][tx] = W;
+        tile[tx][ty] = W;
     }
     __syncthreads();
     const int rb = rp / mr, rr = rp % mr;
@@ -462,7 +396,7 @@ __device__ __forceinline__ void site_group_steps(const int* __restrict__ colext,
 __global__ void __launch_bounds__(RS_THREADS, 1)
     k_tc_site(const __grid_constant__ SiteMaps maps, const int* __restrict__ colext, int ncols, int NZ,
               int mr, int ncb, int NB, int m, int ntx, int ntiles, const float2* __restrict__ XY, int64_t n,
-              const float2* __restrict__ qabs, float wmax, float* __restrict__ partial,
+              const float* __restrict__ qsum, float wmax, float* __restrict__ partial,
               unsigned* __restrict__ status, uint64_t wait_ns) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = align1024(smem_raw);
@@ -596,7 +530,7 @@ __global__ void __launch_bounds__(RS_THREADS, 1)
                 }
                 const int r = rb * mr + rr;
                 if (r < m && i < n)
-                    partial[((int64_t)r * ncb + cb) * n + i] = sacc * (zinv / pow2_below(wmax * qabs[r].y, 14));
+                    partial[((int64_t)r * ncb + cb) * n + i] = sacc * (zinv / pow2_below(wmax * qsum[r], 14));
             }
             tc_fence_before();
             __syncwarp();
@@ -644,19 +578,28 @@ __global__ void k_tc_site_xy(const double2* __restrict__ SX, const double2* __re
 }
 
 // ----------------------------------------------------------------------------- host side
-bool tc_recip_supported(const KTable& k) { return k.nk > 0 && (k.NX + 1) + (2 * k.NY + 1) <= RF_XYROWS; }
-
 TcRecipDims tc_recip_dims(const cpm_ctx* c, int m, int64_t ne) {
     const KTable& k = c->kt;
     TcRecipDims d;
-    d.mtiles = (k.ncols + RF_BM - 1) / RF_BM;
-    d.cpad = d.mtiles * RF_BM;
-    d.ntiles = (k.nzw + RF_ZT - 1) / RF_ZT;
-    const int base = std::max(1, d.mtiles * d.ntiles * m);
-    const int64_t maxs = std::max<int64_t>(1, (ne + 4 * RF_KC - 1) / (4 * RF_KC));   // >= 4 K steps per CTA
-    d.splits = (int)std::max<int64_t>(1, std::min<int64_t>(std::max(1, 152 / base), maxs));
-    d.chunk = (ne + d.splits - 1) / d.splits;
-    d.chunk = ((d.chunk + RF_KC - 1) / RF_KC) * RF_KC;
+    d.nep = ((ne + RF_KC - 1) / RF_KC) * RF_KC;
+    d.cw = ((2 * (k.NZ + 1) + 31) / 32) * 32;
+    // charge ranges: the fewest K steps one after the other (whole waves of CTAs, one per SM, times the
+    // steps of a range and about three more for its set-up and epilogue); every extra range is written and
+    // read back, so it has to gain 3 %
+    const int64_t steps = std::max<int64_t>(1, d.nep / RF_KC), base = (int64_t)std::max(1, c->rows.tcitems) * m;
+    d.splits = (int)((steps + RF_RANGE - 1) / RF_RANGE);
+    d.spc = RF_RANGE;
+    double best = 1e300;
+    for (int s = (int)((steps + RF_RANGE - 1) / RF_RANGE); s <= steps && s <= (int)((steps + RF_RANGE - 1) / RF_RANGE) + 64; ++s) {
+        const int64_t spc = (steps + s - 1) / s, used = (steps + spc - 1) / spc;
+        if (used != s) continue;
+        const double t = (double)((base * s + 151) / 152) * (double)(spc + 3);
+        if (t < 0.97 * best) {
+            best = t;
+            d.splits = s;
+            d.spc = (int)spc;
+        }
+    }
     d.mr = std::min(m, RS_MR);
     d.nrb = (m + d.mr - 1) / d.mr;
     d.CT = RS_CT;
@@ -668,9 +611,6 @@ TcRecipDims tc_recip_dims(const cpm_ctx* c, int m, int64_t ne) {
     return d;
 }
 
-size_t tc_recip_part_bytes(const TcRecipDims& d, int m, int nzw) {
-    return sizeof(float2) * (size_t)d.splits * m * nzw * d.cpad;
-}
 size_t tc_recip_w16_bytes(const TcRecipDims& d) { return 2 * sizeof(uint16_t) * (size_t)d.ngroups * d.NB * d.KZ; }
 
 // site operands that stay fixed with the geometry: phase planes and column factors X_i Y_i
@@ -680,7 +620,6 @@ cpm_status tc_recip_prepare(cpm_ctx* c) {
     dev_free(c, c->tcxy);
     c->tcz = nullptr;
     c->tcxy = nullptr;
-    if (!tc_recip_supported(k)) return CPM_OK;
     const TcRecipDims d = tc_recip_dims(c, 1, 0);
     const int64_t n = c->n;
     CPM_TRY(dev_alloc(c, &c->tcz, sizeof(uint16_t) * 2 * (size_t)d.npad * d.KZ));
@@ -700,51 +639,37 @@ cpm_status tc_recip_prepare(cpm_ctx* c) {
         kmin2 = std::min(kmin2, kk * kk);
     }
     c->tc_wmax = (float)(1.01 * 8.0 * PI / c->g.V / kmin2);
-    // largest harmonic extent of each 128-column tile of the structure-factor stage
-    c->tc_nmx = 0;
-    if (d.mtiles <= 32) {
-        std::vector<int> ext(k.ncols);
-        CPM_CUDA(c, cudaMemcpyAsync(ext.data(), k.colext, sizeof(int) * k.ncols, cudaMemcpyDeviceToHost, c->stream));
-        CPM_CUDA(c, cudaStreamSynchronize(c->stream));
-        for (int t = 0; t < d.mtiles; ++t) {
-            int mx = -1;
-            for (int cc = t * RF_BM; cc < std::min(k.ncols, (t + 1) * RF_BM); ++cc) mx = std::max(mx, ext[cc]);
-            c->tc_mx[t] = mx;
-        }
-        c->tc_nmx = d.mtiles;
-    }
     return CPM_OK;
 }
 
-cpm_status tc_recip_run(cpm_ctx* c, int m, int64_t ne, const float2* EX, const float2* EY, const float2* EZ,
-                        const float* Qv, const float2* qabs, void* part, void* w16, float* site_partial) {
+cpm_status tc_recip_scales(cpm_ctx* c, cudaStream_t st, int m, int64_t ne, const double* Q, float* qsum) {
+    k_qsum_abs<<<m, 1024, 0, st>>>(Q, ne, qsum);
+    CPM_LAUNCH(c, "k_qsum_abs");
+    return CPM_OK;
+}
+
+cpm_status tc_recip_sf(cpm_ctx* c, cudaStream_t st, const TcRecipDims& d, int m, const float2* tab, const float* qmax,
+                       const int* qlast, float* part) {
     const KTable& k = c->kt;
-    const TcRecipDims d = tc_recip_dims(c, m, ne);
-    cudaStream_t st = c->stream;
-    const int64_t n = c->n, ptot = (int64_t)m * ne;
+    const RowTable& t = c->rows;
+    CPM_CUDA(c, cudaFuncSetAttribute(k_tc_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, RF_SMEM));
+    k_tc_rows<<<(unsigned)(t.tcitems * (int64_t)m * d.splits), RF_THREADS, RF_SMEM, st>>>(
+        t.tcitem, t.tcrange, t.pairs, tab, (int64_t)m * d.nep, d.nep, k.NX, k.NY, k.NZ, qmax, qlast, t.tcitems, d.splits,
+        d.spc, m, t.np, d.cw, part, c->status, RT_WAIT_NS);
+    CPM_LAUNCH(c, "k_tc_rows");
+    return CPM_OK;
+}
+
+cpm_status tc_recip_sites(cpm_ctx* c, cudaStream_t st, const TcRecipDims& d, int m, const float2* wrho,
+                          const float* qsum, void* w16, float* site_partial) {
+    const KTable& k = c->kt;
+    const int64_t n = c->n;
     if (!c->tcz || !c->tcxy) return set_err(c, CPM_E_STATE, "tensor-core reciprocal operands not prepared");
-
-    prof_begin(c, CPM_K_SF);
-    CPM_CUDA(c, cudaFuncSetAttribute(k_tc_sf, cudaFuncAttributeMaxDynamicSharedMemorySize, RF_SMEM));
-    TileMx tmx;
-    tmx.n = c->tc_nmx;
-    for (int t = 0; t < 32; ++t) tmx.mx[t] = c->tc_mx[t];
-    k_tc_sf<<<dim3(d.mtiles, d.ntiles, m * d.splits), RF_THREADS, RF_SMEM, st>>>(
-        k.cols, k.colext, k.ncols, k.NX, k.NY, k.NZ, k.nzw, EX, EY, EZ, Qv, qabs, ptot, ne, d.splits, d.chunk, m, d.cpad,
-        tmx, (float2*)part, c->status, RT_WAIT_NS);
-    prof_end(c, CPM_K_SF);
-    CPM_LAUNCH(c, "k_tc_sf");
-
-    prof_begin(c, CPM_K_SFRED);
     const int64_t plane_words = (int64_t)d.ngroups * d.NB * (d.KZ / 2);
-    if (d.NB != 2 * d.CT * d.mr) CPM_CUDA(c, cudaMemsetAsync(w16, 0, tc_recip_w16_bytes(d), st));
     dim3 gw((unsigned)((d.KZ / 2 + 31) / 32), (unsigned)((d.ncb * d.CT + 31) / 32), (unsigned)(d.nrb * d.mr));
-    k_tc_wsplit<<<gw, 1024, 0, st>>>((const float2*)part, d.splits, m, d.cpad, k.nzw, k.NZ, k.colext, k.w32, k.ncols,
-                                    qabs, c->tc_wmax, d.CT, d.mr, d.ncb, d.NB, d.KZ, (uint32_t*)w16, plane_words);
-    prof_end(c, CPM_K_SFRED);
+    k_tc_wsplit<<<gw, 1024, 0, st>>>(wrho, m, k.nzw, k.ncols, qsum, c->tc_wmax, d.CT, d.mr, d.ncb, d.NB, d.KZ,
+                                     (uint32_t*)w16, plane_words);
     CPM_LAUNCH(c, "k_tc_wsplit");
-
-    prof_begin(c, CPM_K_SITE);
     SiteMaps maps;
     const uint16_t* za = (const uint16_t*)c->tcz;
     const uint16_t* wb = (const uint16_t*)w16;
@@ -757,9 +682,8 @@ cpm_status tc_recip_run(cpm_ctx* c, int m, int64_t ne, const float2* EX, const f
     CPM_CUDA(c, cudaFuncSetAttribute(k_tc_site, cudaFuncAttributeMaxDynamicSharedMemorySize, RS_SMEM));
     const int ntx = (int)(d.npad / RS_BM), ntiles = ntx * d.ngroups;
     k_tc_site<<<(unsigned)std::min(ntiles, 152), RS_THREADS, RS_SMEM, st>>>(
-        maps, k.colext, k.ncols, k.NZ, d.mr, d.ncb, d.NB, m, ntx, ntiles, c->tcxy, n, qabs, c->tc_wmax, site_partial,
+        maps, k.colext, k.ncols, k.NZ, d.mr, d.ncb, d.NB, m, ntx, ntiles, c->tcxy, n, qsum, c->tc_wmax, site_partial,
         c->status, RT_WAIT_NS);
-    prof_end(c, CPM_K_SITE);
     CPM_LAUNCH(c, "k_tc_site");
     return CPM_OK;
 }
