@@ -180,10 +180,10 @@ __global__ void k_scatter(const int* key, const int* start, int* cursor, int64_t
 
 // One warp per cell: every charge's rank in the cell is the number of the cell's charges with a
 // smaller input index, so the sorted order (and every sum over a cell) is the same on every
-// call, whatever order the atomic scatter produced.
+// call, whatever order the atomic scatter produced.  sorted32 (FP64): the same charges in single precision too.
 template <typename T>
 __global__ void k_cellsort(const int* start, int ncells_total, const int* order, const typename V4<T>::t* wpos,
-                           typename V4<T>::t* sorted) {
+                           typename V4<T>::t* sorted, float4* sorted32) {
     const int c = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     const int lane = threadIdx.x & 31;
     if (c >= ncells_total) return;
@@ -192,7 +192,9 @@ __global__ void k_cellsort(const int* start, int ncells_total, const int* order,
         const int v = order[i];
         int rank = 0;
         for (int j = b; j < e; ++j) rank += order[j] < v ? 1 : 0;
-        sorted[b + rank] = wpos[v];
+        const typename V4<T>::t p = wpos[v];
+        sorted[b + rank] = p;
+        if (sorted32) sorted32[b + rank] = make_float4((float)p.x, (float)p.y, (float)p.z, (float)p.w);
     }
 }
 
@@ -1046,8 +1048,8 @@ struct BvecPlan {
         off_ewT, off_pm, off_p3m, total;
     int c0chunks;
     bool p3m;                           // reciprocal part of b by P3M (p3m.cu)
-    bool tc;
-    size_t off_qmax, off_spart;
+    bool tc, real64;
+    size_t off_sorted32, off_qmax, off_spart;
 };
 
 template <typename T>
@@ -1101,6 +1103,8 @@ static BvecPlan<T> plan_bvec(const cpm_ctx* c, int m, int64_t ne) {
     p.off_wpos = o; o += al(sizeof(typename V4<T>::t) * ptot);
     p.off_sorted = o; o += al(sizeof(typename V4<T>::t) * ptot);
     p.off_order = o; o += al(sizeof(int) * ptot);
+    p.real64 = std::is_same<T, double>::value && c->r64n > 0;
+    p.off_sorted32 = o; o += p.real64 ? al(sizeof(float4) * ptot) : 0;
     p.c0chunks = (int)std::max<int64_t>(1, (ne + C0_THREADS - 1) / C0_THREADS);
     const int nz0 = std::max(std::min(k.ext0, COL0_NZ), 1);
     p.off_c0part = o; o += al(sizeof(double2) * (size_t)m * p.c0chunks * nz0);
@@ -1150,6 +1154,7 @@ cpm_status bvec_run(cpm_ctx* c, int m, int64_t ne, const double* xyz, const doub
     V4T* wpos = (V4T*)(scr + p.off_wpos);
     V4T* sorted = (V4T*)(scr + p.off_sorted);
     int* order = (int*)(scr + p.off_order);
+    float4* sorted32 = (float4*)(scr + p.off_sorted32);
     float* qmax = (float*)(scr + p.off_qmax);     // per replica: max |Q|, index past the last nonzero charge, sum |Q|
     int* qlast = (int*)(qmax + m);
     float* qsum = (float*)(qlast + m);
@@ -1259,13 +1264,16 @@ cpm_status bvec_run(cpm_ctx* c, int m, int64_t ne, const double* xyz, const doub
     if (ptot > 0) {
         k_scatter<<<(unsigned)((ptot + 255) / 256), 256, 0, st>>>(key, start, cur, ptot, order);
         CPM_LAUNCH(c, "k_scatter");
-        k_cellsort<T><<<(unsigned)(((int64_t)nc * 32 + 255) / 256), 256, 0, st>>>(start, nc, order, wpos, sorted);
+        k_cellsort<T><<<(unsigned)(((int64_t)nc * 32 + 255) / 256), 256, 0, st>>>(start, nc, order, wpos, sorted,
+                                                                                  p.real64 ? sorted32 : nullptr);
         CPM_LAUNCH(c, "k_cellsort");
     }
     prof_end(c, CPM_K_CELLS);
     prof_begin(c, CPM_K_REAL);
     if (std::is_same<T, float>::value && c->rpoly.deg) {
         CPM_TRY(real_poly_run(c, st, m, p.cg, start, (const float4*)sorted, real));
+    } else if (p.real64) {
+        CPM_TRY(real64_run(c, st, m, p.cg, start, sorted, sorted32, real));
     } else if (std::is_same<T, float>::value && c->rtab && c->schunks) {
         const int4* ch4 = (const int4*)c->schunks;
         const float4* tab4 = (const float4*)c->rtab;

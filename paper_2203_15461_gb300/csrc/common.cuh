@@ -149,6 +149,8 @@ struct RowTable {
     float2* zu32 = nullptr;
     int* lperm = nullptr;                // [n] sites by height
     int4* ltiles = nullptr;              // [ntiles] (height, first, count, 0)
+    int4* atiles = nullptr;              // the same in tiles of at most 64 sites (elastance assembly)
+    std::vector<int4> hatiles;
     int tcitems = 0;                     // work items of the tensor-core structure factor, 0: it does not fit
     int4* tcitem = nullptr;              // (first pair, pairs, harmonic tile, harmonics of the tile)
     int4* tcrange = nullptr;             // (first nx, count, first ny, count) of the item's pairs
@@ -246,6 +248,8 @@ struct cpm_ctx {
                                  // the last (cell indices within one replica's cell list)
     float4* rrun_sh = nullptr;   // the image shift of each run
     int rrun_stride = 0;         // run slots per chunk
+    double* r64tab = nullptr;    // FP64 pair function in r^2: [widths][r64n intervals][coefficients, centre]
+    int r64n = 0, r64e0 = 0;     // intervals, exponent of the end of the first
     cpm::RealPoly rpoly{};       // fitted pair function of the gathered real-space kernel
     int rpoly_blocks = 0;        // its persistent grid (resident blocks per SM x SMs)
     cpm::KTable kt;
@@ -466,6 +470,11 @@ RealPoly fit_real_poly(double alpha, double rcut, double rlo);
 cpm_status build_real_poly(cpm_ctx* c, const std::vector<double>& etas);
 cpm_status real_poly_run(cpm_ctx* c, cudaStream_t st, int m, const CellGrid& cg, const int* start,
                          const float4* sorted, double* out);
+
+// real64.cu: the FP64 real-space sum (r64n = 0: the geometry keeps k_real_b)
+cpm_status build_real64(cpm_ctx* c, const std::vector<double>& etas);
+cpm_status real64_run(cpm_ctx* c, cudaStream_t st, int m, const CellGrid& cg, const int* start, const void* sorted,
+                      const float4* sorted32, double* out);
 
 // update.cu
 // bhl_ready: the split of b is already in update_bhl(c, m) (written by bvec in the same step)

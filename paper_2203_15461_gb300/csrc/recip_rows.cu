@@ -67,7 +67,7 @@ __global__ void k_layer_phases(const double* __restrict__ zu, int nzu, double iz
 void free_rows(cpm_ctx* c) {
     RowTable& t = c->rows;
     for (void* p : {(void*)t.pairs, (void*)t.list, (void*)t.W, (void*)t.W32, (void*)t.nxoff, (void*)t.chunkb,
-                    (void*)t.zu64, (void*)t.zu32, (void*)t.lperm, (void*)t.ltiles, (void*)t.colpair, (void*)t.tcitem,
+                    (void*)t.zu64, (void*)t.zu32, (void*)t.lperm, (void*)t.ltiles, (void*)t.colpair, (void*)t.tcitem, (void*)t.atiles,
                     (void*)t.tcrange})
         dev_free(c, p);
     t = RowTable{};
@@ -185,6 +185,9 @@ cpm_status build_rows(cpm_ctx* c) {
             for (int f = cnt[u]; f < cnt[u + 1]; f += ROW_TILE)
                 tiles.push_back(make_int4(u, f, std::min(ROW_TILE, cnt[u + 1] - f), 0));
         t.ntiles = (int)tiles.size();
+        for (int u = 0; u < c->nzu; ++u)
+            for (int f = cnt[u]; f < cnt[u + 1]; f += 64) t.hatiles.push_back(make_int4(u, f, std::min(64, cnt[u + 1] - f), 0));
+        CPM_TRY(upload(c, &t.atiles, t.hatiles));
         CPM_TRY(upload(c, &t.lperm, perm));
         CPM_TRY(upload(c, &t.ltiles, tiles));
         CPM_CUDA(c, cudaStreamSynchronize(c->stream));
@@ -331,6 +334,7 @@ __global__ void __launch_bounds__(RW_THREADS) k_rows_sf(const int4* __restrict__
     __syncthreads();
     if (cb > 2 * s_mx + 1) return;   // no row of the tile reaches these harmonics (block-uniform)
     const int tx = threadIdx.x & 7, ty = threadIdx.x >> 3;
+    const int qn = min(TN, (2 * (s_mx + 1) - cb + 7) / 8);   // groups of eight functions inside the ball
     T acc[TM][TN];
 #pragma unroll
     for (int p = 0; p < TM; ++p)
@@ -369,9 +373,12 @@ __global__ void __launch_bounds__(RW_THREADS) k_rows_sf(const int4* __restrict__
 #pragma unroll
             for (int q = 0; q < TN; ++q) b[q] = Zs[q0][tx + 8 * q];
 #pragma unroll
-            for (int p = 0; p < TM; ++p)
+            for (int q = 0; q < TN; ++q) {
+                // FP64: the eight functions past the tile's extent cost more than the test
+                if (std::is_same<T, double>::value && q >= qn) break;
 #pragma unroll
-                for (int q = 0; q < TN; ++q) acc[p][q] = fma(a[p], b[q], acc[p][q]);
+                for (int p = 0; p < TM; ++p) acc[p][q] = fma(a[p], b[q], acc[p][q]);
+            }
         }
         __syncthreads();
     }

@@ -20,11 +20,7 @@ constexpr int GT_COLS = 128;   // outputs (threads) per block
 constexpr int GT_JT = 64;      // rows of S staged per iteration
 constexpr int GT_MR = 8;       // replicas per block
 
-template <typename TS> struct LaneSum {
-    TS s = 0;
-    __device__ __forceinline__ void add(TS x) { s += x; }
-    __device__ __forceinline__ double value() const { return (double)s; }
-};
+template <typename TS> struct LaneSum;
 template <> struct LaneSum<float> {
     float s = 0.f, c = 0.f;
     __device__ __forceinline__ void add(float x) {
@@ -45,66 +41,70 @@ __global__ void k_split_b(const double* __restrict__ b, int64_t cnt, float2* __r
     bhl[t] = make_float2(hi, (float)(v - (double)hi));
 }
 
-template <typename TS> struct BVal;
-template <> struct BVal<float> { using t = float2; };
-template <> struct BVal<double> { using t = double; };
-
-__device__ __forceinline__ float centred(float2 bj, float2 bi) { return (bj.x - bi.x) + (bj.y - bi.y); }
-__device__ __forceinline__ double centred(double bj, double) { return bj; }
-
-// part[split][r][i] = sum over this split's rows j of S_ji x_j (x_j = b_j - b_i in FP32, b_j in FP64)
-template <typename TS>
-__global__ void __launch_bounds__(GT_COLS) k_gemv_t(const TS* __restrict__ S, const typename BVal<TS>::t* __restrict__ bv,
-                                                     int64_t n, int m, int64_t jchunk, double* __restrict__ part) {
-    typedef typename BVal<TS>::t B;
-    __shared__ B bs[GT_MR][GT_JT];
-    const int64_t i = (int64_t)blockIdx.x * GT_COLS + threadIdx.x;
-    const int split = blockIdx.y;
-    const int r0 = blockIdx.z * GT_MR;
-    const int mm = min(GT_MR, m - r0);
+// FP64: part[split][r][i] = sum over this split's rows j of S_ji b_j for MR replicas, two columns per thread
+// (16-byte loads, n even) or one, sixteen rows of S in flight.  Compiled for the replica count: tested per
+// element instead, one replica of 4,320 sites took 299 us where S streams from HBM in 22 and the FP64 pipe
+// needs 31.
+constexpr int G6_T = 128, G6_U = 16;
+template <int MR, int NC>
+__global__ void __launch_bounds__(G6_T) k_gemv64(const double* __restrict__ S, const double* __restrict__ bv, int64_t n,
+                                                 int m, int64_t jchunk, double* __restrict__ part) {
+    __shared__ double bs[GT_JT][MR];
+    const int64_t i0 = ((int64_t)blockIdx.x * G6_T + threadIdx.x) * NC;
+    const int split = blockIdx.y, r0 = blockIdx.z * MR;
     const int64_t jb = (int64_t)split * jchunk, je = min(n, jb + jchunk);
-    B bi[GT_MR];
-    LaneSum<TS> acc[GT_MR];
+    const bool live = i0 < n;
+    double acc[MR][NC];
 #pragma unroll
-    for (int t = 0; t < GT_MR; ++t) bi[t] = (t < mm && i < n) ? bv[(int64_t)(r0 + t) * n + i] : B{};
+    for (int t = 0; t < MR; ++t)
+#pragma unroll
+        for (int c = 0; c < NC; ++c) acc[t][c] = 0.0;
+    auto row = [&](int64_t j, double* v) {
+        // volatile: all rows of the unrolled group are requested before the first is used
+        if (NC == 2)
+            asm volatile("ld.global.nc.v2.f64 {%0, %1}, [%2];" : "=d"(v[0]), "=d"(v[NC - 1]) : "l"(S + j * n + i0));
+        else
+            asm volatile("ld.global.nc.f64 %0, [%1];" : "=d"(v[0]) : "l"(S + j * n + i0));
+    };
     for (int64_t j0 = jb; j0 < je; j0 += GT_JT) {
-        for (int e = threadIdx.x; e < GT_MR * GT_JT; e += GT_COLS) {
-            int t = e / GT_JT, jj = e % GT_JT;
-            int64_t j = j0 + jj;
-            bs[t][jj] = (t < mm && j < je) ? bv[(int64_t)(r0 + t) * n + j] : B{};
-        }
-        __syncthreads();
         const int jn = (int)min((int64_t)GT_JT, je - j0);
-        if (i < n) {
-            // eight loads of S in flight before they are used
-            int jj = 0;
-            for (; jj + 8 <= jn; jj += 8) {
-                TS sv[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) sv[u] = S[(j0 + jj + u) * n + i];
-#pragma unroll
-                for (int u = 0; u < 8; ++u)
-#pragma unroll
-                    for (int t = 0; t < GT_MR; ++t)
-                        if (t < mm) acc[t].add(sv[u] * (TS)centred(bs[t][jj + u], bi[t]));
-            }
-            for (; jj < jn; ++jj) {
-                const TS sv = S[(j0 + jj) * n + i];
-#pragma unroll
-                for (int t = 0; t < GT_MR; ++t)
-                    if (t < mm) acc[t].add(sv * (TS)centred(bs[t][jj], bi[t]));
-            }
+        __syncthreads();
+        for (int e = threadIdx.x; e < MR * GT_JT; e += G6_T) {
+            const int t = e / GT_JT, jj = e % GT_JT;
+            bs[jj][t] = (r0 + t < m && jj < jn) ? bv[(int64_t)(r0 + t) * n + j0 + jj] : 0.0;
         }
         __syncthreads();
-    }
-    if (i < n) {
+        if (!live) continue;
+        int jj = 0;
+        for (; jj + G6_U <= jn; jj += G6_U) {
+            double v[G6_U][NC];
 #pragma unroll
-        for (int t = 0; t < GT_MR; ++t)
-            if (t < mm) part[((int64_t)split * m + r0 + t) * n + i] = acc[t].value();
+            for (int u = 0; u < G6_U; ++u) row(j0 + jj + u, v[u]);
+#pragma unroll
+            for (int u = 0; u < G6_U; ++u)
+#pragma unroll
+                for (int t = 0; t < MR; ++t)
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) acc[t][c] = fma(v[u][c], bs[jj + u][t], acc[t][c]);
+        }
+        for (; jj < jn; ++jj) {
+            double v[NC];
+            row(j0 + jj, v);
+#pragma unroll
+            for (int t = 0; t < MR; ++t)
+#pragma unroll
+                for (int c = 0; c < NC; ++c) acc[t][c] = fma(v[c], bs[jj][t], acc[t][c]);
+        }
     }
+    if (!live) return;
+#pragma unroll
+    for (int t = 0; t < MR; ++t)
+        if (r0 + t < m)
+#pragma unroll
+            for (int c = 0; c < NC; ++c) part[((int64_t)split * m + r0 + t) * n + i0 + c] = acc[t][c];
 }
 
-// Single-precision variant of k_gemv_t: the hi/lo pairs of b are staged jj-major in shared memory so
+// Single precision: the hi/lo pairs of b are staged jj-major in shared memory so
 // one 16-byte load serves two replicas, and eight loads of S are in flight before use.  Each tile
 // of GT_JT terms is summed plainly in FP32 as S_ij (hi_j - hi_i) + S_ij lo_j (the hi difference
 // is exact; centring the tiny lo part would change nothing), and the tile sums are added with
@@ -474,18 +474,24 @@ static cpm_status launch_neutral(cpm_ctx* c, int m, double* q, double* qtot, boo
 
 // split count and row chunk of the centred product; grows the scratch when needed
 static bool gemv_pairs(const cpm_ctx* c) { return c->p.s_prec == CPM_PREC_FP32 && c->n % 2 == 0; }
+static bool gemv_fp64(const cpm_ctx* c) { return c->p.s_prec == CPM_PREC_FP64; }
+static int gemv64_mr(int m) { return m >= 5 ? 8 : m >= 3 ? 4 : m; }
 static int64_t gemv_colblocks(const cpm_ctx* c) {
+    if (gemv_fp64(c)) return c->n % 2 == 0 ? (c->n + 2 * G6_T - 1) / (2 * G6_T) : (c->n + G6_T - 1) / G6_T;
     return gemv_pairs(c) ? (c->n + 2 * G2_T - 1) / (2 * G2_T) : (c->n + GT_COLS - 1) / GT_COLS;
 }
 
 static cpm_status reserve_update_plan(cpm_ctx* c, int m, int64_t* splits_out, int64_t* jchunk_out) {
     const int64_t n = c->n;
     const int64_t colblocks = gemv_colblocks(c);
-    const int rchunks = (m + GT_MR - 1) / GT_MR;
+    const int mr = gemv_fp64(c) ? gemv64_mr(m) : GT_MR;
+    const int rchunks = (m + mr - 1) / mr;
     const int64_t want = gemv_pairs(c) ? 2 * 152 : 4 * 152;   // resident blocks: about one wave
+    // rows per split in whole tiles; FP64 in steps of the rows in flight, so that a small S is not one long chain
+    const int64_t jt = gemv_fp64(c) ? G6_U : GT_JT;
     int64_t splits = (want + colblocks * rchunks - 1) / (colblocks * rchunks);
-    splits = std::max<int64_t>(1, std::min<int64_t>(splits, (n + GT_JT - 1) / GT_JT));
-    int64_t jchunk = (((n + splits - 1) / splits + GT_JT - 1) / GT_JT) * GT_JT;
+    splits = std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(splits, gemv_fp64(c) ? 64 : splits), (n + jt - 1) / jt));
+    int64_t jchunk = (((n + splits - 1) / splits + jt - 1) / jt) * jt;
     splits = (n + jchunk - 1) / jchunk;
     if (gemv_tma_supported(c)) {
         int64_t cb;
@@ -552,7 +558,19 @@ cpm_status update(cpm_ctx* c, int m, const double* psi, const double* b, double*
         else k_gemv32<<<grid, GT_COLS, 0, st>>>(c->S32, bhl, n, m, jchunk, part);
     } else {
         prof_begin(c, CPM_K_GEMV);
-        k_gemv_t<double><<<grid, GT_COLS, 0, st>>>(c->S, b, n, m, jchunk, part);
+        const int mr = gemv64_mr(m);
+        dim3 g6((unsigned)colblocks, (unsigned)splits, (unsigned)((m + mr - 1) / mr));
+        if (n % 2 == 0) {
+            if (mr == 1) k_gemv64<1, 2><<<g6, G6_T, 0, st>>>(c->S, b, n, m, jchunk, part);
+            else if (mr == 2) k_gemv64<2, 2><<<g6, G6_T, 0, st>>>(c->S, b, n, m, jchunk, part);
+            else if (mr == 4) k_gemv64<4, 2><<<g6, G6_T, 0, st>>>(c->S, b, n, m, jchunk, part);
+            else k_gemv64<8, 2><<<g6, G6_T, 0, st>>>(c->S, b, n, m, jchunk, part);
+        } else {
+            if (mr == 1) k_gemv64<1, 1><<<g6, G6_T, 0, st>>>(c->S, b, n, m, jchunk, part);
+            else if (mr == 2) k_gemv64<2, 1><<<g6, G6_T, 0, st>>>(c->S, b, n, m, jchunk, part);
+            else if (mr == 4) k_gemv64<4, 1><<<g6, G6_T, 0, st>>>(c->S, b, n, m, jchunk, part);
+            else k_gemv64<8, 1><<<g6, G6_T, 0, st>>>(c->S, b, n, m, jchunk, part);
+        }
     }
     prof_end(c, CPM_K_GEMV);
     CPM_TRY(reserve_neutral(c, m));
