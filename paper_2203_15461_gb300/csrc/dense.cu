@@ -11,15 +11,18 @@ namespace cpm {
 // lower: skip tiles strictly above the diagonal of C.  tri & 1: op(A)[i][k] = 0 for k < i;
 // tri & 2: op(B)[k][j] = 0 for k < j (triangular operands; the K loop starts past the zeros).
 // status: when non-null and nonzero the kernel returns without touching C.
-constexpr int DG_BM = 64, DG_BK = 16;
+//
+// The FP64 pipe retires two multiply-adds per clock and SM, so a 64 x 64 tile with 4 x 4 accumulators per
+// thread is far from load-bound once the next K step is fetched while the current one is multiplied; what
+// matters is that every SM has a tile.
+constexpr int DG_BM = 64, DG_BK = 16, DG_T = 256;
 
+// one tile at (r0, c0), K range [kbeg, kend), kbeg a multiple of DG_BK
 template <bool TA, bool TB>
-__global__ void __launch_bounds__(256) k_dgemm(int M, int N, int K, double alpha, const double* A,
-                                               int64_t lda, const double* B, int64_t ldb, double beta,
-                                               double* C, int64_t ldc, int lower, int tri, const unsigned* status) {
-    if (status && *status) return;
-    const int r0 = blockIdx.y * DG_BM, c0 = blockIdx.x * DG_BM;
-    if (lower && c0 > r0 + DG_BM - 1) return;
+__device__ __forceinline__ void dgemm_tile(int r0, int c0, int M, int N, int K, int kbeg, int kend, double alpha,
+                                           const double* A, int64_t lda, const double* B, int64_t ldb, double beta,
+                                           double* C, int64_t ldc) {
+    constexpr int PER = DG_BK * DG_BM / DG_T;
     __shared__ double As[DG_BK][DG_BM + 1];
     __shared__ double Bs[DG_BK][DG_BM + 1];
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
@@ -28,27 +31,33 @@ __global__ void __launch_bounds__(256) k_dgemm(int M, int N, int K, double alpha
     for (int p = 0; p < 4; ++p)
 #pragma unroll
         for (int q = 0; q < 4; ++q) acc[p][q] = 0.0;
-    int kbeg = 0;
-    if (tri & 1) kbeg = max(kbeg, r0);
-    if (tri & 2) kbeg = max(kbeg, c0);
-    kbeg = (kbeg / DG_BK) * DG_BK;
-    for (int k0 = kbeg; k0 < K; k0 += DG_BK) {
-        for (int e = threadIdx.x; e < DG_BK * DG_BM; e += 256) {
+    kend = min(kend, K);
+    double va[PER], vb[PER];
+    auto fetch = [&](int k0) {
+#pragma unroll
+        for (int u = 0; u < PER; ++u) {
+            const int e = threadIdx.x + u * DG_T;
             int m, kk;
             if (TA) { m = e % DG_BM; kk = e / DG_BM; } else { kk = e % DG_BK; m = e / DG_BK; }
             int gi = r0 + m, gk = k0 + kk;
-            double v = 0.0;
-            if (gi < M && gk < K) v = TA ? A[(int64_t)gk * lda + gi] : A[(int64_t)gi * lda + gk];
-            As[kk][m] = v;
+            va[u] = (gi < M && gk < kend) ? (TA ? A[(int64_t)gk * lda + gi] : A[(int64_t)gi * lda + gk]) : 0.0;
             int nn;
             if (TB) { kk = e % DG_BK; nn = e / DG_BK; } else { nn = e % DG_BM; kk = e / DG_BM; }
             int gj = c0 + nn;
             gk = k0 + kk;
-            v = 0.0;
-            if (gj < N && gk < K) v = TB ? B[(int64_t)gj * ldb + gk] : B[(int64_t)gk * ldb + gj];
-            Bs[kk][nn] = v;
+            vb[u] = (gj < N && gk < kend) ? (TB ? B[(int64_t)gj * ldb + gk] : B[(int64_t)gk * ldb + gj]) : 0.0;
+        }
+    };
+    if (kbeg < kend) fetch(kbeg);
+    for (int k0 = kbeg; k0 < kend; k0 += DG_BK) {
+#pragma unroll
+        for (int u = 0; u < PER; ++u) {
+            const int e = threadIdx.x + u * DG_T;
+            if (TA) As[e / DG_BM][e % DG_BM] = va[u]; else As[e % DG_BK][e / DG_BK] = va[u];
+            if (TB) Bs[e % DG_BK][e / DG_BK] = vb[u]; else Bs[e / DG_BM][e % DG_BM] = vb[u];
         }
         __syncthreads();
+        if (k0 + DG_BK < kend) fetch(k0 + DG_BK);
 #pragma unroll
         for (int kk = 0; kk < DG_BK; ++kk) {
             double a[4], b[4];
@@ -77,15 +86,47 @@ __global__ void __launch_bounds__(256) k_dgemm(int M, int N, int K, double alpha
     }
 }
 
+template <bool TA, bool TB>
+__global__ void __launch_bounds__(DG_T) k_dgemm(int M, int N, int K, double alpha, const double* A,
+                                               int64_t lda, const double* B, int64_t ldb, double beta,
+                                               double* C, int64_t ldc, int lower, int tri, const unsigned* status) {
+    if (status && *status) return;
+    const int r0 = blockIdx.y * DG_BM, c0 = blockIdx.x * DG_BM;
+    if (lower && c0 > r0 + DG_BM - 1) return;
+    int kbeg = 0;
+    if (tri & 1) kbeg = max(kbeg, r0);
+    if (tri & 2) kbeg = max(kbeg, c0);
+    dgemm_tile<TA, TB>(r0, c0, M, N, K, (kbeg / DG_BK) * DG_BK, K, alpha, A, lda, B, ldb, beta, C, ldc);
+}
+
+// One level of the blocked inverse of a lower-triangular W whose diagonal blocks of size s are inverted:
+// for every pair of blocks (rows [r, r + s2) below columns [r - s, r), s2 the rows that exist),
+//   step 1: T = W_21 W_11,   step 2: W_21 <- -W_22 T      (W_11, W_22 lower triangular: K skips their zeros).
+// grid (s / 64, s / 64, pairs); T is an n x n scratch, used at the place of W_21.  Every level is two launches
+// over all pairs; block row by block row the inverse of 2,048 rows was 62 launches of at most 32 tiles each
+// (36 of the 62 ms of an inversion).
+__global__ void __launch_bounds__(DG_T) k_trinv_level(double* W, double* T, int64_t n, int s, int step,
+                                                      const unsigned* status) {
+    if (status && *status) return;
+    const int64_t c = (int64_t)blockIdx.z * 2 * s, r = c + s;
+    const int s2 = (int)min((int64_t)s, n - r);
+    const int r0 = blockIdx.y * DG_BM, c0 = blockIdx.x * DG_BM;
+    if (r0 >= s2) return;
+    double* W21 = W + r * n + c;
+    double* T21 = T + r * n + c;
+    if (step == 1) dgemm_tile<false, false>(r0, c0, s2, s, s, c0, s, 1.0, W21, n, W + c * n + c, n, 0.0, T21, n);
+    else dgemm_tile<false, false>(r0, c0, s2, s, s2, 0, r0 + DG_BM, -1.0, W + r * n + r, n, T21, n, 0.0, W21, n);
+}
+
 cpm_status launch_dgemm(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double alpha, const double* A,
                         int64_t lda, const double* B, int64_t ldb, double beta, double* C, int64_t ldc, int lower,
                         int tri, const unsigned* status) {
     if (M <= 0 || N <= 0) return CPM_OK;
     dim3 grid((N + DG_BM - 1) / DG_BM, (M + DG_BM - 1) / DG_BM);
-    if (ta && tb) k_dgemm<true, true><<<grid, 256, 0, s>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, lower, tri, status);
-    else if (ta) k_dgemm<true, false><<<grid, 256, 0, s>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, lower, tri, status);
-    else if (tb) k_dgemm<false, true><<<grid, 256, 0, s>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, lower, tri, status);
-    else k_dgemm<false, false><<<grid, 256, 0, s>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, lower, tri, status);
+    if (ta && tb) k_dgemm<true, true><<<grid, DG_T, 0, s>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, lower, tri, status);
+    else if (ta) k_dgemm<true, false><<<grid, DG_T, 0, s>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, lower, tri, status);
+    else if (tb) k_dgemm<false, true><<<grid, DG_T, 0, s>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, lower, tri, status);
+    else k_dgemm<false, false><<<grid, DG_T, 0, s>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, lower, tri, status);
     return cudaGetLastError() == cudaSuccess ? CPM_OK : CPM_E_CUDA;
 }
 
@@ -95,30 +136,47 @@ constexpr int NB = 64;
 // Unblocked Cholesky of one kb x kb diagonal block (in place, lower), and the inverse of
 // its factor written to Linv (NB x NB, zero above the diagonal).  A pivot that is not
 // positive and finite sets ST_NOT_SPD and stops the factorisation.
-__global__ void __launch_bounds__(256) k_potrf(double* Ab, int64_t lda, int kb, double* Linv, unsigned* status) {
+// One pass eliminates both: after column j, row i > j gets its rank-one update of the trailing columns
+// k = j + 1 .. i and of the inverse's columns c = 0 .. j, i + 1 terms over sixteen threads per row.  The inverse shares
+// the array: its entry (i, c) sits at [c][i + 1].  About 30 us, near what one SM's FP64 pipe needs for 64^3 / 3
+// multiply-adds; with the inverse as 64 serial columns after the factor it took 250.
+constexpr int PF_T = 1024, PF_L = PF_T / NB;
+__global__ void __launch_bounds__(PF_T) k_potrf(double* Ab, int64_t lda, int kb, double* Linv, unsigned* status) {
     if (*status) return;
-    __shared__ double L[NB][NB + 1];
+    __shared__ double L[NB][NB + 3];
     __shared__ int bad;
-    for (int e = threadIdx.x; e < NB * NB; e += blockDim.x) {
-        int i = e / NB, j = e % NB;
-        L[i][j] = (i < kb && j <= i) ? Ab[(int64_t)i * lda + j] : 0.0;
+    for (int e = threadIdx.x; e < NB * NB; e += PF_T) {
+        const int i = e / NB, j = e % NB;
+        if (j <= i) {
+            L[i][j] = i < kb ? Ab[(int64_t)i * lda + j] : (i == j ? 1.0 : 0.0);
+            L[j][i + 1] = 0.0;   // minus the sum over k of L_ik Linv_kj so far
+        }
     }
     if (threadIdx.x == 0) bad = 0;
     __syncthreads();
-    for (int j = 0; j < kb; ++j) {
-        if (threadIdx.x == 0) {
-            double pv = L[j][j];
-            if (!(pv > 0.0) || !isfinite(pv)) bad = 1;
-            else L[j][j] = sqrt(pv);
+    const int i = threadIdx.x / PF_L, q = threadIdx.x % PF_L;
+    for (int j = 0; j < NB; ++j) {
+        const double pv = L[j][j];
+        if (threadIdx.x == 0 && (!(pv > 0.0) || !isfinite(pv))) bad = 1;
+        __syncthreads();   // every thread has read the pivot
+        if (bad) break;
+        const double piv = sqrt(pv);
+        if ((int)threadIdx.x < NB) {   // column j of the factor, row j of the inverse
+            const int t = threadIdx.x;
+            if (t > j) L[t][j] /= piv;
+            else if (t == j) L[j][j] = piv;
+        } else if ((int)threadIdx.x < 2 * NB) {
+            const int t = threadIdx.x - NB;
+            if (t < j) L[t][j + 1] /= piv;
+            else if (t == j) L[j][j + 1] = 1.0 / piv;
         }
         __syncthreads();
-        if (bad) break;
-        for (int i = j + 1 + threadIdx.x; i < kb; i += blockDim.x) L[i][j] /= L[j][j];
-        __syncthreads();
-        const int rem = kb - j - 1;
-        for (int e = threadIdx.x; e < rem * rem; e += blockDim.x) {
-            int i = j + 1 + e / rem, k = j + 1 + e % rem;
-            if (k <= i) L[i][k] -= L[i][j] * L[k][j];
+        if (i > j) {
+            const double lij = L[i][j];
+            for (int c = q; c <= i; c += PF_L) {
+                if (c > j) L[i][c] = fma(-lij, L[c][j], L[i][c]);
+                else L[c][i + 1] = fma(-lij, L[c][j + 1], L[c][i + 1]);
+            }
         }
         __syncthreads();
     }
@@ -126,35 +184,27 @@ __global__ void __launch_bounds__(256) k_potrf(double* Ab, int64_t lda, int kb, 
         if (threadIdx.x == 0) atomicOr(status, ST_NOT_SPD);
         return;
     }
-    for (int e = threadIdx.x; e < kb * kb; e += blockDim.x) {
-        int i = e / kb, j = e % kb;
-        Ab[(int64_t)i * lda + j] = j <= i ? L[i][j] : 0.0;
+    for (int e = threadIdx.x; e < kb * kb; e += PF_T) {
+        const int r = e / kb, j = e % kb;
+        Ab[(int64_t)r * lda + j] = j <= r ? L[r][j] : 0.0;
     }
-    // inverse of the lower-triangular factor, one column per thread
-    for (int col = threadIdx.x; col < NB; col += blockDim.x) {
-        for (int i = 0; i < NB; ++i) {
-            double x = 0.0;
-            if (col < kb && i < kb && i >= col) {
-                if (i == col) x = 1.0 / L[i][i];
-                else {
-                    double s = 0.0;
-                    for (int k = col; k < i; ++k) s += L[i][k] * Linv[k * NB + col];
-                    x = -s / L[i][i];
-                }
-            }
-            Linv[i * NB + col] = x;
-        }
+    for (int e = threadIdx.x; e < NB * NB; e += PF_T) {
+        const int r = e / NB, j = e % NB;
+        Linv[e] = (j <= r && r < kb) ? L[j][r + 1] : 0.0;
     }
 }
 
-// Inverse of a kb x kb lower-triangular diagonal block, in place (the factor is staged in
-// shared memory; each thread writes one column of the inverse straight to the block).
-__global__ void __launch_bounds__(64) k_trtri(double* Ab, int64_t lda, int kb, const unsigned* status) {
+// Inverse of every NB x NB lower-triangular diagonal block of an n x n factor, in place (the factor is staged in
+// shared memory; each thread writes one column of the inverse straight to the block); one CTA per block.
+__global__ void __launch_bounds__(64) k_trtri(double* W, int64_t n, const unsigned* status) {
     if (*status) return;
     __shared__ double L[NB][NB + 1];
+    const int64_t k0 = (int64_t)blockIdx.x * NB;
+    const int kb = (int)min((int64_t)NB, n - k0);
+    double* Ab = W + k0 * n + k0;
     for (int e = threadIdx.x; e < NB * NB; e += blockDim.x) {
         int i = e / NB, j = e % NB;
-        L[i][j] = (i < kb && j <= i) ? Ab[(int64_t)i * lda + j] : 0.0;
+        L[i][j] = (i < kb && j <= i) ? Ab[(int64_t)i * n + j] : 0.0;
     }
     __syncthreads();
     const int col = threadIdx.x;
@@ -164,10 +214,10 @@ __global__ void __launch_bounds__(64) k_trtri(double* Ab, int64_t lda, int kb, c
             if (i == col) x = 1.0 / L[i][i];
             else if (i > col) {
                 double s = 0.0;
-                for (int k = col; k < i; ++k) s += L[i][k] * Ab[(int64_t)k * lda + col];
+                for (int k = col; k < i; ++k) s += L[i][k] * Ab[(int64_t)k * n + col];
                 x = -s / L[i][i];
             }
-            Ab[(int64_t)i * lda + col] = x;
+            Ab[(int64_t)i * n + col] = x;
         }
     }
 }
@@ -250,7 +300,7 @@ cpm_status invert_and_project(cpm_ctx* c) {
     // blocked right-looking Cholesky, lower triangle
     for (int64_t k0 = 0; k0 < n; k0 += NB) {
         const int kb = (int)std::min<int64_t>(NB, n - k0);
-        k_potrf<<<1, 256, 0, st>>>(W + k0 * n + k0, n, kb, Linv, c->status);
+        k_potrf<<<1, PF_T, 0, st>>>(W + k0 * n + k0, n, kb, Linv, c->status);
         CPM_LAUNCH(c, "k_potrf");
         const int rows = (int)(n - k0 - kb);
         if (rows > 0) {
@@ -266,18 +316,14 @@ cpm_status invert_and_project(cpm_ctx* c) {
     CPM_CUDA(c, cudaMemcpyAsync(&hst, c->status, sizeof(unsigned), cudaMemcpyDeviceToHost, st));
     CPM_CUDA(c, cudaStreamSynchronize(st));
     if (hst & ST_NOT_SPD) return set_err(c, CPM_E_NOT_SPD, "elastance matrix is not positive definite");
-    // W <- L^-1, block row by block row; R is an NB x n scratch held in S
-    double* R = c->S;
-    for (int64_t i0 = 0; i0 < n; i0 += NB) {
-        const int kb = (int)std::min<int64_t>(NB, n - i0);
-        k_trtri<<<1, 64, 0, st>>>(W + i0 * n + i0, n, kb, c->status);
-        CPM_LAUNCH(c, "k_trtri");
-        if (i0 > 0) {
-            CPM_TRY(launch_dgemm(st, false, false, kb, (int)i0, (int)i0, 1.0, W + i0 * n, n, W, n, 0.0, R, n, 0, 2,
-                                 c->status));
-            CPM_TRY(launch_dgemm(st, false, false, kb, (int)i0, kb, -1.0, W + i0 * n + i0, n, R, n, 0.0, W + i0 * n, n,
-                                 0, 0, c->status));
-        }
+    // W <- L^-1: the diagonal blocks, then pairs of blocks of doubling size, with S as scratch
+    k_trtri<<<(unsigned)((n + NB - 1) / NB), 64, 0, st>>>(W, n, c->status);
+    CPM_LAUNCH(c, "k_trtri");
+    for (int64_t s = NB; s < n; s *= 2) {
+        const dim3 gl((unsigned)(s / DG_BM), (unsigned)(s / DG_BM), (unsigned)((n - s + 2 * s - 1) / (2 * s)));
+        k_trinv_level<<<gl, DG_T, 0, st>>>(W, c->S, n, (int)s, 1, c->status);
+        k_trinv_level<<<gl, DG_T, 0, st>>>(W, c->S, n, (int)s, 2, c->status);
+        CPM_LAUNCH(c, "k_trinv_level");
     }
     // A^-1 = W^T W, lower tiles, then mirrored
     CPM_TRY(launch_dgemm(st, true, false, (int)n, (int)n, (int)n, 1.0, W, n, W, n, 0.0, c->S, n, 1, 3, c->status));
