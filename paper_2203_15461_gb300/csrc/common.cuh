@@ -86,6 +86,12 @@ struct PartSumF2 {
     }
     __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
 };
+struct PartSumF {   // single FP32 partials, the same two-sum
+    PartSumF2 s;
+    __device__ __forceinline__ void add(float x) { s.add(make_float2(x, 0.f)); }
+    __device__ __forceinline__ double value() const { return s.value(); }
+};
+
 // ----------------------------------------------------------------------------- device status word
 // Kernels never trap: they set one of these bits and return.  The host reads the
 // word when it synchronises.
@@ -238,16 +244,17 @@ struct cpm_ctx {
     int* rtab_id = nullptr;      // [n] table of each site
     int nrtab = 0;
     float* s32 = nullptr;        // [4 * n] wrapped single-precision x | y | z | eta
-    float4* rsite = nullptr;     // [nschunk * 32] sites of each chunk (x, y, z, r_eta^2), slots past the
+    float4* rsite = nullptr;     // [nrchunk * 32] sites of each chunk (x, y, z, r_eta^2), slots past the
                                  // chunk's count repeat its first site
-    int* rsite_tab = nullptr;    // [nschunk * 32] pair-table offset of each slot
-    int* rsite_idx = nullptr;    // [nschunk * 32] site index of each slot
-    float4* rbox = nullptr;      // [nschunk * 2] bounding box of each chunk's single-precision sites
-    int4* rchunk = nullptr;      // [nschunk] per chunk: first site in sperm, site count, run count
-    int2* rrun_cell = nullptr;   // [nschunk * rrun_stride] runs of each chunk: first cell and one past
+    int* rsite_tab = nullptr;    // [nrchunk * 32] pair-table offset of each slot
+    int* rsite_idx = nullptr;    // [nrchunk * 32] site index of each slot
+    float4* rbox = nullptr;      // [nrchunk * 2] bounding box of each chunk's single-precision sites
+    int4* rchunk = nullptr;      // [nrchunk] per chunk: first site in sperm, site count, run count
+    int2* rrun_cell = nullptr;   // [nrchunk * rrun_stride] runs of each chunk: first cell and one past
                                  // the last (cell indices within one replica's cell list)
     float4* rrun_sh = nullptr;   // the image shift of each run
     int rrun_stride = 0;         // run slots per chunk
+    int nrchunk = 0;             // its chunks (of up to 32 sites near one another)
     double* r64tab = nullptr;    // FP64 pair function in r^2: [widths][r64n intervals][coefficients, centre]
     int r64n = 0, r64e0 = 0;     // intervals, exponent of the end of the first
     cpm::RealPoly rpoly{};       // fitted pair function of the gathered real-space kernel
@@ -321,6 +328,7 @@ struct cpm_ctx {
     void* Sb = nullptr;          // S as three bf16 planes [3][n][ld] for the tensor-core update
     double* SZ = nullptr;        // [n][tc_ngrp] S times the centring-group indicators
     int tc_ngrp = 0;
+    int* tc_gperm = nullptr;     // [n] sites by centring group, then [tc_ngrp + 1] offsets
     bool tc_use_z = false;
     void* tbuf = nullptr;        // tensor-core update scratch (K-split partials, b planes)
     size_t tbuf_bytes = 0;
@@ -331,6 +339,9 @@ struct cpm_ctx {
     float tc_wmax = 0.f;         // bound on the k-space weights
     void* p3m_G = nullptr;       // P3M (kspace = CPM_KSPACE_P3M): influence function / V on the mesh (k_prec's T)
     void* p3m_tw = nullptr;      // its FFT twiddles exp(-2 pi i j / K), j < K / 2, for K = Kx, Ky, Kz
+    int* p3m_zlist = nullptr;    // mesh planes that the interpolation at the sites reads, and a mark per plane
+    unsigned char* p3m_need = nullptr;
+    int p3m_nz = 0;
     void* p3m_G64 = nullptr;     // the same in FP64 for the P3M elastance when k_prec is single precision
     void* p3m_tw64 = nullptr;
 
@@ -491,7 +502,7 @@ inline int upd_ng(const cpm_ctx* c) { return c->sg_over ? c->ng_over : c->ng; }
 void ccm_invalidate(cpm_ctx* c);
 
 // tc_gemm.cu
-cpm_status tc_update(cpm_ctx* c, int m, const double* psi, const double* b, double* q);
+cpm_status tc_product(cpm_ctx* c, int m, const double* b, const float** part, int* splits, const double** gmean);
 cpm_status tc_reserve(cpm_ctx* c, int m);
 cpm_status tc_selftest_timeout(cpm_ctx* c, double wait_ms);
 // tile plan of the tensor-core product for m replicas: BN, stages, splits, CTAs, candidates timed

@@ -206,25 +206,33 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_sb(const __grid_constant__
 }
 
 // ----------------------------------------------------------------------------- operand splits
-// x = x0 + x1 + x2 with bf16 terms: x0 = bf16(x), x1 = bf16(x - x0), x2 = bf16(x - x0 - x1).
-// With `gmean`, row r is first centred by its group means: x[r][c] - gmean[r][gid[c]].
+// x = x0 + x1 + x2 with bf16 terms: x0 = bf16(x), x1 = bf16(x - x0), x2 = bf16(x - x0 - x1), two columns per
+// thread.  With `gmean`, row r is first centred by its group means: x[r][c] - gmean[r][gid[c]].  The terms are
+// formed from x as an FP32 pair (48 bits): five FP64 instructions per value where three conversions and
+// differences in FP64 take nine of a pipe that retires two per clock and SM.
 __global__ void k_split3(const double* __restrict__ x, int64_t rows, int64_t cols, int64_t ld,
                          __nv_bfloat16* __restrict__ out, const double* __restrict__ gmean = nullptr,
                          const int* __restrict__ gid = nullptr, int ngrp = 0) {
-    int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= rows * ld) return;
-    const int64_t r = t / ld, c = t % ld;
-    double v = c < cols ? x[r * cols + c] : 0.0;
-    if (gmean && c < cols) v -= gmean[r * ngrp + gid[c]];
-    __nv_bfloat16 h0 = __double2bfloat16(v);
-    double r1 = v - (double)__bfloat162float(h0);
-    __nv_bfloat16 h1 = __double2bfloat16(r1);
-    double r2 = r1 - (double)__bfloat162float(h1);
-    __nv_bfloat16 h2 = __double2bfloat16(r2);
-    const int64_t plane = rows * ld;
-    out[t] = h0;
-    out[plane + t] = h1;
-    out[2 * plane + t] = h2;
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, half = ld / 2;
+    if (t >= rows * half) return;
+    const int64_t r = t / half, c = 2 * (t % half);
+    __nv_bfloat162 h[3];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        double v = c + k < cols ? x[r * cols + c + k] : 0.0;
+        if (gmean && c + k < cols) v -= gmean[r * ngrp + gid[c + k]];
+        const float vh = (float)v, vl = (float)(v - (double)vh);
+        const __nv_bfloat16 h0 = __float2bfloat16_rn(vh);
+        const float r1 = (vh - __bfloat162float(h0)) + vl;
+        const __nv_bfloat16 h1 = __float2bfloat16_rn(r1);
+        const __nv_bfloat16 h2 = __float2bfloat16_rn(r1 - __bfloat162float(h1));
+        if (k == 0) { h[0].x = h0; h[1].x = h1; h[2].x = h2; } else { h[0].y = h0; h[1].y = h1; h[2].y = h2; }
+    }
+    const int64_t plane = rows * half;
+    __nv_bfloat162* o = (__nv_bfloat162*)out + t;
+    o[0] = h[0];
+    o[plane] = h[1];
+    o[2 * plane] = h[2];
 }
 
 // ----------------------------------------------------------------------------- host side
@@ -236,7 +244,7 @@ cpm_status tc_prepare_s(cpm_ctx* c) {
     dev_free(c, c->Sb);
     c->Sb = nullptr;
     CPM_TRY(dev_alloc(c, (void**)&c->Sb, sizeof(__nv_bfloat16) * 3 * n * ld));
-    k_split3<<<(unsigned)((n * ld + 255) / 256), 256, 0, c->stream>>>(c->S, n, n, ld, (__nv_bfloat16*)c->Sb);
+    k_split3<<<(unsigned)((n * (ld / 2) + 255) / 256), 256, 0, c->stream>>>(c->S, n, n, ld, (__nv_bfloat16*)c->Sb);
     CPM_LAUNCH(c, "k_split3(S)");
     return CPM_OK;
 }
@@ -440,7 +448,7 @@ cpm_status tc_sb(cpm_ctx* c, int m, const double* b, float* part, int* splits, v
     const int64_t n = c->n, ld = tc_ld(n);
     TcPlan p;
     CPM_TRY(tc_plan_for(c, m, part, bsplit, &p));
-    k_split3<<<(unsigned)((m * ld + 255) / 256), 256, 0, c->stream>>>(b, m, n, ld, (__nv_bfloat16*)bsplit, gmean, gid,
+    k_split3<<<(unsigned)((m * (ld / 2) + 255) / 256), 256, 0, c->stream>>>(b, m, n, ld, (__nv_bfloat16*)bsplit, gmean, gid,
                                                                       ngrp);
     CPM_LAUNCH(c, "k_split3(b)");
     TcMaps maps;
@@ -468,38 +476,24 @@ __global__ void k_sgroups(const double* __restrict__ S, const int* __restrict__ 
     SZ[t] = a;
 }
 
-// gmean[r][g] = mean of b[r][i] over the sites of group g; one warp per (r, g), fixed order
-__global__ void k_gmeans(const double* __restrict__ b, const int* __restrict__ gid, int64_t n, int m, int ngrp,
-                         double* __restrict__ gmean) {
+// gmean[r][g] = mean of b[r][i] over the sites of group g (perm[off[g]] .. perm[off[g + 1] - 1]); one warp per
+// (r, g), four sums per lane in flight, fixed order
+__global__ void k_gmeans(const double* __restrict__ b, const int* __restrict__ perm, const int* __restrict__ off,
+                         int64_t n, int m, int ngrp, double* __restrict__ gmean) {
     const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (w >= (int64_t)m * ngrp) return;
     const int r = (int)(w / ngrp), g = (int)(w % ngrp);
-    double a = 0.0;
-    int cnt = 0;
-    for (int64_t i = lane; i < n; i += 32)
-        if (gid[i] == g) { a += b[(int64_t)r * n + i]; ++cnt; }
-    for (int o = 16; o > 0; o >>= 1) {
-        a += __shfl_down_sync(0xffffffffu, a, o);
-        cnt += __shfl_down_sync(0xffffffffu, cnt, o);
-    }
-    if (lane == 0) gmean[w] = cnt ? a / cnt : 0.0;
-}
-
-// q[r][i] = sum_g SG[i][g] psi[r][g] - sum_g' SZ[i][g'] gmean[r][g'] - sum_split part[split][r][i]
-__global__ void k_tc_reduce(const float* __restrict__ part, int splits, const double* __restrict__ SG, int ng,
-                            const double* __restrict__ psi, const double* __restrict__ SZ,
-                            const double* __restrict__ gmean, int ngrp, int64_t n, int m, double* __restrict__ q) {
-    int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= (int64_t)m * n) return;
-    const int r = (int)(t / n);
-    const int64_t i = t % n;
-    double v = 0.0;
-    for (int sp = 0; sp < splits; ++sp) v += (double)part[((int64_t)sp * m + r) * n + i];
-    for (int g = 0; g < ngrp; ++g) v += SZ[i * ngrp + g] * gmean[(int64_t)r * ngrp + g];
-    double sv = 0.0;
-    for (int g = 0; g < ng; ++g) sv += SG[i * ng + g] * psi[(int64_t)r * ng + g];
-    q[t] = sv - v;
+    const double* br = b + (int64_t)r * n;
+    const int k0 = off[g], k1 = off[g + 1];
+    double a[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int k = k0 + lane; k < k1; k += 128)
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (k + 32 * u < k1) a[u] += br[perm[k + 32 * u]];
+    double s = (a[0] + a[1]) + (a[2] + a[3]);
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (lane == 0) gmean[w] = k1 > k0 ? s / (k1 - k0) : 0.0;
 }
 
 cpm_status tc_reserve(cpm_ctx* c, int m) {
@@ -516,6 +510,20 @@ cpm_status tc_reserve(cpm_ctx* c, int m) {
         const int* gid = c->tc_use_z ? c->zmap : c->group;
         k_sgroups<<<(unsigned)((n * c->tc_ngrp + 255) / 256), 256, 0, c->stream>>>(c->S, gid, n, c->tc_ngrp, c->SZ);
         CPM_LAUNCH(c, "k_sgroups");
+        // the sites of every group, in index order
+        std::vector<int> gi(n), perm(n), off(c->tc_ngrp + 1, 0);
+        CPM_CUDA(c, cudaMemcpyAsync(gi.data(), gid, sizeof(int) * n, cudaMemcpyDeviceToHost, c->stream));
+        CPM_CUDA(c, cudaStreamSynchronize(c->stream));
+        for (int64_t i = 0; i < n; ++i) ++off[gi[i] + 1];
+        for (int g = 0; g < c->tc_ngrp; ++g) off[g + 1] += off[g];
+        std::vector<int> at(off.begin(), off.end() - 1);
+        for (int64_t i = 0; i < n; ++i) perm[at[gi[i]]++] = (int)i;
+        dev_free(c, c->tc_gperm);
+        c->tc_gperm = nullptr;
+        CPM_TRY(dev_alloc(c, (void**)&c->tc_gperm, sizeof(int) * (n + c->tc_ngrp + 1)));
+        CPM_CUDA(c, cudaMemcpyAsync(c->tc_gperm, perm.data(), sizeof(int) * n, cudaMemcpyHostToDevice, c->stream));
+        CPM_CUDA(c, cudaMemcpyAsync(c->tc_gperm + n, off.data(), sizeof(int) * off.size(), cudaMemcpyHostToDevice, c->stream));
+        CPM_CUDA(c, cudaStreamSynchronize(c->stream));
     }
     const size_t pb = std::max(tc_part_need(c->device, n, m), c->tc_pbytes);
     const size_t need = pb + ((tc_bsplit_bytes(n, m) + 255) & ~(size_t)255) + sizeof(double) * (size_t)m * c->tc_ngrp;
@@ -534,22 +542,21 @@ cpm_status tc_reserve(cpm_ctx* c, int m) {
     return tc_plan_for(c, m, (float*)c->tbuf, (char*)c->tbuf + c->tc_pbytes, &p);
 }
 
-cpm_status tc_update(cpm_ctx* c, int m, const double* psi, const double* b, double* q) {
+// the product alone: part[split][r][i] and the group means; the caller adds SZ gmean and reduces (update.cu)
+cpm_status tc_product(cpm_ctx* c, int m, const double* b, const float** part_out, int* splits, const double** gmean_out) {
     const int64_t n = c->n;
     CPM_TRY(tc_reserve(c, m));
     float* part = (float*)c->tbuf;
     void* bsplit = (char*)c->tbuf + c->tc_pbytes;
     double* gmean = (double*)((char*)bsplit + ((tc_bsplit_bytes(n, m) + 255) & ~(size_t)255));
     const int* gid = c->tc_use_z ? c->zmap : c->group;
-    k_gmeans<<<(unsigned)(((int64_t)m * c->tc_ngrp * 32 + 255) / 256), 256, 0, c->stream>>>(b, gid, n, m, c->tc_ngrp,
-                                                                                              gmean);
+    k_gmeans<<<(unsigned)(((int64_t)m * c->tc_ngrp * 32 + 127) / 128), 128, 0, c->stream>>>(b, c->tc_gperm, c->tc_gperm + n, n,
+                                                                                            m, c->tc_ngrp, gmean);
     CPM_LAUNCH(c, "k_gmeans");
-    int splits = 0;
-    CPM_TRY(tc_sb(c, m, b, part, &splits, bsplit, gmean, gid, c->tc_ngrp));
-    k_tc_reduce<<<(unsigned)((m * n + 255) / 256), 256, 0, c->stream>>>(part, splits, upd_sg(c), upd_ng(c), psi, c->SZ, gmean,
-                                                                        c->tc_ngrp, n, m, q);
-    CPM_LAUNCH(c, "k_tc_reduce");
-    c->launches += 4;
+    CPM_TRY(tc_sb(c, m, b, part, splits, bsplit, gmean, gid, c->tc_ngrp));
+    *part_out = part;
+    *gmean_out = gmean;
+    c->launches += 3;
     return CPM_OK;
 }
 

@@ -259,8 +259,10 @@ constexpr int NB_T = 256;
 template <typename P> struct PartSum;
 template <> struct PartSum<double> { using type = PartSumD; };
 template <> struct PartSum<float2> { using type = PartSumF2; };
+template <> struct PartSum<float> { using type = PartSumF; };   // partials of the tensor-core product
 
-// q = SG psi - sum of the split partials, then the neutrality fix of Sec. II.B in the last block of
+// q = SG psi - sum of the split partials (tensor-core product: - SZ gmean, the share of the group means taken out
+// of its operand), then the neutrality fix of Sec. II.B in the last block of
 // each replica: every block writes its slice of q and the slice's sum p1[r][b]; the replica's last
 // block (ticket) adds the p1 in block order, applies q <- q - u (e^T q) with symm, and writes
 // qtot[r] = e^T q of the result (plain FP64 sums in a fixed order: the rounding, about n eps max|q|,
@@ -272,7 +274,9 @@ __global__ void __launch_bounds__(NB_T) k_gemv_reduce(const P* __restrict__ part
                                                       double* __restrict__ q, double* __restrict__ p1,
                                                       const double* __restrict__ u, int symm,
                                                       int* __restrict__ tickets, double* __restrict__ qtot,
-                                                      const double* __restrict__ b, const double* __restrict__ srow) {
+                                                      const double* __restrict__ b, const double* __restrict__ srow,
+                                                      const double* __restrict__ SZ, const double* __restrict__ gmean,
+                                                      int ngrp) {
     __shared__ double sh[NB_T / 32];
     __shared__ double buf[NB_T];
     __shared__ double s_sum;
@@ -294,6 +298,7 @@ __global__ void __launch_bounds__(NB_T) k_gemv_reduce(const P* __restrict__ part
         }
         double sv = 0.0;
         for (int g = 0; g < ng; ++g) sv += SG[i * ng + g] * psi[(int64_t)r * ng + g];
+        for (int g = 0; g < ngrp; ++g) sv -= SZ[i * ngrp + g] * gmean[(int64_t)r * ngrp + g];
         // the centred products give sum_j S_ij (b_j - b_i): add b_i sum_j S_ij back where rows do not sum to zero
         qi = sv - (srow ? v.value() + b[(int64_t)r * n + i] * srow[i] : v.value());
         qr[i] = qi;
@@ -354,95 +359,11 @@ __global__ void __launch_bounds__(NB_T) k_gemv_reduce(const P* __restrict__ part
     if (threadIdx.x == 0 && qtot) qtot[r] = tot;
 }
 
-__device__ __forceinline__ void neumaier_add(double& a, double& comp, double v) {
-    const double t = a + v;
-    comp += fabs(a) >= fabs(v) ? (a - t) + v : (v - t) + a;
-    a = t;
-}
-
-// Neutrality fix and total charge, Sec. II.B (q <- q - u e^T q with u = A^-1 e / (e^T A^-1 e), then
-// the FP64 total): grid (slices of the sites, m); two passes because the fix needs the replica's
-// whole sum first (the first pass is k_qsum, or the GEMV reduction when it writes p1).
-
-// p1[r][b] = sum of q[r][i] over slice b
-__global__ void __launch_bounds__(NB_T) k_qsum(const double* __restrict__ q, int64_t n, double* __restrict__ p1) {
-    __shared__ double sh[NB_T / 32];
-    const int b = blockIdx.x, nb = gridDim.x, r = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t chunk = (n + nb - 1) / nb, ib = (int64_t)b * chunk, ie = min(n, ib + chunk);
-    double s = 0.0;
-    for (int64_t i = ib + threadIdx.x; i < ie; i += NB_T) s += q[(int64_t)r * n + i];
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if (lane == 0) sh[warp] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = sh[0];
-        for (int w = 1; w < NB_T / 32; ++w) t += sh[w];
-        p1[(int64_t)r * nb + b] = t;
-    }
-}
-
-// with symm: q[r][i] -= u[i] * sum_b p1[r][b] (np1 block sums); then p2[r][b] = sum of the new q over
-// slice b, and the replica's last block writes qtot[r] = sum of p2 in slice order (plain FP64 sums in
-// a fixed order: the rounding, about n eps max|q|, is far below the 1e-12 e the total is held to)
-__global__ void __launch_bounds__(NB_T) k_neutral_fix(double* __restrict__ q, const double* __restrict__ u, int64_t n,
-                                                      int symm, const double* __restrict__ p1, int np1,
-                                                      double* __restrict__ p2, int* __restrict__ tickets,
-                                                      double* __restrict__ qtot) {
-    __shared__ double sh[NB_T / 32];
-    __shared__ double buf[NB_T];
-    __shared__ double s_sum;
-    const int b = blockIdx.x, nb = gridDim.x, r = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t chunk = (n + nb - 1) / nb, ib = (int64_t)b * chunk, ie = min(n, ib + chunk);
-    double* qr = q + (int64_t)r * n;
-    double s = 0.0;
-    if (symm) {
-        // sum of the np1 block sums in order: loaded by all threads at once, added by thread 0
-        for (int k0 = 0; k0 < np1; k0 += NB_T) {
-            if (k0 + (int)threadIdx.x < np1) buf[threadIdx.x] = p1[(int64_t)r * np1 + k0 + threadIdx.x];
-            __syncthreads();
-            if (threadIdx.x == 0)
-                for (int k = 0; k < min(NB_T, np1 - k0); ++k) s += buf[k];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) s_sum = s;
-        __syncthreads();
-        s = s_sum;
-    }
-    double a = 0.0;
-    for (int64_t i = ib + threadIdx.x; i < ie; i += NB_T) {
-        double v = qr[i];
-        if (symm) {
-            v -= u[i] * s;
-            qr[i] = v;
-        }
-        a += v;
-    }
-    for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
-    if (lane == 0) sh[warp] = a;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = sh[0];
-        for (int w = 1; w < NB_T / 32; ++w) t += sh[w];
-        p2[(int64_t)r * nb + b] = t;
-    }
-    if (!last_block_of(&tickets[r], nb)) return;
-    if (!qtot) return;
-    const volatile double* pv = p2 + (int64_t)r * nb;
-    if ((int)threadIdx.x < nb) buf[threadIdx.x] = pv[threadIdx.x];   // nb <= 64 slices
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int k = 0; k < nb; ++k) t += buf[k];
-        qtot[r] = t;
-    }
-}
-
-static int neutral_blocks(int64_t n) { return (int)std::max<int64_t>(1, std::min<int64_t>(64, (n + 1023) / 1024)); }
 static int reduce_blocks(int64_t n) { return (int)((n + NB_T - 1) / NB_T); }
 
 static cpm_status reserve_neutral(cpm_ctx* c, int m) {
     CPM_TRY(ensure_tickets(c, m));
-    const size_t need = sizeof(double) * (size_t)m * (reduce_blocks(c->n) + neutral_blocks(c->n));
+    const size_t need = sizeof(double) * (size_t)m * reduce_blocks(c->n);
     if (c->nbuf_bytes >= need) return CPM_OK;
     c->graph_valid = false;
     dev_free(c, c->nbuf);
@@ -450,25 +371,6 @@ static cpm_status reserve_neutral(cpm_ctx* c, int m) {
     c->nbuf_bytes = 0;
     CPM_TRY(dev_alloc(c, (void**)&c->nbuf, need));
     c->nbuf_bytes = need;
-    return CPM_OK;
-}
-
-// have_p1: the block sums p1 were written by the GEMV reduction; else k_qsum writes them
-static cpm_status launch_neutral(cpm_ctx* c, int m, double* q, double* qtot, bool have_p1) {
-    CPM_TRY(reserve_neutral(c, m));
-    const int nb = neutral_blocks(c->n);
-    const int np1 = have_p1 ? reduce_blocks(c->n) : nb;
-    double* p1 = c->nbuf;
-    double* p2 = c->nbuf + (size_t)m * reduce_blocks(c->n);
-    prof_begin(c, CPM_K_NEUTRAL);
-    if (c->p.symm && !have_p1) {
-        k_qsum<<<dim3(nb, m), NB_T, 0, c->stream>>>(q, c->n, p1);
-        c->launches += 1;
-    }
-    k_neutral_fix<<<dim3(nb, m), NB_T, 0, c->stream>>>(q, c->u, c->n, c->p.symm, p1, np1, p2, c->tickets, qtot);
-    prof_end(c, CPM_K_NEUTRAL);
-    CPM_LAUNCH(c, "k_neutral_fix");
-    c->launches += 1;
     return CPM_OK;
 }
 
@@ -529,10 +431,21 @@ cpm_status update(cpm_ctx* c, int m, const double* psi, const double* b, double*
     const int64_t n = c->n;
     cudaStream_t st = c->stream;
     if (c->p.s_prec == CPM_PREC_BF16X3) {
+        const float* part = nullptr;
+        const double* gmean = nullptr;
+        int splits = 0;
         prof_begin(c, CPM_K_GEMV);
-        CPM_TRY(tc_update(c, m, psi, b, q));
+        CPM_TRY(tc_product(c, m, b, &part, &splits, &gmean));
         prof_end(c, CPM_K_GEMV);
-        return launch_neutral(c, m, q, qtot, false);
+        CPM_TRY(reserve_neutral(c, m));
+        prof_begin(c, CPM_K_NEUTRAL);
+        k_gemv_reduce<float><<<dim3((unsigned)reduce_blocks(n), m), NB_T, 0, st>>>(
+            part, splits, upd_sg(c), upd_ng(c), psi, n, m, q, c->nbuf, c->u, c->p.symm, c->tickets, qtot, b, nullptr, c->SZ,
+            gmean, c->tc_ngrp);
+        prof_end(c, CPM_K_NEUTRAL);
+        CPM_LAUNCH(c, "k_gemv_reduce");
+        c->launches += 1;
+        return CPM_OK;
     }
     const bool f32 = c->p.s_prec == CPM_PREC_FP32;
     int64_t splits = 0, jchunk = 0;
@@ -579,10 +492,10 @@ cpm_status update(cpm_ctx* c, int m, const double* psi, const double* b, double*
     const double* srow = (f32 && !c->p.symm) ? c->dvec : nullptr;
     if (f32 && gemv_tma_supported(c))
         k_gemv_reduce<float2><<<rgrid, NB_T, 0, st>>>((const float2*)part, (int)splits, upd_sg(c), upd_ng(c), psi, n, m, q,
-                                                      c->nbuf, c->u, c->p.symm, c->tickets, qtot, b, srow);
+                                                      c->nbuf, c->u, c->p.symm, c->tickets, qtot, b, srow, nullptr, nullptr, 0);
     else
         k_gemv_reduce<double><<<rgrid, NB_T, 0, st>>>(part, (int)splits, upd_sg(c), upd_ng(c), psi, n, m, q, c->nbuf, c->u,
-                                                      c->p.symm, c->tickets, qtot, b, srow);
+                                                      c->p.symm, c->tickets, qtot, b, srow, nullptr, nullptr, 0);
     prof_end(c, CPM_K_NEUTRAL);
     CPM_LAUNCH(c, "k_gemv");
     return CPM_OK;
