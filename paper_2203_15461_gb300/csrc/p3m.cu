@@ -15,12 +15,13 @@
 // * Two replicas share one complex mesh (real part, imaginary part).  G is real and even on the
 //   mesh, so IFFT(G FFT(rho_a + i rho_b)) = phi_a + i phi_b exactly: one complex transform serves
 //   two replicas.
-// * Charge assignment: one CTA per (mesh brick, replica pair) owns the brick's points in shared
+// * Charge assignment: one CTA per (mesh brick, replica) owns the brick's points in shared
 //   memory and takes every charge whose stencil reaches into the brick, adding only the points it
 //   owns.  Every mesh point is written by exactly one CTA, with a plain store: no halo exchange and
 //   no global atomics.  Inside the brick the contributions are added as exact fixed-point integers
 //   with 32-bit shared-memory atomics, so the mesh charge does not depend on the order of the
-//   atomics and the whole path is deterministic.
+//   atomics and the whole path is deterministic.  Bricks that no charge reaches are not written, only marked,
+//   and planes of such bricks are not transformed (an electrolyte fills a third of a slab cell).
 // * Transforms: radix-2 decimation in time in shared memory with twiddles tabulated in FP64 on the
 //   host.  The forward and inverse xy transforms take a whole plane per CTA; the z pass loads
 //   16 z lines per CTA, transforms them forward, multiplies by G, transforms back and stores, so
@@ -145,150 +146,169 @@ __device__ __forceinline__ void bspline_weights(T f, T* w) {
 }
 
 // ----------------------------------------------------------------------------- charge assignment
-// grid (bricks, replica pairs, charge splits); a brick is BX x BY x BZ mesh points (x fastest), brick
-// index bx fastest; split sp takes the chunks [sp cps, (sp + 1) cps) of NT charges of each replica.
+// grid (bricks, replicas, charge splits); a brick is BX x BY x BZ mesh points (x fastest), brick
+// index bx fastest; split sp takes the chunks [sp cps, (sp + 1) cps) of NT charges of the replica.
 // Those whose stencil reaches into the brick are compacted (warp ballots, then warp offsets) into
-// shared memory with their 3 p weights and their stencil origin relative to the brick; then the
-// chunk's (charge, z offset, y offset) items are spread over the threads, each adding its p x
-// contributions that land in the brick.
+// shared memory with their 3 p weights and their stencil origin relative to the brick; then a warp takes one charge
+// at a time, lane = (plane of the brick, y offset), each lane adding its p x contributions.
 // Every contribution is rounded to 2^-40 e (FP64: 2^-60 e) and added as exact integers split over
 // 32-bit words, a = floor(v 2^20), then the next 20 bits (FP64: and 20 more), with native 32-bit
 // shared-memory atomics; integer addition is associative, so the brick's charge does not depend on
-// the order of the atomics.  The low words carry into the next after every chunk (a chunk adds at
-// most 1,024 x 2^20 to a low word), and a wraps modulo 2^32, exact while the final charge of a mesh
-// point stays below 2,048 e.  Brick
-// rows are padded to BX + 1 words so that the x offsets of one charge fall in distinct banks.  The
-// split's brick goes to its own partial mesh; the first transform sums the splits in split order.
+// the order of the atomics.  The low words carry into the next at least every P3M_CARRY charges (each adds at
+// most 2^20 to a low word), and a wraps modulo 2^32, exact while the final charge of a mesh
+// point stays below 2,048 e.
+// Layout: with the whole y period and four planes in a brick, 28 of 32 lanes have a row for order 7 (all of them
+// in the brick but for its first and last planes); rows are padded to BX + 1 words and planes by 8, so the rows of
+// one charge fall in distinct banks.  Bricks of half a y period and eight planes with the rows spread over
+// threads left three of four lanes without work: 136 us for 8 EDL replicas.
+// The split's brick goes to its own partial mesh (part, real and imaginary part for even and odd replicas) if a
+// charge reached it (flag); the first transform sums the splits in split order.
 template <typename T> struct P3mWords { static constexpr int n = std::is_same<T, double>::value ? 3 : 2; };
-template <typename T> struct P3mSpreadThreads { static constexpr int n = std::is_same<T, double>::value ? 512 : 1024; };
+constexpr int P3M_NT = 512;          // threads and charges per chunk of the assignment
+constexpr int P3M_CARRY = 1024;
+constexpr int P3M_BZ = 4;            // planes per brick (lanes 8 z + y)
 
 template <typename T, int P>
-__global__ void __launch_bounds__(P3mSpreadThreads<T>::n) k_p3m_spread(const int* __restrict__ key,
-                                                                      const typename P3mV4<T>::t* __restrict__ fq,
-                                                                      int64_t ne, int m, int Kx, int Ky, int Kz, int BX,
-                                                                      int BY, int BZ, int cps,
-                                                                      c2<T>* __restrict__ part) {
-    constexpr int NW = P3mWords<T>::n;
-    constexpr int NT = P3mSpreadThreads<T>::n;
+__global__ void __launch_bounds__(P3M_NT) k_p3m_spread(const int* __restrict__ key,
+                                                       const typename P3mV4<T>::t* __restrict__ fq, int64_t ne, int m,
+                                                       int Kx, int Ky, int Kz, int BX, int BY, int cps,
+                                                       c2<T>* __restrict__ part, int* __restrict__ flag) {
+    constexpr int NW = P3mWords<T>::n, BZ = P3M_BZ;
     extern __shared__ __align__(16) unsigned char p3m_smem[];
-    const int RX = BX + 1;                              // padded row
-    const int NB = RX * BY * BZ;
-    int* acc = (int*)p3m_smem;                          // [2 replicas][NW words][NB]
-    T* sw = (T*)(acc + ((2 * NW * NB + 3) & ~3));       // [NT][3 p + 1]: weights x | y | z, then Q
-    int* so = (int*)(sw + NT * (3 * P + 1));            // [NT]: origin sx | sy << 10 | sz << 20
-    __shared__ int wcount[NT / 32];
+    const int RX = BX + 1, PS = BY * RX + 8;            // padded row and plane
+    const int NB = PS * BZ;
+    int* A = (int*)p3m_smem;                            // [NW words][NB]
+    T* sw = (T*)(A + ((NW * NB + 3) & ~3));             // [NT][3 p + 1]: weights x | y | z, then Q
+    int* so = (int*)(sw + P3M_NT * (3 * P + 1));        // [NT]: origin sx | sy << 10 | sz << 20
+    __shared__ int wcount[P3M_NT / 32];
     const int nbx = Kx / BX, nby = Ky / BY;
-    const int bi = blockIdx.x;
+    const int bi = blockIdx.x, rep = blockIdx.y;
     const int b0x = (bi % nbx) * BX, b0y = ((bi / nbx) % nby) * BY, b0z = (bi / (nbx * nby)) * BZ;
-    const int pair = blockIdx.y;
-    const int nrep = min(2, m - 2 * pair);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int64_t jbeg = (int64_t)blockIdx.z * cps * NT;
-    const int64_t jend = min(ne, jbeg + (int64_t)cps * NT);
-    for (int i = threadIdx.x; i < 2 * NW * NB; i += NT) acc[i] = 0;
-    for (int rep = 0; rep < nrep; ++rep) {
-        const int64_t base = (int64_t)(2 * pair + rep) * ne;
-        int* A = acc + rep * NW * NB;
-        for (int64_t j0 = jbeg; j0 < jend; j0 += NT) {
-            const int64_t j = j0 + threadIdx.x;
-            bool sel = false;
-            int sx = 0, sy = 0, sz = 0;
-            if (j < jend) {
-                const int kv = key[base + j];
-                if (kv >= 0) {
-                    sx = ((kv & 1023) - b0x + Kx) & (Kx - 1);
-                    sy = (((kv >> 10) & 1023) - b0y + Ky) & (Ky - 1);
-                    sz = ((kv >> 20) - b0z + Kz) & (Kz - 1);
-                    sel = (sx < BX || sx + P - 1 >= Kx) && (sy < BY || sy + P - 1 >= Ky) &&
-                          (sz < BZ || sz + P - 1 >= Kz);
-                }
+    const int64_t jbeg = (int64_t)blockIdx.z * cps * P3M_NT;
+    const int64_t jend = min(ne, jbeg + (int64_t)cps * P3M_NT);
+    const int64_t base = (int64_t)rep * ne;
+    auto carry = [&]() {   // every point's words belong to one thread here
+        __syncthreads();
+        for (int i = threadIdx.x; i < NB; i += P3M_NT) {
+            int lo = A[NB + i];
+            if (NW == 3) {
+                const int c = A[2 * NB + i];
+                lo += c >> 20;
+                A[2 * NB + i] = c & 0xFFFFF;
             }
-            const unsigned bal = __ballot_sync(0xffffffffu, sel);
-            if (lane == 0) wcount[wid] = __popc(bal);
-            __syncthreads();   // also orders the previous chunk's reads of sw / so before the writes below
-            int off = 0, L = 0;
+            A[i] += lo >> 20;
+            A[NB + i] = lo & 0xFFFFF;
+        }
+        __syncthreads();
+    };
+    int added = -1;        // charges since the last carry; -1: nothing reached the brick yet
+    for (int64_t j0 = jbeg; j0 < jend; j0 += P3M_NT) {
+        const int64_t j = j0 + threadIdx.x;
+        bool sel = false;
+        int sx = 0, sy = 0, sz = 0;
+        if (j < jend) {
+            const int kv = key[base + j];
+            if (kv >= 0) {
+                sx = ((kv & 1023) - b0x + Kx) & (Kx - 1);
+                sy = (((kv >> 10) & 1023) - b0y + Ky) & (Ky - 1);
+                sz = ((kv >> 20) - b0z + Kz) & (Kz - 1);
+                sel = (sx < BX || sx + P - 1 >= Kx) && (sy < BY || sy + P - 1 >= Ky) &&
+                      (sz < BZ || sz + P - 1 >= Kz);
+            }
+        }
+        const unsigned bal = __ballot_sync(0xffffffffu, sel);
+        if (lane == 0) wcount[wid] = __popc(bal);
+        __syncthreads();   // also orders the previous chunk's reads of sw / so before the writes below
+        int off = 0, L = 0;
 #pragma unroll
-            for (int w = 0; w < NT / 32; ++w) {
-                const int cw = wcount[w];
-                off += w < wid ? cw : 0;
-                L += cw;
-            }
-            if (sel) {
-                const int slot = off + __popc(bal & ((1u << lane) - 1u));
-                const typename P3mV4<T>::t v = fq[base + j];
-                T* w = sw + slot * (3 * P + 1);
-                bspline_weights<T, P>(v.x, w);
-                bspline_weights<T, P>(v.y, w + P);
-                bspline_weights<T, P>(v.z, w + 2 * P);
-                w[3 * P] = v.w;
-                so[slot] = sx | (sy << 10) | (sz << 20);
-            }
+        for (int w = 0; w < P3M_NT / 32; ++w) {
+            const int cw = wcount[w];
+            off += w < wid ? cw : 0;
+            L += cw;
+        }
+        if (L == 0) {   // uniform
             __syncthreads();
-            // items (charge, z offset c, y offset b): the y and z rows inside the brick, then p x points
-            for (int it = threadIdx.x; it < L * P * P; it += NT) {
-                const int sl = it / (P * P), cb = it - sl * (P * P);
-                const int c = cb / P, b = cb - c * P;
-                const int o = so[sl];
-                int gy = ((o >> 10) & 1023) + b;
-                if (gy >= Ky) gy -= Ky;
-                int gz = (o >> 20) + c;
-                if (gz >= Kz) gz -= Kz;
-                if (gy >= BY || gz >= BZ) continue;
-                const T* w = sw + sl * (3 * P + 1);
-                const T wyz = w[3 * P] * w[P + b] * w[2 * P + c];
-                const int ox = o & 1023;
-                int* row = A + (gz * BY + gy) * RX;
+            continue;
+        }
+        if (added < 0) {
+            for (int i = threadIdx.x; i < NW * NB; i += P3M_NT) A[i] = 0;
+            added = 0;
+        } else if (added + L > P3M_CARRY) {
+            carry();
+            added = 0;
+        }
+        added += L;
+        if (sel) {
+            const int slot = off + __popc(bal & ((1u << lane) - 1u));
+            const typename P3mV4<T>::t v = fq[base + j];
+            T* w = sw + slot * (3 * P + 1);
+            bspline_weights<T, P>(v.x, w);
+            bspline_weights<T, P>(v.y, w + P);
+            bspline_weights<T, P>(v.z, w + 2 * P);
+            w[3 * P] = v.w;
+            so[slot] = sx | (sy << 10) | (sz << 20);
+        }
+        __syncthreads();
+        const int zz = lane >> 3, b = lane & 7;
+        for (int sl = wid; sl < L; sl += P3M_NT / 32) {
+            const int o = so[sl];
+            const T* w = sw + sl * (3 * P + 1);
+            const int c = (zz - (o >> 20)) & (Kz - 1);   // z offset whose plane is zz
+            int gy = ((o >> 10) & 1023) + b;
+            if (gy >= Ky) gy -= Ky;
+            const bool in = b < P && c < P && gy < BY;
+            const T q = w[3 * P];
+            const T wyz = in ? q * w[P + b] * w[2 * P + c] : (T)0;
+            const int ox = o & 1023;
+            int* row = A + zz * PS + gy * RX;
+            const bool small = fabs(q) <= (T)2;          // warp-uniform
 #pragma unroll
-                for (int a = 0; a < P; ++a) {
-                    int gx = ox + a;
-                    if (gx >= Kx) gx -= Kx;
-                    if (gx < BX) {
-                        // v = hi 2^-20 + lo 2^-40 (+ lo2 2^-60): exact splits of the scaled contribution
-                        if (std::is_same<T, double>::value) {
-                            const double x = (double)(wyz * w[a]) * 1048576.0;   // 2^20
-                            const double h = floor(x);
-                            const double y = (x - h) * 1048576.0;
-                            const double l = floor(y);
-                            atomicAdd(&row[gx], (int)h);
-                            atomicAdd(&row[NB + gx], (int)l);
-                            atomicAdd(&row[2 * NB + gx], __double2int_rn((y - l) * 1048576.0));
-                        } else {
-                            const float x = (float)(wyz * w[a]) * 1048576.0f;
-                            const float h = floorf(x);
-                            atomicAdd(&row[gx], (int)h);
-                            atomicAdd(&row[NB + gx], __float2int_rn((x - h) * 1048576.0f));
-                        }
+            for (int a = 0; a < P; ++a) {
+                int gx = ox + a;
+                if (gx >= Kx) gx -= Kx;
+                if (gx >= BX) continue;                  // uniform
+                // v = hi 2^-20 + lo 2^-40 (+ lo2 2^-60): exact splits of the scaled contribution
+                if (std::is_same<T, double>::value) {
+                    if (!in) continue;
+                    const double x = (double)(wyz * w[a]) * 1048576.0;   // 2^20
+                    const double h = floor(x);
+                    const double y = (x - h) * 1048576.0;
+                    const double l = floor(y);
+                    atomicAdd(&row[gx], (int)h);
+                    atomicAdd(&row[NB + gx], (int)l);
+                    atomicAdd(&row[2 * NB + gx], __double2int_rn((y - l) * 1048576.0));
+                } else {
+                    const float x = (float)(wyz * w[a]) * 1048576.0f;
+                    int hi, lo;
+                    if (small) {   // |x| < 2^22: rounding by adding 1.5 2^23, no conversion instructions
+                        const float t = x + 12582912.0f;
+                        hi = __float_as_int(t) - 0x4B400000;
+                        lo = __float_as_int(fmaf(x - (t - 12582912.0f), 1048576.0f, 12582912.0f)) - 0x4B400000;
+                    } else {
+                        const float h = floorf(x);
+                        hi = (int)h;
+                        lo = __float2int_rn((x - h) * 1048576.0f);
                     }
-                }
-            }
-            {   // carry the low words (every point's words belong to one thread here)
-                __syncthreads();
-                for (int i = threadIdx.x; i < NB; i += NT) {
-                    int lo = A[NB + i];
-                    if (NW == 3) {
-                        const int c = A[2 * NB + i];
-                        lo += c >> 20;
-                        A[2 * NB + i] = c & 0xFFFFF;
+                    if (in) {
+                        atomicAdd(&row[gx], hi);
+                        atomicAdd(&row[NB + gx], lo);
                     }
-                    A[i] += lo >> 20;
-                    A[NB + i] = lo & 0xFFFFF;
                 }
             }
         }
     }
+    if (threadIdx.x == 0) flag[((int64_t)blockIdx.z * m + rep) * gridDim.x + bi] = added >= 0;
+    if (added < 0) return;   // uniform
     __syncthreads();
     const int64_t N = (int64_t)Kx * Ky * Kz;
-    c2<T>* out = part + ((int64_t)blockIdx.z * gridDim.y + pair) * N;
-    for (int i = threadIdx.x; i < BX * BY * BZ; i += NT) {
+    T* out = (T*)(part + ((int64_t)blockIdx.z * ((m + 1) / 2) + rep / 2) * N) + (rep & 1);
+    for (int i = threadIdx.x; i < BX * BY * BZ; i += P3M_NT) {
         const int lx = i % BX, ly = (i / BX) % BY, lz = i / (BX * BY);
-        const int at = (lz * BY + ly) * RX + lx;
-        double v[2] = {0.0, 0.0};
-        for (int r = 0; r < nrep; ++r) {
-            const int* W = acc + r * NW * NB;
-            v[r] = (double)W[at] * 0x1p-20 + (double)W[NB + at] * 0x1p-40;
-            if (NW == 3) v[r] += (double)W[2 * NB + at] * 0x1p-60;
-        }
-        out[((int64_t)(b0z + lz) * Ky + (b0y + ly)) * Kx + (b0x + lx)] = cmake<T>((T)v[0], (T)v[1]);
+        const int at = lz * PS + ly * RX + lx;
+        double v = (double)A[at] * 0x1p-20 + (double)A[NB + at] * 0x1p-40;
+        if (NW == 3) v += (double)A[2 * NB + at] * 0x1p-60;
+        out[2 * (((int64_t)(b0z + lz) * Ky + (b0y + ly)) * Kx + (b0x + lx))] = (T)v;
     }
 }
 
@@ -319,28 +339,55 @@ __device__ __forceinline__ void dit_stages(c2<T>* x, int K, int lg, int lines, i
     }
 }
 
-// 2D transform of every (z plane, replica pair) over x and y; INV: exp(+i ...) (unnormalised).  The
-// forward transform first sums the nsplit partial meshes of the charge assignment (split_stride
-// elements apart) in split order.  Dynamic shared memory: the plane [Ky][Kx], then Kx/2 + Ky/2 twiddles.
+// 2D transform of (z plane, replica pair) over x and y; INV: exp(+i ...) (unnormalised), of the planes zlist that a
+// site's interpolation reads.  The forward transform takes every plane and first sums the nsplit partial meshes of
+// the charge assignment (split_stride elements apart) in split order, of the bricks that are marked; a plane without
+// any is zero.  Dynamic shared memory: the plane [Ky][Kx], then Kx/2 + Ky/2 twiddles.
+constexpr int P3M_FLAGS = 2048;   // marks of one plane: splits x 2 replicas x bricks, at most 8 x 2 x 128
 template <typename T, bool INV>
 __global__ void __launch_bounds__(P3M_THREADS) k_p3m_plane(c2<T>* __restrict__ mesh, int Kx, int Ky, int Kz,
                                                           const c2<T>* __restrict__ twx, const c2<T>* __restrict__ twy,
-                                                          int nsplit, int64_t split_stride) {
+                                                          int nsplit, int64_t split_stride, int m, int BX, int BY,
+                                                          const int* __restrict__ flag, const int* __restrict__ zlist) {
     extern __shared__ __align__(16) unsigned char p3m_smem[];
+    __shared__ unsigned char fl[INV ? 1 : P3M_FLAGS];
     c2<T>* pl = (c2<T>*)p3m_smem;
     c2<T>* tx = pl + Kx * Ky;
     c2<T>* ty = tx + Kx / 2;
     const int lx = ilog2i(Kx), ly = ilog2i(Ky);
+    const int z = INV ? zlist[blockIdx.x] : blockIdx.x;
+    c2<T>* g = mesh + ((int64_t)blockIdx.y * Kz + z) * Kx * Ky;
+    const int nbx = Kx / BX, nbp = nbx * (Ky / BY);   // bricks of one plane
+    if (!INV) {
+        const int nb = nbp * (Kz / P3M_BZ);
+        bool any = false;
+        for (int e = threadIdx.x; e < nsplit * 2 * nbp; e += P3M_THREADS) {
+            const int b = e % nbp, h = (e / nbp) & 1, sp = e / (2 * nbp), r = 2 * blockIdx.y + h;
+            const bool f = r < m && flag[((int64_t)sp * m + r) * nb + (z / P3M_BZ) * nbp + b] != 0;
+            fl[e] = f;
+            any |= f;
+        }
+        if (!__syncthreads_or(any)) {
+            for (int i = threadIdx.x; i < Kx * Ky; i += P3M_THREADS) g[i] = cmake<T>(0, 0);
+            return;
+        }
+    }
     for (int j = threadIdx.x; j < Kx / 2; j += P3M_THREADS) { c2<T> w = twx[j]; if (INV) w.y = -w.y; tx[j] = w; }
     for (int j = threadIdx.x; j < Ky / 2; j += P3M_THREADS) { c2<T> w = twy[j]; if (INV) w.y = -w.y; ty[j] = w; }
-    c2<T>* g = mesh + ((int64_t)blockIdx.y * Kz + blockIdx.x) * Kx * Ky;
     for (int i = threadIdx.x; i < Kx * Ky; i += P3M_THREADS) {
         const int x = i & (Kx - 1), y = i >> lx;
-        c2<T> v = g[i];
-        for (int sp = 1; sp < nsplit; ++sp) {   // the charge splits of the assignment, in split order
-            const c2<T> u = g[sp * split_stride + i];
-            v.x += u.x;
-            v.y += u.y;
+        c2<T> v = cmake<T>(0, 0);
+        if (INV) {
+            v = g[i];
+        } else {
+            const int b = (y / BY) * nbx + x / BX;
+            for (int sp = 0; sp < nsplit; ++sp) {   // the charge splits of the assignment, in split order
+                const bool f0 = fl[(2 * sp) * nbp + b], f1 = fl[(2 * sp + 1) * nbp + b];
+                if (!f0 && !f1) continue;
+                const c2<T> u = g[sp * split_stride + i];   // an unmarked half is not defined
+                if (f0) v.x += u.x;
+                if (f1) v.y += u.y;
+            }
         }
         pl[bitrev(y, ly) * Kx + bitrev(x, lx)] = v;
     }
@@ -351,10 +398,12 @@ __global__ void __launch_bounds__(P3M_THREADS) k_p3m_plane(c2<T>* __restrict__ m
 }
 
 // z pass: for P3M_ZTX adjacent x at one (y, replica pair): forward transform along z, times G / V,
-// inverse transform along z.  Dynamic shared memory: [Kz][tx] lines, then Kz/2 twiddles.
+// inverse transform along z, stored where a site's interpolation reads (need[z]).  Dynamic shared memory: [Kz][tx]
+// lines, then Kz/2 twiddles.
 template <typename T>
 __global__ void __launch_bounds__(P3M_THREADS) k_p3m_zline(c2<T>* __restrict__ mesh, int Kx, int Ky, int Kz, int tx,
-                                                          const T* __restrict__ G, const c2<T>* __restrict__ twz) {
+                                                          const T* __restrict__ G, const c2<T>* __restrict__ twz,
+                                                          const unsigned char* __restrict__ need) {
     extern __shared__ __align__(16) unsigned char p3m_smem[];
     c2<T>* ln = (c2<T>*)p3m_smem;
     c2<T>* tw = ln + Kz * tx;
@@ -389,7 +438,7 @@ __global__ void __launch_bounds__(P3M_THREADS) k_p3m_zline(c2<T>* __restrict__ m
     dit_stages<T>(ln, Kz, lz, tx, 1, tx, tw);
     for (int i = threadIdx.x; i < Kz * tx; i += P3M_THREADS) {
         const int z = i / tx, x = i - z * tx;
-        g[z * plane + x] = ln[i];
+        if (need[z]) g[z * plane + x] = ln[i];
     }
 }
 
@@ -457,21 +506,19 @@ static int64_t mesh_pts(const cpm_ctx* c) {
     return (int64_t)c->p.p3m_mesh[0] * c->p.p3m_mesh[1] * c->p.p3m_mesh[2];
 }
 
-// Assignment bricks (32 x 16 x 8 points at most: 2 x 3 words of 33 x 16 x 8 points and the staged
-// weights of a chunk fit in 227 KiB of shared memory) and charge splits: enough CTAs for four per SM of
-// 152, no split without a chunk of charges, at most 8 partial meshes.
-struct P3mSpread { int BX, BY, BZ, nbricks, nsplit, cps; };
-template <typename T>
+// Assignment bricks of 32 x 32 x 4 points at most and charge splits: enough CTAs that the bricks within the
+// electrolyte, about a third, still fill two CTAs per SM a few times; no split without a chunk of charges, at
+// most 8 partial meshes.
+struct P3mSpread { int BX, BY, nbricks, nsplit, cps; };
 static P3mSpread p3m_spread_plan(const cpm_ctx* c, int m, int64_t ne) {
     P3mSpread sp;
     const int Kx = c->p.p3m_mesh[0], Ky = c->p.p3m_mesh[1], Kz = c->p.p3m_mesh[2];
     sp.BX = std::min(Kx, 32);
-    sp.BY = std::min(Ky, 16);
-    sp.BZ = std::min(Kz, 8);
-    sp.nbricks = (Kx / sp.BX) * (Ky / sp.BY) * (Kz / sp.BZ);
-    const int64_t ctas = (int64_t)sp.nbricks * ((m + 1) / 2);
-    const int64_t nchunks = std::max<int64_t>(1, (ne + P3mSpreadThreads<T>::n - 1) / P3mSpreadThreads<T>::n);
-    int64_t ns = std::max<int64_t>(1, (4 * 152 + ctas - 1) / ctas);
+    sp.BY = std::min(Ky, 32);
+    sp.nbricks = (Kx / sp.BX) * (Ky / sp.BY) * (Kz / P3M_BZ);
+    const int64_t ctas = (int64_t)sp.nbricks * m;
+    const int64_t nchunks = std::max<int64_t>(1, (ne + P3M_NT - 1) / P3M_NT);
+    int64_t ns = std::max<int64_t>(1, (16 * 152 + ctas - 1) / ctas);
     ns = std::min<int64_t>(std::min<int64_t>(ns, 8), nchunks);
     sp.cps = (int)((nchunks + ns - 1) / ns);
     sp.nsplit = (int)((nchunks + sp.cps - 1) / sp.cps);
@@ -481,8 +528,9 @@ static P3mSpread p3m_spread_plan(const cpm_ctx* c, int m, int64_t ne) {
 template <typename T>
 size_t p3m_scratch_bytes(const cpm_ctx* c, int m, int64_t ne) {
     const int64_t ptot = (int64_t)m * ne;
-    const P3mSpread sp = p3m_spread_plan<T>(c, m, ne);
+    const P3mSpread sp = p3m_spread_plan(c, m, ne);
     return p3m_al(sizeof(int) * ptot) + p3m_al(sizeof(typename P3mV4<T>::t) * ptot) +
+           p3m_al(sizeof(int) * (size_t)sp.nsplit * m * sp.nbricks) +
            p3m_al(sizeof(c2<T>) * (size_t)sp.nsplit * ((m + 1) / 2) * mesh_pts(c));
 }
 template size_t p3m_scratch_bytes<float>(const cpm_ctx*, int, int64_t);
@@ -511,7 +559,34 @@ static cpm_status p3m_prepare_t(cpm_ctx* c, void** Gp, void** twp) {
     return CPM_OK;
 }
 
+// the planes that the interpolation at the sites reads (one more on either side of each stencil, so that no
+// rounding of the origin can matter)
+static cpm_status p3m_planes(cpm_ctx* c) {
+    const int Kz = c->p.p3m_mesh[2], P = c->p.p3m_order;
+    std::vector<double> zu(c->nzu);
+    CPM_CUDA(c, cudaMemcpyAsync(zu.data(), c->zuniq, sizeof(double) * zu.size(), cudaMemcpyDeviceToHost, c->stream));
+    CPM_CUDA(c, cudaStreamSynchronize(c->stream));
+    std::vector<unsigned char> need(Kz, 0);
+    for (double z : zu) {
+        double s = z * c->g.inv[2];
+        s -= std::floor(s);
+        const int b = (int)std::floor(s * Kz - 0.5 * P);
+        for (int a = 0; a < P + 2; ++a) need[((b + a) % Kz + Kz) % Kz] = 1;
+    }
+    std::vector<int> list;
+    for (int z = 0; z < Kz; ++z)
+        if (need[z]) list.push_back(z);
+    CPM_TRY(dev_alloc(c, (void**)&c->p3m_need, Kz));
+    CPM_TRY(dev_alloc(c, (void**)&c->p3m_zlist, sizeof(int) * list.size()));
+    CPM_CUDA(c, cudaMemcpyAsync(c->p3m_need, need.data(), Kz, cudaMemcpyHostToDevice, c->stream));
+    CPM_CUDA(c, cudaMemcpyAsync(c->p3m_zlist, list.data(), sizeof(int) * list.size(), cudaMemcpyHostToDevice, c->stream));
+    CPM_CUDA(c, cudaStreamSynchronize(c->stream));
+    c->p3m_nz = (int)list.size();
+    return CPM_OK;
+}
+
 cpm_status p3m_prepare(cpm_ctx* c) {
+    CPM_TRY(p3m_planes(c));
     if (c->p3m_G) return CPM_OK;   // depends on the cell and the parameters only
     if (c->p.k_prec == CPM_PREC_FP64) return p3m_prepare_t<double>(c, &c->p3m_G, &c->p3m_tw);
     CPM_TRY(p3m_prepare_t<float>(c, &c->p3m_G, &c->p3m_tw));
@@ -529,29 +604,29 @@ template <typename T> static const c2<T>* p3m_twiddles(const cpm_ctx* c) {
 
 template <typename T, int P>
 static cpm_status launch_p3m_pp(cudaStream_t st, cpm_ctx* c, int m, int64_t ne, const int* key,
-                          const typename P3mV4<T>::t* fq, c2<T>* mesh, double* pm) {
+                          const typename P3mV4<T>::t* fq, int* flag, c2<T>* mesh, double* pm) {
     const int Kx = c->p.p3m_mesh[0], Ky = c->p.p3m_mesh[1], Kz = c->p.p3m_mesh[2];
-    const P3mSpread sp = p3m_spread_plan<T>(c, m, ne);
+    const P3mSpread sp = p3m_spread_plan(c, m, ne);
     const int npairs = (m + 1) / 2;
-    constexpr int NT = P3mSpreadThreads<T>::n;
-    const size_t ssm = sizeof(int) * ((2 * P3mWords<T>::n * (sp.BX + 1) * sp.BY * sp.BZ + 3) & ~3) +
-                       sizeof(T) * NT * (3 * P + 1) + sizeof(int) * NT;
+    const size_t ssm = sizeof(int) * ((P3mWords<T>::n * P3M_BZ * (sp.BY * (sp.BX + 1) + 8) + 3) & ~3) +
+                       sizeof(T) * P3M_NT * (3 * P + 1) + sizeof(int) * P3M_NT;
     CPM_CUDA(c, cudaFuncSetAttribute(k_p3m_spread<T, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssm));
-    k_p3m_spread<T, P><<<dim3(sp.nbricks, npairs, sp.nsplit), NT, ssm, st>>>(key, fq, ne, m, Kx, Ky, Kz, sp.BX, sp.BY,
-                                                                             sp.BZ, sp.cps, mesh);
+    k_p3m_spread<T, P><<<dim3(sp.nbricks, m, sp.nsplit), P3M_NT, ssm, st>>>(key, fq, ne, m, Kx, Ky, Kz, sp.BX, sp.BY,
+                                                                            sp.cps, mesh, flag);
     const int64_t sstride = (int64_t)npairs * Kx * Ky * Kz;
     const c2<T>* tw = p3m_twiddles<T>(c);
     const size_t psm = sizeof(c2<T>) * ((size_t)Kx * Ky + Kx / 2 + Ky / 2);
     CPM_CUDA(c, cudaFuncSetAttribute(k_p3m_plane<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psm));
     CPM_CUDA(c, cudaFuncSetAttribute(k_p3m_plane<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psm));
     k_p3m_plane<T, false><<<dim3(Kz, npairs), P3M_THREADS, psm, st>>>(mesh, Kx, Ky, Kz, tw, tw + Kx / 2, sp.nsplit,
-                                                                      sstride);
+                                                                      sstride, m, sp.BX, sp.BY, flag, nullptr);
     const int tx = std::min(Kx, P3M_ZTX);
     const size_t zsm = sizeof(c2<T>) * ((size_t)Kz * tx + Kz / 2);
     CPM_CUDA(c, cudaFuncSetAttribute(k_p3m_zline<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)zsm));
     k_p3m_zline<T><<<dim3(Kx / tx, Ky, npairs), P3M_THREADS, zsm, st>>>(mesh, Kx, Ky, Kz, tx, p3m_green<T>(c),
-                                                                        tw + Kx / 2 + Ky / 2);
-    k_p3m_plane<T, true><<<dim3(Kz, npairs), P3M_THREADS, psm, st>>>(mesh, Kx, Ky, Kz, tw, tw + Kx / 2, 1, 0);
+                                                                        tw + Kx / 2 + Ky / 2, c->p3m_need);
+    k_p3m_plane<T, true><<<dim3(c->p3m_nz, npairs), P3M_THREADS, psm, st>>>(mesh, Kx, Ky, Kz, tw, tw + Kx / 2, 1, 0, m,
+                                                                            sp.BX, sp.BY, nullptr, c->p3m_zlist);
     const int64_t warps = c->n * npairs;
     k_p3m_interp<T, P><<<(unsigned)((warps + P3M_THREADS / 32 - 1) / (P3M_THREADS / 32)), P3M_THREADS, 0, st>>>(
         c->sx, c->n, m, c->g, Kx, Ky, Kz, mesh, pm);
@@ -566,19 +641,21 @@ cpm_status p3m_run(cpm_ctx* c, cudaStream_t st, int m, int64_t ne, const double*
     int* key = (int*)scr;
     typedef typename P3mV4<T>::t V4T;
     V4T* fq = (V4T*)(scr + p3m_al(sizeof(int) * ptot));
-    c2<T>* mesh = (c2<T>*)(scr + p3m_al(sizeof(int) * ptot) + p3m_al(sizeof(V4T) * ptot));
+    int* flag = (int*)((char*)fq + p3m_al(sizeof(V4T) * ptot));
+    const P3mSpread sp = p3m_spread_plan(c, m, ne);
+    c2<T>* mesh = (c2<T>*)((char*)flag + p3m_al(sizeof(int) * (size_t)sp.nsplit * m * sp.nbricks));
     const int P = c->p.p3m_order;
     const int Kx = c->p.p3m_mesh[0], Ky = c->p.p3m_mesh[1], Kz = c->p.p3m_mesh[2];
     k_p3m_prep<T><<<(unsigned)((ptot + 255) / 256), 256, 0, st>>>(xyz, Q, ptot, c->g, Kx, Ky, Kz, P, key, fq);
     CPM_LAUNCH(c, "k_p3m_prep");
     c->launches += 6;
     switch (P) {
-        case 2: return launch_p3m_pp<T, 2>(st, c, m, ne, key, fq, mesh, pm);
-        case 3: return launch_p3m_pp<T, 3>(st, c, m, ne, key, fq, mesh, pm);
-        case 4: return launch_p3m_pp<T, 4>(st, c, m, ne, key, fq, mesh, pm);
-        case 5: return launch_p3m_pp<T, 5>(st, c, m, ne, key, fq, mesh, pm);
-        case 6: return launch_p3m_pp<T, 6>(st, c, m, ne, key, fq, mesh, pm);
-        default: return launch_p3m_pp<T, 7>(st, c, m, ne, key, fq, mesh, pm);
+        case 2: return launch_p3m_pp<T, 2>(st, c, m, ne, key, fq, flag, mesh, pm);
+        case 3: return launch_p3m_pp<T, 3>(st, c, m, ne, key, fq, flag, mesh, pm);
+        case 4: return launch_p3m_pp<T, 4>(st, c, m, ne, key, fq, flag, mesh, pm);
+        case 5: return launch_p3m_pp<T, 5>(st, c, m, ne, key, fq, flag, mesh, pm);
+        case 6: return launch_p3m_pp<T, 6>(st, c, m, ne, key, fq, flag, mesh, pm);
+        default: return launch_p3m_pp<T, 7>(st, c, m, ne, key, fq, flag, mesh, pm);
     }
 }
 // ----------------------------------------------------------------------------- the P3M elastance

@@ -1,0 +1,39 @@
+"""P3M charge assignment and the planes left out: b against the oracle's P3M (1e-12 in FP64, 2e-6 in single precision,
+as the other P3M tests) with charges above and below 2 e, more charges at one place than are added between two carries,
+one replica more than a pair, an empty replica, and meshes with one and several bricks per axis."""
+import numpy as np
+import pytest
+
+from gpu_util import dev, make_ctx, need_gpu, rel_l2, run_bvec, torch
+from oracle import cpm_oracle as o
+from paper_2203_15461_gb300 import systems as s
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("k_prec,tol", [("fp64", 1e-12), ("fp32", 2e-6)])
+@pytest.mark.parametrize("mesh,order", [((32, 32, 64), 7), ((64, 64, 64), 5), ((8, 128, 32), 3), ((64, 16, 128), 6)])
+def test_p3m_assignment(mesh, order, k_prec, tol):
+    need_gpu()
+    base = s.au111_slab(seed_layers=1, nx=5, ny=6, gap=24.0)
+    el = s.Electrodes(**{**base.__dict__, "p3m_mesh": mesh, "p3m_order": order})
+    rng = np.random.default_rng(12)
+    zc = 0.5 * (el.z_inner[0] + el.z_inner[1])
+
+    def cloud(n, spread, qmax):
+        x = np.column_stack([rng.uniform(0, el.box[0], n), rng.uniform(0, el.box[1], n), zc + rng.uniform(-spread, spread, n)])
+        return s.Electrolyte(xyz=x, Q=rng.uniform(-qmax, qmax, n))
+
+    crowd = cloud(2600, 0.02, 0.8)                      # one chunk after the other in the same planes
+    crowd.xyz[:, :2] = crowd.xyz[0, :2] + rng.uniform(-0.05, 0.05, (2600, 2))
+    elyts = [crowd, cloud(90, 6.0, 40.0), s.Electrolyte(xyz=np.zeros((0, 3)), Q=np.zeros(0)), cloud(513, 8.0, 1.9),
+             cloud(1, 1.0, 1.0)]
+    ctx = make_ctx(el, k_prec=k_prec)
+    ctx.cpm_prepare(dev(el.xyz), dev(el.eta), dev(el.group, torch.int32), el.n_groups)
+    b = run_bvec(ctx, elyts)
+    for r, e in enumerate(elyts):
+        if e.n == 0:
+            # the rounding of the partner in the shared mesh, which has the partner's relative accuracy
+            assert np.abs(b[r]).max() <= tol * np.abs(b[r + 1]).max()
+        else:
+            assert rel_l2(b[r], o.bvec(el, e)) <= tol, r
