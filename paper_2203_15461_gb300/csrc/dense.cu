@@ -7,77 +7,85 @@
 namespace cpm {
 
 // ----------------------------------------------------------------------------- DGEMM
-// C = alpha op(A) op(B) + beta C, row-major, 64 x 64 tiles, 256 threads (4 x 4 each).
+// C = alpha op(A) op(B) + beta C, row-major, BM x BN tiles, 256 threads (BM / 16 x BN / 16 each).
 // lower: skip tiles strictly above the diagonal of C.  tri & 1: op(A)[i][k] = 0 for k < i;
 // tri & 2: op(B)[k][j] = 0 for k < j (triangular operands; the K loop starts past the zeros).
 // status: when non-null and nonzero the kernel returns without touching C.
 //
-// The FP64 pipe retires two multiply-adds per clock and SM, so a 64 x 64 tile with 4 x 4 accumulators per
-// thread is far from load-bound once the next K step is fetched while the current one is multiplied; what
-// matters is that every SM has a tile.
-constexpr int DG_BM = 64, DG_BK = 16, DG_T = 256;
+// The FP64 pipe retires two multiply-adds per clock and SM, so even a 2 x 2 block of accumulators per
+// thread is not load-bound once the next K step is fetched while the current one is multiplied; what
+// matters is that every SM has a tile: 64 x 64 x 64 takes 68 us on one.  64 x 64 tiles are taken from DG_MANY of
+// them on (four per SM), 32 x 32 below.
+constexpr int DG_BM = 64, DG_BK = 16, DG_T = 256, DG_MANY = 4 * 152;
 
 // one tile at (r0, c0), K range [kbeg, kend), kbeg a multiple of DG_BK
-template <bool TA, bool TB>
+template <bool TA, bool TB, int BM, int BN>
 __device__ __forceinline__ void dgemm_tile(int r0, int c0, int M, int N, int K, int kbeg, int kend, double alpha,
                                            const double* A, int64_t lda, const double* B, int64_t ldb, double beta,
                                            double* C, int64_t ldc) {
-    constexpr int PER = DG_BK * DG_BM / DG_T;
-    __shared__ double As[DG_BK][DG_BM + 1];
-    __shared__ double Bs[DG_BK][DG_BM + 1];
+    constexpr int TM = BM / 16, TN = BN / 16, PA = DG_BK * BM / DG_T, PB = DG_BK * BN / DG_T;
+    __shared__ double As[DG_BK][BM + 1];
+    __shared__ double Bs[DG_BK][BN + 1];
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    double acc[4][4];
+    double acc[TM][TN];
 #pragma unroll
-    for (int p = 0; p < 4; ++p)
+    for (int p = 0; p < TM; ++p)
 #pragma unroll
-        for (int q = 0; q < 4; ++q) acc[p][q] = 0.0;
+        for (int q = 0; q < TN; ++q) acc[p][q] = 0.0;
     kend = min(kend, K);
-    double va[PER], vb[PER];
+    double va[PA], vb[PB];
     auto fetch = [&](int k0) {
 #pragma unroll
-        for (int u = 0; u < PER; ++u) {
+        for (int u = 0; u < PA; ++u) {
             const int e = threadIdx.x + u * DG_T;
             int m, kk;
-            if (TA) { m = e % DG_BM; kk = e / DG_BM; } else { kk = e % DG_BK; m = e / DG_BK; }
-            int gi = r0 + m, gk = k0 + kk;
+            if (TA) { m = e % BM; kk = e / BM; } else { kk = e % DG_BK; m = e / DG_BK; }
+            const int gi = r0 + m, gk = k0 + kk;
             va[u] = (gi < M && gk < kend) ? (TA ? A[(int64_t)gk * lda + gi] : A[(int64_t)gi * lda + gk]) : 0.0;
-            int nn;
-            if (TB) { kk = e % DG_BK; nn = e / DG_BK; } else { nn = e % DG_BM; kk = e / DG_BM; }
-            int gj = c0 + nn;
-            gk = k0 + kk;
+        }
+#pragma unroll
+        for (int u = 0; u < PB; ++u) {
+            const int e = threadIdx.x + u * DG_T;
+            int nn, kk;
+            if (TB) { kk = e % DG_BK; nn = e / DG_BK; } else { nn = e % BN; kk = e / BN; }
+            const int gj = c0 + nn, gk = k0 + kk;
             vb[u] = (gj < N && gk < kend) ? (TB ? B[(int64_t)gj * ldb + gk] : B[(int64_t)gk * ldb + gj]) : 0.0;
         }
     };
     if (kbeg < kend) fetch(kbeg);
     for (int k0 = kbeg; k0 < kend; k0 += DG_BK) {
 #pragma unroll
-        for (int u = 0; u < PER; ++u) {
+        for (int u = 0; u < PA; ++u) {
             const int e = threadIdx.x + u * DG_T;
-            if (TA) As[e / DG_BM][e % DG_BM] = va[u]; else As[e % DG_BK][e / DG_BK] = va[u];
-            if (TB) Bs[e % DG_BK][e / DG_BK] = vb[u]; else Bs[e / DG_BM][e % DG_BM] = vb[u];
+            if (TA) As[e / BM][e % BM] = va[u]; else As[e % DG_BK][e / DG_BK] = va[u];
+        }
+#pragma unroll
+        for (int u = 0; u < PB; ++u) {
+            const int e = threadIdx.x + u * DG_T;
+            if (TB) Bs[e % DG_BK][e / DG_BK] = vb[u]; else Bs[e / BN][e % BN] = vb[u];
         }
         __syncthreads();
         if (k0 + DG_BK < kend) fetch(k0 + DG_BK);
 #pragma unroll
         for (int kk = 0; kk < DG_BK; ++kk) {
-            double a[4], b[4];
+            double a[TM], b[TN];
 #pragma unroll
-            for (int p = 0; p < 4; ++p) a[p] = As[kk][ty + 16 * p];
+            for (int p = 0; p < TM; ++p) a[p] = As[kk][ty + 16 * p];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) b[q] = Bs[kk][tx + 16 * q];
+            for (int q = 0; q < TN; ++q) b[q] = Bs[kk][tx + 16 * q];
 #pragma unroll
-            for (int p = 0; p < 4; ++p)
+            for (int p = 0; p < TM; ++p)
 #pragma unroll
-                for (int q = 0; q < 4; ++q) acc[p][q] = fma(a[p], b[q], acc[p][q]);
+                for (int q = 0; q < TN; ++q) acc[p][q] = fma(a[p], b[q], acc[p][q]);
         }
         __syncthreads();
     }
 #pragma unroll
-    for (int p = 0; p < 4; ++p) {
+    for (int p = 0; p < TM; ++p) {
         int i = r0 + ty + 16 * p;
         if (i >= M) continue;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
+        for (int q = 0; q < TN; ++q) {
             int j = c0 + tx + 16 * q;
             if (j >= N) continue;
             double* cp = C + (int64_t)i * ldc + j;
@@ -86,47 +94,59 @@ __device__ __forceinline__ void dgemm_tile(int r0, int c0, int M, int N, int K, 
     }
 }
 
-template <bool TA, bool TB>
+template <bool TA, bool TB, int BM, int BN>
 __global__ void __launch_bounds__(DG_T) k_dgemm(int M, int N, int K, double alpha, const double* A,
                                                int64_t lda, const double* B, int64_t ldb, double beta,
                                                double* C, int64_t ldc, int lower, int tri, const unsigned* status) {
     if (status && *status) return;
-    const int r0 = blockIdx.y * DG_BM, c0 = blockIdx.x * DG_BM;
-    if (lower && c0 > r0 + DG_BM - 1) return;
+    const int r0 = blockIdx.y * BM, c0 = blockIdx.x * BN;
+    if (lower && c0 > r0 + BM - 1) return;
     int kbeg = 0;
     if (tri & 1) kbeg = max(kbeg, r0);
     if (tri & 2) kbeg = max(kbeg, c0);
-    dgemm_tile<TA, TB>(r0, c0, M, N, K, (kbeg / DG_BK) * DG_BK, K, alpha, A, lda, B, ldb, beta, C, ldc);
+    dgemm_tile<TA, TB, BM, BN>(r0, c0, M, N, K, (kbeg / DG_BK) * DG_BK, K, alpha, A, lda, B, ldb, beta, C, ldc);
 }
 
 // One level of the blocked inverse of a lower-triangular W whose diagonal blocks of size s are inverted:
 // for every pair of blocks (rows [r, r + s2) below columns [r - s, r), s2 the rows that exist),
 //   step 1: T = W_21 W_11,   step 2: W_21 <- -W_22 T      (W_11, W_22 lower triangular: K skips their zeros).
-// grid (s / 64, s / 64, pairs); T is an n x n scratch, used at the place of W_21.  Every level is two launches
+// grid (s / BM, s / BM, pairs); T is an n x n scratch, used at the place of W_21.  Every level is two launches
 // over all pairs; block row by block row the inverse of 2,048 rows was 62 launches of at most 32 tiles each
 // (36 of the 62 ms of an inversion).
+template <int BM>
 __global__ void __launch_bounds__(DG_T) k_trinv_level(double* W, double* T, int64_t n, int s, int step,
                                                       const unsigned* status) {
     if (status && *status) return;
     const int64_t c = (int64_t)blockIdx.z * 2 * s, r = c + s;
     const int s2 = (int)min((int64_t)s, n - r);
-    const int r0 = blockIdx.y * DG_BM, c0 = blockIdx.x * DG_BM;
+    const int r0 = blockIdx.y * BM, c0 = blockIdx.x * BM;
     if (r0 >= s2) return;
     double* W21 = W + r * n + c;
     double* T21 = T + r * n + c;
-    if (step == 1) dgemm_tile<false, false>(r0, c0, s2, s, s, c0, s, 1.0, W21, n, W + c * n + c, n, 0.0, T21, n);
-    else dgemm_tile<false, false>(r0, c0, s2, s, s2, 0, r0 + DG_BM, -1.0, W + r * n + r, n, T21, n, 0.0, W21, n);
+    if (step == 1) dgemm_tile<false, false, BM, BM>(r0, c0, s2, s, s, c0, s, 1.0, W21, n, W + c * n + c, n, 0.0, T21, n);
+    else dgemm_tile<false, false, BM, BM>(r0, c0, s2, s, s2, 0, r0 + BM, -1.0, W + r * n + r, n, T21, n, 0.0, W21, n);
+}
+
+template <bool TA, bool TB>
+static void dgemm_tiles(cudaStream_t s, int M, int N, int K, double alpha, const double* A, int64_t lda, const double* B,
+                        int64_t ldb, double beta, double* C, int64_t ldc, int lower, int tri, const unsigned* status) {
+    const int64_t tm = (M + 63) / 64, tn = (N + 63) / 64, tiles = lower ? tm * (tm + 1) / 2 : tm * tn;
+    if (tiles >= DG_MANY)
+        k_dgemm<TA, TB, 64, 64><<<dim3((unsigned)tn, (unsigned)tm), DG_T, 0, s>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc,
+                                                                                 lower, tri, status);
+    else
+        k_dgemm<TA, TB, 32, 32><<<dim3((N + 31) / 32, (M + 31) / 32), DG_T, 0, s>>>(M, N, K, alpha, A, lda, B, ldb, beta, C,
+                                                                                   ldc, lower, tri, status);
 }
 
 cpm_status launch_dgemm(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double alpha, const double* A,
                         int64_t lda, const double* B, int64_t ldb, double beta, double* C, int64_t ldc, int lower,
                         int tri, const unsigned* status) {
     if (M <= 0 || N <= 0) return CPM_OK;
-    dim3 grid((N + DG_BM - 1) / DG_BM, (M + DG_BM - 1) / DG_BM);
-    if (ta && tb) k_dgemm<true, true><<<grid, DG_T, 0, s>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, lower, tri, status);
-    else if (ta) k_dgemm<true, false><<<grid, DG_T, 0, s>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, lower, tri, status);
-    else if (tb) k_dgemm<false, true><<<grid, DG_T, 0, s>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, lower, tri, status);
-    else k_dgemm<false, false><<<grid, DG_T, 0, s>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, lower, tri, status);
+    if (ta && tb) dgemm_tiles<true, true>(s, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, lower, tri, status);
+    else if (ta) dgemm_tiles<true, false>(s, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, lower, tri, status);
+    else if (tb) dgemm_tiles<false, true>(s, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, lower, tri, status);
+    else dgemm_tiles<false, false>(s, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, lower, tri, status);
     return cudaGetLastError() == cudaSuccess ? CPM_OK : CPM_E_CUDA;
 }
 
@@ -137,13 +157,15 @@ constexpr int NB = 64;
 // its factor written to Linv (NB x NB, zero above the diagonal).  A pivot that is not
 // positive and finite sets ST_NOT_SPD and stops the factorisation.
 // One pass eliminates both: after column j, row i > j gets its rank-one update of the trailing columns
-// k = j + 1 .. i and of the inverse's columns c = 0 .. j, i + 1 terms over sixteen threads per row.  The inverse shares
-// the array: its entry (i, c) sits at [c][i + 1].  About 30 us, near what one SM's FP64 pipe needs for 64^3 / 3
-// multiply-adds; with the inverse as 64 serial columns after the factor it took 250.
-constexpr int PF_T = 1024, PF_L = PF_T / NB;
+// k = j + 1 .. i and of the inverse's columns c = 0 .. j, i + 1 terms over eight threads per row.  The inverse shares
+// the array: its entry (i, c) sits at [c][i + 1].  One SM's FP64 pipe takes 16 clocks per warp instruction, so
+// nothing is computed twice: two warps form the square root and the reciprocal square root of the next pivot
+// beside the update, and the column is scaled by a product.
+constexpr int PF_L = 8, PF_U = NB * PF_L, PF_T = PF_U + 64;   // update threads, then the two pivot warps
 __global__ void __launch_bounds__(PF_T) k_potrf(double* Ab, int64_t lda, int kb, double* Linv, unsigned* status) {
     if (*status) return;
     __shared__ double L[NB][NB + 3];
+    __shared__ double s_piv[2], s_inv[2];
     __shared__ int bad;
     for (int e = threadIdx.x; e < NB * NB; e += PF_T) {
         const int i = e / NB, j = e % NB;
@@ -155,31 +177,43 @@ __global__ void __launch_bounds__(PF_T) k_potrf(double* Ab, int64_t lda, int kb,
     if (threadIdx.x == 0) bad = 0;
     __syncthreads();
     const int i = threadIdx.x / PF_L, q = threadIdx.x % PF_L;
+    const bool root = threadIdx.x == PF_U, rroot = threadIdx.x == PF_U + 32;
+    auto pivot = [&](int j, double pv) {
+        if (root) {
+            if (!(pv > 0.0) || !isfinite(pv)) bad = 1;
+            s_piv[j & 1] = sqrt(pv);
+        } else {
+            s_inv[j & 1] = rsqrt(pv);
+        }
+    };
+    if (root || rroot) pivot(0, L[0][0]);
     for (int j = 0; j < NB; ++j) {
-        const double pv = L[j][j];
-        if (threadIdx.x == 0 && (!(pv > 0.0) || !isfinite(pv))) bad = 1;
-        __syncthreads();   // every thread has read the pivot
-        if (bad) break;
-        const double piv = sqrt(pv);
+        __syncthreads();
+        if (bad) break;   // set before the barrier; nobody writes it until the next one
+        const double piv = s_piv[j & 1], inv = s_inv[j & 1];
         if ((int)threadIdx.x < NB) {   // column j of the factor, row j of the inverse
             const int t = threadIdx.x;
-            if (t > j) L[t][j] /= piv;
+            if (t > j) L[t][j] *= inv;
             else if (t == j) L[j][j] = piv;
         } else if ((int)threadIdx.x < 2 * NB) {
             const int t = threadIdx.x - NB;
-            if (t < j) L[t][j + 1] /= piv;
-            else if (t == j) L[j][j + 1] = 1.0 / piv;
+            if (t < j) L[t][j + 1] *= inv;
+            else if (t == j) L[j][j + 1] = inv;
         }
         __syncthreads();
-        if (i > j) {
-            const double lij = L[i][j];
-            for (int c = q; c <= i; c += PF_L) {
-                if (c > j) L[i][c] = fma(-lij, L[c][j], L[i][c]);
-                else L[c][i + 1] = fma(-lij, L[c][j + 1], L[c][i + 1]);
+        if ((int)threadIdx.x < PF_U) {
+            if (i > j) {
+                const double lij = L[i][j];
+                for (int c = q; c <= i; c += PF_L) {
+                    if (c <= j) L[c][i + 1] = fma(-lij, L[c][j + 1], L[c][i + 1]);
+                    else if (c < i || i > j + 1) L[i][c] = fma(-lij, L[c][j], L[i][c]);   // the next pivot: below
+                }
             }
+        } else if ((root || rroot) && j + 1 < NB) {
+            pivot(j + 1, fma(-L[j + 1][j], L[j + 1][j], L[j + 1][j + 1]));
         }
-        __syncthreads();
     }
+    __syncthreads();
     if (bad) {
         if (threadIdx.x == 0) atomicOr(status, ST_NOT_SPD);
         return;
@@ -305,8 +339,11 @@ cpm_status invert_and_project(cpm_ctx* c) {
         const int rows = (int)(n - k0 - kb);
         if (rows > 0) {
             double* P = W + (k0 + kb) * n + k0;
-            // panel: P <- P L_kk^-T (in place; one 64-wide tile column, so every block owns its rows)
-            CPM_TRY(launch_dgemm(st, false, true, rows, kb, kb, 1.0, P, n, Linv, NB, 0.0, P, n, 0, 0, c->status));
+            // panel: P <- P L_kk^-T (in place; one 64-wide tile column, so every block owns its rows; 16 rows each,
+            // for as many blocks as there are SMs)
+            k_dgemm<false, true, 16, NB><<<dim3(1, (rows + 15) / 16), DG_T, 0, st>>>(rows, kb, kb, 1.0, P, n, Linv, NB, 0.0,
+                                                                                    P, n, 0, 0, c->status);
+            CPM_LAUNCH(c, "k_dgemm(panel)");
             // trailing update, lower triangle: A22 <- A22 - P P^T
             CPM_TRY(launch_dgemm(st, false, true, rows, rows, kb, -1.0, P, n, P, n, 1.0, W + (k0 + kb) * (n + 1), n, 1,
                                  0, c->status));
@@ -320,9 +357,15 @@ cpm_status invert_and_project(cpm_ctx* c) {
     k_trtri<<<(unsigned)((n + NB - 1) / NB), 64, 0, st>>>(W, n, c->status);
     CPM_LAUNCH(c, "k_trtri");
     for (int64_t s = NB; s < n; s *= 2) {
-        const dim3 gl((unsigned)(s / DG_BM), (unsigned)(s / DG_BM), (unsigned)((n - s + 2 * s - 1) / (2 * s)));
-        k_trinv_level<<<gl, DG_T, 0, st>>>(W, c->S, n, (int)s, 1, c->status);
-        k_trinv_level<<<gl, DG_T, 0, st>>>(W, c->S, n, (int)s, 2, c->status);
+        const int64_t pairs = (n - s + 2 * s - 1) / (2 * s);
+        for (int step = 1; step <= 2; ++step) {
+            if ((s / 64) * (s / 64) * pairs >= DG_MANY)
+                k_trinv_level<64><<<dim3((unsigned)(s / 64), (unsigned)(s / 64), (unsigned)pairs), DG_T, 0, st>>>(
+                    W, c->S, n, (int)s, step, c->status);
+            else
+                k_trinv_level<32><<<dim3((unsigned)(s / 32), (unsigned)(s / 32), (unsigned)pairs), DG_T, 0, st>>>(
+                    W, c->S, n, (int)s, step, c->status);
+        }
         CPM_LAUNCH(c, "k_trinv_level");
     }
     // A^-1 = W^T W, lower tiles, then mirrored
