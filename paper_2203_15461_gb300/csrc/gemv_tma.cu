@@ -35,9 +35,12 @@ constexpr int GV_RJ = 16;                      // rows of S per stage
 constexpr int GV_STAGES = 3;                   // per block; two blocks per SM
 constexpr int GV_STAGE_BYTES = GV_RJ * GV_BC * 4;
 constexpr int GV_JMAX = 192;                   // rows of b staged per block
-constexpr int GV_MR = 8;                       // replicas per block
-constexpr int GV_SPT = (GV_JMAX * GV_MR + GV_T - 1) / GV_T;   // staged entries per consumer thread
-constexpr int GV_SMEM = 1024 + GV_STAGES * GV_STAGE_BYTES + GV_JMAX * 2 * GV_MR * 4 + 256;
+constexpr int GV_MR = 8;                       // replicas per block, at most
+// Replicas per block: a step of one or two replicas does the arithmetic of two, not of eight (the consumers, two
+// warps per scheduler, take longer over a stage for eight than the copies do).  A step of one replica over 4,320
+// sites: 119 -> 115.6 us; four replicas over 512 sites: 55 -> 54 us; eight replicas take the same code as before.
+static int gv_mr(int m) { return m <= 2 ? 2 : m <= 4 ? 4 : GV_MR; }
+constexpr int gv_smem(int mr) { return 1024 + GV_STAGES * GV_STAGE_BYTES + GV_JMAX * 2 * mr * 4 + 256; }
 constexpr uint64_t GV_WAIT_NS = 2000000000ull;
 
 // compensated sum of packed pairs (Kahan): the sum is s - c; every step is one rounding
@@ -73,22 +76,24 @@ __device__ __forceinline__ DF df_sub(DF a, DF b) {
     return df_norm(s.hi, __fadd_rn(s.lo, __fsub_rn(a.lo, b.lo)));
 }
 
-// grid (column blocks, splits, replica chunks of eight)
+// grid (column blocks, splits, replica chunks of MR)
+template <int MR>
 __global__ void __launch_bounds__(GV_T + 32, 2)
     k_gemv_tma(const __grid_constant__ CUtensorMap smap, const float2* __restrict__ bv, int64_t n, int m,
                int64_t jchunk, float2* __restrict__ part, unsigned* __restrict__ status, uint64_t wait_ns) {
+    constexpr int SPT = (GV_JMAX * MR + GV_T - 1) / GV_T;   // staged entries per consumer thread
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = align1024(smem_raw);
-    float* shi = (float*)(smem + GV_STAGES * GV_STAGE_BYTES);   // [jj][8] high parts of b
-    float* slo = shi + GV_JMAX * GV_MR;                          // [jj][8] low parts
-    uint64_t* full = (uint64_t*)(slo + GV_JMAX * GV_MR);
+    float* shi = (float*)(smem + GV_STAGES * GV_STAGE_BYTES);   // [jj][MR] high parts of b
+    float* slo = shi + GV_JMAX * MR;                          // [jj][MR] low parts
+    uint64_t* full = (uint64_t*)(slo + GV_JMAX * MR);
     uint64_t* empty = full + GV_STAGES;
     volatile int* abort = (volatile int*)(empty + GV_STAGES);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int64_t i0 = (int64_t)blockIdx.x * GV_BC;
-    const int split = blockIdx.y, r0 = blockIdx.z * GV_MR;
-    const int mm = min(GV_MR, m - r0);
+    const int split = blockIdx.y, r0 = blockIdx.z * MR;
+    const int mm = min(MR, m - r0);
     const int64_t jb = (int64_t)split * jchunk, je = min(n, jb + jchunk);
     const int nrow = (int)max((int64_t)0, je - jb);
     const int nst = (nrow + GV_RJ - 1) / GV_RJ;
@@ -131,31 +136,31 @@ __global__ void __launch_bounds__(GV_T + 32, 2)
     const int64_t ic = i0 + GV_CPT * tid;
     const bool live = ic < n;   // n is a multiple of 4: a thread's columns are all in range or all out
     {
-        float2 v[GV_SPT];
+        float2 v[SPT];
 #pragma unroll
-        for (int k = 0; k < GV_SPT; ++k) {
+        for (int k = 0; k < SPT; ++k) {
             const int e = tid + GV_T * k, t = e / GV_JMAX, jj = e % GV_JMAX;
             v[k] = (t < mm && jj < nrow) ? bv[(int64_t)(r0 + t) * n + jb + jj] : make_float2(0.f, 0.f);
         }
 #pragma unroll
-        for (int k = 0; k < GV_SPT; ++k) {
+        for (int k = 0; k < SPT; ++k) {
             const int e = tid + GV_T * k, t = e / GV_JMAX, jj = e % GV_JMAX;
-            if (t < GV_MR) {
-                shi[jj * GV_MR + t] = v[k].x;
-                slo[jj * GV_MR + t] = v[k].y;
+            if (t < MR) {
+                shi[jj * MR + t] = v[k].x;
+                slo[jj * MR + t] = v[k].y;
             }
         }
     }
     // beta_r = bh of this thread's first column, as replica pairs
-    uint64_t beta[GV_MR / 2];
+    uint64_t beta[MR / 2];
 #pragma unroll
-    for (int h = 0; h < GV_MR / 2; ++h) {
+    for (int h = 0; h < MR / 2; ++h) {
         const int ta = 2 * h, tb = 2 * h + 1;
         beta[h] = pk2((ta < mm && live) ? bv[(int64_t)(r0 + ta) * n + ic].x : 0.f,
                       (tb < mm && live) ? bv[(int64_t)(r0 + tb) * n + ic].x : 0.f);
     }
     asm volatile("bar.sync 1, %0;" ::"n"(GV_T) : "memory");
-    Kahan2 acc[GV_CPT][GV_MR / 2], rsum[GV_CPT / 2];
+    Kahan2 acc[GV_CPT][MR / 2], rsum[GV_CPT / 2];
     // this thread's 16-byte run of a staged row: box (4 tid) / 256, offset (4 tid) % 256
     const uint32_t col_off = (uint32_t)((GV_CPT * tid / 256) * (GV_STAGE_BYTES / 2) + (GV_CPT * tid % 256) * 4);
     bool ok = true;
@@ -164,30 +169,36 @@ __global__ void __launch_bounds__(GV_T + 32, 2)
         if (!mbar_wait(&full[s], (t / GV_STAGES) & 1, abort, wait_ns)) { ok = false; break; }
         const uint8_t* st = smem + s * GV_STAGE_BYTES + col_off;
         const int rows = min(GV_RJ, nrow - t * GV_RJ);
-        uint64_t tile[GV_CPT][GV_MR / 2], rs[GV_CPT / 2] = {0ull, 0ull};
+        uint64_t tile[GV_CPT][MR / 2], rs[GV_CPT / 2] = {0ull, 0ull};
 #pragma unroll
         for (int c = 0; c < GV_CPT; ++c)
 #pragma unroll
-            for (int h = 0; h < GV_MR / 2; ++h) tile[c][h] = 0ull;
+            for (int h = 0; h < MR / 2; ++h) tile[c][h] = 0ull;
 #pragma unroll 2
         for (int u = 0; u < rows; ++u) {
             const float4 s4 = *reinterpret_cast<const float4*>(st + u * 256 * 4);   // S_j,i0 .. S_j,i0+3
             const int jj = t * GV_RJ + u;
-            const float4 h0 = *reinterpret_cast<const float4*>(shi + jj * GV_MR);
-            const float4 h1 = *reinterpret_cast<const float4*>(shi + jj * GV_MR + 4);
-            const float4 l0 = *reinterpret_cast<const float4*>(slo + jj * GV_MR);
-            const float4 l1 = *reinterpret_cast<const float4*>(slo + jj * GV_MR + 4);
-            const uint64_t hp[4] = {pk2(h0.x, h0.y), pk2(h0.z, h0.w), pk2(h1.x, h1.y), pk2(h1.z, h1.w)};
-            const uint64_t lp[4] = {pk2(l0.x, l0.y), pk2(l0.z, l0.w), pk2(l1.x, l1.y), pk2(l1.z, l1.w)};
-            uint64_t d[GV_MR / 2];
+            uint64_t hp[MR / 2], lp[MR / 2], d[MR / 2];
+            if (MR == 2) {
+                hp[0] = *reinterpret_cast<const uint64_t*>(shi + jj * MR);
+                lp[0] = *reinterpret_cast<const uint64_t*>(slo + jj * MR);
+            } else {
 #pragma unroll
-            for (int h = 0; h < GV_MR / 2; ++h) d[h] = add2(sub2(hp[h], beta[h]), lp[h]);
+                for (int h = 0; h < MR / 4; ++h) {
+                    const float4 hv = *reinterpret_cast<const float4*>(shi + jj * MR + 4 * h);
+                    const float4 lv = *reinterpret_cast<const float4*>(slo + jj * MR + 4 * h);
+                    hp[2 * h] = pk2(hv.x, hv.y); hp[2 * h + 1] = pk2(hv.z, hv.w);
+                    lp[2 * h] = pk2(lv.x, lv.y); lp[2 * h + 1] = pk2(lv.z, lv.w);
+                }
+            }
+#pragma unroll
+            for (int h = 0; h < MR / 2; ++h) d[h] = add2(sub2(hp[h], beta[h]), lp[h]);
             const float sc[GV_CPT] = {s4.x, s4.y, s4.z, s4.w};
 #pragma unroll
             for (int c = 0; c < GV_CPT; ++c) {
                 const uint64_t sp = pk2(sc[c], sc[c]);
 #pragma unroll
-                for (int h = 0; h < GV_MR / 2; ++h) tile[c][h] = fma2(sp, d[h], tile[c][h]);
+                for (int h = 0; h < MR / 2; ++h) tile[c][h] = fma2(sp, d[h], tile[c][h]);
             }
             rs[0] = add2(rs[0], pk2(s4.x, s4.y));
             rs[1] = add2(rs[1], pk2(s4.z, s4.w));
@@ -197,7 +208,7 @@ __global__ void __launch_bounds__(GV_T + 32, 2)
 #pragma unroll
         for (int c = 0; c < GV_CPT; ++c)
 #pragma unroll
-            for (int h = 0; h < GV_MR / 2; ++h) acc[c][h].add(tile[c][h]);
+            for (int h = 0; h < MR / 2; ++h) acc[c][h].add(tile[c][h]);
         rsum[0].add(rs[0]);
         rsum[1].add(rs[1]);
     }
@@ -216,7 +227,7 @@ __global__ void __launch_bounds__(GV_T + 32, 2)
         rsc[3] = df_norm(s23.y, -c23.y);
     }
 #pragma unroll
-    for (int t = 0; t < GV_MR; ++t) {
+    for (int t = 0; t < MR; ++t) {
         if (t >= mm) continue;
         const float2* br = bv + (int64_t)(r0 + t) * n + ic;
         const float bt = br[0].x;   // beta_t
@@ -241,7 +252,8 @@ bool gemv_tma_supported(const cpm_ctx* c) { return c->p.s_prec == CPM_PREC_FP32 
 
 void gemv_tma_plan(int64_t n, int m, int64_t* colblocks, int64_t* splits, int64_t* jchunk) {
     *colblocks = (n + GV_BC - 1) / GV_BC;
-    const int64_t rchunks = (m + GV_MR - 1) / GV_MR;
+    const int mr = gv_mr(m);
+    const int64_t rchunks = (m + mr - 1) / mr;
     // one wave: two blocks per SM
     int64_t sp = std::max<int64_t>(1, 2 * 152 / (*colblocks * rchunks));
     sp = std::max<int64_t>(sp, (n + GV_JMAX - 1) / GV_JMAX);
@@ -267,9 +279,15 @@ cpm_status gemv_tma(cpm_ctx* c, int m, const float2* bhl, float2* part, int64_t 
     int64_t colblocks, sp, jc;
     gemv_tma_plan(n, m, &colblocks, &sp, &jc);
     if (sp != splits || jc != jchunk) return set_err(c, CPM_E_STATE, "gemv_tma: plan mismatch");
-    CPM_CUDA(c, cudaFuncSetAttribute(k_gemv_tma, cudaFuncAttributeMaxDynamicSharedMemorySize, GV_SMEM));
-    const dim3 grid((unsigned)colblocks, (unsigned)splits, (unsigned)((m + GV_MR - 1) / GV_MR));
-    k_gemv_tma<<<grid, GV_T + 32, GV_SMEM, c->stream>>>(smap, bhl, n, m, jchunk, part, c->status, GV_WAIT_NS);
+    const int mr = gv_mr(m);
+    const dim3 grid((unsigned)colblocks, (unsigned)splits, (unsigned)((m + mr - 1) / mr));
+    auto launch = [&](auto kern) {
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, gv_smem(mr));
+        if (e == cudaSuccess)
+            kern<<<grid, GV_T + 32, gv_smem(mr), c->stream>>>(smap, bhl, n, m, jchunk, part, c->status, GV_WAIT_NS);
+        return e;
+    };
+    CPM_CUDA(c, mr == 2 ? launch(k_gemv_tma<2>) : mr == 4 ? launch(k_gemv_tma<4>) : launch(k_gemv_tma<8>));
     CPM_LAUNCH(c, "k_gemv_tma");
     return CPM_OK;
 }
