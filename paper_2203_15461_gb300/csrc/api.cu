@@ -143,7 +143,7 @@ static void free_geometry(cpm_ctx* c) {
                     c->sperm, c->schunks, c->rqueue, c->tcz, c->tcxy, c->c0e, c->c0tab, c->ccm_buf, c->ccm_scr, c->SGx,
                     c->h2d_idx, c->h2d_norm, c->rsite, c->rsite_tab, c->rrun_cell, c->rrun_sh,
                     c->rchunk, c->rsite_idx, c->rbox, c->r64tab, c->tc_gperm, c->p3m_zlist,
-                    c->p3m_need};
+                    c->p3m_need, c->p3m_base, c->p3m_lb, c->p3m_w32, c->p3m_lw32, c->p3m_w64, c->p3m_lw64};
     for (void* p : ptrs) dev_free(c, p);
     c->sx = nullptr; c->group = nullptr; c->s32 = nullptr; c->sxyz = nullptr;
     c->zmap = nullptr; c->zuniq = nullptr; c->nzu = 0;
@@ -156,7 +156,8 @@ static void free_geometry(cpm_ctx* c) {
     c->rsite = nullptr; c->rsite_tab = nullptr; c->rpoly = cpm::RealPoly{}; c->rpoly_blocks = 0;
     c->rrun_cell = nullptr; c->rrun_sh = nullptr; c->rchunk = nullptr; c->rrun_stride = 0;
     c->rsite_idx = nullptr; c->rbox = nullptr; c->r64tab = nullptr; c->r64n = 0;
-    c->tc_gperm = nullptr; c->p3m_zlist = nullptr; c->p3m_need = nullptr; c->p3m_nz = 0;
+    c->tc_gperm = nullptr; c->p3m_zlist = nullptr; c->p3m_need = nullptr; c->p3m_nz = c->p3m_nl = 0;
+    c->p3m_base = c->p3m_lb = nullptr; c->p3m_w32 = c->p3m_lw32 = nullptr; c->p3m_w64 = c->p3m_lw64 = nullptr;
     c->site64 = Phases<double>{}; c->site32 = Phases<float>{};
     c->A = c->W = c->S = c->SG = c->u = c->dvec = nullptr;
     c->S32 = nullptr;

@@ -342,6 +342,10 @@ struct cpm_ctx {
     int* p3m_zlist = nullptr;    // mesh planes that the interpolation at the sites reads, and a mark per plane
     unsigned char* p3m_need = nullptr;
     int p3m_nz = 0;
+    int p3m_nl = 0;              // > 0: the sites share this many heights, one transformed plane each
+    int *p3m_base = nullptr, *p3m_lb = nullptr;          // [n][2], [nzu] first mesh index of the sites (x, y) and heights
+    float *p3m_w32 = nullptr, *p3m_lw32 = nullptr;       // [n][2][8], [nzu][8] their weights
+    double *p3m_w64 = nullptr, *p3m_lw64 = nullptr;
     void* p3m_G64 = nullptr;     // the same in FP64 for the P3M elastance when k_prec is single precision
     void* p3m_tw64 = nullptr;
 

@@ -28,6 +28,11 @@
 //   the reciprocal-space product never leaves shared memory.
 // * Interpolation: one warp per (site, replica pair); lanes take the p^2 (x, y) columns, each runs
 //   over the p z points; the warp sum is a fixed butterfly.
+//   Sites that share few heights (at most one per LAYER_MIN_SITES sites, as in the product basis): the z pass
+//   applies each height's z weights while the line is in shared memory, the inverse xy transform runs on one plane
+//   per height instead of on every plane a stencil reads, and a site sums p^2 points with weights kept since the
+//   preparation.  Inverse xy transform and interpolation together: 4,320 sites x 8 replicas, 128 mesh planes,
+//   29 -> 14 us; 16,384 sites x 16 replicas, 64 planes, 141 -> 43 us.
 // Arithmetic in T = double (k_prec = FP64) or float (the single-precision paths); the influence
 // function is computed in FP64 and stored in T.
 #include "common.cuh"
@@ -262,37 +267,42 @@ __global__ void __launch_bounds__(P3M_NT) k_p3m_spread(const int* __restrict__ k
             const T wyz = in ? q * w[P + b] * w[2 * P + c] : (T)0;
             const int ox = o & 1023;
             int* row = A + zz * PS + gy * RX;
-            const bool small = fabs(q) <= (T)2;          // warp-uniform
+            // v = hi 2^-20 + lo 2^-40 (+ lo2 2^-60): exact splits of the scaled contribution
+            if (std::is_same<T, float>::value && fabs(q) <= (T)2 && ox + P <= BX) {
+                // the usual case, uniform in the warp: no wrap or clipping in x, and |v| 2^20 < 2^22, so that
+                // adding 1.5 2^23 rounds without a conversion instruction; index arithmetic of the general branch
+                // taken out, 16,384 sites x 16 replicas of 32,768 charges: 656 -> 538 us
+                const float s20 = (float)wyz * 1048576.0f;
+                int* r0 = row + ox;
 #pragma unroll
-            for (int a = 0; a < P; ++a) {
-                int gx = ox + a;
-                if (gx >= Kx) gx -= Kx;
-                if (gx >= BX) continue;                  // uniform
-                // v = hi 2^-20 + lo 2^-40 (+ lo2 2^-60): exact splits of the scaled contribution
-                if (std::is_same<T, double>::value) {
-                    if (!in) continue;
-                    const double x = (double)(wyz * w[a]) * 1048576.0;   // 2^20
-                    const double h = floor(x);
-                    const double y = (x - h) * 1048576.0;
-                    const double l = floor(y);
-                    atomicAdd(&row[gx], (int)h);
-                    atomicAdd(&row[NB + gx], (int)l);
-                    atomicAdd(&row[2 * NB + gx], __double2int_rn((y - l) * 1048576.0));
-                } else {
-                    const float x = (float)(wyz * w[a]) * 1048576.0f;
-                    int hi, lo;
-                    if (small) {   // |x| < 2^22: rounding by adding 1.5 2^23, no conversion instructions
-                        const float t = x + 12582912.0f;
-                        hi = __float_as_int(t) - 0x4B400000;
-                        lo = __float_as_int(fmaf(x - (t - 12582912.0f), 1048576.0f, 12582912.0f)) - 0x4B400000;
-                    } else {
-                        const float h = floorf(x);
-                        hi = (int)h;
-                        lo = __float2int_rn((x - h) * 1048576.0f);
-                    }
+                for (int a = 0; a < P; ++a) {
+                    const float x = s20 * (float)w[a];
+                    const float t = x + 12582912.0f;
+                    const float l = fmaf(x - (t - 12582912.0f), 1048576.0f, 12582912.0f);
                     if (in) {
-                        atomicAdd(&row[gx], hi);
-                        atomicAdd(&row[NB + gx], lo);
+                        atomicAdd(&r0[a], __float_as_int(t) - 0x4B400000);
+                        atomicAdd(&r0[NB + a], __float_as_int(l) - 0x4B400000);
+                    }
+                }
+            } else if (in) {
+#pragma unroll
+                for (int a = 0; a < P; ++a) {
+                    int gx = ox + a;
+                    if (gx >= Kx) gx -= Kx;
+                    if (gx >= BX) continue;                  // uniform
+                    if (std::is_same<T, double>::value) {
+                        const double x = (double)(wyz * w[a]) * 1048576.0;   // 2^20
+                        const double h = floor(x);
+                        const double y = (x - h) * 1048576.0;
+                        const double l = floor(y);
+                        atomicAdd(&row[gx], (int)h);
+                        atomicAdd(&row[NB + gx], (int)l);
+                        atomicAdd(&row[2 * NB + gx], __double2int_rn((y - l) * 1048576.0));
+                    } else {
+                        const float x = (float)(wyz * w[a]) * 1048576.0f;
+                        const float h = floorf(x);
+                        atomicAdd(&row[gx], (int)h);
+                        atomicAdd(&row[NB + gx], __float2int_rn((x - h) * 1048576.0f));
                     }
                 }
             }
@@ -403,7 +413,8 @@ __global__ void __launch_bounds__(P3M_THREADS) k_p3m_plane(c2<T>* __restrict__ m
 template <typename T>
 __global__ void __launch_bounds__(P3M_THREADS) k_p3m_zline(c2<T>* __restrict__ mesh, int Kx, int Ky, int Kz, int tx,
                                                           const T* __restrict__ G, const c2<T>* __restrict__ twz,
-                                                          const unsigned char* __restrict__ need) {
+                                                          const unsigned char* __restrict__ need, int nl,
+                                                          const int* __restrict__ lb, const T* __restrict__ lw, int P) {
     extern __shared__ __align__(16) unsigned char p3m_smem[];
     c2<T>* ln = (c2<T>*)p3m_smem;
     c2<T>* tw = ln + Kz * tx;
@@ -438,7 +449,20 @@ __global__ void __launch_bounds__(P3M_THREADS) k_p3m_zline(c2<T>* __restrict__ m
     dit_stages<T>(ln, Kz, lz, tx, 1, tx, tw);
     for (int i = threadIdx.x; i < Kz * tx; i += P3M_THREADS) {
         const int z = i / tx, x = i - z * tx;
-        if (need[z]) g[z * plane + x] = ln[i];
+        if (nl == 0 && need[z]) g[z * plane + x] = ln[i];
+    }
+    // sites of few heights: the z weights of each height applied here, before the inverse xy transform, which then
+    // has nl planes (stored as planes 0 .. nl - 1 of this line's own column)
+    for (int i = threadIdx.x; i < nl * tx; i += P3M_THREADS) {
+        const int u = i / tx, x = i - u * tx, b = lb[u];
+        T re = 0, im = 0;
+        for (int a = 0; a < P; ++a) {
+            const c2<T> v = ln[((b + a) & (Kz - 1)) * tx + x];
+            const T w = lw[8 * u + a];
+            re += w * v.x;
+            im += w * v.y;
+        }
+        g[u * plane + x] = cmake<T>(re, im);
     }
 }
 
@@ -486,6 +510,70 @@ __global__ void __launch_bounds__(P3M_THREADS) k_p3m_interp(const double* __rest
             const T ww = wxy * sw[wid][2][c];
             re += ww * v.x;
             im += ww * v.y;
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        re += __shfl_xor_sync(0xffffffffu, re, o);
+        im += __shfl_xor_sync(0xffffffffu, im, o);
+    }
+    if (lane == 0) {
+        pm[(int64_t)(2 * pair) * n + i] = (double)re;
+        if (2 * pair + 1 < m) pm[(int64_t)(2 * pair + 1) * n + i] = (double)im;
+    }
+}
+
+// The fixed interpolation of the sites: per point (site or height) and axis the first mesh index and the P weights.
+// axes x and y: base[2 i + d], w[8 (2 i + d) + a]; heights (axis 2): base[u], w[8 u + a].
+template <typename T, int P>
+__global__ void k_p3m_weights(const double* __restrict__ x, int64_t cnt, int64_t stride, int naxes, Geometry g, int Kx,
+                              int Ky, int Kz, int axis0, int* __restrict__ base, T* __restrict__ w) {
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= cnt * naxes) return;
+    const int64_t i = t / naxes;
+    const int d = axis0 + (int)(t % naxes);
+    const int K = d == 0 ? Kx : (d == 1 ? Ky : Kz);
+    double s = x[(int64_t)(d - axis0) * stride + i] * (d == 0 ? g.inv[0] : d == 1 ? g.inv[1] : g.inv[2]);
+    s -= floor(s);
+    const double u = s * K - 0.5 * P;
+    const double fl = floor(u);
+    int bi = ((int)fl + 1) % K;
+    if (bi < 0) bi += K;
+    base[t] = bi;
+    T wt[P];
+    bspline_weights<T, P>((T)(u - fl), wt);
+#pragma unroll
+    for (int a = 0; a < 8; ++a) w[8 * t + a] = a < P ? wt[a] : (T)0;
+}
+
+// Sites of few heights: one warp per (site, replica pair) over the P x P points of its height's plane, lane =
+// (x offset, y offset modulo 4); the weights, fixed with the geometry, are read, not formed (each warp of
+// k_p3m_interp spends more instructions on them than on the sum).
+template <typename T>
+__global__ void __launch_bounds__(P3M_THREADS) k_p3m_interp2(const int* __restrict__ zmap, const int* __restrict__ base,
+                                                            const T* __restrict__ w, int64_t n, int m, int P, int Kx,
+                                                            int Ky, int Kz, const c2<T>* __restrict__ mesh,
+                                                            double* __restrict__ pm) {
+    const int lane = threadIdx.x & 31;
+    const int64_t wid = (int64_t)blockIdx.x * (P3M_THREADS / 32) + (threadIdx.x >> 5);
+    if (wid >= n * ((m + 1) / 2)) return;
+    const int64_t i = wid % n;
+    const int pair = (int)(wid / n);
+    const c2<T>* ph = mesh + ((int64_t)pair * Kz + zmap[i]) * Kx * Ky;
+    const int bx = base[2 * i], by = base[2 * i + 1], a = lane & 7, b = lane >> 3;
+    const int gx = (bx + a) & (Kx - 1);
+    const T wx = w[16 * i + a], w0 = w[16 * i + 8 + b], w1 = w[16 * i + 12 + b];   // zero from P on
+    T re = 0, im = 0;
+    if (a < P) {
+        if (b < P) {
+            const c2<T> v = ph[(int64_t)((by + b) & (Ky - 1)) * Kx + gx];
+            re = wx * w0 * v.x;
+            im = wx * w0 * v.y;
+        }
+        if (b + 4 < P) {
+            const c2<T> v = ph[(int64_t)((by + b + 4) & (Ky - 1)) * Kx + gx];
+            re += wx * w1 * v.x;
+            im += wx * w1 * v.y;
         }
     }
 #pragma unroll
@@ -559,23 +647,56 @@ static cpm_status p3m_prepare_t(cpm_ctx* c, void** Gp, void** twp) {
     return CPM_OK;
 }
 
-// the planes that the interpolation at the sites reads (one more on either side of each stencil, so that no
-// rounding of the origin can matter)
+template <typename T, int P>
+static cpm_status p3m_weights_p(cpm_ctx* c, T** w, T** lw) {
+    const int Kx = c->p.p3m_mesh[0], Ky = c->p.p3m_mesh[1], Kz = c->p.p3m_mesh[2];
+    CPM_TRY(dev_alloc(c, (void**)w, sizeof(T) * 16 * c->n));
+    CPM_TRY(dev_alloc(c, (void**)lw, sizeof(T) * 8 * c->nzu));
+    k_p3m_weights<T, P><<<(unsigned)((2 * c->n + 127) / 128), 128, 0, c->stream>>>(c->sx, c->n, c->n, 2, c->g, Kx, Ky, Kz, 0,
+                                                                                  c->p3m_base, *w);
+    k_p3m_weights<T, P><<<(unsigned)((c->nzu + 127) / 128), 128, 0, c->stream>>>(c->zuniq, c->nzu, 0, 1, c->g, Kx, Ky, Kz, 2,
+                                                                                c->p3m_lb, *lw);
+    CPM_LAUNCH(c, "k_p3m_weights");
+    return CPM_OK;
+}
+template <typename T> static cpm_status p3m_weights(cpm_ctx* c, T** w, T** lw) {
+    switch (c->p.p3m_order) {
+        case 2: return p3m_weights_p<T, 2>(c, w, lw);
+        case 3: return p3m_weights_p<T, 3>(c, w, lw);
+        case 4: return p3m_weights_p<T, 4>(c, w, lw);
+        case 5: return p3m_weights_p<T, 5>(c, w, lw);
+        case 6: return p3m_weights_p<T, 6>(c, w, lw);
+        default: return p3m_weights_p<T, 7>(c, w, lw);
+    }
+}
+
+// What the inverse transform has to give.  Sites that share few heights (as in recip_rows.cu): one plane per
+// height.  Otherwise the planes that the interpolation at the sites reads (one more on either side of each
+// stencil, so that no rounding of the origin can matter).
 static cpm_status p3m_planes(cpm_ctx* c) {
     const int Kz = c->p.p3m_mesh[2], P = c->p.p3m_order;
-    std::vector<double> zu(c->nzu);
-    CPM_CUDA(c, cudaMemcpyAsync(zu.data(), c->zuniq, sizeof(double) * zu.size(), cudaMemcpyDeviceToHost, c->stream));
-    CPM_CUDA(c, cudaStreamSynchronize(c->stream));
     std::vector<unsigned char> need(Kz, 0);
-    for (double z : zu) {
-        double s = z * c->g.inv[2];
-        s -= std::floor(s);
-        const int b = (int)std::floor(s * Kz - 0.5 * P);
-        for (int a = 0; a < P + 2; ++a) need[((b + a) % Kz + Kz) % Kz] = 1;
-    }
     std::vector<int> list;
-    for (int z = 0; z < Kz; ++z)
-        if (need[z]) list.push_back(z);
+    c->p3m_nl = (int64_t)c->nzu * LAYER_MIN_SITES <= c->n && c->nzu <= Kz ? c->nzu : 0;
+    if (c->p3m_nl) {
+        for (int u = 0; u < c->nzu; ++u) list.push_back(u);
+        CPM_TRY(dev_alloc(c, (void**)&c->p3m_base, sizeof(int) * 2 * c->n));
+        CPM_TRY(dev_alloc(c, (void**)&c->p3m_lb, sizeof(int) * c->nzu));
+        if (c->p.k_prec != CPM_PREC_FP64) CPM_TRY(p3m_weights<float>(c, &c->p3m_w32, &c->p3m_lw32));
+        if (c->p.k_prec == CPM_PREC_FP64 || c->p.p3m_matrix) CPM_TRY(p3m_weights<double>(c, &c->p3m_w64, &c->p3m_lw64));
+    } else {
+        std::vector<double> zu(c->nzu);
+        CPM_CUDA(c, cudaMemcpyAsync(zu.data(), c->zuniq, sizeof(double) * zu.size(), cudaMemcpyDeviceToHost, c->stream));
+        CPM_CUDA(c, cudaStreamSynchronize(c->stream));
+        for (double z : zu) {
+            double s = z * c->g.inv[2];
+            s -= std::floor(s);
+            const int b = (int)std::floor(s * Kz - 0.5 * P);
+            for (int a = 0; a < P + 2; ++a) need[((b + a) % Kz + Kz) % Kz] = 1;
+        }
+        for (int z = 0; z < Kz; ++z)
+            if (need[z]) list.push_back(z);
+    }
     CPM_TRY(dev_alloc(c, (void**)&c->p3m_need, Kz));
     CPM_TRY(dev_alloc(c, (void**)&c->p3m_zlist, sizeof(int) * list.size()));
     CPM_CUDA(c, cudaMemcpyAsync(c->p3m_need, need.data(), Kz, cudaMemcpyHostToDevice, c->stream));
@@ -584,6 +705,12 @@ static cpm_status p3m_planes(cpm_ctx* c) {
     c->p3m_nz = (int)list.size();
     return CPM_OK;
 }
+template <typename T> static const T* p3m_site_w(const cpm_ctx* c);
+template <> const float* p3m_site_w<float>(const cpm_ctx* c) { return c->p3m_w32; }
+template <> const double* p3m_site_w<double>(const cpm_ctx* c) { return c->p3m_w64; }
+template <typename T> static const T* p3m_height_w(const cpm_ctx* c);
+template <> const float* p3m_height_w<float>(const cpm_ctx* c) { return c->p3m_lw32; }
+template <> const double* p3m_height_w<double>(const cpm_ctx* c) { return c->p3m_lw64; }
 
 cpm_status p3m_prepare(cpm_ctx* c) {
     CPM_TRY(p3m_planes(c));
@@ -624,12 +751,17 @@ static cpm_status launch_p3m_pp(cudaStream_t st, cpm_ctx* c, int m, int64_t ne, 
     const size_t zsm = sizeof(c2<T>) * ((size_t)Kz * tx + Kz / 2);
     CPM_CUDA(c, cudaFuncSetAttribute(k_p3m_zline<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)zsm));
     k_p3m_zline<T><<<dim3(Kx / tx, Ky, npairs), P3M_THREADS, zsm, st>>>(mesh, Kx, Ky, Kz, tx, p3m_green<T>(c),
-                                                                        tw + Kx / 2 + Ky / 2, c->p3m_need);
+                                                                        tw + Kx / 2 + Ky / 2, c->p3m_need, c->p3m_nl,
+                                                                        c->p3m_lb, p3m_height_w<T>(c), P);
     k_p3m_plane<T, true><<<dim3(c->p3m_nz, npairs), P3M_THREADS, psm, st>>>(mesh, Kx, Ky, Kz, tw, tw + Kx / 2, 1, 0, m,
                                                                             sp.BX, sp.BY, nullptr, c->p3m_zlist);
     const int64_t warps = c->n * npairs;
-    k_p3m_interp<T, P><<<(unsigned)((warps + P3M_THREADS / 32 - 1) / (P3M_THREADS / 32)), P3M_THREADS, 0, st>>>(
-        c->sx, c->n, m, c->g, Kx, Ky, Kz, mesh, pm);
+    if (c->p3m_nl)
+        k_p3m_interp2<T><<<(unsigned)((warps + P3M_THREADS / 32 - 1) / (P3M_THREADS / 32)), P3M_THREADS, 0, st>>>(
+            c->zmap, c->p3m_base, p3m_site_w<T>(c), c->n, m, P, Kx, Ky, Kz, mesh, pm);
+    else
+        k_p3m_interp<T, P><<<(unsigned)((warps + P3M_THREADS / 32 - 1) / (P3M_THREADS / 32)), P3M_THREADS, 0, st>>>(
+            c->sx, c->n, m, c->g, Kx, Ky, Kz, mesh, pm);
     CPM_LAUNCH(c, "k_p3m (spread, transforms, interpolation)");
     return CPM_OK;
 }

@@ -37,3 +37,21 @@ def test_p3m_assignment(mesh, order, k_prec, tol):
             assert np.abs(b[r]).max() <= tol * np.abs(b[r + 1]).max()
         else:
             assert rel_l2(b[r], o.bvec(el, e)) <= tol, r
+
+
+@pytest.mark.parametrize("k_prec,tol", [("fp64", 1e-12), ("fp32", 2e-6)])
+@pytest.mark.parametrize("sites_per_height", [1, 7, 8, 30])
+def test_p3m_shared_and_single_heights(sites_per_height, k_prec, tol):
+    """Every site on a height of its own (interpolation over the mesh) to whole layers (one plane per height)."""
+    need_gpu()
+    base = s.au111_slab(seed_layers=2, nx=5, ny=6, gap=24.0)
+    first = (np.arange(base.n) // sites_per_height) * sites_per_height
+    xyz = base.xyz.copy()
+    xyz[:, 2] = (base.xyz[:, 2] + 0.2 * np.sin(first * 1.7 + 0.3))[first]
+    el = s.Electrodes(**{**base.__dict__, "xyz": xyz, "p3m_mesh": (32, 16, 64), "p3m_order": 5})
+    elyts = [s.ions_in_gap(el, 40 + 9 * r, seed=60 + r, dmin=2.0) for r in range(3)]
+    ctx = make_ctx(el, k_prec=k_prec)
+    ctx.cpm_prepare(dev(el.xyz), dev(el.eta), dev(el.group, torch.int32), el.n_groups)
+    b = run_bvec(ctx, elyts)
+    for r, e in enumerate(elyts):
+        assert rel_l2(b[r], o.bvec(el, e)) <= tol, r
