@@ -841,17 +841,20 @@ __global__ void __launch_bounds__(C0_THREADS) k_col0(const double* __restrict__ 
     const int chunk = blockIdx.x, r = blockIdx.y;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // a zero charge, also past the end, contributes exact zeros
-    dfl q = {0.f, 0.f};
     dcx e1 = {{1.f, 0.f}, {0.f, 0.f}};
+    double qd = 0.0;
     const int64_t j = (int64_t)chunk * C0_THREADS + threadIdx.x;
     if (j < ne) {
         const int64_t p = (int64_t)r * ne + j;
-        const double qd = Q[p];
-        if (qd != 0.0) {
-            q = df_of(qd);
-            e1 = c0_phase(z_fraction(xyz[3 * p + 2], invLz), tab);
-        }
+        qd = Q[p];
+        if (qd != 0.0) e1 = c0_phase(z_fraction(xyz[3 * p + 2], invLz), tab);
     }
+    // the warp's charges are scaled by a power of two below 2: FP32 pairs hold FP64's range that way
+    int qe = exp_bits(qd);
+    for (int o = 16; o > 0; o >>= 1) qe = max(qe, __shfl_xor_sync(0xffffffffu, qe, o));
+    qe = min(max(qe, 1), 2045);
+    const dfl q = df_of(qd * pow2_bits(2046 - qe));
+    const double unscale = pow2_bits(qe);
     dcx e = {df_mul(q, e1.re), df_mul(q, e1.im)};
     for (int k = 0; k < nz0; ++k) {   // warp sums in double-float, one FP64 value per warp
         dfl re = e.re, im = e.im;
@@ -862,7 +865,7 @@ __global__ void __launch_bounds__(C0_THREADS) k_col0(const double* __restrict__ 
             re = df_add(re, ore);
             im = df_add(im, oim);
         }
-        if (lane == k) red[warp][k] = make_double2((double)re.hi + (double)re.lo, (double)im.hi + (double)im.lo);
+        if (lane == k) red[warp][k] = make_double2(unscale * ((double)re.hi + (double)re.lo), unscale * ((double)im.hi + (double)im.lo));
         e = dcx_mul(e, e1);
     }
     __syncthreads();

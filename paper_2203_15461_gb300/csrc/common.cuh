@@ -118,6 +118,10 @@ __device__ __forceinline__ float pow2_below(float bound, int top) {
     return ldexpf(1.f, top - e);
 }
 
+// biased exponent of |x| (2047: infinity or not a number) and 2^(e - 1023)
+__device__ __forceinline__ int exp_bits(double x) { return (__double2hiint(x) >> 20) & 0x7FF; }
+__device__ __forceinline__ double pow2_bits(int e) { return __hiloint2double(e << 20, 0); }
+
 struct KTable {
     int NX = 0, NY = 0, NZ = 0;
     int ncols = 0, nzw = 0;
