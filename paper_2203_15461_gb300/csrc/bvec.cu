@@ -1058,13 +1058,14 @@ struct BvecPlan {
     bool rows;                          // reciprocal sums in the product basis: on the CUDA cores (rd, recip_rows.cu)
     RowDims rd;                         // or the tensor cores (tc, td, tc_recip.cu)
     TcRecipDims td;
+    Rows64Dims r64;                     // FP64 by integer products (tc_rows64.cu)
     size_t off_EX, off_EY, off_EZ, off_rp, off_wr, off_part, off_real, off_stats, off_key, off_cnt, off_cur,
         off_nzc, off_start, off_wpos, off_sorted, off_order, off_c0part, off_b0, off_T, off_w16, off_ew,
         off_ewT, off_pm, off_p3m, total;
     int c0chunks;
     bool p3m;                           // reciprocal part of b by P3M (p3m.cu)
     bool tc, real64;
-    size_t off_sorted32, off_qmax, off_spart;
+    size_t off_sorted32, off_ipart, off_qmax, off_spart;
 };
 
 template <typename T>
@@ -1083,13 +1084,15 @@ static BvecPlan<T> plan_bvec(const cpm_ctx* c, int m, int64_t ne) {
         p.splits = p.td.splits;
         p.nctiles = p.td.ncb;
     } else if (p.rows) {
+        if (std::is_same<T, double>::value) p.r64 = rows64_dims(c, m, ne);
         p.rd = row_dims<T>(c, m, ne);
         p.cw = p.rd.cw;
-        p.splits = p.rd.splits;
+        p.splits = p.r64.use ? 1 : p.rd.splits;
     }
     if (p.rows && c->rows.layered) p.nctiles = c->rows.nchunk;
     const int64_t ptot = (int64_t)m * ne;
-    const int64_t pph = p.p3m ? 0 : ptot;   // points with electrolyte phase tables (none with P3M)
+    // points with electrolyte phase tables (none with P3M)
+    const int64_t pph = p.p3m ? 0 : p.r64.use ? (int64_t)m * p.r64.nep : ptot;
     const size_t grid = (size_t)k.ncols * k.nzw;
     size_t o = 0;
     if (p.tc) {
@@ -1099,6 +1102,7 @@ static BvecPlan<T> plan_bvec(const cpm_ctx* c, int m, int64_t ne) {
         p.off_EY = o; o += al(sizeof(c2<T>) * (k.NY + 1) * pph);
         p.off_EZ = o; o += al(sizeof(c2<T>) * (k.NZ + 1) * pph);
     }
+    p.off_ipart = o; o += p.r64.use ? al(sizeof(longlong2) * (size_t)p.r64.splits * m * 4 * c->rows.np * p.cw) : 0;
     p.off_rp = p.off_wr = p.off_T = p.off_w16 = o;
     if (p.rows) {
         p.off_rp = o; o += al(sizeof(T) * (size_t)p.splits * m * 4 * c->rows.np * p.cw);
@@ -1174,7 +1178,7 @@ cpm_status bvec_run(cpm_ctx* c, int m, int64_t ne, const double* xyz, const doub
     int* qlast = (int*)(qmax + m);
     float* qsum = (float*)(qlast + m);
     const int nc = m * p.cg.ncells;
-    c->launches += 5 + (ptot > 0 ? 2 : 0) + ((k.nk > 0 && ptot > 0 && !p.p3m) ? 4 + (c->rows.layered || !p.tc ? 0 : 2) : 0);
+    c->launches += 5 + (ptot > 0 ? 2 : 0) + ((k.nk > 0 && ptot > 0 && !p.p3m) ? 4 + (p.r64.use ? 2 : 0) + (c->rows.layered || !p.tc ? 0 : 2) : 0);
 
     // Three chains: the origin stream bins the charges (per-replica totals) and runs the cell list and
     // the real-space sum; side stream 1 takes the phase tables and the reciprocal sums; side stream 2 sums the
@@ -1196,6 +1200,10 @@ cpm_status bvec_run(cpm_ctx* c, int m, int64_t ne, const double* xyz, const doub
         if (p.tc) {
             CPM_TRY(launch_charge_slots(c, s1, m, ne, p.td.nep, xyz, Q, (float2*)EX, qmax, qlast));
             if (!c->rows.layered) CPM_TRY(tc_recip_scales(c, s1, m, ne, Q, qsum));
+        } else if (p.r64.use) {
+            CPM_TRY(launch_qexp(c, s1, m, ne, Q, qlast));
+            CPM_TRY(launch_charge_fixed(c, s1, m, ne, p.r64.nep, xyz, Q, qlast, (longlong2*)EX, (longlong2*)EY,
+                                        (longlong2*)EZ));
         } else {
             CPM_TRY(launch_charge_phases<T>(c, s1, ptot, xyz, Q, EX, EY, EZ));
         }
@@ -1233,6 +1241,9 @@ cpm_status bvec_run(cpm_ctx* c, int m, int64_t ne, const double* xyz, const doub
         const float* qs = p.tc ? qmax : nullptr;
         prof_begin(c, CPM_K_SF);
         if (p.tc) CPM_TRY(tc_recip_sf(c, s1, p.td, m, (const float2*)EX, qmax, qlast, (float*)rp));
+        else if (p.r64.use)
+            CPM_TRY(rows64_sf(c, s1, p.r64, m, (const longlong2*)EX, (const longlong2*)EY, (const longlong2*)EZ, qlast,
+                              (longlong2*)(scr + p.off_ipart), (double*)rp));
         else CPM_TRY(rows_sf<T>(c, s1, p.rd, m, ne, EX, EY, EZ, rp));
         prof_end(c, CPM_K_SF);
         const Phases<T>& sp = site_tables<T>(c);

@@ -143,6 +143,9 @@ constexpr int LAYER_MIN_SITES = 8;     // sites per distinct height from which t
 constexpr int ROW_TC_PAIRS = 64;       // pairs, charges per step and staged x and y harmonics of a CTA of the
 constexpr int ROW_TC_STEP = 64;        // tensor-core structure factor (tc_recip.cu)
 constexpr int ROW_TC_SLOTS = 50;
+constexpr int ROW64_PAIRS = 32, ROW64_HARM = 32, ROW64_STEP = 32;   // the same of the FP64 one (tc_rows64.cu), with its
+                                                                    // harmonics per CTA
+constexpr int ROW64_EMAX = 2044;       // largest biased exponent of a charge that it can scale (|Q| < 2^1022)
 struct RowTable {
     int np = 0, nrows = 0, nslots = 0;   // pairs, rows that are not identically zero, (nx, ny) slots
     int nchunk = 0, ntiles = 0;          // nx ranges and site tiles of the site stage
@@ -164,6 +167,8 @@ struct RowTable {
     int tcitems = 0;                     // work items of the tensor-core structure factor, 0: it does not fit
     int4* tcitem = nullptr;              // (first pair, pairs, harmonic tile, harmonics of the tile)
     int4* tcrange = nullptr;             // (first nx, count, first ny, count) of the item's pairs
+    int items64 = 0;                     // work items of the FP64 structure factor by integer products
+    int4* item64 = nullptr;              // (first pair, pairs, first harmonic, harmonics)
     std::vector<int> hext, hlist;        // host copies: extents of the pairs, the row list
 };
 struct RowDims {
@@ -441,6 +446,10 @@ cpm_status rows_sf(cpm_ctx* c, cudaStream_t st, const RowDims& d, int m, int64_t
 int64_t charge_slots(const KTable& k);
 cpm_status launch_charge_slots(cpm_ctx* c, cudaStream_t st, int m, int64_t ne, int64_t nep, const double* xyz,
                                const double* Q, float2* tab, float* qmax, int* qlast);
+// the same as fixed point, (cos, sin) in 64 bits: x times Q, scaled by a power of two to |Q| < 1 (qexp: the replica's
+// largest exponent), and y times 2^62, z times 2^55
+cpm_status launch_charge_fixed(cpm_ctx* c, cudaStream_t st, int m, int64_t ne, int64_t nep, const double* xyz,
+                               const double* Q, const int* qexp, longlong2* X, longlong2* Y, longlong2* Z);
 // qmax (tensor-core stage 1): part is scaled by 2^14 pow2_below(max |Q|, 14)
 template <typename T>
 cpm_status rows_layers(cpm_ctx* c, cudaStream_t st, int cw, int splits, int m, const T* part, const float* qmax, T* Tbuf);
@@ -540,6 +549,18 @@ cpm_status tc_recip_sf(cpm_ctx* c, cudaStream_t st, const TcRecipDims& d, int m,
 // the site stage of electrodes whose sites hardly share heights, from w rho of the signed columns
 cpm_status tc_recip_sites(cpm_ctx* c, cudaStream_t st, const TcRecipDims& d, int m, const float2* wrho,
                           const float* qsum, void* w16, float* site_partial);
+
+// tc_rows64.cu: the FP64 structure factor by exact integer products on the tensor cores
+struct Rows64Dims {
+    bool use;                           // enough work for it
+    int64_t nep;                        // charges per replica, padded to whole steps
+    int steps, splits, spc, cw;         // steps, charge ranges, steps per range, stored functions per row
+};
+Rows64Dims rows64_dims(const cpm_ctx* c, int m, int64_t ne);
+cpm_status launch_qexp(cpm_ctx* c, cudaStream_t st, int m, int64_t ne, const double* Q, int* qexp);
+// part: as rows_sf with one range; ipart: splits x m x 4 np x cw integer pairs
+cpm_status rows64_sf(cpm_ctx* c, cudaStream_t st, const Rows64Dims& d, int m, const longlong2* X, const longlong2* Y,
+                     const longlong2* Z, const int* qexp, longlong2* ipart, double* part);
 
 // p3m.cu: the reciprocal part of b by P3M (cpm_params.kspace = CPM_KSPACE_P3M)
 constexpr int P3M_MAX_MESH = 512;                 // mesh points per axis (powers of two, at least 8)

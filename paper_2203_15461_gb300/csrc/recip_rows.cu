@@ -67,7 +67,7 @@ __global__ void k_layer_phases(const double* __restrict__ zu, int nzu, double iz
 void free_rows(cpm_ctx* c) {
     RowTable& t = c->rows;
     for (void* p : {(void*)t.pairs, (void*)t.list, (void*)t.W, (void*)t.W32, (void*)t.nxoff, (void*)t.chunkb,
-                    (void*)t.zu64, (void*)t.zu32, (void*)t.lperm, (void*)t.ltiles, (void*)t.colpair, (void*)t.tcitem, (void*)t.atiles,
+                    (void*)t.zu64, (void*)t.zu32, (void*)t.lperm, (void*)t.ltiles, (void*)t.colpair, (void*)t.tcitem, (void*)t.atiles, (void*)t.item64,
                     (void*)t.tcrange})
         dev_free(c, p);
     t = RowTable{};
@@ -150,6 +150,19 @@ cpm_status build_rows(cpm_ctx* c) {
     }
     for (int q = 0; q < k.ncols; ++q)   // the pair of every signed column
         cpair[q] = slotpair[off[cols[q].x] + std::abs(cols[q].y)];
+    if (c->p.k_prec == CPM_PREC_FP64) {
+        std::vector<int4> i64;
+        for (size_t f = 0; f < pairs.size(); f += ROW64_PAIRS) {
+            const size_t e = std::min(pairs.size(), f + ROW64_PAIRS);
+            int mx = 0;
+            for (size_t q = f; q < e; ++q) mx = std::max(mx, pairs[q].z);
+            for (int z = 0; z <= mx; z += ROW64_HARM)
+                i64.push_back(make_int4((int)f, (int)(e - f), z, std::min(ROW64_HARM, mx + 1 - z)));
+        }
+        t.items64 = (int)i64.size();
+        CPM_TRY(upload(c, &t.item64, i64));
+        CPM_CUDA(c, cudaStreamSynchronize(c->stream));
+    }
     t.np = (int)pairs.size();
     t.nrows = (int)list.size();
     t.hext.resize(t.np);
@@ -222,16 +235,19 @@ cpm_status build_rows(cpm_ctx* c) {
 // evaluated phases, so that an axis of H harmonics needs about 8 + H / 8 sincospi and the rest are four
 // multiply-adds (one rounding more than a direct evaluation).  The fractions, FP64 work, are made once per
 // (charge, axis) by three warps: with one per thread the FP64 pipe took 9 us for 45,600 charges.
-// SPLIT (the tensor-core stage): the z phases stay two factors, k = 0..7 and 2^14 times the steps 8 a, which
-// that kernel multiplies itself, and p runs over replicas padded to nep charges.
+// CP_SPLIT (the tensor-core stage): the z phases stay two factors, k = 0..7 and 2^14 times the steps 8 a, which
+// that kernel multiplies itself, and p runs over replicas padded to nep charges; qmax and qlast are written.
+// CP_FIXED (FP64 on the tensor cores): padded as well, written as fixed point; qlast holds the replicas' exponents (k_qexp).
 constexpr int CP_PTS = 32;
-template <typename T, bool SPLIT>
+enum { CP_PLAIN = 0, CP_SPLIT = 1, CP_FIXED = 2 };
+template <typename T, int MODE>
 __global__ void __launch_bounds__(8 * CP_PTS) k_charge_phases(const double* __restrict__ xyz,
                                                               const double* __restrict__ Q, int64_t P, int64_t ne,
                                                               int64_t nep, double ix, double iy, double iz, int NX,
                                                               int NY, int NZ, c2<T>* __restrict__ X,
                                                               c2<T>* __restrict__ Y, c2<T>* __restrict__ Z,
                                                               float* __restrict__ qmax, int* __restrict__ qlast) {
+    constexpr bool SPLIT = MODE == CP_SPLIT;
     __shared__ c2<T> sg[8][CP_PTS];
     __shared__ uint64_t sf[3][CP_PTS];
     __shared__ T sq[CP_PTS];
@@ -241,7 +257,7 @@ __global__ void __launch_bounds__(8 * CP_PTS) k_charge_phases(const double* __re
     if (k < 3) {
         int64_t src = p;
         bool real = live;
-        if (SPLIT) {
+        if (MODE != CP_PLAIN) {
             const int64_t r = p / nep, j = p - r * nep;
             real = live && j < ne;
             src = r * ne + j;
@@ -264,6 +280,7 @@ __global__ void __launch_bounds__(8 * CP_PTS) k_charge_phases(const double* __re
         }
     }
     __syncthreads();
+    const double qs = MODE == CP_FIXED && live ? pow2_bits(2045 - min(max(qlast[p / nep], 1), ROW64_EMAX)) : 1.0;
     for (int axis = 0; axis < 3; ++axis) {
         const int H = axis == 0 ? NX : axis == 1 ? NY : NZ, na = H / 8 + 1;
         c2<T>* out = axis == 0 ? X : axis == 1 ? Y : Z;
@@ -281,7 +298,11 @@ __global__ void __launch_bounds__(8 * CP_PTS) k_charge_phases(const double* __re
             }
             break;
         }
-        if (axis == 0) { base.x *= sq[pt]; base.y *= sq[pt]; }
+        if (axis == 0) {
+            const T q = MODE == CP_FIXED ? (T)(sq[pt] * qs) : sq[pt];
+            base.x *= q;
+            base.y *= q;
+        }
         for (int a0 = 0; a0 < na; a0 += 8) {   // eight steps 8 a at a time
             const int a = a0 + k;
             __syncthreads();
@@ -289,7 +310,14 @@ __global__ void __launch_bounds__(8 * CP_PTS) k_charge_phases(const double* __re
             __syncthreads();
             for (int b = 0; b < min(8, na - a0); ++b) {
                 const int h = 8 * (a0 + b) + k;
-                if (h <= H && live) out[(int64_t)h * P + p] = a0 + b == 0 ? base : cmul(sg[b][pt], base);
+                if (h > H || !live) continue;
+                const c2<T> v = a0 + b == 0 ? base : cmul(sg[b][pt], base);
+                if (MODE == CP_FIXED) {
+                    const double f = axis == 2 ? 0x1p55 : 0x1p62;
+                    ((longlong2*)out)[(int64_t)h * P + p] = make_longlong2(__double2ll_rn((double)v.x * f), __double2ll_rn((double)v.y * f));
+                } else {
+                    out[(int64_t)h * P + p] = v;
+                }
             }
         }
     }
@@ -583,7 +611,7 @@ template <typename T>
 cpm_status launch_charge_phases(cpm_ctx* c, cudaStream_t st, int64_t P, const double* xyz, const double* Q, c2<T>* X,
                                 c2<T>* Y, c2<T>* Z) {
     const KTable& k = c->kt;
-    k_charge_phases<T, false><<<(unsigned)((P + CP_PTS - 1) / CP_PTS), 8 * CP_PTS, 0, st>>>(
+    k_charge_phases<T, CP_PLAIN><<<(unsigned)((P + CP_PTS - 1) / CP_PTS), 8 * CP_PTS, 0, st>>>(
         xyz, Q, P, P, P, c->g.inv[0], c->g.inv[1], c->g.inv[2], k.NX, k.NY, k.NZ, X, Y, Z, nullptr, nullptr);
     CPM_LAUNCH(c, "k_charge_phases");
     return CPM_OK;
@@ -598,9 +626,20 @@ cpm_status launch_charge_slots(cpm_ctx* c, cudaStream_t st, int m, int64_t ne, i
     const KTable& k = c->kt;
     const int64_t P = (int64_t)m * nep;
     float2* Y = tab + (int64_t)(k.NX + 1) * P;
-    k_charge_phases<float, true><<<(unsigned)((P + CP_PTS - 1) / CP_PTS), 8 * CP_PTS, 0, st>>>(
+    k_charge_phases<float, CP_SPLIT><<<(unsigned)((P + CP_PTS - 1) / CP_PTS), 8 * CP_PTS, 0, st>>>(
         xyz, Q, P, ne, nep, c->g.inv[0], c->g.inv[1], c->g.inv[2], k.NX, k.NY, k.NZ, tab, Y, Y + (int64_t)(k.NY + 1) * P,
         qmax, qlast);
+    CPM_LAUNCH(c, "k_charge_phases");
+    return CPM_OK;
+}
+
+cpm_status launch_charge_fixed(cpm_ctx* c, cudaStream_t st, int m, int64_t ne, int64_t nep, const double* xyz,
+                               const double* Q, const int* qexp, longlong2* X, longlong2* Y, longlong2* Z) {
+    const KTable& k = c->kt;
+    const int64_t P = (int64_t)m * nep;
+    k_charge_phases<double, CP_FIXED><<<(unsigned)((P + CP_PTS - 1) / CP_PTS), 8 * CP_PTS, 0, st>>>(
+        xyz, Q, P, ne, nep, c->g.inv[0], c->g.inv[1], c->g.inv[2], k.NX, k.NY, k.NZ, (double2*)X, (double2*)Y, (double2*)Z,
+        nullptr, const_cast<int*>(qexp));
     CPM_LAUNCH(c, "k_charge_phases");
     return CPM_OK;
 }
