@@ -5,7 +5,7 @@
 // for m replicas sharing one capacitance matrix S.  Both operands are split into three bf16
 // terms, S = S0 + S1 + S2 and b = B0 + B1 + B2 (24 significant bits each), and the six
 // products of combined order <= 2 (S0B0, S0B1, S1B0, S0B2, S1B1, S2B0) are accumulated in
-// FP32 in tensor memory, which keeps the single-precision accuracy of S.
+// FP32 in tensor memory (S0B0 apart from the other five), which keeps the single-precision accuracy of S.
 //
 // The product runs as a persistent kernel: a grid of at most one CTA per SM walks a static list
 // of work items (row tile of 128 sites, replica tile of BN, K split), the replica tile varying
@@ -41,7 +41,7 @@ template <int BN, int STAGES> struct TcCfg {
     static constexpr int A_BYTES = TC_BM * 128;            // one bf16 split of the S tile
     static constexpr int B_BYTES = BN * 128;               // one bf16 split of the b tile
     static constexpr int STAGE = 3 * A_BYTES + 3 * B_BYTES;
-    static constexpr int TMEM_COLS = 2 * BN;               // two accumulators
+    static constexpr int TMEM_COLS = 4 * BN;               // two items, two accumulators each
     static constexpr int SMEM = 1024 + STAGES * STAGE + 256;
     static_assert(SMEM <= 227 * 1024, "stage ring exceeds shared memory");
 };
@@ -131,7 +131,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_sb(const __grid_constant__
         }
     } else if (warp == 1) {
         if (lane == 0) {
-            // MMA issuer: item li accumulates into TMEM columns (li & 1) * BN
+            // MMA issuer: item li accumulates S0 B0 into TMEM columns 2 (li & 1) BN and the five smaller products into the
+            // next BN: the tensor core rounds the sum at every step, and the large sum takes a sixth of the steps this way
             const uint32_t idesc = idesc_bf16(TC_BM, BN);
             const int pa[6] = {0, 0, 1, 0, 1, 2};
             const int pb[6] = {0, 1, 0, 2, 1, 0};
@@ -143,7 +144,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_sb(const __grid_constant__
                 const uint32_t acc = li & 1;
                 if (li >= 2 && !mbar_wait(&acce[acc], ((li >> 1) - 1) & 1, abort, wait_ns)) { ok = false; break; }
                 tc_fence_after();
-                const uint32_t dt = tmem + acc * BN;
+                const uint32_t dt = tmem + acc * 2 * BN;
                 for (int t = kb; t < ke; ++t, ++g) {
                     const int s = (int)(g % STAGES);
                     if (!mbar_wait(&full[s], (g / STAGES) & 1, abort, wait_ns)) { ok = false; break; }
@@ -156,7 +157,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_sb(const __grid_constant__
                         for (int p = 0; p < 6; ++p) {
                             const uint64_t ad = sdesc_sw128(sa + pa[p] * C::A_BYTES + kk * 32);
                             const uint64_t bd = sdesc_sw128(sb + pb[p] * C::B_BYTES + kk * 32);
-                            umma_f16(dt, ad, bd, idesc, (t > kb || kk > 0 || p > 0) ? 1u : 0u);
+                            umma_f16(dt + (p > 0 ? BN : 0), ad, bd, idesc, (t > kb || kk > 0 || p > 1) ? 1u : 0u);
                         }
                     }
                     umma_commit(&empty[s]);
@@ -176,17 +177,18 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_sb(const __grid_constant__
             if (!have) break;
             tc_fence_after();
             const int i = row * TC_BM + quarter * 32 + lane;
-            const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16) + acc * BN;
+            const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16) + acc * 2 * BN;
             float* pout = part + (int64_t)split * m * n;
 #pragma unroll
             for (int c0 = 0; c0 < BN; c0 += 16) {
-                float v[16];
+                float v[16], w[16];
                 tmem_ld16(trow + c0, v);
+                tmem_ld16(trow + BN + c0, w);
                 if (i < n) {
 #pragma unroll
                     for (int k = 0; k < 16; ++k) {
                         const int r = rep * BN + c0 + k;
-                        if (r < m) pout[(int64_t)r * n + i] = v[k];
+                        if (r < m) pout[(int64_t)r * n + i] = v[k] + w[k];
                     }
                 }
             }
@@ -476,24 +478,34 @@ __global__ void k_sgroups(const double* __restrict__ S, const int* __restrict__ 
     SZ[t] = a;
 }
 
-// gmean[r][g] = mean of b[r][i] over the sites of group g (perm[off[g]] .. perm[off[g + 1] - 1]); one warp per
-// (r, g), four sums per lane in flight, fixed order
-__global__ void k_gmeans(const double* __restrict__ b, const int* __restrict__ perm, const int* __restrict__ off,
-                         int64_t n, int m, int ngrp, double* __restrict__ gmean) {
-    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (w >= (int64_t)m * ngrp) return;
-    const int r = (int)(w / ngrp), g = (int)(w % ngrp);
+// gmean[r][g] = mean of b[r][i] over the sites of group g (perm[off[g]] .. perm[off[g + 1] - 1]); one block per
+// (g, r), four sums per thread in flight, fixed order.  A chain of two dependent loads: one round of it for 1,024
+// sites (4,320 sites in six groups, 64 replicas: a warp per pair took 12 us, a block 7).
+constexpr int GM_T = 256;
+__global__ void __launch_bounds__(GM_T) k_gmeans(const double* __restrict__ b, const int* __restrict__ perm,
+                                                 const int* __restrict__ off, int64_t n, int ngrp,
+                                                 double* __restrict__ gmean) {
+    __shared__ double sh[GM_T / 32];
+    const int g = blockIdx.x, r = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const double* br = b + (int64_t)r * n;
     const int k0 = off[g], k1 = off[g + 1];
     double a[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int k = k0 + lane; k < k1; k += 128)
+    for (int k = k0 + (int)threadIdx.x; k < k1; k += 4 * GM_T) {
+        int id[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) id[u] = k + GM_T * u < k1 ? perm[k + GM_T * u] : -1;
 #pragma unroll
         for (int u = 0; u < 4; ++u)
-            if (k + 32 * u < k1) a[u] += br[perm[k + 32 * u]];
+            if (id[u] >= 0) a[u] += br[id[u]];
+    }
     double s = (a[0] + a[1]) + (a[2] + a[3]);
     for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if (lane == 0) gmean[w] = k1 > k0 ? s / (k1 - k0) : 0.0;
+    if (lane == 0) sh[warp] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < GM_T / 32; ++w) s += sh[w];
+        gmean[(int64_t)r * ngrp + g] = k1 > k0 ? s / (k1 - k0) : 0.0;
+    }
 }
 
 cpm_status tc_reserve(cpm_ctx* c, int m) {
@@ -550,8 +562,7 @@ cpm_status tc_product(cpm_ctx* c, int m, const double* b, const float** part_out
     void* bsplit = (char*)c->tbuf + c->tc_pbytes;
     double* gmean = (double*)((char*)bsplit + ((tc_bsplit_bytes(n, m) + 255) & ~(size_t)255));
     const int* gid = c->tc_use_z ? c->zmap : c->group;
-    k_gmeans<<<(unsigned)(((int64_t)m * c->tc_ngrp * 32 + 127) / 128), 128, 0, c->stream>>>(b, c->tc_gperm, c->tc_gperm + n, n,
-                                                                                            m, c->tc_ngrp, gmean);
+    k_gmeans<<<dim3((unsigned)c->tc_ngrp, (unsigned)m), GM_T, 0, c->stream>>>(b, c->tc_gperm, c->tc_gperm + n, n, c->tc_ngrp, gmean);
     CPM_LAUNCH(c, "k_gmeans");
     CPM_TRY(tc_sb(c, m, b, part, splits, bsplit, gmean, gid, c->tc_ngrp));
     *part_out = part;
