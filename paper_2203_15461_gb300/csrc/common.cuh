@@ -169,6 +169,7 @@ struct RowTable {
     int4* tcrange = nullptr;             // (first nx, count, first ny, count) of the item's pairs
     int items64 = 0;                     // work items of the FP64 structure factor by integer products
     int4* item64 = nullptr;              // (first pair, pairs, first harmonic, harmonics)
+    longlong2* fxtab = nullptr;          // cos and sin tables of its phases
     std::vector<int> hext, hlist;        // host copies: extents of the pairs, the row list
 };
 struct RowDims {
@@ -291,8 +292,6 @@ struct cpm_ctx {
     int tickets_n = 0;
     float4* c0tab = nullptr;     // double-float cos and sin of 256 angles (k_perp = 0 column)
     double2* c0e = nullptr;      // [nzu][min(ext0, COL0_NZ)] exp(i kz z_u) of the k_perp = 0 column at the sites
-    double* nbuf = nullptr;      // neutrality fix: per-block partial sums of q
-    size_t nbuf_bytes = 0;
     bool assembled = false, inverted = false;
     bool has_A = false;          // A (and the factor workspace W) allocated and valid
     double etd = 0.0;            // e^T A^-1 e (FP64), kept with S

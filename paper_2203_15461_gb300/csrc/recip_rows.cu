@@ -64,10 +64,12 @@ __global__ void k_layer_phases(const double* __restrict__ zu, int nzu, double iz
     ZU[t] = row_phase<T>(row_frac(zu[t % nzu], iz), t / nzu);
 }
 
+static cpm_status charge_fixed_table(cpm_ctx* c);
+
 void free_rows(cpm_ctx* c) {
     RowTable& t = c->rows;
     for (void* p : {(void*)t.pairs, (void*)t.list, (void*)t.W, (void*)t.W32, (void*)t.nxoff, (void*)t.chunkb,
-                    (void*)t.zu64, (void*)t.zu32, (void*)t.lperm, (void*)t.ltiles, (void*)t.colpair, (void*)t.tcitem, (void*)t.atiles, (void*)t.item64,
+                    (void*)t.zu64, (void*)t.zu32, (void*)t.lperm, (void*)t.ltiles, (void*)t.colpair, (void*)t.tcitem, (void*)t.atiles, (void*)t.item64, (void*)t.fxtab,
                     (void*)t.tcrange})
         dev_free(c, p);
     t = RowTable{};
@@ -161,6 +163,7 @@ cpm_status build_rows(cpm_ctx* c) {
         }
         t.items64 = (int)i64.size();
         CPM_TRY(upload(c, &t.item64, i64));
+        CPM_TRY(charge_fixed_table(c));
         CPM_CUDA(c, cudaStreamSynchronize(c->stream));
     }
     t.np = (int)pairs.size();
@@ -236,18 +239,15 @@ cpm_status build_rows(cpm_ctx* c) {
 // multiply-adds (one rounding more than a direct evaluation).  The fractions, FP64 work, are made once per
 // (charge, axis) by three warps: with one per thread the FP64 pipe took 9 us for 45,600 charges.
 // CP_SPLIT (the tensor-core stage): the z phases stay two factors, k = 0..7 and 2^14 times the steps 8 a, which
-// that kernel multiplies itself, and p runs over replicas padded to nep charges; qmax and qlast are written.
-// CP_FIXED (FP64 on the tensor cores): padded as well, written as fixed point; qlast holds the replicas' exponents (k_qexp).
+// that kernel multiplies itself, and p runs over replicas padded to nep charges.
 constexpr int CP_PTS = 32;
-enum { CP_PLAIN = 0, CP_SPLIT = 1, CP_FIXED = 2 };
-template <typename T, int MODE>
+template <typename T, bool SPLIT>
 __global__ void __launch_bounds__(8 * CP_PTS) k_charge_phases(const double* __restrict__ xyz,
                                                               const double* __restrict__ Q, int64_t P, int64_t ne,
                                                               int64_t nep, double ix, double iy, double iz, int NX,
                                                               int NY, int NZ, c2<T>* __restrict__ X,
                                                               c2<T>* __restrict__ Y, c2<T>* __restrict__ Z,
                                                               float* __restrict__ qmax, int* __restrict__ qlast) {
-    constexpr bool SPLIT = MODE == CP_SPLIT;
     __shared__ c2<T> sg[8][CP_PTS];
     __shared__ uint64_t sf[3][CP_PTS];
     __shared__ T sq[CP_PTS];
@@ -257,7 +257,7 @@ __global__ void __launch_bounds__(8 * CP_PTS) k_charge_phases(const double* __re
     if (k < 3) {
         int64_t src = p;
         bool real = live;
-        if (MODE != CP_PLAIN) {
+        if (SPLIT) {
             const int64_t r = p / nep, j = p - r * nep;
             real = live && j < ne;
             src = r * ne + j;
@@ -280,7 +280,6 @@ __global__ void __launch_bounds__(8 * CP_PTS) k_charge_phases(const double* __re
         }
     }
     __syncthreads();
-    const double qs = MODE == CP_FIXED && live ? pow2_bits(2045 - min(max(qlast[p / nep], 1), ROW64_EMAX)) : 1.0;
     for (int axis = 0; axis < 3; ++axis) {
         const int H = axis == 0 ? NX : axis == 1 ? NY : NZ, na = H / 8 + 1;
         c2<T>* out = axis == 0 ? X : axis == 1 ? Y : Z;
@@ -298,11 +297,7 @@ __global__ void __launch_bounds__(8 * CP_PTS) k_charge_phases(const double* __re
             }
             break;
         }
-        if (axis == 0) {
-            const T q = MODE == CP_FIXED ? (T)(sq[pt] * qs) : sq[pt];
-            base.x *= q;
-            base.y *= q;
-        }
+        if (axis == 0) { base.x *= sq[pt]; base.y *= sq[pt]; }
         for (int a0 = 0; a0 < na; a0 += 8) {   // eight steps 8 a at a time
             const int a = a0 + k;
             __syncthreads();
@@ -310,17 +305,89 @@ __global__ void __launch_bounds__(8 * CP_PTS) k_charge_phases(const double* __re
             __syncthreads();
             for (int b = 0; b < min(8, na - a0); ++b) {
                 const int h = 8 * (a0 + b) + k;
-                if (h > H || !live) continue;
-                const c2<T> v = a0 + b == 0 ? base : cmul(sg[b][pt], base);
-                if (MODE == CP_FIXED) {
-                    const double f = axis == 2 ? 0x1p55 : 0x1p62;
-                    ((longlong2*)out)[(int64_t)h * P + p] = make_longlong2(__double2ll_rn((double)v.x * f), __double2ll_rn((double)v.y * f));
-                } else {
-                    out[(int64_t)h * P + p] = v;
-                }
+                if (h <= H && live) out[(int64_t)h * P + p] = a0 + b == 0 ? base : cmul(sg[b][pt], base);
             }
         }
     }
+}
+
+// The same in fixed point (tc_rows64.cu): cos and sin times 2^62 in 64-bit integers, X times the scaled charge, Z
+// rounded to 2^55.  FP64 arithmetic took 34 us for 5,700 charges of 110 harmonics, the integers 9.5 us: the 64-bit
+// product of two phases is some 40 instructions of a pipe with thirty times the rate.  A phase is evaluated as
+// T1[top ten bits] T2[next ten] (1 - d^2 / 2, d - d^3 / 6) with the angle d < 2 pi 2^-20 of the other 44 bits: the
+// terms left out are below 2^-72, T1 is FP64's own cosine and sine, and T2's are kept as 1 - cos, exact to 2^-62.
+constexpr int FX_TAB = 1024;
+__global__ void k_fixed_tab(longlong2* __restrict__ tab) {   // grid 2 x FX_TAB: T1 | T2
+    const int t = threadIdx.x;
+    double s, c;
+    if (blockIdx.x == 0) {
+        sincospi(2.0 * t / FX_TAB, &s, &c);
+        tab[t] = make_longlong2(__double2ll_rn(c * 0x1p62), __double2ll_rn(s * 0x1p62));
+    } else {
+        const double a = t * (1.0 / (FX_TAB * (double)FX_TAB));   // half the angle, in half turns
+        sincospi(a, &s, &c);
+        tab[FX_TAB + t] = make_longlong2((1ll << 62) - __double2ll_rn(2.0 * s * s * 0x1p62), __double2ll_rn(2.0 * s * c * 0x1p62));
+    }
+}
+__device__ __forceinline__ longlong2 fx_mul(longlong2 a, longlong2 b) {   // the floors of the two halves cancel, or cost one
+    return make_longlong2((__mul64hi(a.x, b.x) - __mul64hi(a.y, b.y)) * 4,
+                          (__mul64hi(a.x, b.y) + __mul64hi(a.y, b.x) + 1) * 4);
+}
+__device__ __forceinline__ longlong2 fx_phase(uint64_t f, const longlong2* __restrict__ tab) {
+    const longlong2 b = fx_mul(__ldg(&tab[f >> 54]), __ldg(&tab[FX_TAB + ((f >> 44) & (FX_TAB - 1))]));
+    const uint64_t D = __umul64hi(f << 20, 0x1921FB54442D1846ull);            // d 2^78 = (f mod 2^44) 2 pi 2^14
+    const uint64_t d2 = __umul64hi(D, D);                                     // d^2 2^92
+    const int64_t v4 = (int64_t)(d2 >> 31) * 4;                               // d^2 / 2 times 2^64
+    const int64_t sn = (int64_t)(D - (uint32_t)(__umul64hi(D, d2) >> 28) / 6);   // (d - d^3 / 6) 2^78
+    return make_longlong2(b.x - __mul64hi(b.x, v4) - (__mul64hi(b.y, sn) >> 14),
+                          b.y - __mul64hi(b.y, v4) + (__mul64hi(b.x, sn) >> 14));
+}
+// grid (P / CP_PTS, axis); P and nep are multiples of CP_PTS
+__global__ void __launch_bounds__(8 * CP_PTS) k_charge_fixed(const double* __restrict__ xyz, const double* __restrict__ Q,
+                                                             int64_t P, int64_t ne, int64_t nep, double3 inv, int NX,
+                                                             int NY, int NZ, const int* __restrict__ qexp,
+                                                             const longlong2* __restrict__ tab, longlong2* __restrict__ X,
+                                                             longlong2* __restrict__ Y, longlong2* __restrict__ Z) {
+    __shared__ longlong2 sg[8][CP_PTS];
+    __shared__ uint64_t sf[CP_PTS];
+    __shared__ int64_t sq[CP_PTS];
+    const int pt = threadIdx.x % CP_PTS, k = threadIdx.x / CP_PTS, axis = blockIdx.y;
+    const int64_t p = (int64_t)blockIdx.x * CP_PTS + pt;
+    if (k == 0) {
+        const int64_t r = p / nep, j = p - r * nep, src = r * ne + j;
+        const double q = j < ne ? Q[src] : 0.0;
+        // a zero charge (padding) contributes nothing wherever it sits
+        sf[pt] = q != 0.0 ? row_frac(xyz[3 * src + axis], axis == 0 ? inv.x : axis == 1 ? inv.y : inv.z) : 0ull;
+        sq[pt] = __double2ll_rn(q * pow2_bits(2045 - min(max(qexp[r], 1), ROW64_EMAX)) * 0x1p62);
+    }
+    __syncthreads();
+    const int H = axis == 0 ? NX : axis == 1 ? NY : NZ, na = H / 8 + 1;
+    longlong2* out = axis == 0 ? X : axis == 1 ? Y : Z;
+    const uint64_t f = sf[pt];
+    longlong2 base = make_longlong2(1ll << 62, 0);
+    if (k > 0 && k <= H) base = fx_phase(f * (uint64_t)k, tab);
+    if (axis == 0) base = make_longlong2(__mul64hi(base.x, sq[pt]) * 4 + 2, __mul64hi(base.y, sq[pt]) * 4 + 2);
+    for (int a0 = 0; a0 < na; a0 += 8) {   // eight steps 8 a at a time
+        const int a = a0 + k;
+        __syncthreads();
+        if (a < na && a > 0) sg[k][pt] = fx_phase(f * (uint64_t)(8 * a), tab);
+        __syncthreads();
+        for (int b = 0; b < min(8, na - a0); ++b) {
+            const int h = 8 * (a0 + b) + k;
+            if (h > H) continue;
+            longlong2 v = a0 + b == 0 ? base : fx_mul(sg[b][pt], base);
+            if (axis == 2) v = make_longlong2((v.x + 64) >> 7, (v.y + 64) >> 7);
+            out[(int64_t)h * P + p] = v;
+        }
+    }
+}
+static cpm_status charge_fixed_table(cpm_ctx* c) {
+    dev_free(c, c->rows.fxtab);
+    c->rows.fxtab = nullptr;
+    CPM_TRY(dev_alloc(c, (void**)&c->rows.fxtab, sizeof(longlong2) * 2 * FX_TAB));
+    k_fixed_tab<<<2, FX_TAB, 0, c->stream>>>(c->rows.fxtab);
+    CPM_LAUNCH(c, "k_fixed_tab");
+    return CPM_OK;
 }
 
 // ----------------------------------------------------------------------------- stage 1, CUDA cores
@@ -611,7 +678,7 @@ template <typename T>
 cpm_status launch_charge_phases(cpm_ctx* c, cudaStream_t st, int64_t P, const double* xyz, const double* Q, c2<T>* X,
                                 c2<T>* Y, c2<T>* Z) {
     const KTable& k = c->kt;
-    k_charge_phases<T, CP_PLAIN><<<(unsigned)((P + CP_PTS - 1) / CP_PTS), 8 * CP_PTS, 0, st>>>(
+    k_charge_phases<T, false><<<(unsigned)((P + CP_PTS - 1) / CP_PTS), 8 * CP_PTS, 0, st>>>(
         xyz, Q, P, P, P, c->g.inv[0], c->g.inv[1], c->g.inv[2], k.NX, k.NY, k.NZ, X, Y, Z, nullptr, nullptr);
     CPM_LAUNCH(c, "k_charge_phases");
     return CPM_OK;
@@ -626,7 +693,7 @@ cpm_status launch_charge_slots(cpm_ctx* c, cudaStream_t st, int m, int64_t ne, i
     const KTable& k = c->kt;
     const int64_t P = (int64_t)m * nep;
     float2* Y = tab + (int64_t)(k.NX + 1) * P;
-    k_charge_phases<float, CP_SPLIT><<<(unsigned)((P + CP_PTS - 1) / CP_PTS), 8 * CP_PTS, 0, st>>>(
+    k_charge_phases<float, true><<<(unsigned)((P + CP_PTS - 1) / CP_PTS), 8 * CP_PTS, 0, st>>>(
         xyz, Q, P, ne, nep, c->g.inv[0], c->g.inv[1], c->g.inv[2], k.NX, k.NY, k.NZ, tab, Y, Y + (int64_t)(k.NY + 1) * P,
         qmax, qlast);
     CPM_LAUNCH(c, "k_charge_phases");
@@ -637,10 +704,9 @@ cpm_status launch_charge_fixed(cpm_ctx* c, cudaStream_t st, int m, int64_t ne, i
                                const double* Q, const int* qexp, longlong2* X, longlong2* Y, longlong2* Z) {
     const KTable& k = c->kt;
     const int64_t P = (int64_t)m * nep;
-    k_charge_phases<double, CP_FIXED><<<(unsigned)((P + CP_PTS - 1) / CP_PTS), 8 * CP_PTS, 0, st>>>(
-        xyz, Q, P, ne, nep, c->g.inv[0], c->g.inv[1], c->g.inv[2], k.NX, k.NY, k.NZ, (double2*)X, (double2*)Y, (double2*)Z,
-        nullptr, const_cast<int*>(qexp));
-    CPM_LAUNCH(c, "k_charge_phases");
+    k_charge_fixed<<<dim3((unsigned)(P / CP_PTS), 3), 8 * CP_PTS, 0, st>>>(
+        xyz, Q, P, ne, nep, make_double3(c->g.inv[0], c->g.inv[1], c->g.inv[2]), k.NX, k.NY, k.NZ, qexp, c->rows.fxtab, X, Y, Z);
+    CPM_LAUNCH(c, "k_charge_fixed");
     return CPM_OK;
 }
 

@@ -19,7 +19,7 @@
 // with 64-byte rows (64-byte swizzle).  B digits lie one after the other, so digit i of A meets digits 0 .. 7 - i of B
 // in one MMA of up to 256 columns, column block i + j.  One thread issues; two stages of 96 KB; every wait is
 // bounded as in tc_recip.cu.
-// EDL capacitor, one replica of 5,700 charges: this kernel 31 us and its sum, where the FP64 pipe took 571 us for two
+// EDL capacitor, one replica of 5,700 charges: this kernel 31 us and its sum 9, where the FP64 pipe took 571 us for two
 // multiply-adds per (charge, k).  What bounds it: forming the digits (96 registers, one CTA per SM by shared memory).
 #include <cuda_fp16.h>
 
@@ -244,7 +244,7 @@ __global__ void __launch_bounds__(R4_THREADS, 1)
 }
 
 // out[r][4 p + t][c]: the ranges added as integers, then FP64; the replica's scale removed.  A charge that is no
-// finite number makes the replica's sums not a number.  grid (pairs, m)
+// finite number makes the replica's sums not a number.  grid (pairs, m, 4 rows t); one function per thread
 __global__ void __launch_bounds__(128) k_rows64_sum(const int4* __restrict__ pairs, int np, int cw,
                                                     const longlong2* __restrict__ part, int splits, int m,
                                                     const int* __restrict__ qexp, double* __restrict__ out) {
@@ -253,8 +253,8 @@ __global__ void __launch_bounds__(128) k_rows64_sum(const int4* __restrict__ pai
     const int64_t stride = (int64_t)m * np * 4 * cw;
     const int qe = qexp[r];
     const double f = qe > R4_EMAX ? nan("") : pow2_bits(max(qe, 1) + 1);
-    for (int e = threadIdx.x; e < 4 * nc; e += 128) {
-        const int t = e / nc, c = e - t * nc;
+    const int t = blockIdx.z;
+    for (int c = threadIdx.x; c < nc; c += 128) {
         const int64_t at = (((int64_t)r * np + p) * 4 + t) * cw + c;
         long long hi = 0, lo = 0;
         for (int s0 = 0; s0 < splits; s0 += 8) {   // eight loads in flight
@@ -315,7 +315,7 @@ cpm_status rows64_sf(cpm_ctx* c, cudaStream_t st, const Rows64Dims& d, int m, co
         t.item64, t.pairs, X, Y, Z, (int64_t)m * d.nep, d.nep, c->kt.NZ, t.items64, d.splits, d.spc, d.steps, m, t.np,
         d.cw, ipart, c->status, R4_WAIT_NS);
     CPM_LAUNCH(c, "k_tc_rows64");
-    k_rows64_sum<<<dim3(t.np, m), 128, 0, st>>>(t.pairs, t.np, d.cw, ipart, d.splits, m, qexp, part);
+    k_rows64_sum<<<dim3(t.np, m, 4), 128, 0, st>>>(t.pairs, t.np, d.cw, ipart, d.splits, m, qexp, part);
     CPM_LAUNCH(c, "k_rows64_sum");
     return CPM_OK;
 }
