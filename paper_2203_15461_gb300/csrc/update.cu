@@ -2,9 +2,13 @@
 // followed by the FP64 neutrality fix q <- q - u (e^T q), u = A^-1 e / (e^T A^-1 e), and the
 // total charge e^T q.  In exact arithmetic S e = 0 already (Eq. S); the fix removes the
 // rounding left by a single-precision S.
+#include <cooperative_groups.h>
+
 #include "common.cuh"
 
 namespace cpm {
+
+namespace cg = cooperative_groups;
 
 // S is symmetric, so q_i = sum_j S_ji b_j: one thread per output i reads column i of S (row
 // j = column j, coalesced across the block), the b_j are broadcast from shared memory, and the
@@ -253,124 +257,109 @@ __global__ void __launch_bounds__(G2_T, 2) k_gemv32x2(const float* __restrict__ 
     }
 }
 
-// q[r][i] = sum_g SG[i][g] psi[r][g] - sum_split part[split][r][i]; grid (sites / NB_T, m); with p1,
-// each block also writes the sum of its q values (the first pass of the neutrality fix)
-constexpr int NB_T = 256;
 template <typename P> struct PartSum;
 template <> struct PartSum<double> { using type = PartSumD; };
 template <> struct PartSum<float2> { using type = PartSumF2; };
 template <> struct PartSum<float> { using type = PartSumF; };   // partials of the tensor-core product
 
 // q = SG psi - sum of the split partials (tensor-core product: - SZ gmean, the share of the group means taken out
-// of its operand), then the neutrality fix of Sec. II.B in the last block of
-// each replica: every block writes its slice of q and the slice's sum p1[r][b]; the replica's last
-// block (ticket) adds the p1 in block order, applies q <- q - u (e^T q) with symm, and writes
-// qtot[r] = e^T q of the result (plain FP64 sums in a fixed order: the rounding, about n eps max|q|,
-// is far below the 1e-12 e the total is held to)
+// of its operand), then the neutrality fix of Sec. II.B: q <- q - u (e^T q) with symm, and qtot[r] = e^T q of the
+// result (plain FP64 sums in a fixed order: the rounding, about n eps max|q|, is far below the 1e-12 e the total
+// is held to).
+//
+// Grid (cluster of up to eight blocks, m): one cluster per replica, one thread per site (slices beyond 640 sites take
+// several passes), the block sums exchanged through distributed shared memory, so that every thread still holds
+// its q when e^T q is known.  With a replica's last block (a ticket) doing the fix, that block read the whole q
+// back.  Whole steps, before and now: 4,320 sites x 8 replicas 158.3 and 155.4 us, the product alone x 64 80.0 and
+// 74.5, 512 sites x 4 54.0 and 51.2, 256 small replicas 184 and 178.  Bounded by the latency of the loads and of
+// two cluster barriers; 48 registers let two blocks of 640 threads share an SM (with 64, one: the product took 89 us).
+constexpr int NB_CLUSTER = 8;
+constexpr int NB_T = 640;      // threads per block, at most
+constexpr int NB_LEAST = 128;   // sites per block that a cluster of several blocks has at least
 template <typename P>
-__global__ void __launch_bounds__(NB_T) k_gemv_reduce(const P* __restrict__ part, int splits,
+__global__ void __launch_bounds__(NB_T, 2) k_gemv_reduce(const P* __restrict__ part, int splits,
                                                       const double* __restrict__ SG, int ng,
                                                       const double* __restrict__ psi, int64_t n, int m,
-                                                      double* __restrict__ q, double* __restrict__ p1,
-                                                      const double* __restrict__ u, int symm,
-                                                      int* __restrict__ tickets, double* __restrict__ qtot,
-                                                      const double* __restrict__ b, const double* __restrict__ srow,
-                                                      const double* __restrict__ SZ, const double* __restrict__ gmean,
-                                                      int ngrp) {
+                                                      double* __restrict__ q, const double* __restrict__ u, int symm,
+                                                      double* __restrict__ qtot, const double* __restrict__ b,
+                                                      const double* __restrict__ srow, const double* __restrict__ SZ,
+                                                      const double* __restrict__ gmean, int ngrp) {
     __shared__ double sh[NB_T / 32];
-    __shared__ double buf[NB_T];
-    __shared__ double s_sum;
-    const int r = blockIdx.y, nb = gridDim.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t i = (int64_t)blockIdx.x * NB_T + threadIdx.x;
+    __shared__ double csum[2][NB_CLUSTER];   // block sums of the cluster before and after the fix
+    const cg::cluster_group cluster = cg::this_cluster();
+    const int r = blockIdx.y, cl = gridDim.x, rank = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t slice = (n + cl - 1) / cl, lo = rank * slice, hi = min(n, lo + slice);
     double* qr = q + (int64_t)r * n;
-    double qi = 0.0;
-    if (i < n) {
+    auto exchange = [&](double a, int which) {   // fixed order: warp trees, warps in order, blocks in order
+        for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
+        if (lane == 0) sh[warp] = a;
+        __syncthreads();
+        if ((int)threadIdx.x < cl) {
+            double t = sh[0];
+            for (int w = 1; w < (int)blockDim.x / 32; ++w) t += sh[w];
+            *cluster.map_shared_rank(&csum[which][rank], threadIdx.x) = t;
+        }
+        cluster.sync();
+        double t = csum[which][0];
+        for (int k = 1; k < cl; ++k) t += csum[which][k];
+        return t;
+    };
+    double q0 = 0.0, u0 = 0.0, a = 0.0;   // this thread's first site
+    if (symm && lo + threadIdx.x < hi) u0 = u[lo + threadIdx.x];
+    for (int64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) {
         typename PartSum<P>::type v;
         const P* pi = part + (int64_t)r * n + i;
         const int64_t stride = (int64_t)m * n;
-        for (int sp = 0; sp < splits; sp += 16) {   // sixteen loads in flight, added in split order
-            P x[16];
+        constexpr int LD = sizeof(P) == 4 ? 16 : 8;   // loads in flight, added in split order
+        for (int sp = 0; sp < splits; sp += LD) {
+            P x[LD];
 #pragma unroll
-            for (int k = 0; k < 16; ++k) x[k] = sp + k < splits ? pi[(int64_t)(sp + k) * stride] : P{};
+            for (int k = 0; k < LD; ++k) x[k] = sp + k < splits ? pi[(int64_t)(sp + k) * stride] : P{};
 #pragma unroll
-            for (int k = 0; k < 16; ++k)
+            for (int k = 0; k < LD; ++k)
                 if (sp + k < splits) v.add(x[k]);
         }
         double sv = 0.0;
         for (int g = 0; g < ng; ++g) sv += SG[i * ng + g] * psi[(int64_t)r * ng + g];
         for (int g = 0; g < ngrp; ++g) sv -= SZ[i * ngrp + g] * gmean[(int64_t)r * ngrp + g];
         // the centred products give sum_j S_ij (b_j - b_i): add b_i sum_j S_ij back where rows do not sum to zero
-        qi = sv - (srow ? v.value() + b[(int64_t)r * n + i] * srow[i] : v.value());
-        qr[i] = qi;
-        __threadfence();   // this slice of q is visible device-wide before the block takes its ticket
+        const double qi = sv - (srow ? v.value() + b[(int64_t)r * n + i] * srow[i] : v.value());
+        if (i == lo + threadIdx.x) q0 = qi;
+        else qr[i] = qi;                        // read back by this thread alone
+        a += qi;
     }
-    auto block_sum = [&](double a) {   // fixed order: warp trees, then warps in order
-        for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
-        if (lane == 0) sh[warp] = a;
-        __syncthreads();
-        double t = 0.0;
-        if (threadIdx.x == 0) {
-            t = sh[0];
-            for (int w = 1; w < NB_T / 32; ++w) t += sh[w];
-        }
-        __syncthreads();
-        return t;   // valid in thread 0
-    };
-    const double bsum = block_sum(qi);
-    if (threadIdx.x == 0) p1[(int64_t)r * nb + blockIdx.x] = bsum;
-    if (!last_block_of(&tickets[r], nb)) return;
-    double s = 0.0;
-    if (symm) {
-        const volatile double* pv = p1 + (int64_t)r * nb;
-        for (int k0 = 0; k0 < nb; k0 += NB_T) {
-            if (k0 + (int)threadIdx.x < nb) buf[threadIdx.x] = pv[k0 + threadIdx.x];
-            __syncthreads();
-            if (threadIdx.x == 0)
-                for (int k = 0; k < min(NB_T, nb - k0); ++k) s += buf[k];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) s_sum = s;
-        __syncthreads();
-        s = s_sum;
+    const double s = exchange(a, 0);
+    a = 0.0;
+    for (int64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) {
+        const bool first = i == lo + threadIdx.x;
+        double v = first ? q0 : qr[i];
+        if (symm) v -= (first ? u0 : u[i]) * s;
+        qr[i] = v;
+        a += v;
     }
-    // the replica's q, written by the other blocks: loaded past L1 (__ldcg), eight per thread in
-    // flight, fixed and summed in index order per thread
-    double a = 0.0;
-    for (int64_t k0 = 0; k0 < n; k0 += 8 * NB_T) {
-        double v[8];
-#pragma unroll
-        for (int w = 0; w < 8; ++w) {
-            const int64_t k = k0 + (int64_t)w * NB_T + threadIdx.x;
-            v[w] = k < n ? __ldcg(qr + k) : 0.0;
-        }
-#pragma unroll
-        for (int w = 0; w < 8; ++w) {
-            const int64_t k = k0 + (int64_t)w * NB_T + threadIdx.x;
-            if (k < n) {
-                if (symm) {
-                    v[w] -= u[k] * s;
-                    qr[k] = v[w];
-                }
-                a += v[w];
-            }
-        }
-    }
-    const double tot = block_sum(a);
-    if (threadIdx.x == 0 && qtot) qtot[r] = tot;
+    if (!qtot) return;   // uniform
+    const double tot = exchange(a, 1);
+    if (rank == 0 && threadIdx.x == 0) qtot[r] = tot;
 }
 
-static int reduce_blocks(int64_t n) { return (int)((n + NB_T - 1) / NB_T); }
-
-static cpm_status reserve_neutral(cpm_ctx* c, int m) {
-    CPM_TRY(ensure_tickets(c, m));
-    const size_t need = sizeof(double) * (size_t)m * reduce_blocks(c->n);
-    if (c->nbuf_bytes >= need) return CPM_OK;
-    c->graph_valid = false;
-    dev_free(c, c->nbuf);
-    c->nbuf = nullptr;
-    c->nbuf_bytes = 0;
-    CPM_TRY(dev_alloc(c, (void**)&c->nbuf, need));
-    c->nbuf_bytes = need;
+template <typename P>
+static cpm_status launch_reduce(cpm_ctx* c, const void* part, int splits, int m, const double* psi, double* q, double* qtot,
+                                const double* b, const double* srow, const double* SZ, const double* gmean, int ngrp) {
+    int cl = NB_CLUSTER;
+    while (cl > 1 && c->n < (int64_t)cl * NB_LEAST) cl /= 2;
+    const int64_t slice = (c->n + cl - 1) / cl;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)cl, (unsigned)m);
+    cfg.blockDim = dim3((unsigned)std::min<int64_t>(NB_T, (slice + 31) / 32 * 32));
+    cfg.stream = c->stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)cl;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    CPM_CUDA(c, cudaLaunchKernelEx(&cfg, k_gemv_reduce<P>, (const P*)part, splits, (const double*)upd_sg(c), (int)upd_ng(c), psi,
+                                   c->n, m, q, (const double*)c->u, (int)c->p.symm, qtot, b, srow, SZ, gmean, ngrp));
     return CPM_OK;
 }
 
@@ -414,7 +403,6 @@ static cpm_status reserve_update_plan(cpm_ctx* c, int m, int64_t* splits_out, in
 }
 
 cpm_status reserve_update(cpm_ctx* c, int m) {
-    CPM_TRY(reserve_neutral(c, m));
     if (c->p.s_prec == CPM_PREC_BF16X3) return tc_reserve(c, m);
     int64_t s, j;
     return reserve_update_plan(c, m, &s, &j);
@@ -437,11 +425,8 @@ cpm_status update(cpm_ctx* c, int m, const double* psi, const double* b, double*
         prof_begin(c, CPM_K_GEMV);
         CPM_TRY(tc_product(c, m, b, &part, &splits, &gmean));
         prof_end(c, CPM_K_GEMV);
-        CPM_TRY(reserve_neutral(c, m));
         prof_begin(c, CPM_K_NEUTRAL);
-        k_gemv_reduce<float><<<dim3((unsigned)reduce_blocks(n), m), NB_T, 0, st>>>(
-            part, splits, upd_sg(c), upd_ng(c), psi, n, m, q, c->nbuf, c->u, c->p.symm, c->tickets, qtot, b, nullptr, c->SZ,
-            gmean, c->tc_ngrp);
+        CPM_TRY(launch_reduce<float>(c, part, splits, m, psi, q, qtot, b, nullptr, c->SZ, gmean, c->tc_ngrp));
         prof_end(c, CPM_K_NEUTRAL);
         CPM_LAUNCH(c, "k_gemv_reduce");
         c->launches += 1;
@@ -486,16 +471,12 @@ cpm_status update(cpm_ctx* c, int m, const double* psi, const double* b, double*
         }
     }
     prof_end(c, CPM_K_GEMV);
-    CPM_TRY(reserve_neutral(c, m));
     prof_begin(c, CPM_K_NEUTRAL);
-    const dim3 rgrid((unsigned)reduce_blocks(n), m);
     const double* srow = (f32 && !c->p.symm) ? c->dvec : nullptr;
     if (f32 && gemv_tma_supported(c))
-        k_gemv_reduce<float2><<<rgrid, NB_T, 0, st>>>((const float2*)part, (int)splits, upd_sg(c), upd_ng(c), psi, n, m, q,
-                                                      c->nbuf, c->u, c->p.symm, c->tickets, qtot, b, srow, nullptr, nullptr, 0);
+        CPM_TRY(launch_reduce<float2>(c, part, (int)splits, m, psi, q, qtot, b, srow, nullptr, nullptr, 0));
     else
-        k_gemv_reduce<double><<<rgrid, NB_T, 0, st>>>(part, (int)splits, upd_sg(c), upd_ng(c), psi, n, m, q, c->nbuf, c->u,
-                                                      c->p.symm, c->tickets, qtot, b, srow, nullptr, nullptr, 0);
+        CPM_TRY(launch_reduce<double>(c, part, (int)splits, m, psi, q, qtot, b, srow, nullptr, nullptr, 0));
     prof_end(c, CPM_K_NEUTRAL);
     CPM_LAUNCH(c, "k_gemv");
     return CPM_OK;
