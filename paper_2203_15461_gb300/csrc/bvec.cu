@@ -45,6 +45,7 @@ template <typename T>
 __global__ void __launch_bounds__(ST_THREADS) k_bin(const double* __restrict__ xyz, const double* __restrict__ Q,
                                                   int64_t ne, Geometry g, CellGrid cg, float3 inv_h, int* key,
                                                   int* count, typename V4<T>::t* wpos, int* nzc) {
+    grid_go();
     const int r = blockIdx.y, lane = threadIdx.x & 31;
     const int64_t j = (int64_t)blockIdx.x * ST_THREADS + threadIdx.x;
     bool nz = false;
@@ -135,6 +136,8 @@ __global__ void __launch_bounds__(ST_THREADS) k_totals(const double* __restrict_
 constexpr int CS_THREADS = 256, CS_PER = 8;
 __global__ void __launch_bounds__(CS_THREADS) k_cellscan(const int* count, int* start, int ncells, int64_t ne, int m,
                                                          const int* nzc) {
+    grid_wait();
+    grid_go();
     __shared__ int warp_tot[CS_THREADS / 32];
     __shared__ int carry;
     const int r = blockIdx.x;
@@ -183,6 +186,8 @@ __global__ void __launch_bounds__(CS_THREADS) k_cellscan(const int* count, int* 
 }
 
 __global__ void k_scatter(const int* key, const int* start, int* cursor, int64_t ptot, int* order) {
+    grid_wait();
+    grid_go();
     int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= ptot) return;
     int k = key[p];
@@ -196,6 +201,8 @@ __global__ void k_scatter(const int* key, const int* start, int* cursor, int64_t
 template <typename T>
 __global__ void k_cellsort(const int* start, int ncells_total, const int* order, const typename V4<T>::t* wpos,
                            typename V4<T>::t* sorted, float4* sorted32) {
+    grid_wait();
+    grid_go();
     const int c = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     const int lane = threadIdx.x & 31;
     if (c >= ncells_total) return;
@@ -1006,6 +1013,7 @@ template <typename T>
 __global__ void k_combine(const T* partial, int nctiles, const double* real, const double* b0, const int* zmap,
                           int nzu, const double* stats, const double* sx, int64_t n, int m, Geometry g, double* b,
                           float2* bhl, const double* ew, const double* pm) {
+    grid_go();
     int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= (int64_t)m * n) return;
     const int r = (int)(t / n);
@@ -1286,13 +1294,13 @@ cpm_status bvec_run(cpm_ctx* c, int m, int64_t ne, const double* xyz, const doub
         prof_end(c, CPM_K_SF);
     }
     prof_begin(c, CPM_K_CELLS);
-    k_cellscan<<<m, CS_THREADS, 0, st>>>(cnt, start, p.cg.ncells, ne, m, nzc);
+    CPM_CUDA(c, launch_after(k_cellscan, dim3(m), dim3(CS_THREADS), 0, st, cnt, start, p.cg.ncells, ne, m, nzc));
     CPM_LAUNCH(c, "k_cellscan");
     if (ptot > 0) {
-        k_scatter<<<(unsigned)((ptot + 255) / 256), 256, 0, st>>>(key, start, cur, ptot, order);
+        CPM_CUDA(c, launch_after(k_scatter, dim3((unsigned)((ptot + 255) / 256)), dim3(256), 0, st, key, start, cur, ptot, order));
         CPM_LAUNCH(c, "k_scatter");
-        k_cellsort<T><<<(unsigned)(((int64_t)nc * 32 + 255) / 256), 256, 0, st>>>(start, nc, order, wpos, sorted,
-                                                                                  p.real64 ? sorted32 : nullptr);
+        CPM_CUDA(c, launch_after(k_cellsort<T>, dim3((unsigned)(((int64_t)nc * 32 + 255) / 256)), dim3(256), 0, st, start, nc, order, wpos, sorted,
+                                                                                  p.real64 ? sorted32 : nullptr));
         CPM_LAUNCH(c, "k_cellsort");
     }
     prof_end(c, CPM_K_CELLS);

@@ -107,7 +107,8 @@ __global__ void __launch_bounds__(GV_T + 32, 2)
     __syncthreads();
 
     if (warp == GV_T / 32) {
-        // producer
+        // producer: S alone, which no kernel just in front of this one writes, so that the first stages are under way
+        // while b is finished
         if (lane == 0) {
             int issued = 0;
             for (int t = 0; t < nst; ++t) {
@@ -128,8 +129,11 @@ __global__ void __launch_bounds__(GV_T + 32, 2)
                 }
             }
         }
+        __syncwarp();
+        grid_wait();
         return;
     }
+    grid_wait();
 
     // consumers: stage b of the block's rows, replica-minor, high and low parts apart (coalesced
     // loads along the rows, all in flight before the first store)
@@ -283,9 +287,9 @@ cpm_status gemv_tma(cpm_ctx* c, int m, const float2* bhl, float2* part, int64_t 
     const dim3 grid((unsigned)colblocks, (unsigned)splits, (unsigned)((m + mr - 1) / mr));
     auto launch = [&](auto kern) {
         const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, gv_smem(mr));
-        if (e == cudaSuccess)
-            kern<<<grid, GV_T + 32, gv_smem(mr), c->stream>>>(smap, bhl, n, m, jchunk, part, c->status, GV_WAIT_NS);
-        return e;
+        return e != cudaSuccess ? e
+                                : launch_after(kern, grid, dim3(GV_T + 32), gv_smem(mr), c->stream, smap, bhl, n, m, jchunk,
+                                               part, c->status, GV_WAIT_NS);
     };
     CPM_CUDA(c, mr == 2 ? launch(k_gemv_tma<2>) : mr == 4 ? launch(k_gemv_tma<4>) : launch(k_gemv_tma<8>));
     CPM_LAUNCH(c, "k_gemv_tma");

@@ -106,6 +106,7 @@ template <> struct P3mV4<double> { using t = double4_32a; };
 template <typename T>
 __global__ void k_p3m_prep(const double* __restrict__ xyz, const double* __restrict__ Q, int64_t ptot, Geometry g,
                            int Kx, int Ky, int Kz, int P, int* __restrict__ key, typename P3mV4<T>::t* __restrict__ fq) {
+    grid_go();
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= ptot) return;
     const double q = Q[t];
@@ -178,6 +179,7 @@ __global__ void __launch_bounds__(P3M_NT) k_p3m_spread(const int* __restrict__ k
                                                        const typename P3mV4<T>::t* __restrict__ fq, int64_t ne, int m,
                                                        int Kx, int Ky, int Kz, int BX, int BY, int cps,
                                                        c2<T>* __restrict__ part, int* __restrict__ flag) {
+    grid_wait();
     constexpr int NW = P3mWords<T>::n, BZ = P3M_BZ;
     extern __shared__ __align__(16) unsigned char p3m_smem[];
     const int RX = BX + 1, PS = BY * RX + 8;            // padded row and plane
@@ -359,6 +361,7 @@ __global__ void __launch_bounds__(P3M_THREADS) k_p3m_plane(c2<T>* __restrict__ m
                                                           const c2<T>* __restrict__ twx, const c2<T>* __restrict__ twy,
                                                           int nsplit, int64_t split_stride, int m, int BX, int BY,
                                                           const int* __restrict__ flag, const int* __restrict__ zlist) {
+    grid_wait();
     extern __shared__ __align__(16) unsigned char p3m_smem[];
     __shared__ unsigned char fl[INV ? 1 : P3M_FLAGS];
     c2<T>* pl = (c2<T>*)p3m_smem;
@@ -415,6 +418,7 @@ __global__ void __launch_bounds__(P3M_THREADS) k_p3m_zline(c2<T>* __restrict__ m
                                                           const T* __restrict__ G, const c2<T>* __restrict__ twz,
                                                           const unsigned char* __restrict__ need, int nl,
                                                           const int* __restrict__ lb, const T* __restrict__ lw, int P) {
+    grid_wait();
     extern __shared__ __align__(16) unsigned char p3m_smem[];
     c2<T>* ln = (c2<T>*)p3m_smem;
     c2<T>* tw = ln + Kz * tx;
@@ -472,6 +476,7 @@ template <typename T, int P>
 __global__ void __launch_bounds__(P3M_THREADS) k_p3m_interp(const double* __restrict__ sx, int64_t n, int m,
                                                            Geometry g, int Kx, int Ky, int Kz,
                                                            const c2<T>* __restrict__ mesh, double* __restrict__ pm) {
+    grid_wait();
     __shared__ T sw[P3M_THREADS / 32][3][8];
     __shared__ int sb[P3M_THREADS / 32][3];
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -554,6 +559,7 @@ __global__ void __launch_bounds__(P3M_THREADS) k_p3m_interp2(const int* __restri
                                                             const T* __restrict__ w, int64_t n, int m, int P, int Kx,
                                                             int Ky, int Kz, const c2<T>* __restrict__ mesh,
                                                             double* __restrict__ pm) {
+    grid_wait();
     const int lane = threadIdx.x & 31;
     const int64_t wid = (int64_t)blockIdx.x * (P3M_THREADS / 32) + (threadIdx.x >> 5);
     if (wid >= n * ((m + 1) / 2)) return;
@@ -738,30 +744,30 @@ static cpm_status launch_p3m_pp(cudaStream_t st, cpm_ctx* c, int m, int64_t ne, 
     const size_t ssm = sizeof(int) * ((P3mWords<T>::n * P3M_BZ * (sp.BY * (sp.BX + 1) + 8) + 3) & ~3) +
                        sizeof(T) * P3M_NT * (3 * P + 1) + sizeof(int) * P3M_NT;
     CPM_CUDA(c, cudaFuncSetAttribute(k_p3m_spread<T, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssm));
-    k_p3m_spread<T, P><<<dim3(sp.nbricks, m, sp.nsplit), P3M_NT, ssm, st>>>(key, fq, ne, m, Kx, Ky, Kz, sp.BX, sp.BY,
-                                                                            sp.cps, mesh, flag);
+    CPM_CUDA(c, launch_after(k_p3m_spread<T, P>, dim3(sp.nbricks, m, sp.nsplit), dim3(P3M_NT), ssm, st, key, fq, ne, m, Kx, Ky, Kz, sp.BX, sp.BY,
+                                                                            sp.cps, mesh, flag));
     const int64_t sstride = (int64_t)npairs * Kx * Ky * Kz;
     const c2<T>* tw = p3m_twiddles<T>(c);
     const size_t psm = sizeof(c2<T>) * ((size_t)Kx * Ky + Kx / 2 + Ky / 2);
     CPM_CUDA(c, cudaFuncSetAttribute(k_p3m_plane<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psm));
     CPM_CUDA(c, cudaFuncSetAttribute(k_p3m_plane<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psm));
-    k_p3m_plane<T, false><<<dim3(Kz, npairs), P3M_THREADS, psm, st>>>(mesh, Kx, Ky, Kz, tw, tw + Kx / 2, sp.nsplit,
-                                                                      sstride, m, sp.BX, sp.BY, flag, nullptr);
+    CPM_CUDA(c, launch_after(k_p3m_plane<T, false>, dim3(Kz, npairs), dim3(P3M_THREADS), psm, st, mesh, Kx, Ky, Kz, tw, tw + Kx / 2, sp.nsplit,
+                                                                      sstride, m, sp.BX, sp.BY, flag, nullptr));
     const int tx = std::min(Kx, P3M_ZTX);
     const size_t zsm = sizeof(c2<T>) * ((size_t)Kz * tx + Kz / 2);
     CPM_CUDA(c, cudaFuncSetAttribute(k_p3m_zline<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)zsm));
-    k_p3m_zline<T><<<dim3(Kx / tx, Ky, npairs), P3M_THREADS, zsm, st>>>(mesh, Kx, Ky, Kz, tx, p3m_green<T>(c),
+    CPM_CUDA(c, launch_after(k_p3m_zline<T>, dim3(Kx / tx, Ky, npairs), dim3(P3M_THREADS), zsm, st, mesh, Kx, Ky, Kz, tx, p3m_green<T>(c),
                                                                         tw + Kx / 2 + Ky / 2, c->p3m_need, c->p3m_nl,
-                                                                        c->p3m_lb, p3m_height_w<T>(c), P);
-    k_p3m_plane<T, true><<<dim3(c->p3m_nz, npairs), P3M_THREADS, psm, st>>>(mesh, Kx, Ky, Kz, tw, tw + Kx / 2, 1, 0, m,
-                                                                            sp.BX, sp.BY, nullptr, c->p3m_zlist);
+                                                                        c->p3m_lb, p3m_height_w<T>(c), P));
+    CPM_CUDA(c, launch_after(k_p3m_plane<T, true>, dim3(c->p3m_nz, npairs), dim3(P3M_THREADS), psm, st, mesh, Kx, Ky, Kz, tw, tw + Kx / 2, 1, 0, m,
+                                                                            sp.BX, sp.BY, nullptr, c->p3m_zlist));
     const int64_t warps = c->n * npairs;
     if (c->p3m_nl)
-        k_p3m_interp2<T><<<(unsigned)((warps + P3M_THREADS / 32 - 1) / (P3M_THREADS / 32)), P3M_THREADS, 0, st>>>(
-            c->zmap, c->p3m_base, p3m_site_w<T>(c), c->n, m, P, Kx, Ky, Kz, mesh, pm);
+        CPM_CUDA(c, launch_after(k_p3m_interp2<T>, dim3((unsigned)((warps + P3M_THREADS / 32 - 1) / (P3M_THREADS / 32))), dim3(P3M_THREADS), 0, st, 
+            c->zmap, c->p3m_base, p3m_site_w<T>(c), c->n, m, P, Kx, Ky, Kz, mesh, pm));
     else
-        k_p3m_interp<T, P><<<(unsigned)((warps + P3M_THREADS / 32 - 1) / (P3M_THREADS / 32)), P3M_THREADS, 0, st>>>(
-            c->sx, c->n, m, c->g, Kx, Ky, Kz, mesh, pm);
+        CPM_CUDA(c, launch_after(k_p3m_interp<T, P>, dim3((unsigned)((warps + P3M_THREADS / 32 - 1) / (P3M_THREADS / 32))), dim3(P3M_THREADS), 0, st, 
+            c->sx, c->n, m, c->g, Kx, Ky, Kz, mesh, pm));
     CPM_LAUNCH(c, "k_p3m (spread, transforms, interpolation)");
     return CPM_OK;
 }

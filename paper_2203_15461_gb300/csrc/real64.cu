@@ -95,6 +95,7 @@ __global__ void __launch_bounds__(32 * R6_WARPS)
     k_real64(const double* __restrict__ sx, int64_t n, int m, Geometry g, CellGrid cg, const int* __restrict__ start,
              const double4_32a* __restrict__ sorted, const float4* __restrict__ sorted32, const double* __restrict__ tab,
              int nint, int e0, const int* __restrict__ tabid, float slack, double* __restrict__ out) {
+    grid_wait();
     __shared__ R6Row s_row[R6_WARPS][33];
     __shared__ float4 s_sh[R6_WARPS][32];            // image shift of a run, w: the shift counts packed
     __shared__ int2 s_q[R6_WARPS][64];               // queue: (charge, shift counts)
@@ -233,9 +234,9 @@ cpm_status real64_run(cpm_ctx* c, cudaStream_t st, int m, const CellGrid& cg, co
     // a coordinate and an image shift round to 2^-24 of at most a few box lengths each
     const double lmax = std::max(c->g.boxL[0], std::max(c->g.boxL[1], c->g.boxL[2])) + c->g.rcut;
     const float slack = (float)(4e-6 * c->g.rcut * lmax);
-    k_real64<<<(unsigned)(((int64_t)m * c->n + R6_WARPS - 1) / R6_WARPS), 32 * R6_WARPS, 0, st>>>(
+    CPM_CUDA(c, launch_after(k_real64, dim3((unsigned)(((int64_t)m * c->n + R6_WARPS - 1) / R6_WARPS)), dim3(32 * R6_WARPS), 0, st, 
         c->sx, c->n, m, c->g, cg, start, (const double4_32a*)sorted, sorted32, c->r64tab, c->r64n, c->r64e0, c->rtab_id,
-        slack, out);
+        slack, out));
     CPM_LAUNCH(c, "k_real64");
     return CPM_OK;
 }

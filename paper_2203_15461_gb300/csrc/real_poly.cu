@@ -331,6 +331,7 @@ __global__ void __launch_bounds__(RB_T, 4)
     k_real_blk(RbInputs in, RbGrid gr, int ncells, const int* __restrict__ start, const float4* __restrict__ sorted,
                const float4* __restrict__ tab, RealPoly rp, int m, int64_t n, int* __restrict__ rqueue,
                double* __restrict__ out) {
+    grid_wait();
     __shared__ RbShared sm;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const float rc2 = rp.rc2;
@@ -661,9 +662,9 @@ cpm_status real_poly_run(cpm_ctx* c, cudaStream_t st, int m, const CellGrid& cg,
     in.stride = c->rrun_stride;
     in.nchunks = c->nschunk;
     if (c->rpoly.deg == 12)
-        k_real_blk<12><<<grid, RB_T, 0, st>>>(in, gr, cg.ncells, start, sorted, tab, c->rpoly, m, c->n, c->rqueue, out);
+        CPM_CUDA(c, launch_after(k_real_blk<12>, dim3(grid), dim3(RB_T), 0, st, in, gr, cg.ncells, start, sorted, tab, c->rpoly, m, c->n, c->rqueue, out));
     else
-        k_real_blk<14><<<grid, RB_T, 0, st>>>(in, gr, cg.ncells, start, sorted, tab, c->rpoly, m, c->n, c->rqueue, out);
+        CPM_CUDA(c, launch_after(k_real_blk<14>, dim3(grid), dim3(RB_T), 0, st, in, gr, cg.ncells, start, sorted, tab, c->rpoly, m, c->n, c->rqueue, out));
     CPM_LAUNCH(c, "k_real_blk");
     return CPM_OK;
 }

@@ -348,6 +348,7 @@ __global__ void __launch_bounds__(8 * CP_PTS) k_charge_fixed(const double* __res
                                                              int NY, int NZ, const int* __restrict__ qexp,
                                                              const longlong2* __restrict__ tab, longlong2* __restrict__ X,
                                                              longlong2* __restrict__ Y, longlong2* __restrict__ Z) {
+    grid_wait();
     __shared__ longlong2 sg[8][CP_PTS];
     __shared__ uint64_t sf[CP_PTS];
     __shared__ int64_t sq[CP_PTS];
@@ -407,6 +408,7 @@ __global__ void __launch_bounds__(RW_THREADS) k_rows_sf(const int4* __restrict__
                                                         const c2<T>* __restrict__ Y, const c2<T>* __restrict__ Z,
                                                         int64_t P, int64_t ne, int splits, int64_t chunk, int m,
                                                         T* __restrict__ part) {
+    grid_wait();
     constexpr int TM = RowTileOf<T>::TM, TN = RowTileOf<T>::TN, BM = 16 * TM, BN = 8 * TN;
     __shared__ T Ps[RW_BK][BM + 1];
     __shared__ T Zs[RW_BK][BN + 1];
@@ -500,6 +502,8 @@ __global__ void __launch_bounds__(RL_THREADS) k_rows_layers(const int4* __restri
                                                             const T* __restrict__ W, const c2<T>* __restrict__ ZU,
                                                             int nzu, int nslots, const float* __restrict__ qmax,
                                                             T* __restrict__ Tout) {
+    grid_wait();
+    grid_go();
     extern __shared__ __align__(16) unsigned char rl_smem[];
     const int p = blockIdx.x, r = blockIdx.y;
     const int4 pr = pairs[p];
@@ -561,6 +565,7 @@ __global__ void __launch_bounds__(ROW_TILE) k_rows_sites(const int4* __restrict_
                                                          int nslots, const c2<T>* __restrict__ SX,
                                                          const c2<T>* __restrict__ SY, int64_t n, int m, int nchunk,
                                                          T* __restrict__ partial) {
+    grid_wait();
     extern __shared__ __align__(32) unsigned char rs_smem[];
     typename T4of<T>::t* st = (typename T4of<T>::t*)rs_smem;   // [slot of the chunk][MR]
     const int4 tl = tiles[blockIdx.x];
@@ -704,8 +709,8 @@ cpm_status launch_charge_fixed(cpm_ctx* c, cudaStream_t st, int m, int64_t ne, i
                                const double* Q, const int* qexp, longlong2* X, longlong2* Y, longlong2* Z) {
     const KTable& k = c->kt;
     const int64_t P = (int64_t)m * nep;
-    k_charge_fixed<<<dim3((unsigned)(P / CP_PTS), 3), 8 * CP_PTS, 0, st>>>(
-        xyz, Q, P, ne, nep, make_double3(c->g.inv[0], c->g.inv[1], c->g.inv[2]), k.NX, k.NY, k.NZ, qexp, c->rows.fxtab, X, Y, Z);
+    CPM_CUDA(c, launch_after(k_charge_fixed, dim3((unsigned)(P / CP_PTS), 3), dim3(8 * CP_PTS), 0, st, 
+        xyz, Q, P, ne, nep, make_double3(c->g.inv[0], c->g.inv[1], c->g.inv[2]), k.NX, k.NY, k.NZ, qexp, c->rows.fxtab, X, Y, Z));
     CPM_LAUNCH(c, "k_charge_fixed");
     return CPM_OK;
 }
@@ -714,8 +719,8 @@ template <typename T>
 cpm_status rows_sf(cpm_ctx* c, cudaStream_t st, const RowDims& d, int m, int64_t ne, const c2<T>* X, const c2<T>* Y,
                    const c2<T>* Z, T* part) {
     const RowTable& t = c->rows;
-    k_rows_sf<T><<<dim3(d.xt, d.yt, (unsigned)(m * d.splits)), RW_THREADS, 0, st>>>(
-        t.pairs, t.list, t.nrows, t.np, d.cw, X, Y, Z, (int64_t)m * ne, ne, d.splits, d.chunk, m, part);
+    CPM_CUDA(c, launch_after(k_rows_sf<T>, dim3(d.xt, d.yt, (unsigned)(m * d.splits)), dim3(RW_THREADS), 0, st, 
+        t.pairs, t.list, t.nrows, t.np, d.cw, X, Y, Z, (int64_t)m * ne, ne, d.splits, d.chunk, m, part));
     CPM_LAUNCH(c, "k_rows_sf");
     return CPM_OK;
 }
@@ -727,8 +732,8 @@ cpm_status rows_layers(cpm_ctx* c, cudaStream_t st, int cw, int splits, int m, c
     const RowTable& t = c->rows;
     const size_t sm = sizeof(T) * 4 * 2 * (c->kt.NZ + 1);
     if (sm > 48 * 1024) CPM_CUDA(c, cudaFuncSetAttribute(k_rows_layers<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    k_rows_layers<T><<<dim3(t.np, m), RL_THREADS, sm, st>>>(t.pairs, t.np, cw, c->kt.NZ, part, splits, m,
-                                                            row_weights<T>(c), row_zu<T>(c), c->nzu, t.nslots, qmax, Tbuf);
+    CPM_CUDA(c, launch_after(k_rows_layers<T>, dim3(t.np, m), dim3(RL_THREADS), sm, st, t.pairs, t.np, cw, c->kt.NZ, part, splits, m,
+                                                            row_weights<T>(c), row_zu<T>(c), c->nzu, t.nslots, qmax, Tbuf));
     CPM_LAUNCH(c, "k_rows_layers");
     return CPM_OK;
 }
@@ -736,14 +741,15 @@ template cpm_status rows_layers<double>(cpm_ctx*, cudaStream_t, int, int, int, c
 template cpm_status rows_layers<float>(cpm_ctx*, cudaStream_t, int, int, int, const float*, const float*, float*);
 
 template <typename T, int MR>
-static void rows_sites_mr(cpm_ctx* c, cudaStream_t st, int m, const T* Tbuf, T* partial) {
+static cpm_status rows_sites_mr(cpm_ctx* c, cudaStream_t st, int m, const T* Tbuf, T* partial) {
     const RowTable& t = c->rows;
     const Phases<T>& s = row_sites<T>(c);
     const size_t sm = sizeof(T) * 4 * MR * t.chunkmax;
     if (sm > 48 * 1024) cudaFuncSetAttribute(k_rows_sites<T, MR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k_rows_sites<T, MR><<<dim3(t.ntiles, t.nchunk, (m + MR - 1) / MR), ROW_TILE, sm, st>>>(
+    CPM_CUDA(c, launch_after(k_rows_sites<T, MR>, dim3(t.ntiles, t.nchunk, (m + MR - 1) / MR), dim3(ROW_TILE), sm, st, 
         t.ltiles, t.lperm, t.chunkb, t.nxoff, (const typename T4of<T>::t*)Tbuf, c->nzu, t.nslots, s.X,
-        s.Y + (int64_t)c->kt.NY * c->n, c->n, m, t.nchunk, partial);
+        s.Y + (int64_t)c->kt.NY * c->n, c->n, m, t.nchunk, partial));
+    return CPM_OK;
 }
 // replicas per thread: the site phases are read once for all of them; one replica alone keeps the
 // registers of one
@@ -757,9 +763,9 @@ template int64_t rows_T_elems<float>(const cpm_ctx*, int);
 
 template <typename T>
 cpm_status rows_sites(cpm_ctx* c, cudaStream_t st, int m, const T* Tbuf, T* partial) {
-    if (rows_mr<T>(m) == 1) rows_sites_mr<T, 1>(c, st, m, Tbuf, partial);
-    else if (rows_mr<T>(m) == 4) rows_sites_mr<T, 4>(c, st, m, Tbuf, partial);
-    else rows_sites_mr<T, 8>(c, st, m, Tbuf, partial);
+    if (rows_mr<T>(m) == 1) CPM_TRY((rows_sites_mr<T, 1>(c, st, m, Tbuf, partial)));
+    else if (rows_mr<T>(m) == 4) CPM_TRY((rows_sites_mr<T, 4>(c, st, m, Tbuf, partial)));
+    else CPM_TRY((rows_sites_mr<T, 8>(c, st, m, Tbuf, partial)));
     CPM_LAUNCH(c, "k_rows_sites");
     return CPM_OK;
 }

@@ -101,6 +101,18 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_sb(const __grid_constant__
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
+    // the first item's S tiles, which no kernel just in front of this one writes, are fetched while b's terms are formed
+    uint32_t early = 0;
+    if (warp == 0 && lane == 0 && !skip_loads && (int)blockIdx.x < items) {
+        int row, rep, split, kb, ke;
+        W.get(blockIdx.x, row, rep, split, kb, ke);
+        for (; early < (uint32_t)STAGES && kb + (int)early < ke; ++early) {
+            mbar_expect_tx(&full[early], C::STAGE);
+            for (int q = 0; q < 3; ++q)
+                tma_load_2d(smem + early * C::STAGE + q * C::A_BYTES, &maps.a[q], (kb + early) * TC_BK, row * TC_BM, &full[early]);
+        }
+    }
+    grid_wait();
     if (warp == 0) {
         if (lane == 0 && !skip_loads) {
             // producer: six TMA tiles per K step, continuing across items without a break
@@ -112,9 +124,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_sb(const __grid_constant__
                     const int s = (int)(g % STAGES);
                     if (g >= (uint32_t)STAGES && !mbar_wait(&empty[s], ((g / STAGES) - 1) & 1, abort, wait_ns)) break;
                     uint8_t* st = smem + s * C::STAGE;
-                    mbar_expect_tx(&full[s], C::STAGE);
                     const int kx = t * TC_BK;
-                    for (int q = 0; q < 3; ++q) tma_load_2d(st + q * C::A_BYTES, &maps.a[q], kx, row * TC_BM, &full[s]);
+                    if (g >= early) {
+                        mbar_expect_tx(&full[s], C::STAGE);
+                        for (int q = 0; q < 3; ++q) tma_load_2d(st + q * C::A_BYTES, &maps.a[q], kx, row * TC_BM, &full[s]);
+                    }
                     for (int q = 0; q < 3; ++q)
                         tma_load_2d(st + 3 * C::A_BYTES + q * C::B_BYTES, &maps.b[q], kx, rep * BN, &full[s]);
                     ++issued;
@@ -215,6 +229,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_sb(const __grid_constant__
 __global__ void k_split3(const double* __restrict__ x, int64_t rows, int64_t cols, int64_t ld,
                          __nv_bfloat16* __restrict__ out, const double* __restrict__ gmean = nullptr,
                          const int* __restrict__ gid = nullptr, int ngrp = 0) {
+    grid_wait();
+    grid_go();
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, half = ld / 2;
     if (t >= rows * half) return;
     const int64_t r = t / half, c = 2 * (t % half);
@@ -281,7 +297,8 @@ static cpm_status launch_tc_t(cpm_ctx* c, const TcMaps& maps, const TcItems& W, 
                              int skip_loads, uint64_t wait_ns) {
     typedef TcCfg<BN, STAGES> C;
     CPM_CUDA(c, cudaFuncSetAttribute(k_tc_sb<BN, STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
-    k_tc_sb<BN, STAGES><<<grid, TC_THREADS, C::SMEM, c->stream>>>(maps, W, n, m, part, c->status, skip_loads, wait_ns);
+    CPM_CUDA(c, launch_after(k_tc_sb<BN, STAGES>, dim3(grid), dim3(TC_THREADS), C::SMEM, c->stream, maps, W, n, m, part, c->status,
+                             skip_loads, wait_ns));
     CPM_LAUNCH(c, "k_tc_sb");
     return CPM_OK;
 }
@@ -450,8 +467,8 @@ cpm_status tc_sb(cpm_ctx* c, int m, const double* b, float* part, int* splits, v
     const int64_t n = c->n, ld = tc_ld(n);
     TcPlan p;
     CPM_TRY(tc_plan_for(c, m, part, bsplit, &p));
-    k_split3<<<(unsigned)((m * (ld / 2) + 255) / 256), 256, 0, c->stream>>>(b, m, n, ld, (__nv_bfloat16*)bsplit, gmean, gid,
-                                                                      ngrp);
+    CPM_CUDA(c, launch_after(k_split3, dim3((unsigned)((m * (ld / 2) + 255) / 256)), dim3(256), 0, c->stream, b, m, n, ld, (__nv_bfloat16*)bsplit, gmean, gid,
+                                                                      ngrp));
     CPM_LAUNCH(c, "k_split3(b)");
     TcMaps maps;
     CPM_TRY(tc_maps(c, m, p.bn, bsplit, &maps));
@@ -485,6 +502,7 @@ constexpr int GM_T = 256;
 __global__ void __launch_bounds__(GM_T) k_gmeans(const double* __restrict__ b, const int* __restrict__ perm,
                                                  const int* __restrict__ off, int64_t n, int ngrp,
                                                  double* __restrict__ gmean) {
+    grid_go();
     __shared__ double sh[GM_T / 32];
     const int g = blockIdx.x, r = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const double* br = b + (int64_t)r * n;

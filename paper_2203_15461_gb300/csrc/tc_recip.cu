@@ -119,6 +119,7 @@ __global__ void __launch_bounds__(RF_THREADS, 1)
               const float2* __restrict__ tab, int64_t P, int64_t nep, int NX, int NY, int NZ,
               const float* __restrict__ qmax, const int* __restrict__ qlast, int nitems, int splits, int spc, int m, int np,
               int cw, float* __restrict__ part, unsigned* __restrict__ status, uint64_t wait_ns) {
+    grid_wait();
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = align1024(smem_raw);
     uint8_t* aux = smem + RF_STAGES * RF_STAGE;
@@ -653,9 +654,9 @@ cpm_status tc_recip_sf(cpm_ctx* c, cudaStream_t st, const TcRecipDims& d, int m,
     const KTable& k = c->kt;
     const RowTable& t = c->rows;
     CPM_CUDA(c, cudaFuncSetAttribute(k_tc_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, RF_SMEM));
-    k_tc_rows<<<(unsigned)(t.tcitems * (int64_t)m * d.splits), RF_THREADS, RF_SMEM, st>>>(
+    CPM_CUDA(c, launch_after(k_tc_rows, dim3((unsigned)(t.tcitems * (int64_t)m * d.splits)), dim3(RF_THREADS), RF_SMEM, st, 
         t.tcitem, t.tcrange, t.pairs, tab, (int64_t)m * d.nep, d.nep, k.NX, k.NY, k.NZ, qmax, qlast, t.tcitems, d.splits,
-        d.spc, m, t.np, d.cw, part, c->status, RT_WAIT_NS);
+        d.spc, m, t.np, d.cw, part, c->status, RT_WAIT_NS));
     CPM_LAUNCH(c, "k_tc_rows");
     return CPM_OK;
 }

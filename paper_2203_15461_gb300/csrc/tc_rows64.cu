@@ -93,6 +93,7 @@ __global__ void __launch_bounds__(R4_THREADS, 1)
                 const longlong2* __restrict__ Y, const longlong2* __restrict__ Z, int64_t P, int64_t nep, int NZ,
                 int nitems, int splits, int spc, int steps, int m, int np, int cw, longlong2* __restrict__ part,
                 unsigned* __restrict__ status, uint64_t wait_ns) {
+    grid_wait();
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = align1024(smem_raw);
     uint64_t* full = (uint64_t*)(smem + R4_STAGES * R4_STAGE);
@@ -248,6 +249,8 @@ __global__ void __launch_bounds__(R4_THREADS, 1)
 __global__ void __launch_bounds__(128) k_rows64_sum(const int4* __restrict__ pairs, int np, int cw,
                                                     const longlong2* __restrict__ part, int splits, int m,
                                                     const int* __restrict__ qexp, double* __restrict__ out) {
+    grid_wait();
+    grid_go();
     const int p = blockIdx.x, r = blockIdx.y;
     const int nc = 2 * (pairs[p].z + 1);
     const int64_t stride = (int64_t)m * np * 4 * cw;
@@ -270,6 +273,7 @@ __global__ void __launch_bounds__(128) k_rows64_sum(const int4* __restrict__ pai
 
 // largest biased exponent of Q per replica (zero before)
 __global__ void __launch_bounds__(256) k_qexp(const double* __restrict__ Q, int64_t ne, int* __restrict__ qexp) {
+    grid_go();
     const int64_t j = (int64_t)blockIdx.x * 256 + threadIdx.x;
     int v = j < ne ? exp_bits(Q[(int64_t)blockIdx.y * ne + j]) : 0;
     for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
@@ -311,11 +315,11 @@ cpm_status rows64_sf(cpm_ctx* c, cudaStream_t st, const Rows64Dims& d, int m, co
                      const longlong2* Z, const int* qexp, longlong2* ipart, double* part) {
     const RowTable& t = c->rows;
     CPM_CUDA(c, cudaFuncSetAttribute(k_tc_rows64, cudaFuncAttributeMaxDynamicSharedMemorySize, R4_SMEM));
-    k_tc_rows64<<<(unsigned)(t.items64 * (int64_t)m * d.splits), R4_THREADS, R4_SMEM, st>>>(
+    CPM_CUDA(c, launch_after(k_tc_rows64, dim3((unsigned)(t.items64 * (int64_t)m * d.splits)), dim3(R4_THREADS), R4_SMEM, st, 
         t.item64, t.pairs, X, Y, Z, (int64_t)m * d.nep, d.nep, c->kt.NZ, t.items64, d.splits, d.spc, d.steps, m, t.np,
-        d.cw, ipart, c->status, R4_WAIT_NS);
+        d.cw, ipart, c->status, R4_WAIT_NS));
     CPM_LAUNCH(c, "k_tc_rows64");
-    k_rows64_sum<<<dim3(t.np, m, 4), 128, 0, st>>>(t.pairs, t.np, d.cw, ipart, d.splits, m, qexp, part);
+    CPM_CUDA(c, launch_after(k_rows64_sum, dim3(t.np, m, 4), dim3(128), 0, st, t.pairs, t.np, d.cw, ipart, d.splits, m, qexp, part));
     CPM_LAUNCH(c, "k_rows64_sum");
     return CPM_OK;
 }

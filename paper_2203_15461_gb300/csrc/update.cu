@@ -38,6 +38,7 @@ template <> struct LaneSum<float> {
 
 // bhl[t] = (hi, lo) with hi = float(b[t]) and lo = float(b[t] - hi)
 __global__ void k_split_b(const double* __restrict__ b, int64_t cnt, float2* __restrict__ bhl) {
+    grid_go();
     int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= cnt) return;
     double v = b[t];
@@ -53,6 +54,7 @@ constexpr int G6_T = 128, G6_U = 16;
 template <int MR, int NC>
 __global__ void __launch_bounds__(G6_T) k_gemv64(const double* __restrict__ S, const double* __restrict__ bv, int64_t n,
                                                  int m, int64_t jchunk, double* __restrict__ part) {
+    grid_wait();
     __shared__ double bs[GT_JT][MR];
     const int64_t i0 = ((int64_t)blockIdx.x * G6_T + threadIdx.x) * NC;
     const int split = blockIdx.y, r0 = blockIdx.z * MR;
@@ -115,6 +117,7 @@ __global__ void __launch_bounds__(G6_T) k_gemv64(const double* __restrict__ S, c
 // compensation.
 __global__ void __launch_bounds__(GT_COLS) k_gemv32(const float* __restrict__ S, const float2* __restrict__ bv,
                                                    int64_t n, int m, int64_t jchunk, double* __restrict__ part) {
+    grid_wait();
     __shared__ __align__(16) float2 bs[GT_JT][GT_MR];
     const int64_t i = (int64_t)blockIdx.x * GT_COLS + threadIdx.x;
     const int split = blockIdx.y;
@@ -180,6 +183,7 @@ __global__ void __launch_bounds__(GT_COLS) k_gemv32(const float* __restrict__ S,
 constexpr int G2_T = 256;
 __global__ void __launch_bounds__(G2_T, 2) k_gemv32x2(const float* __restrict__ S, const float2* __restrict__ bv,
                                                       int64_t n, int m, int64_t jchunk, double* __restrict__ part) {
+    grid_wait();
     __shared__ __align__(16) float2 bs[GT_JT][GT_MR];
     const int64_t i0 = ((int64_t)blockIdx.x * G2_T + threadIdx.x) * 2;
     const int split = blockIdx.y;
@@ -284,6 +288,7 @@ __global__ void __launch_bounds__(NB_T, 2) k_gemv_reduce(const P* __restrict__ p
                                                       double* __restrict__ qtot, const double* __restrict__ b,
                                                       const double* __restrict__ srow, const double* __restrict__ SZ,
                                                       const double* __restrict__ gmean, int ngrp) {
+    grid_wait();
     __shared__ double sh[NB_T / 32];
     __shared__ double csum[2][NB_CLUSTER];   // block sums of the cluster before and after the fix
     const cg::cluster_group cluster = cg::this_cluster();
@@ -352,12 +357,14 @@ static cpm_status launch_reduce(cpm_ctx* c, const void* part, int splits, int m,
     cfg.gridDim = dim3((unsigned)cl, (unsigned)m);
     cfg.blockDim = dim3((unsigned)std::min<int64_t>(NB_T, (slice + 31) / 32 * 32));
     cfg.stream = c->stream;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = (unsigned)cl;
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // as launch_after()
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     CPM_CUDA(c, cudaLaunchKernelEx(&cfg, k_gemv_reduce<P>, (const P*)part, splits, (const double*)upd_sg(c), (int)upd_ng(c), psi,
                                    c->n, m, q, (const double*)c->u, (int)c->p.symm, qtot, b, srow, SZ, gmean, ngrp));
     return CPM_OK;
@@ -452,22 +459,22 @@ cpm_status update(cpm_ctx* c, int m, const double* psi, const double* b, double*
         }
         prof_begin(c, CPM_K_GEMV);
         if (gemv_tma_supported(c)) CPM_TRY(gemv_tma(c, m, bhl, (float2*)part, splits, jchunk));
-        else if (gemv_pairs(c)) k_gemv32x2<<<grid, G2_T, 0, st>>>(c->S32, bhl, n, m, jchunk, part);
-        else k_gemv32<<<grid, GT_COLS, 0, st>>>(c->S32, bhl, n, m, jchunk, part);
+        else if (gemv_pairs(c)) CPM_CUDA(c, launch_after(k_gemv32x2, dim3(grid), dim3(G2_T), 0, st, c->S32, bhl, n, m, jchunk, part));
+        else CPM_CUDA(c, launch_after(k_gemv32, dim3(grid), dim3(GT_COLS), 0, st, c->S32, bhl, n, m, jchunk, part));
     } else {
         prof_begin(c, CPM_K_GEMV);
         const int mr = gemv64_mr(m);
         dim3 g6((unsigned)colblocks, (unsigned)splits, (unsigned)((m + mr - 1) / mr));
         if (n % 2 == 0) {
-            if (mr == 1) k_gemv64<1, 2><<<g6, G6_T, 0, st>>>(c->S, b, n, m, jchunk, part);
-            else if (mr == 2) k_gemv64<2, 2><<<g6, G6_T, 0, st>>>(c->S, b, n, m, jchunk, part);
-            else if (mr == 4) k_gemv64<4, 2><<<g6, G6_T, 0, st>>>(c->S, b, n, m, jchunk, part);
-            else k_gemv64<8, 2><<<g6, G6_T, 0, st>>>(c->S, b, n, m, jchunk, part);
+            if (mr == 1) CPM_CUDA(c, launch_after(k_gemv64<1, 2>, dim3(g6), dim3(G6_T), 0, st, c->S, b, n, m, jchunk, part));
+            else if (mr == 2) CPM_CUDA(c, launch_after(k_gemv64<2, 2>, dim3(g6), dim3(G6_T), 0, st, c->S, b, n, m, jchunk, part));
+            else if (mr == 4) CPM_CUDA(c, launch_after(k_gemv64<4, 2>, dim3(g6), dim3(G6_T), 0, st, c->S, b, n, m, jchunk, part));
+            else CPM_CUDA(c, launch_after(k_gemv64<8, 2>, dim3(g6), dim3(G6_T), 0, st, c->S, b, n, m, jchunk, part));
         } else {
-            if (mr == 1) k_gemv64<1, 1><<<g6, G6_T, 0, st>>>(c->S, b, n, m, jchunk, part);
-            else if (mr == 2) k_gemv64<2, 1><<<g6, G6_T, 0, st>>>(c->S, b, n, m, jchunk, part);
-            else if (mr == 4) k_gemv64<4, 1><<<g6, G6_T, 0, st>>>(c->S, b, n, m, jchunk, part);
-            else k_gemv64<8, 1><<<g6, G6_T, 0, st>>>(c->S, b, n, m, jchunk, part);
+            if (mr == 1) CPM_CUDA(c, launch_after(k_gemv64<1, 1>, dim3(g6), dim3(G6_T), 0, st, c->S, b, n, m, jchunk, part));
+            else if (mr == 2) CPM_CUDA(c, launch_after(k_gemv64<2, 1>, dim3(g6), dim3(G6_T), 0, st, c->S, b, n, m, jchunk, part));
+            else if (mr == 4) CPM_CUDA(c, launch_after(k_gemv64<4, 1>, dim3(g6), dim3(G6_T), 0, st, c->S, b, n, m, jchunk, part));
+            else CPM_CUDA(c, launch_after(k_gemv64<8, 1>, dim3(g6), dim3(G6_T), 0, st, c->S, b, n, m, jchunk, part));
         }
     }
     prof_end(c, CPM_K_GEMV);
