@@ -1254,6 +1254,12 @@ cpm_status bvec_run(cpm_ctx* c, int m, int64_t ne, const double* xyz, const doub
                               (longlong2*)(scr + p.off_ipart), (double*)rp));
         else CPM_TRY(rows_sf<T>(c, s1, p.rd, m, ne, EX, EY, EZ, rp));
         prof_end(c, CPM_K_SF);
+        if (fork && p.r64.use) {
+            // its CTAs need a whole SM each: behind the real-space sum, which fills every SM with small blocks for longer,
+            // the rest of this chain would start only then (EDL capacitor: 228 against 208 us)
+            CPM_CUDA(c, cudaEventRecord(c->fev[2], s1));
+            CPM_CUDA(c, cudaStreamWaitEvent(s0, c->fev[2], 0));
+        }
         const Phases<T>& sp = site_tables<T>(c);
         prof_begin(c, CPM_K_SFRED);
         if (c->rows.layered) CPM_TRY(rows_layers<T>(c, s1, p.cw, p.splits, m, rp, qs, (T*)(scr + p.off_T)));
@@ -1308,7 +1314,7 @@ cpm_status bvec_run(cpm_ctx* c, int m, int64_t ne, const double* xyz, const doub
     if (std::is_same<T, float>::value && c->rpoly.deg) {
         CPM_TRY(real_poly_run(c, st, m, p.cg, start, (const float4*)sorted, real));
     } else if (p.real64) {
-        CPM_TRY(real64_run(c, st, m, p.cg, start, sorted, sorted32, real));
+        CPM_TRY(real64_run(c, st, m, p.cg, start, sorted, sorted32, real, !(recip && p.r64.use)));
     } else if (std::is_same<T, float>::value && c->rtab && c->schunks) {
         const int4* ch4 = (const int4*)c->schunks;
         const float4* tab4 = (const float4*)c->rtab;

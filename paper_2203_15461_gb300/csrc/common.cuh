@@ -525,7 +525,7 @@ cpm_status real_poly_run(cpm_ctx* c, cudaStream_t st, int m, const CellGrid& cg,
 // real64.cu: the FP64 real-space sum (r64n = 0: the geometry keeps k_real_b)
 cpm_status build_real64(cpm_ctx* c, const std::vector<double>& etas);
 cpm_status real64_run(cpm_ctx* c, cudaStream_t st, int m, const CellGrid& cg, const int* start, const void* sorted,
-                      const float4* sorted32, double* out);
+                      const float4* sorted32, double* out, bool chained);
 
 // update.cu
 // bhl_ready: the split of b is already in update_bhl(c, m) (written by bvec in the same step)

@@ -230,12 +230,17 @@ __global__ void __launch_bounds__(32 * R6_WARPS)
 }
 
 cpm_status real64_run(cpm_ctx* c, cudaStream_t st, int m, const CellGrid& cg, const int* start, const void* sorted,
-                      const float4* sorted32, double* out) {
+                      const float4* sorted32, double* out, bool chained) {
     // a coordinate and an image shift round to 2^-24 of at most a few box lengths each
     const double lmax = std::max(c->g.boxL[0], std::max(c->g.boxL[1], c->g.boxL[2])) + c->g.rcut;
     const float slack = (float)(4e-6 * c->g.rcut * lmax);
-    CPM_CUDA(c, launch_after(k_real64, dim3((unsigned)(((int64_t)m * c->n + R6_WARPS - 1) / R6_WARPS)), dim3(32 * R6_WARPS), 0, st, 
-        c->sx, c->n, m, c->g, cg, start, (const double4_32a*)sorted, sorted32, c->r64tab, c->r64n, c->r64e0, c->rtab_id,
+    const unsigned grid = (unsigned)(((int64_t)m * c->n + R6_WARPS - 1) / R6_WARPS);
+    auto launch = [&](auto... a) {   // chained: the kernel in front of this one in the stream is all it waits for
+        if (chained) return launch_after(k_real64, dim3(grid), dim3(32 * R6_WARPS), 0, st, a...);
+        k_real64<<<grid, 32 * R6_WARPS, 0, st>>>(a...);
+        return cudaSuccess;
+    };
+    CPM_CUDA(c, launch(c->sx, c->n, m, c->g, cg, start, (const double4_32a*)sorted, sorted32, c->r64tab, c->r64n, c->r64e0, c->rtab_id,
         slack, out));
     CPM_LAUNCH(c, "k_real64");
     return CPM_OK;
