@@ -271,15 +271,16 @@ template <> struct PartSum<float> { using type = PartSumF; };   // partials of t
 // result (plain FP64 sums in a fixed order: the rounding, about n eps max|q|, is far below the 1e-12 e the total
 // is held to).
 //
-// Grid (cluster of up to eight blocks, m): one cluster per replica, one thread per site (slices beyond 640 sites take
+// Grid (cluster of up to sixteen blocks, m): one cluster per replica, one thread per site (slices beyond 640 sites take
 // several passes), the block sums exchanged through distributed shared memory, so that every thread still holds
 // its q when e^T q is known.  With a replica's last block (a ticket) doing the fix, that block read the whole q
 // back.  Whole steps, before and now: 4,320 sites x 8 replicas 158.3 and 155.4 us, the product alone x 64 80.0 and
 // 74.5, 512 sites x 4 54.0 and 51.2, 256 small replicas 184 and 178.  Bounded by the latency of the loads and of
-// two cluster barriers; 48 registers let two blocks of 640 threads share an SM (with 64, one: the product took 89 us).
-constexpr int NB_CLUSTER = 8;
+// two cluster barriers, and FP64 at sixteen clocks a warp and SM: one warp adds a block's values (the product x 64
+// 67.9 with a tree per warp, 65.5 now).  48 registers let two blocks of 640 threads share an SM (with 64, one: the product took 89 us).
+constexpr int NB_CLUSTER = 16;  // blocks per replica, at most; more than eight where the replicas are few
 constexpr int NB_T = 640;      // threads per block, at most
-constexpr int NB_LEAST = 128;   // sites per block that a cluster of several blocks has at least
+constexpr int NB_LEAST = 64;    // sites per block that a cluster of several blocks has at least
 template <typename P>
 __global__ void __launch_bounds__(NB_T, 2) k_gemv_reduce(const P* __restrict__ part, int splits,
                                                       const double* __restrict__ SG, int ng,
@@ -289,20 +290,20 @@ __global__ void __launch_bounds__(NB_T, 2) k_gemv_reduce(const P* __restrict__ p
                                                       const double* __restrict__ srow, const double* __restrict__ SZ,
                                                       const double* __restrict__ gmean, int ngrp) {
     grid_wait();
-    __shared__ double sh[NB_T / 32];
+    __shared__ double sh[NB_T];
     __shared__ double csum[2][NB_CLUSTER];   // block sums of the cluster before and after the fix
     const cg::cluster_group cluster = cg::this_cluster();
     const int r = blockIdx.y, cl = gridDim.x, rank = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t slice = (n + cl - 1) / cl, lo = rank * slice, hi = min(n, lo + slice);
     double* qr = q + (int64_t)r * n;
-    auto exchange = [&](double a, int which) {   // fixed order: warp trees, warps in order, blocks in order
-        for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
-        if (lane == 0) sh[warp] = a;
+    auto exchange = [&](double a, int which) {   // fixed order: lanes over the block's values, a warp tree, blocks in order
+        sh[threadIdx.x] = a;
         __syncthreads();
-        if ((int)threadIdx.x < cl) {
-            double t = sh[0];
-            for (int w = 1; w < (int)blockDim.x / 32; ++w) t += sh[w];
-            *cluster.map_shared_rank(&csum[which][rank], threadIdx.x) = t;
+        if (warp == 0) {   // one warp: an FP64 instruction occupies the SM for sixteen clocks whatever its lanes do
+            double t = sh[lane];
+            for (int k = lane + 32; k < (int)blockDim.x; k += 32) t += sh[k];
+            for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+            if (lane < cl) *cluster.map_shared_rank(&csum[which][rank], lane) = t;
         }
         cluster.sync();
         double t = csum[which][0];
@@ -350,8 +351,10 @@ __global__ void __launch_bounds__(NB_T, 2) k_gemv_reduce(const P* __restrict__ p
 template <typename P>
 static cpm_status launch_reduce(cpm_ctx* c, const void* part, int splits, int m, const double* psi, double* q, double* qtot,
                                 const double* b, const double* srow, const double* SZ, const double* gmean, int ngrp) {
-    int cl = NB_CLUSTER;
-    while (cl > 1 && c->n < (int64_t)cl * NB_LEAST) cl /= 2;
+    // sixteen blocks up to four replicas (one replica of 4,320 sites: 108 against 109.5 us a step; eight: 143.0 against 142.4)
+    int cl = m <= 4 ? NB_CLUSTER : 8;
+    while (cl > 1 && c->n < (int64_t)cl * (cl > 8 ? 2 * NB_LEAST : NB_LEAST)) cl /= 2;
+    if (cl > 8) CPM_CUDA(c, cudaFuncSetAttribute(k_gemv_reduce<P>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     const int64_t slice = (c->n + cl - 1) / cl;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)cl, (unsigned)m);
