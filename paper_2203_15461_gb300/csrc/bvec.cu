@@ -1017,6 +1017,7 @@ __global__ void __launch_bounds__(256, 2) k_site32(const int2* __restrict__ cols
 // b[r][i] = K_E (recip + real - pi Q_tot / (V alpha^2) + boundary)
 // with bhl also the two-float split of b for the single-precision S product (the same arithmetic as
 // k_split_b, so the update gives bit-identical results either way)
+constexpr int CB_T = 64;
 template <typename T>
 __global__ void k_combine(const T* partial, int nctiles, const double* real, const double* b0, const int* zmap,
                           int nzu, const double* stats, const double* sx, int64_t n, int m, Geometry g, double* b,
@@ -1028,7 +1029,7 @@ __global__ void k_combine(const T* partial, int nctiles, const double* real, con
     const int64_t i = t % n;
     const double rl = real[t];   // issued with the tile loads below
     const double bz = b0 ? b0[(int64_t)r * nzu + zmap[i]] : 0.0;
-    double s = 0.0;
+    TermSum<T> tiles;
     const T* pp = partial + (int64_t)r * nctiles * n + i;
     int k = 0;
     for (; k + 16 <= nctiles; k += 16) {   // sixteen loads in flight, added in tile order
@@ -1036,17 +1037,18 @@ __global__ void k_combine(const T* partial, int nctiles, const double* real, con
 #pragma unroll
         for (int u = 0; u < 16; ++u) x[u] = pp[(int64_t)(k + u) * n];
 #pragma unroll
-        for (int u = 0; u < 16; ++u) s += (double)x[u];
+        for (int u = 0; u < 16; ++u) tiles.add(x[u]);
     }
     if (k + 8 <= nctiles) {
         T x[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) x[u] = pp[(int64_t)(k + u) * n];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) s += (double)x[u];
+        for (int u = 0; u < 8; ++u) tiles.add(x[u]);
         k += 8;
     }
-    for (; k < nctiles; ++k) s += (double)pp[(int64_t)k * n];
+    for (; k < nctiles; ++k) tiles.add(pp[(int64_t)k * n]);
+    double s = tiles.value();
     s += rl;
     if (b0) s += bz;
     if (pm) s += pm[t];   // P3M: the mesh potential in place of the Ewald tiles
@@ -1353,7 +1355,8 @@ cpm_status bvec_run(cpm_ctx* c, int m, int64_t ne, const double* xyz, const doub
         CPM_CUDA(c, cudaStreamWaitEvent(s0, c->fev[4], 0));
     }
     prof_begin(c, CPM_K_COMBINE);
-    k_combine<T><<<(unsigned)(((int64_t)m * n + 255) / 256), 256, 0, st>>>(part, p.nctiles, real, b0, c->zmap, c->nzu,
+    // small blocks: 16,000 outputs (four replicas of the tubes) in blocks of 256 used 63 SMs
+    k_combine<T><<<(unsigned)(((int64_t)m * n + CB_T - 1) / CB_T), CB_T, 0, st>>>(part, p.nctiles, real, b0, c->zmap, c->nzu,
                                                                           stats, c->sx, n, m, c->g, b_out, bhl, ew,
                                                                           pm);
     prof_end(c, CPM_K_COMBINE);

@@ -92,6 +92,29 @@ struct PartSumF {   // single FP32 partials, the same two-sum
     __device__ __forceinline__ double value() const { return s.value(); }
 };
 
+// sum of terms of type T without loss against FP64: FP32 terms in three FP32 words by two exact two-sums (13
+// instructions of the FP32 pipe; a conversion and an addition in FP64 hold the SM for 32 clocks)
+template <typename T> struct TermSum;
+template <> struct TermSum<double> {
+    double v = 0.0;
+    __device__ __forceinline__ void add(double x) { v += x; }
+    __device__ __forceinline__ double value() const { return v; }
+};
+template <> struct TermSum<float> {
+    float a = 0.f, b = 0.f, c = 0.f;
+    __device__ __forceinline__ static float err(float s, float x, float y) {   // x + y - s, exactly
+        const float t = __fsub_rn(s, x);
+        return __fadd_rn(__fsub_rn(x, __fsub_rn(s, t)), __fsub_rn(y, t));
+    }
+    __device__ __forceinline__ void add(float x) {
+        const float s = __fadd_rn(a, x), e = err(s, a, x), t = __fadd_rn(b, e);
+        c = __fadd_rn(c, err(t, b, e));
+        a = s;
+        b = t;
+    }
+    __device__ __forceinline__ double value() const { return (double)a + ((double)b + (double)c); }
+};
+
 // ----------------------------------------------------------------------------- device status word
 // Kernels never trap: they set one of these bits and return.  The host reads the
 // word when it synchronises.
