@@ -311,8 +311,8 @@ __global__ void __launch_bounds__(8 * CP_PTS) k_charge_phases(const double* __re
     }
 }
 
-// The same in fixed point (tc_rows64.cu): cos and sin times 2^62 in 64-bit integers, X times the scaled charge, Z
-// rounded to 2^55.  FP64 arithmetic took 34 us for 5,700 charges of 110 harmonics, the integers 9.5 us: the 64-bit
+// The same in fixed point, for FP64: cos and sin times 2^62 in 64-bit integers (tc_rows64.cu takes them as they are, X
+// times the scaled charge, Z rounded to 2^55; k_rows_sf<double> converted at the end).  FP64 arithmetic took 34 us for 5,700 charges of 110 harmonics, the integers 9.5 us (100 charges in k_rows_sf<double>: 11 and 3 us): the 64-bit
 // product of two phases is some 40 instructions of a pipe with thirty times the rate.  A phase is evaluated as
 // T1[top ten bits] T2[next ten] (1 - d^2 / 2, d - d^3 / 6) with the angle d < 2 pi 2^-20 of the other 44 bits: the
 // terms left out are below 2^-72, T1 is FP64's own cosine and sine, and T2's are kept as 1 - cos, exact to 2^-62.
@@ -342,7 +342,14 @@ __device__ __forceinline__ longlong2 fx_phase(uint64_t f, const longlong2* __res
     return make_longlong2(b.x - __mul64hi(b.x, v4) - (__mul64hi(b.y, sn) >> 14),
                           b.y - __mul64hi(b.y, v4) + (__mul64hi(b.x, sn) >> 14));
 }
-// grid (P / CP_PTS, axis); P and nep are multiples of CP_PTS
+// v 2^-62, the exponent changed in integers
+__device__ __forceinline__ double fx_double(int64_t v) {
+    const double d = (double)v;
+    return v ? __hiloint2double(__double2hiint(d) - (62 << 20), __double2loint(d)) : 0.0;
+}
+// grid (P / CP_PTS, axis).  FIXED: X, Y, Z in fixed point, replicas padded to nep, a multiple of CP_PTS, charges scaled
+// with qexp.  Otherwise the phases in FP64 (k_rows_sf<double>): nep = ne, and X times the charge itself.
+template <bool FIXED>
 __global__ void __launch_bounds__(8 * CP_PTS) k_charge_fixed(const double* __restrict__ xyz, const double* __restrict__ Q,
                                                              int64_t P, int64_t ne, int64_t nep, double3 inv, int NX,
                                                              int NY, int NZ, const int* __restrict__ qexp,
@@ -356,10 +363,10 @@ __global__ void __launch_bounds__(8 * CP_PTS) k_charge_fixed(const double* __res
     const int64_t p = (int64_t)blockIdx.x * CP_PTS + pt;
     if (k == 0) {
         const int64_t r = p / nep, j = p - r * nep, src = r * ne + j;
-        const double q = j < ne ? Q[src] : 0.0;
+        const double q = p < P && j < ne ? Q[src] : 0.0;
         // a zero charge (padding) contributes nothing wherever it sits
         sf[pt] = q != 0.0 ? row_frac(xyz[3 * src + axis], axis == 0 ? inv.x : axis == 1 ? inv.y : inv.z) : 0ull;
-        sq[pt] = __double2ll_rn(q * pow2_bits(2045 - min(max(qexp[r], 1), ROW64_EMAX)) * 0x1p62);
+        sq[pt] = FIXED ? __double2ll_rn(q * pow2_bits(2045 - min(max(qexp[r], 1), ROW64_EMAX)) * 0x1p62) : __double_as_longlong(q);
     }
     __syncthreads();
     const int H = axis == 0 ? NX : axis == 1 ? NY : NZ, na = H / 8 + 1;
@@ -367,7 +374,7 @@ __global__ void __launch_bounds__(8 * CP_PTS) k_charge_fixed(const double* __res
     const uint64_t f = sf[pt];
     longlong2 base = make_longlong2(1ll << 62, 0);
     if (k > 0 && k <= H) base = fx_phase(f * (uint64_t)k, tab);
-    if (axis == 0) base = make_longlong2(__mul64hi(base.x, sq[pt]) * 4 + 2, __mul64hi(base.y, sq[pt]) * 4 + 2);
+    if (FIXED && axis == 0) base = make_longlong2(__mul64hi(base.x, sq[pt]) * 4 + 2, __mul64hi(base.y, sq[pt]) * 4 + 2);
     for (int a0 = 0; a0 < na; a0 += 8) {   // eight steps 8 a at a time
         const int a = a0 + k;
         __syncthreads();
@@ -375,10 +382,17 @@ __global__ void __launch_bounds__(8 * CP_PTS) k_charge_fixed(const double* __res
         __syncthreads();
         for (int b = 0; b < min(8, na - a0); ++b) {
             const int h = 8 * (a0 + b) + k;
-            if (h > H) continue;
+            if (h > H || p >= P) continue;
             longlong2 v = a0 + b == 0 ? base : fx_mul(sg[b][pt], base);
-            if (axis == 2) v = make_longlong2((v.x + 64) >> 7, (v.y + 64) >> 7);
-            out[(int64_t)h * P + p] = v;
+            if (FIXED) {
+                if (axis == 2) v = make_longlong2((v.x + 64) >> 7, (v.y + 64) >> 7);
+                out[(int64_t)h * P + p] = v;
+            } else {
+                const double q = axis == 0 ? __longlong_as_double(sq[pt]) : 1.0;
+                double2 d = make_double2(fx_double(v.x), fx_double(v.y));
+                if (axis == 0) { d.x *= q; d.y *= q; }
+                ((double2*)out)[(int64_t)h * P + p] = d;
+            }
         }
     }
 }
@@ -679,17 +693,25 @@ template <typename T> static const Phases<T>& row_sites(const cpm_ctx* c);
 template <> const Phases<double>& row_sites<double>(const cpm_ctx* c) { return c->site64; }
 template <> const Phases<float>& row_sites<float>(const cpm_ctx* c) { return c->site32; }
 
-template <typename T>
-cpm_status launch_charge_phases(cpm_ctx* c, cudaStream_t st, int64_t P, const double* xyz, const double* Q, c2<T>* X,
-                                c2<T>* Y, c2<T>* Z) {
+template <>
+cpm_status launch_charge_phases<float>(cpm_ctx* c, cudaStream_t st, int64_t P, const double* xyz, const double* Q, float2* X,
+                                       float2* Y, float2* Z) {
     const KTable& k = c->kt;
-    k_charge_phases<T, false><<<(unsigned)((P + CP_PTS - 1) / CP_PTS), 8 * CP_PTS, 0, st>>>(
+    k_charge_phases<float, false><<<(unsigned)((P + CP_PTS - 1) / CP_PTS), 8 * CP_PTS, 0, st>>>(
         xyz, Q, P, P, P, c->g.inv[0], c->g.inv[1], c->g.inv[2], k.NX, k.NY, k.NZ, X, Y, Z, nullptr, nullptr);
     CPM_LAUNCH(c, "k_charge_phases");
     return CPM_OK;
 }
-template cpm_status launch_charge_phases<double>(cpm_ctx*, cudaStream_t, int64_t, const double*, const double*, double2*, double2*, double2*);
-template cpm_status launch_charge_phases<float>(cpm_ctx*, cudaStream_t, int64_t, const double*, const double*, float2*, float2*, float2*);
+template <>
+cpm_status launch_charge_phases<double>(cpm_ctx* c, cudaStream_t st, int64_t P, const double* xyz, const double* Q, double2* X,
+                                        double2* Y, double2* Z) {
+    const KTable& k = c->kt;
+    k_charge_fixed<false><<<dim3((unsigned)((P + CP_PTS - 1) / CP_PTS), 3), 8 * CP_PTS, 0, st>>>(
+        xyz, Q, P, P, P, make_double3(c->g.inv[0], c->g.inv[1], c->g.inv[2]), k.NX, k.NY, k.NZ, nullptr, c->rows.fxtab,
+        (longlong2*)X, (longlong2*)Y, (longlong2*)Z);
+    CPM_LAUNCH(c, "k_charge_fixed");
+    return CPM_OK;
+}
 
 int64_t charge_slots(const KTable& k) { return (k.NX + 1) + (k.NY + 1) + 8 + (k.NZ / 8 + 1); }
 
@@ -709,7 +731,7 @@ cpm_status launch_charge_fixed(cpm_ctx* c, cudaStream_t st, int m, int64_t ne, i
                                const double* Q, const int* qexp, longlong2* X, longlong2* Y, longlong2* Z) {
     const KTable& k = c->kt;
     const int64_t P = (int64_t)m * nep;
-    CPM_CUDA(c, launch_after(k_charge_fixed, dim3((unsigned)(P / CP_PTS), 3), dim3(8 * CP_PTS), 0, st, 
+    CPM_CUDA(c, launch_after(k_charge_fixed<true>, dim3((unsigned)(P / CP_PTS), 3), dim3(8 * CP_PTS), 0, st, 
         xyz, Q, P, ne, nep, make_double3(c->g.inv[0], c->g.inv[1], c->g.inv[2]), k.NX, k.NY, k.NZ, qexp, c->rows.fxtab, X, Y, Z));
     CPM_LAUNCH(c, "k_charge_fixed");
     return CPM_OK;
