@@ -103,9 +103,37 @@ template <typename T> struct P3mV4;
 template <> struct P3mV4<float> { using t = float4; };
 template <> struct P3mV4<double> { using t = double4_32a; };
 
+// The bricks of a mesh (x fastest) and those that the stencil of a charge reaches, each once.
+constexpr int P3M_BZ = 4;            // planes per brick (lanes 8 z + y of the assignment)
+struct P3mBricks {
+    int BX, BY, nx, ny, nz;
+    __host__ __device__ int n() const { return nx * ny * nz; }
+    template <typename F> __device__ __forceinline__ void each(int kv, int P, F f) const {
+        if (kv < 0) return;   // no charge
+        const int x = kv & 1023, y = (kv >> 10) & 1023, z = kv >> 20;
+        const int x0 = x / BX, y0 = y / BY, z0 = z / P3M_BZ;
+        const int cx = min(nx, (x + P - 1) / BX - x0 + 1), cy = min(ny, (y + P - 1) / BY - y0 + 1),
+                  cz = min(nz, (z + P - 1) / P3M_BZ - z0 + 1);
+        for (int c = 0; c < cz; ++c)
+            for (int b = 0; b < cy; ++b)
+                for (int a = 0; a < cx; ++a) {
+                    int bx = x0 + a, by = y0 + b, bz = z0 + c;
+                    if (bx >= nx) bx -= nx;
+                    if (by >= ny) by -= ny;
+                    if (bz >= nz) bz -= nz;
+                    f((bz * ny + by) * nx + bx);
+                }
+    }
+    // at most this many bricks per charge
+    int most(int P) const {
+        return std::min(nx, (P + BX - 2) / BX + 1) * std::min(ny, (P + BY - 2) / BY + 1) * std::min(nz, (P + P3M_BZ - 2) / P3M_BZ + 1);
+    }
+};
+
 template <typename T>
 __global__ void k_p3m_prep(const double* __restrict__ xyz, const double* __restrict__ Q, int64_t ptot, Geometry g,
-                           int Kx, int Ky, int Kz, int P, int* __restrict__ key, typename P3mV4<T>::t* __restrict__ fq) {
+                           int Kx, int Ky, int Kz, int P, int* __restrict__ key, typename P3mV4<T>::t* __restrict__ fq,
+                           int64_t ne, P3mBricks br, int nsplit, int64_t per, int* __restrict__ count) {
     grid_go();
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= ptot) return;
@@ -123,7 +151,10 @@ __global__ void k_p3m_prep(const double* __restrict__ xyz, const double* __restr
         if (bi < 0) bi += K[d];
         b[d] = bi;
     }
-    key[t] = q == 0.0 ? -1 : (b[0] | (b[1] << 10) | (b[2] << 20));
+    const int kv = q == 0.0 ? -1 : (b[0] | (b[1] << 10) | (b[2] << 20));
+    key[t] = kv;
+    const int64_t r = t / ne, row = r * nsplit + (t - r * ne) / per;
+    br.each(kv, P, [&](int brick) { atomicAdd(&count[row * br.n() + brick], 1); });
     typename P3mV4<T>::t v;
     v.x = (T)f[0]; v.y = (T)f[1]; v.z = (T)f[2]; v.w = (T)q;
     fq[t] = v;
@@ -153,10 +184,13 @@ __device__ __forceinline__ void bspline_weights(T f, T* w) {
 
 // ----------------------------------------------------------------------------- charge assignment
 // grid (bricks, replicas, charge splits); a brick is BX x BY x BZ mesh points (x fastest), brick
-// index bx fastest; split sp takes the chunks [sp cps, (sp + 1) cps) of NT charges of the replica.
-// Those whose stencil reaches into the brick are compacted (warp ballots, then warp offsets) into
-// shared memory with their 3 p weights and their stencil origin relative to the brick; then a warp takes one charge
-// at a time, lane = (plane of the brick, y offset), each lane adding its p x contributions.
+// index bx fastest.  The charges whose stencil reaches into a brick are listed beforehand (counted with the
+// preparation, k_p3m_scan, k_p3m_fill; the order within a list varies, the sums do not): with each brick looking through
+// all keys of its replica, that took half of the time (270 of 538 us for 16,384 sites x 16 replicas), and the
+// weights of the few charges found were formed by warps with two lanes of work.  A split takes a fixed range of
+// the replica's charges, so that its sum does not depend on the order either.  Their 3 p weights and the stencil origins relative to the brick go to shared memory,
+// NT charges at a time; then a warp takes one charge at a time, lane = (plane of the brick, y offset), each lane
+// adding its p x contributions.
 // Every contribution is rounded to 2^-40 e (FP64: 2^-60 e) and added as exact integers split over
 // 32-bit words, a = floor(v 2^20), then the next 20 bits (FP64: and 20 more), with native 32-bit
 // shared-memory atomics; integer addition is associative, so the brick's charge does not depend on
@@ -172,12 +206,57 @@ __device__ __forceinline__ void bspline_weights(T f, T* w) {
 template <typename T> struct P3mWords { static constexpr int n = std::is_same<T, double>::value ? 3 : 2; };
 constexpr int P3M_NT = 512;          // threads and charges per chunk of the assignment
 constexpr int P3M_CARRY = 1024;
-constexpr int P3M_BZ = 4;            // planes per brick (lanes 8 z + y)
+
+// start[r][split][brick]: exclusive sums of the nb counts of a replica, one block each
+constexpr int P3M_SCAN = 256;
+__global__ void __launch_bounds__(P3M_SCAN) k_p3m_scan(const int* __restrict__ count, int nb, int* __restrict__ start) {
+    grid_wait();
+    grid_go();
+    __shared__ int sw[P3M_SCAN / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t r0 = (int64_t)blockIdx.x * nb;
+    int carry = 0;
+    for (int i0 = 0; i0 < nb; i0 += P3M_SCAN) {
+        const int i = i0 + threadIdx.x, c = i < nb ? count[r0 + i] : 0;
+        int v = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(0xffffffffu, v, o);
+            if (lane >= o) v += u;
+        }
+        if (lane == 31) sw[warp] = v;
+        __syncthreads();
+        int before = carry, all = 0;
+#pragma unroll
+        for (int w = 0; w < P3M_SCAN / 32; ++w) {
+            before += w < warp ? sw[w] : 0;
+            all += sw[w];
+        }
+        if (i < nb) start[r0 + i] = before + v - c;
+        carry += all;
+        __syncthreads();
+    }
+}
+
+// list[r ne most + start + ..]: the charges of every brick and split (`per` charges each); the starts become ends
+__global__ void __launch_bounds__(256) k_p3m_fill(const int* __restrict__ key, int64_t ptot, int64_t ne, int P, P3mBricks br,
+                                                int nsplit, int64_t per, int most, int* __restrict__ start, int* __restrict__ list) {
+    grid_wait();
+    const int64_t t = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (t >= ptot) return;
+    const int64_t r = t / ne, j = t - r * ne, row = r * nsplit + j / per;
+    int* mine = list + r * ne * most;
+    br.each(key[t], P, [&](int brick) {
+        mine[atomicAdd(&start[row * br.n() + brick], 1)] = (int)j;
+    });
+}
 
 template <typename T, int P>
 __global__ void __launch_bounds__(P3M_NT) k_p3m_spread(const int* __restrict__ key,
                                                        const typename P3mV4<T>::t* __restrict__ fq, int64_t ne, int m,
-                                                       int Kx, int Ky, int Kz, int BX, int BY, int cps,
+                                                       int Kx, int Ky, int Kz, int BX, int BY,
+                                                       const int* __restrict__ count, const int* __restrict__ start,
+                                                       const int* __restrict__ list, int most,
                                                        c2<T>* __restrict__ part, int* __restrict__ flag) {
     grid_wait();
     constexpr int NW = P3mWords<T>::n, BZ = P3M_BZ;
@@ -187,14 +266,15 @@ __global__ void __launch_bounds__(P3M_NT) k_p3m_spread(const int* __restrict__ k
     int* A = (int*)p3m_smem;                            // [NW words][NB]
     T* sw = (T*)(A + ((NW * NB + 3) & ~3));             // [NT][3 p + 1]: weights x | y | z, then Q
     int* so = (int*)(sw + P3M_NT * (3 * P + 1));        // [NT]: origin sx | sy << 10 | sz << 20
-    __shared__ int wcount[P3M_NT / 32];
     const int nbx = Kx / BX, nby = Ky / BY;
     const int bi = blockIdx.x, rep = blockIdx.y;
     const int b0x = (bi % nbx) * BX, b0y = ((bi / nbx) % nby) * BY, b0z = (bi / (nbx * nby)) * BZ;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int64_t jbeg = (int64_t)blockIdx.z * cps * P3M_NT;
-    const int64_t jend = min(ne, jbeg + (int64_t)cps * P3M_NT);
-    const int64_t base = (int64_t)rep * ne;
+    const int64_t base = (int64_t)rep * ne, at = ((int64_t)rep * gridDim.z + blockIdx.z) * gridDim.x + bi;
+    const int total = count[at];
+    if (threadIdx.x == 0) flag[((int64_t)blockIdx.z * m + rep) * gridDim.x + bi] = total > 0;
+    if (total == 0) return;   // uniform
+    const int* mine = list + base * most + start[at] - total;   // start holds the end
     auto carry = [&]() {   // every point's words belong to one thread here
         __syncthreads();
         for (int i = threadIdx.x; i < NB; i += P3M_NT) {
@@ -209,45 +289,21 @@ __global__ void __launch_bounds__(P3M_NT) k_p3m_spread(const int* __restrict__ k
         }
         __syncthreads();
     };
-    int added = -1;        // charges since the last carry; -1: nothing reached the brick yet
-    for (int64_t j0 = jbeg; j0 < jend; j0 += P3M_NT) {
-        const int64_t j = j0 + threadIdx.x;
-        bool sel = false;
-        int sx = 0, sy = 0, sz = 0;
-        if (j < jend) {
-            const int kv = key[base + j];
-            if (kv >= 0) {
-                sx = ((kv & 1023) - b0x + Kx) & (Kx - 1);
-                sy = (((kv >> 10) & 1023) - b0y + Ky) & (Ky - 1);
-                sz = ((kv >> 20) - b0z + Kz) & (Kz - 1);
-                sel = (sx < BX || sx + P - 1 >= Kx) && (sy < BY || sy + P - 1 >= Ky) &&
-                      (sz < BZ || sz + P - 1 >= Kz);
-            }
-        }
-        const unsigned bal = __ballot_sync(0xffffffffu, sel);
-        if (lane == 0) wcount[wid] = __popc(bal);
-        __syncthreads();   // also orders the previous chunk's reads of sw / so before the writes below
-        int off = 0, L = 0;
-#pragma unroll
-        for (int w = 0; w < P3M_NT / 32; ++w) {
-            const int cw = wcount[w];
-            off += w < wid ? cw : 0;
-            L += cw;
-        }
-        if (L == 0) {   // uniform
-            __syncthreads();
-            continue;
-        }
-        if (added < 0) {
-            for (int i = threadIdx.x; i < NW * NB; i += P3M_NT) A[i] = 0;
-            added = 0;
-        } else if (added + L > P3M_CARRY) {
+    int added = 0;         // charges since the last carry
+    for (int i = threadIdx.x; i < NW * NB; i += P3M_NT) A[i] = 0;
+    for (int j0 = 0; j0 < total; j0 += P3M_NT) {
+        const int L = min(P3M_NT, total - j0);
+        if (added + L > P3M_CARRY) {
             carry();
             added = 0;
         }
         added += L;
-        if (sel) {
-            const int slot = off + __popc(bal & ((1u << lane) - 1u));
+        if ((int)threadIdx.x < L) {
+            const int slot = threadIdx.x;
+            const int64_t j = mine[j0 + slot];
+            const int kv = key[base + j];
+            const int sx = ((kv & 1023) - b0x + Kx) & (Kx - 1), sy = (((kv >> 10) & 1023) - b0y + Ky) & (Ky - 1),
+                      sz = ((kv >> 20) - b0z + Kz) & (Kz - 1);
             const typename P3mV4<T>::t v = fq[base + j];
             T* w = sw + slot * (3 * P + 1);
             bspline_weights<T, P>(v.x, w);
@@ -273,7 +329,7 @@ __global__ void __launch_bounds__(P3M_NT) k_p3m_spread(const int* __restrict__ k
             if (std::is_same<T, float>::value && fabs(q) <= (T)2 && ox + P <= BX) {
                 // the usual case, uniform in the warp: no wrap or clipping in x, and |v| 2^20 < 2^22, so that
                 // adding 1.5 2^23 rounds without a conversion instruction; index arithmetic of the general branch
-                // taken out, 16,384 sites x 16 replicas of 32,768 charges: 656 -> 538 us
+                // taken out, 16,384 sites x 16 replicas of up to 32,768 charges: 656 -> 538 us, before the lists
                 const float s20 = (float)wyz * 1048576.0f;
                 int* r0 = row + ox;
 #pragma unroll
@@ -309,10 +365,8 @@ __global__ void __launch_bounds__(P3M_NT) k_p3m_spread(const int* __restrict__ k
                 }
             }
         }
+        __syncthreads();   // the weights are free, at the end the sums complete
     }
-    if (threadIdx.x == 0) flag[((int64_t)blockIdx.z * m + rep) * gridDim.x + bi] = added >= 0;
-    if (added < 0) return;   // uniform
-    __syncthreads();
     const int64_t N = (int64_t)Kx * Ky * Kz;
     T* out = (T*)(part + ((int64_t)blockIdx.z * ((m + 1) / 2) + rep / 2) * N) + (rep & 1);
     for (int i = threadIdx.x; i < BX * BY * BZ; i += P3M_NT) {
@@ -600,20 +654,22 @@ static int64_t mesh_pts(const cpm_ctx* c) {
     return (int64_t)c->p.p3m_mesh[0] * c->p.p3m_mesh[1] * c->p.p3m_mesh[2];
 }
 
-// Assignment bricks of 32 x 32 x 4 points at most and charge splits: enough CTAs that the bricks within the
-// electrolyte, about a third, still fill two CTAs per SM a few times; no split without a chunk of charges, at
-// most 8 partial meshes.
-struct P3mSpread { int BX, BY, nbricks, nsplit, cps; };
+// Assignment bricks of 32 x 32 x 4 points at most and charge splits: enough CTAs that the uneven bricks within the
+// electrolyte, about a third, even out (16,384 sites x 16 replicas: 1,309 us a step without a split, 1,121 with three,
+// 1,109 with five, 1,130 with eight), no split with less than three chunks of charges (4,320 x 8: 190 us with six splits
+// of two, 182.5 with four of three: every split is a partial mesh to be written and added), at most 8.
+struct P3mSpread { int BX, BY, nbricks, nsplit, cps; P3mBricks br; };
 static P3mSpread p3m_spread_plan(const cpm_ctx* c, int m, int64_t ne) {
     P3mSpread sp;
     const int Kx = c->p.p3m_mesh[0], Ky = c->p.p3m_mesh[1], Kz = c->p.p3m_mesh[2];
     sp.BX = std::min(Kx, 32);
     sp.BY = std::min(Ky, 32);
-    sp.nbricks = (Kx / sp.BX) * (Ky / sp.BY) * (Kz / P3M_BZ);
+    sp.br = P3mBricks{sp.BX, sp.BY, Kx / sp.BX, Ky / sp.BY, Kz / P3M_BZ};
+    sp.nbricks = sp.br.n();
     const int64_t ctas = (int64_t)sp.nbricks * m;
     const int64_t nchunks = std::max<int64_t>(1, (ne + P3M_NT - 1) / P3M_NT);
-    int64_t ns = std::max<int64_t>(1, (16 * 152 + ctas - 1) / ctas);
-    ns = std::min<int64_t>(std::min<int64_t>(ns, 8), nchunks);
+    int64_t ns = std::max<int64_t>(1, (32 * 152 + ctas - 1) / ctas);
+    ns = std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(ns, 8), nchunks / 3));
     sp.cps = (int)((nchunks + ns - 1) / ns);
     sp.nsplit = (int)((nchunks + sp.cps - 1) / sp.cps);
     return sp;
@@ -624,8 +680,8 @@ size_t p3m_scratch_bytes(const cpm_ctx* c, int m, int64_t ne) {
     const int64_t ptot = (int64_t)m * ne;
     const P3mSpread sp = p3m_spread_plan(c, m, ne);
     return p3m_al(sizeof(int) * ptot) + p3m_al(sizeof(typename P3mV4<T>::t) * ptot) +
-           p3m_al(sizeof(int) * (size_t)sp.nsplit * m * sp.nbricks) +
-           p3m_al(sizeof(c2<T>) * (size_t)sp.nsplit * ((m + 1) / 2) * mesh_pts(c));
+           3 * p3m_al(sizeof(int) * (size_t)sp.nsplit * m * sp.nbricks) +   // marks, counts, starts
+           p3m_al(sizeof(int) * (size_t)ptot * sp.br.most(c->p.p3m_order)) + p3m_al(sizeof(c2<T>) * (size_t)sp.nsplit * ((m + 1) / 2) * mesh_pts(c));
 }
 template size_t p3m_scratch_bytes<float>(const cpm_ctx*, int, int64_t);
 template size_t p3m_scratch_bytes<double>(const cpm_ctx*, int, int64_t);
@@ -737,7 +793,8 @@ template <typename T> static const c2<T>* p3m_twiddles(const cpm_ctx* c) {
 
 template <typename T, int P>
 static cpm_status launch_p3m_pp(cudaStream_t st, cpm_ctx* c, int m, int64_t ne, const int* key,
-                          const typename P3mV4<T>::t* fq, int* flag, c2<T>* mesh, double* pm) {
+                          const typename P3mV4<T>::t* fq, int* flag, const int* count, const int* start, const int* list, int most,
+                          c2<T>* mesh, double* pm) {
     const int Kx = c->p.p3m_mesh[0], Ky = c->p.p3m_mesh[1], Kz = c->p.p3m_mesh[2];
     const P3mSpread sp = p3m_spread_plan(c, m, ne);
     const int npairs = (m + 1) / 2;
@@ -745,7 +802,7 @@ static cpm_status launch_p3m_pp(cudaStream_t st, cpm_ctx* c, int m, int64_t ne, 
                        sizeof(T) * P3M_NT * (3 * P + 1) + sizeof(int) * P3M_NT;
     CPM_CUDA(c, cudaFuncSetAttribute(k_p3m_spread<T, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssm));
     CPM_CUDA(c, launch_after(k_p3m_spread<T, P>, dim3(sp.nbricks, m, sp.nsplit), dim3(P3M_NT), ssm, st, key, fq, ne, m, Kx, Ky, Kz, sp.BX, sp.BY,
-                                                                            sp.cps, mesh, flag));
+                                                                            count, start, list, most, mesh, flag));
     const int64_t sstride = (int64_t)npairs * Kx * Ky * Kz;
     const c2<T>* tw = p3m_twiddles<T>(c);
     const size_t psm = sizeof(c2<T>) * ((size_t)Kx * Ky + Kx / 2 + Ky / 2);
@@ -781,19 +838,30 @@ cpm_status p3m_run(cpm_ctx* c, cudaStream_t st, int m, int64_t ne, const double*
     V4T* fq = (V4T*)(scr + p3m_al(sizeof(int) * ptot));
     int* flag = (int*)((char*)fq + p3m_al(sizeof(V4T) * ptot));
     const P3mSpread sp = p3m_spread_plan(c, m, ne);
-    c2<T>* mesh = (c2<T>*)((char*)flag + p3m_al(sizeof(int) * (size_t)sp.nsplit * m * sp.nbricks));
+    const size_t lists = p3m_al(sizeof(int) * (size_t)sp.nsplit * m * sp.nbricks);
+    int* count = (int*)((char*)flag + lists);
+    int* start = (int*)((char*)count + lists);
+    int* list = (int*)((char*)start + lists);
+    const int most = sp.br.most(c->p.p3m_order);
+    c2<T>* mesh = (c2<T>*)((char*)list + p3m_al(sizeof(int) * (size_t)ptot * most));
     const int P = c->p.p3m_order;
     const int Kx = c->p.p3m_mesh[0], Ky = c->p.p3m_mesh[1], Kz = c->p.p3m_mesh[2];
-    k_p3m_prep<T><<<(unsigned)((ptot + 255) / 256), 256, 0, st>>>(xyz, Q, ptot, c->g, Kx, Ky, Kz, P, key, fq);
+    const int64_t per = (int64_t)sp.cps * P3M_NT;
+    CPM_CUDA(c, cudaMemsetAsync(count, 0, lists, st));
+    k_p3m_prep<T><<<(unsigned)((ptot + 255) / 256), 256, 0, st>>>(xyz, Q, ptot, c->g, Kx, Ky, Kz, P, key, fq, ne, sp.br,
+                                                                  sp.nsplit, per, count);
     CPM_LAUNCH(c, "k_p3m_prep");
-    c->launches += 6;
+    CPM_CUDA(c, launch_after(k_p3m_scan, dim3((unsigned)m), dim3(P3M_SCAN), 0, st, count, sp.nsplit * sp.nbricks, start));
+    CPM_CUDA(c, launch_after(k_p3m_fill, dim3((unsigned)((ptot + 255) / 256)), dim3(256), 0, st, key, ptot, ne, P, sp.br, sp.nsplit,
+                             per, most, start, list));
+    c->launches += 8;
     switch (P) {
-        case 2: return launch_p3m_pp<T, 2>(st, c, m, ne, key, fq, flag, mesh, pm);
-        case 3: return launch_p3m_pp<T, 3>(st, c, m, ne, key, fq, flag, mesh, pm);
-        case 4: return launch_p3m_pp<T, 4>(st, c, m, ne, key, fq, flag, mesh, pm);
-        case 5: return launch_p3m_pp<T, 5>(st, c, m, ne, key, fq, flag, mesh, pm);
-        case 6: return launch_p3m_pp<T, 6>(st, c, m, ne, key, fq, flag, mesh, pm);
-        default: return launch_p3m_pp<T, 7>(st, c, m, ne, key, fq, flag, mesh, pm);
+        case 2: return launch_p3m_pp<T, 2>(st, c, m, ne, key, fq, flag, count, start, list, most, mesh, pm);
+        case 3: return launch_p3m_pp<T, 3>(st, c, m, ne, key, fq, flag, count, start, list, most, mesh, pm);
+        case 4: return launch_p3m_pp<T, 4>(st, c, m, ne, key, fq, flag, count, start, list, most, mesh, pm);
+        case 5: return launch_p3m_pp<T, 5>(st, c, m, ne, key, fq, flag, count, start, list, most, mesh, pm);
+        case 6: return launch_p3m_pp<T, 6>(st, c, m, ne, key, fq, flag, count, start, list, most, mesh, pm);
+        default: return launch_p3m_pp<T, 7>(st, c, m, ne, key, fq, flag, count, start, list, most, mesh, pm);
     }
 }
 // ----------------------------------------------------------------------------- the P3M elastance

@@ -55,3 +55,26 @@ def test_p3m_shared_and_single_heights(sites_per_height, k_prec, tol):
     b = run_bvec(ctx, elyts)
     for r, e in enumerate(elyts):
         assert rel_l2(b[r], o.bvec(el, e)) <= tol, r
+
+
+@pytest.mark.parametrize("k_prec,tol", [("fp64", 1e-12), ("fp32", 2e-6)])
+def test_p3m_brick_lists(k_prec, tol):
+    """Enough charges for several splits, bricks on both sides of every face of the cell, and the same bits each time."""
+    need_gpu()
+    base = s.au111_slab(seed_layers=1, nx=5, ny=6, gap=24.0)
+    el = s.Electrodes(**{**base.__dict__, "p3m_mesh": (64, 32, 64), "p3m_order": 7})
+    rng = np.random.default_rng(21)
+
+    def cloud(n):
+        x = rng.uniform(-0.3, 1.3, (n, 3)) * np.array([el.box[0], el.box[1], 0.0])
+        x[:, 2] = rng.uniform(el.z_inner[0] + 3.0, el.z_inner[1] - 3.0, n)
+        return s.Electrolyte(xyz=x, Q=rng.uniform(-1.0, 1.0, n))
+
+    elyts = [cloud(5000), cloud(1537), cloud(4608)]
+    ctx = make_ctx(el, k_prec=k_prec)
+    ctx.cpm_prepare(dev(el.xyz), dev(el.eta), dev(el.group, torch.int32), el.n_groups)
+    b = run_bvec(ctx, elyts)
+    for r, e in enumerate(elyts):
+        assert rel_l2(b[r], o.bvec(el, e)) <= tol, r
+    for _ in range(3):
+        assert np.array_equal(run_bvec(ctx, elyts), b)
