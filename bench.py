@@ -921,8 +921,8 @@ def main():
     alu_src = f"FP32 FMA issue rate 152 SM x 128 lanes x 2 x {peaks.get('sm_max_mhz', 2070.0)} MHz"
     pairs = real_pairs(el, xyz, Q, ne, m, W)
     work = kernel_work(el, nk, ne, m, pairs, tensor=args.k_prec == "f16x2")
-    kname = {"real": "k_real_blk", "sf": "k_tc_sf" if args.k_prec == "f16x2" else "k_sf32",
-             "site": "k_tc_site" if args.k_prec == "f16x2" else "k_site32", "gemv": "k_gemv_tma"}
+    kname = {"real": "k_real_blk", "sf": "k_tc_rows" if args.k_prec == "f16x2" else "k_rows_sf<float>",
+             "site": "k_rows_sites<float>", "gemv": "k_gemv_tma"}
     top, roof = roofline(prof, work, peaks, src, kname, alu_peak, alu_src, ms_prof)
     roof["pairs_in_rcut_per_launch"] = pairs
     roof["flop_per_unit"] = {"real_pair": FLOP_PAIR, "sf_charge_k": FLOP_SF, "site_k": FLOP_SITE,
@@ -935,7 +935,7 @@ def main():
                               "profiles/launches_edl_capacitor_4320.md")
     pairs1 = real_pairs(el, xyz, Q, ne, 1, W)
     work64 = kernel_work(el, nk, ne, 1, pairs1, tensor=False, s_bytes=8)
-    k64 = {"real": "k_real_b<double>", "sf": "k_sf<double>", "site": "k_site<double>", "gemv": "k_gemv_t<double>"}
+    k64 = {"real": "k_real64", "sf": "k_tc_rows64", "site": "k_rows_sites<double>", "gemv": "k_gemv64"}
     fp64_peak = 1.25   # nominal GB300 FP64 rate (TFLOP/s); no measured FP64 peak on this machine
     _, roof64 = roofline(prof64, work64, peaks, src, k64, fp64_peak, "nominal GB300 FP64 rate, 1.25 TFLOP/s", ms64)
 

@@ -16,8 +16,8 @@
 //   mesh, so IFFT(G FFT(rho_a + i rho_b)) = phi_a + i phi_b exactly: one complex transform serves
 //   two replicas.
 // * Charge assignment: one CTA per (mesh brick, replica) owns the brick's points in shared
-//   memory and takes every charge whose stencil reaches into the brick, adding only the points it
-//   owns.  Every mesh point is written by exactly one CTA, with a plain store: no halo exchange and
+//   memory and takes every charge whose stencil reaches into the brick (listed beforehand), adding only
+//   the points it owns.  Every mesh point is written by exactly one CTA, with a plain store: no halo exchange and
 //   no global atomics.  Inside the brick the contributions are added as exact fixed-point integers
 //   with 32-bit shared-memory atomics, so the mesh charge does not depend on the order of the
 //   atomics and the whole path is deterministic.  Bricks that no charge reaches are not written, only marked,
@@ -183,14 +183,14 @@ __device__ __forceinline__ void bspline_weights(T f, T* w) {
 }
 
 // ----------------------------------------------------------------------------- charge assignment
-// grid (bricks, replicas, charge splits); a brick is BX x BY x BZ mesh points (x fastest), brick
-// index bx fastest.  The charges whose stencil reaches into a brick are listed beforehand (counted with the
-// preparation, k_p3m_scan, k_p3m_fill; the order within a list varies, the sums do not): with each brick looking through
-// all keys of its replica, that took half of the time (270 of 538 us for 16,384 sites x 16 replicas), and the
-// weights of the few charges found were formed by warps with two lanes of work.  A split takes a fixed range of
-// the replica's charges, so that its sum does not depend on the order either.  Their 3 p weights and the stencil origins relative to the brick go to shared memory,
-// NT charges at a time; then a warp takes one charge at a time, lane = (plane of the brick, y offset), each lane
-// adding its p x contributions.
+// grid (bricks, replicas, charge splits); a brick is BX x BY x BZ mesh points (x fastest), brick index bx fastest.
+// The charges whose stencil reaches into a brick are listed beforehand (counted with the preparation, k_p3m_scan,
+// k_p3m_fill; the order within a list varies, the sums do not): with each brick looking through all keys of its
+// replica, that took half of the time (270 of 538 us for 16,384 sites x 16 replicas), and the weights of the few
+// charges found were formed by warps with two lanes of work.  A split takes a fixed range of the replica's
+// charges, so that its sum does not depend on the order either.  Their 3 p weights and the stencil origins
+// relative to the brick go to shared memory, NT charges at a time; then a warp takes one charge at a time, lane =
+// (plane of the brick, y offset), each lane adding its p x contributions.
 // Every contribution is rounded to 2^-40 e (FP64: 2^-60 e) and added as exact integers split over
 // 32-bit words, a = floor(v 2^20), then the next 20 bits (FP64: and 20 more), with native 32-bit
 // shared-memory atomics; integer addition is associative, so the brick's charge does not depend on

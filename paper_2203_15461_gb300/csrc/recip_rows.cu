@@ -311,11 +311,12 @@ __global__ void __launch_bounds__(8 * CP_PTS) k_charge_phases(const double* __re
     }
 }
 
-// The same in fixed point, for FP64: cos and sin times 2^62 in 64-bit integers (tc_rows64.cu takes them as they are, X
-// times the scaled charge, Z rounded to 2^55; k_rows_sf<double> converted at the end).  FP64 arithmetic took 34 us for 5,700 charges of 110 harmonics, the integers 9.5 us (100 charges in k_rows_sf<double>: 11 and 3 us): the 64-bit
-// product of two phases is some 40 instructions of a pipe with thirty times the rate.  A phase is evaluated as
-// T1[top ten bits] T2[next ten] (1 - d^2 / 2, d - d^3 / 6) with the angle d < 2 pi 2^-20 of the other 44 bits: the
-// terms left out are below 2^-72, T1 is FP64's own cosine and sine, and T2's are kept as 1 - cos, exact to 2^-62.
+// The same in fixed point, for FP64: cos and sin times 2^62 in 64-bit integers (tc_rows64.cu takes them as they are,
+// X times the scaled charge, Z rounded to 2^55; k_rows_sf<double> converted at the end).  FP64 arithmetic took 34 us
+// for 5,700 charges of 110 harmonics, the integers 9.5 us (100 charges in k_rows_sf<double>: 11 and 3 us): the 64-bit
+// product of two phases is some 40 instructions of a pipe with thirty times the rate.  A phase is evaluated as T1[top
+// ten bits] T2[next ten] (1 - d^2 / 2, d - d^3 / 6) with the angle d < 2 pi 2^-20 of the other 44 bits: the terms
+// left out are below 2^-72, T1 is FP64's own cosine and sine, and T2's are kept as 1 - cos, exact to 2^-62.
 constexpr int FX_TAB = 1024;
 __global__ void k_fixed_tab(longlong2* __restrict__ tab) {   // grid 2 x FX_TAB: T1 | T2
     const int t = threadIdx.x;
