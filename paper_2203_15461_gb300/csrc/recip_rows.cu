@@ -552,7 +552,7 @@ __global__ void __launch_bounds__(RL_THREADS) k_rows_layers(const int4* __restri
         T s = 0;
         if (o < 4 * nzu) {
             const T* v = V + t * ncc;
-            for (int nz = l4; nz <= pr.z; nz += 4) {
+            for (int nz = pr.z - l4; nz >= 0; nz -= 4) {   // the large terms last
                 const c2<T> z = ZU[(int64_t)nz * nzu + u];
                 s = fma(v[2 * nz], z.x, s);
                 s = fma(v[2 * nz + 1], z.y, s);
@@ -598,7 +598,8 @@ __global__ void __launch_bounds__(ROW_TILE) k_rows_sites(const int4* __restrict_
 #pragma unroll
     for (int k = 0; k < MR; ++k) acc[k] = 0;
     __syncthreads();
-    for (int x = x0; x < x1; ++x) {
+    // from the high harmonics down: the large terms, of the long waves, come last and the sums stay small before them
+    for (int x = x1 - 1; x >= x0; --x) {
         const int o0 = nxoff[x] - f0, cnt = nxoff[x + 1] - f0 - o0;
         if (cnt <= 0) continue;
         const c2<T> sx = SX[(int64_t)x * n + i];
@@ -606,7 +607,7 @@ __global__ void __launch_bounds__(ROW_TILE) k_rows_sites(const int4* __restrict_
 #pragma unroll
         for (int k = 0; k < MR; ++k) ic[k] = is[k] = 0;
 #pragma unroll 4
-        for (int y = 0; y < cnt; ++y) {
+        for (int y = cnt - 1; y >= 0; --y) {
             const c2<T> sy = SY[(int64_t)y * n + i];
 #pragma unroll
             for (int k = 0; k < MR; ++k) {
