@@ -415,6 +415,11 @@ void dev_free(cpm_ctx* c, void* ptr);
 // to 145.8.
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// The two halves of a cluster barrier, by every thread of every block.  Distributed shared memory may be touched only
+// once all blocks of the cluster have started: arrive at the top of a kernel, wait in front of its first access, and
+// the loads in between hide the barrier.
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait;" ::: "memory"); }
 template <typename... KA, typename... A>
 inline cudaError_t launch_after(void (*kernel)(KA...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
     cudaLaunchConfig_t cfg = {};

@@ -290,6 +290,7 @@ __global__ void __launch_bounds__(NB_T, 2) k_gemv_reduce(const P* __restrict__ p
                                                       double* __restrict__ qtot, const double* __restrict__ b,
                                                       const double* __restrict__ srow, const double* __restrict__ SZ,
                                                       const double* __restrict__ gmean, int ngrp) {
+    cluster_arrive();   // matched in front of the first store to another block, which must have started by then
     grid_wait();
     __shared__ double sh[NB_T];
     __shared__ double csum[2][NB_CLUSTER];   // block sums of the cluster before and after the fix
@@ -335,6 +336,7 @@ __global__ void __launch_bounds__(NB_T, 2) k_gemv_reduce(const P* __restrict__ p
         else qr[i] = qi;                        // read back by this thread alone
         a += qi;
     }
+    cluster_wait();
     const double s = exchange(a, 0);
     a = 0.0;
     for (int64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) {
