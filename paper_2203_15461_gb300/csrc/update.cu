@@ -351,12 +351,48 @@ __global__ void __launch_bounds__(NB_T, 2) k_gemv_reduce(const P* __restrict__ p
     if (rank == 0 && threadIdx.x == 0) qtot[r] = tot;
 }
 
+// out[r][i] = sum of the split partials, one output per thread over the whole GPU
+template <typename P>
+__global__ void __launch_bounds__(256) k_sum_splits(const P* __restrict__ part, int splits, int64_t cnt,
+                                                    double* __restrict__ out) {
+    grid_wait();
+    grid_go();
+    const int64_t t = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (t >= cnt) return;
+    typename PartSum<P>::type v;
+    for (int sp = 0; sp < splits; sp += 16) {   // sixteen loads in flight, added in split order
+        P x[16];
+#pragma unroll
+        for (int k = 0; k < 16; ++k) x[k] = sp + k < splits ? part[(int64_t)(sp + k) * cnt + t] : P{};
+#pragma unroll
+        for (int k = 0; k < 16; ++k)
+            if (sp + k < splits) v.add(x[k]);
+    }
+    out[t] = v.value();
+}
+
+// Blocks per replica.  Sixteen up to four replicas (one replica of 4,320 sites: 20.9 us an update against 22.8 with
+// eight); beyond, eight while the replicas' blocks are one wave of two per SM, and fewer after that: with eight for
+// every batch, 256 replicas of 4,320 sites took 566 us an update, with one block each 507; of 1,031 sites 113 and 101;
+// 64 of 4,320 on the tensor cores 66 and 56 with four.
+static int reduce_cluster(int64_t n, int m) {
+    int cl = m <= 4 ? NB_CLUSTER : 8;
+    while (cl > 1 && (m > 4 && (int64_t)m * cl > 2 * 152)) cl /= 2;
+    while (cl > 1 && n < (int64_t)cl * (cl > 8 ? 2 * NB_LEAST : NB_LEAST)) cl /= 2;
+    return cl;
+}
+// A replica of more sites than sixteen blocks have threads, its partials in many splits, and fewer blocks of eight
+// than SMs: most of the GPU would wait while a few SMs read the partials, so k_sum_splits adds them beforehand.  16,384
+// sites, 86 splits: one replica 193 -> 181 us an update, five 248 -> 234, eight 261 -> 247, sixteen 463 -> 456, but 32
+// replicas 839 -> 857; 8,192 sites x 8 86 -> 89; 16,384 sites x 8 in the tensor-core product's few splits 280 -> 290.
+static bool reduce_sums_first(int64_t n, int m, int64_t splits) {
+    return n > (int64_t)NB_CLUSTER * NB_T && splits >= 32 && 8 * m <= 152;
+}
+
 template <typename P>
 static cpm_status launch_reduce(cpm_ctx* c, const void* part, int splits, int m, const double* psi, double* q, double* qtot,
                                 const double* b, const double* srow, const double* SZ, const double* gmean, int ngrp) {
-    // sixteen blocks up to four replicas (one replica of 4,320 sites: 108 against 109.5 us a step; eight: 143.0 against 142.4)
-    int cl = m <= 4 ? NB_CLUSTER : 8;
-    while (cl > 1 && c->n < (int64_t)cl * (cl > 8 ? 2 * NB_LEAST : NB_LEAST)) cl /= 2;
+    const int cl = reduce_cluster(c->n, m);
     if (cl > 8) CPM_CUDA(c, cudaFuncSetAttribute(k_gemv_reduce<P>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     const int64_t slice = (c->n + cl - 1) / cl;
     cudaLaunchConfig_t cfg = {};
@@ -374,6 +410,18 @@ static cpm_status launch_reduce(cpm_ctx* c, const void* part, int splits, int m,
     CPM_CUDA(c, cudaLaunchKernelEx(&cfg, k_gemv_reduce<P>, (const P*)part, splits, (const double*)upd_sg(c), (int)upd_ng(c), psi,
                                    c->n, m, q, (const double*)c->u, (int)c->p.symm, qtot, b, srow, SZ, gmean, ngrp));
     return CPM_OK;
+}
+
+// the streamed products: with the splits added first where that is faster (the sums are the same)
+template <typename P>
+static cpm_status reduce_streamed(cpm_ctx* c, const void* part, double* sums, int splits, int m, const double* psi, double* q,
+                                  double* qtot, const double* b, const double* srow) {
+    if (!reduce_sums_first(c->n, m, splits)) return launch_reduce<P>(c, part, splits, m, psi, q, qtot, b, srow, nullptr, nullptr, 0);
+    const int64_t cnt = (int64_t)m * c->n;
+    CPM_CUDA(c, launch_after(k_sum_splits<P>, dim3((unsigned)((cnt + 255) / 256)), dim3(256), 0, c->stream, (const P*)part,
+                             splits, cnt, sums));
+    c->launches += 1;
+    return launch_reduce<double>(c, sums, 1, m, psi, q, qtot, b, srow, nullptr, nullptr, 0);
 }
 
 // split count and row chunk of the centred product; grows the scratch when needed
@@ -401,6 +449,7 @@ static cpm_status reserve_update_plan(cpm_ctx* c, int m, int64_t* splits_out, in
         int64_t cb;
         gemv_tma_plan(n, m, &cb, &splits, &jchunk);
     }
+    // the partials, then the two-float split of b, whose place the sums of the splits take after the product
     const size_t need = ((sizeof(double) * splits * m * n + 255) & ~(size_t)255) + sizeof(float2) * m * n;
     if (c->ubuf_bytes < need) {
         dev_free(c, c->ubuf);
@@ -487,9 +536,9 @@ cpm_status update(cpm_ctx* c, int m, const double* psi, const double* b, double*
     prof_begin(c, CPM_K_NEUTRAL);
     const double* srow = (f32 && !c->p.symm) ? c->dvec : nullptr;
     if (f32 && gemv_tma_supported(c))
-        CPM_TRY(launch_reduce<float2>(c, part, (int)splits, m, psi, q, qtot, b, srow, nullptr, nullptr, 0));
+        CPM_TRY(reduce_streamed<float2>(c, part, (double*)bhl, (int)splits, m, psi, q, qtot, b, srow));
     else
-        CPM_TRY(launch_reduce<double>(c, part, (int)splits, m, psi, q, qtot, b, srow, nullptr, nullptr, 0));
+        CPM_TRY(reduce_streamed<double>(c, part, (double*)bhl, (int)splits, m, psi, q, qtot, b, srow));
     prof_end(c, CPM_K_NEUTRAL);
     CPM_LAUNCH(c, "k_gemv");
     return CPM_OK;
