@@ -433,18 +433,38 @@ static int64_t gemv_colblocks(const cpm_ctx* c) {
     return gemv_pairs(c) ? (c->n + 2 * G2_T - 1) / (2 * G2_T) : (c->n + GT_COLS - 1) / GT_COLS;
 }
 
+// FP64: rows per split in steps of the rows in flight.  The FP64 pipe is what bounds the product, so the time is the rows
+// that the busiest SM takes: blocks per SM times rows per block while all blocks fit at once (four per SM), their mean
+// and half a block beyond; one to three blocks of four warps keep the pipe less than busy (the factors are fitted to
+// 25 split counts at each of 42 sizes).  About one wave of blocks whatever their remainder, the rule before: 2,050 sites
+// x 8 87.5 us an update, 77.5 now, x 64 621 and 509; 8,192 x 16 2,124 and 1,781, x 64 8,286 and 6,950; 16,384 x 1 567
+// and 493.  The fewest splits within 1 % (their partial sums are memory).
+static void gemv64_plan(int64_t n, int64_t blocks, int64_t* splits, int64_t* jchunk) {
+    const double busy[5] = {0.0, 0.5, 0.9, 0.95, 1.0};
+    const int64_t most = std::min<int64_t>(64, (n + G6_U - 1) / G6_U);
+    double cost[65], best = 1e300;
+    for (int64_t s = 1; s <= most; ++s) {
+        const int64_t j = ((n + s - 1) / s + G6_U - 1) / G6_U * G6_U, nb = blocks * ((n + j - 1) / j), k = (nb + 151) / 152;
+        cost[s] = (k <= 4 ? (double)k / busy[k] : (double)nb / 152 + 0.5) * (double)j;
+        best = std::min(best, cost[s]);
+    }
+    int64_t s = 1;
+    while (cost[s] > 1.01 * best) ++s;
+    *jchunk = ((n + s - 1) / s + G6_U - 1) / G6_U * G6_U;
+    *splits = (n + *jchunk - 1) / *jchunk;
+}
+
 static cpm_status reserve_update_plan(cpm_ctx* c, int m, int64_t* splits_out, int64_t* jchunk_out) {
     const int64_t n = c->n;
     const int64_t colblocks = gemv_colblocks(c);
     const int mr = gemv_fp64(c) ? gemv64_mr(m) : GT_MR;
     const int rchunks = (m + mr - 1) / mr;
     const int64_t want = gemv_pairs(c) ? 2 * 152 : 4 * 152;   // resident blocks: about one wave
-    // rows per split in whole tiles; FP64 in steps of the rows in flight, so that a small S is not one long chain
-    const int64_t jt = gemv_fp64(c) ? G6_U : GT_JT;
-    int64_t splits = (want + colblocks * rchunks - 1) / (colblocks * rchunks);
-    splits = std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(splits, gemv_fp64(c) ? 64 : splits), (n + jt - 1) / jt));
-    int64_t jchunk = (((n + splits - 1) / splits + jt - 1) / jt) * jt;
+    int64_t splits = (want + colblocks * rchunks - 1) / (colblocks * rchunks);   // rows per split in whole tiles
+    splits = std::max<int64_t>(1, std::min<int64_t>(splits, (n + GT_JT - 1) / GT_JT));
+    int64_t jchunk = (((n + splits - 1) / splits + GT_JT - 1) / GT_JT) * GT_JT;
     splits = (n + jchunk - 1) / jchunk;
+    if (gemv_fp64(c)) gemv64_plan(n, colblocks * rchunks, &splits, &jchunk);
     if (gemv_tma_supported(c)) {
         int64_t cb;
         gemv_tma_plan(n, m, &cb, &splits, &jchunk);
