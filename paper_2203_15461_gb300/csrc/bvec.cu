@@ -834,6 +834,19 @@ __global__ void k_col0_tab(float4* __restrict__ tab) {
 // recurrence, and the block sums its threads in a fixed order.
 constexpr int C0_THREADS = 128;
 
+// sum_nz Re[conj(e0[nz]) w_nz rho_nz] of one height
+__device__ __forceinline__ double col0_at(const double2* __restrict__ e0, const double2* sw, int nz0) {
+    double s = 0.0;
+#pragma unroll
+    for (int k = 0; k < COL0_NZ; ++k) {
+        if (k < nz0) {
+            const double2 e = e0[k];
+            s += e.x * sw[k].x + e.y * sw[k].y;
+        }
+    }
+    return s;
+}
+
 // grid (charge chunks, m).  The replica's last block (ticket) then adds the chunks (lanes over the
 // chunks, a fixed tree), weights them and leaves b0[r][u] = sum_nz Re[conj(e0[u][nz]) w_nz rho_nz] for every
 // distinct site height: one launch where input, sum, reduction and evaluation were four dependent ones
@@ -842,7 +855,8 @@ __global__ void __launch_bounds__(C0_THREADS) k_col0(const double* __restrict__ 
                                                      int64_t ne, double invLz, int nz0, const double* __restrict__ w,
                                                      int NZ, const double2* __restrict__ e0, int nzu,
                                                      const float4* __restrict__ tab, double2* __restrict__ part,
-                                                     int* __restrict__ tickets, double* __restrict__ b0) {
+                                                     int* __restrict__ tickets, double2* __restrict__ wsum,
+                                                     double* __restrict__ b0) {
     __shared__ float4 red[C0_THREADS / 32][COL0_NZ];   // the warps' sums (re hi, lo, im hi, lo), scaled
     __shared__ double s_un[C0_THREADS / 32];
     __shared__ double2 sw[COL0_NZ];
@@ -911,19 +925,24 @@ __global__ void __launch_bounds__(C0_THREADS) k_col0(const double* __restrict__ 
         for (int g = 1; g < G; ++g) { a.x += sp[g][threadIdx.x].x; a.y += sp[g][threadIdx.x].y; }
         const double wt = w[NZ + threadIdx.x + 1];   // column 0 occupies the first row of the dense grid
         sw[threadIdx.x] = make_double2(wt * a.x, wt * a.y);
+        if (wsum) wsum[r * nz0 + threadIdx.x] = sw[threadIdx.x];
     }
+    if (wsum) return;   // uniform: k_col0_heights
     __syncthreads();
-    for (int u = threadIdx.x; u < nzu; u += C0_THREADS) {
-        double s = 0.0;
-#pragma unroll
-        for (int k = 0; k < COL0_NZ; ++k) {
-            if (k < nz0) {
-                const double2 e = e0[(int64_t)u * nz0 + k];
-                s += e.x * sw[k].x + e.y * sw[k].y;
-            }
-        }
-        b0[(int64_t)r * nzu + u] = s;
-    }
+    for (int u = threadIdx.x; u < nzu; u += C0_THREADS) b0[(int64_t)r * nzu + u] = col0_at(e0 + (int64_t)u * nz0, sw, nz0);
+}
+
+// The same evaluation from the weighted sums, over the whole GPU: past C0_HEIGHTS heights the replica's last block
+// alone takes longer than another launch (4,320 heights, b of one replica: 96.8 us, 77.3 now, of eight: 239 and 106).
+constexpr int C0_HEIGHTS = 2 * C0_THREADS;
+__global__ void __launch_bounds__(C0_THREADS) k_col0_heights(const double2* __restrict__ e0, int nzu, int nz0,
+                                                             const double2* __restrict__ wsum, double* __restrict__ b0) {
+    grid_wait();
+    __shared__ double2 sw[COL0_NZ];
+    const int u = blockIdx.x * C0_THREADS + threadIdx.x, r = blockIdx.y;
+    if ((int)threadIdx.x < nz0) sw[threadIdx.x] = wsum[r * nz0 + threadIdx.x];
+    __syncthreads();
+    if (u < nzu) b0[(int64_t)r * nzu + u] = col0_at(e0 + (int64_t)u * nz0, sw, nz0);
 }
 
 // e0[u][nz - 1] = exp(i kz z_u) for each distinct site height z_u and nz = 1 .. COL0_NZ (fixed with
@@ -1078,7 +1097,7 @@ struct BvecPlan {
     TcRecipDims td;
     Rows64Dims r64;                     // FP64 by integer products (tc_rows64.cu)
     size_t off_EX, off_EY, off_EZ, off_rp, off_wr, off_part, off_real, off_stats, off_key, off_cnt, off_cur,
-        off_nzc, off_start, off_wpos, off_sorted, off_order, off_c0part, off_b0, off_T, off_w16, off_ew,
+        off_nzc, off_start, off_wpos, off_sorted, off_order, off_c0part, off_c0w, off_b0, off_T, off_w16, off_ew,
         off_ewT, off_pm, off_p3m, total;
     int c0chunks;
     bool p3m;                           // reciprocal part of b by P3M (p3m.cu)
@@ -1145,6 +1164,7 @@ static BvecPlan<T> plan_bvec(const cpm_ctx* c, int m, int64_t ne) {
     p.c0chunks = (int)std::max<int64_t>(1, (ne + C0_THREADS - 1) / C0_THREADS);
     const int nz0 = std::max(std::min(k.ext0, COL0_NZ), 1);
     p.off_c0part = o; o += al(sizeof(double2) * (size_t)m * p.c0chunks * nz0);
+    p.off_c0w = o; o += al(sizeof(double2) * (size_t)m * nz0);
     p.off_b0 = o; o += al(sizeof(double) * (size_t)m * std::max(c->nzu, 1));
     p.off_spart = o; o += al(sizeof(double) * ST_Q * (size_t)std::max<int64_t>(1, (ne + ST_THREADS - 1) / ST_THREADS) * m);
     p.off_ew = p.off_ewT = o;
@@ -1237,9 +1257,15 @@ cpm_status bvec_run(cpm_ctx* c, int m, int64_t ne, const double* xyz, const doub
         b0 = (double*)(scr + p.off_b0);
         prof_begin(c, CPM_K_COL0);
         const int nz0 = std::min(k.ext0, COL0_NZ);
+        double2* wsum = c->nzu > C0_HEIGHTS ? (double2*)(scr + p.off_c0w) : nullptr;
         k_col0<<<dim3(p.c0chunks, m), C0_THREADS, 0, s2>>>(xyz, Q, ne, c->g.inv[2], nz0, k.w, k.NZ, c->c0e, c->nzu, c->c0tab,
-                                                           (double2*)(scr + p.off_c0part), c->tickets + m, b0);
+                                                           (double2*)(scr + p.off_c0part), c->tickets + m, wsum, b0);
         CPM_LAUNCH(c, "k_col0");
+        if (wsum) {
+            CPM_CUDA(c, launch_after(k_col0_heights, dim3((unsigned)((c->nzu + C0_THREADS - 1) / C0_THREADS), (unsigned)m),
+                                     dim3(C0_THREADS), 0, s2, c->c0e, c->nzu, nz0, wsum, b0));
+            c->launches += 1;
+        }
         prof_end(c, CPM_K_COL0);
         c->launches += 1;
     }
