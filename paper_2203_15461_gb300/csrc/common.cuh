@@ -176,7 +176,7 @@ struct RowTable {
     bool layered = false;                // the sites share few heights
     int4* pairs = nullptr;               // [np] (nx, ny, largest nz, slot)
     int* list = nullptr;                 // [nrows] 4 pair + part
-    int* colpair = nullptr;              // [ncols] pair of each signed column
+    int2* paircols = nullptr;            // [np] the signed columns (nx, ny) and (nx, -ny) of each pair (-1: none)
     int* nxoff = nullptr;                // [NX + 2] first slot of each nx (slot = nxoff[nx] + ny)
     int* chunkb = nullptr;               // [nchunk + 1] first nx of each range
     double* W = nullptr;                 // [np][NZ + 1] weights of the octant vectors

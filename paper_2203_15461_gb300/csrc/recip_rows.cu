@@ -69,7 +69,7 @@ static cpm_status charge_fixed_table(cpm_ctx* c);
 void free_rows(cpm_ctx* c) {
     RowTable& t = c->rows;
     for (void* p : {(void*)t.pairs, (void*)t.list, (void*)t.W, (void*)t.W32, (void*)t.nxoff, (void*)t.chunkb,
-                    (void*)t.zu64, (void*)t.zu32, (void*)t.lperm, (void*)t.ltiles, (void*)t.colpair, (void*)t.tcitem, (void*)t.atiles, (void*)t.item64, (void*)t.fxtab,
+                    (void*)t.zu64, (void*)t.zu32, (void*)t.lperm, (void*)t.ltiles, (void*)t.paircols, (void*)t.tcitem, (void*)t.atiles, (void*)t.item64, (void*)t.fxtab,
                     (void*)t.tcrange})
         dev_free(c, p);
     t = RowTable{};
@@ -102,7 +102,7 @@ cpm_status build_rows(cpm_ctx* c) {
     for (int x = 0; x <= k.NX; ++x) off[x + 1] = off[x] + ymax[x] + 1;
     t.nslots = off[k.NX + 1];
     std::vector<int4> pairs;
-    std::vector<int> col, list, cpair(k.ncols, 0), slotpair(t.nslots, 0), order;
+    std::vector<int> col, list, slotpair(t.nslots, 0), order;
     for (int q = 0; q < k.ncols; ++q)
         if (cols[q].y >= 0) order.push_back(q);
     // The order of |k_perp| keeps pairs of like extents together.  The tensor-core stage takes 64 pairs per CTA
@@ -150,8 +150,10 @@ cpm_status build_rows(cpm_ctx* c) {
         for (int part = 0; part < 4; ++part)   // sin 0 = 0: no row
             if (!((part & 1) && cols[q].x == 0) && !((part & 2) && cols[q].y == 0)) list.push_back(4 * p + part);
     }
-    for (int q = 0; q < k.ncols; ++q)   // the pair of every signed column
-        cpair[q] = slotpair[off[cols[q].x] + std::abs(cols[q].y)];
+    std::vector<int2> pcols(pairs.size());   // the signed columns (nx, ny) and (nx, -ny) of every pair
+    for (size_t p = 0; p < pairs.size(); ++p) pcols[p] = make_int2(col[p], -1);
+    for (int q = 0; q < k.ncols; ++q)
+        if (cols[q].y < 0) pcols[slotpair[off[cols[q].x] - cols[q].y]].y = q;
     if (c->p.k_prec == CPM_PREC_FP64) {
         std::vector<int4> i64;
         for (size_t f = 0; f < pairs.size(); f += ROW64_PAIRS) {
@@ -212,7 +214,7 @@ cpm_status build_rows(cpm_ctx* c) {
     CPM_TRY(upload(c, &t.pairs, pairs));
     CPM_TRY(upload(c, &t.list, list));
     CPM_TRY(upload(c, &t.nxoff, off));
-    CPM_TRY(upload(c, &t.colpair, cpair));
+    CPM_TRY(upload(c, &t.paircols, pcols));
     CPM_TRY(upload(c, &t.chunkb, cb));
     CPM_TRY(upload(c, &dcol, col));
     const size_t nw = (size_t)t.np * (k.NZ + 1), nu = (size_t)c->nzu * (k.NZ + 1);
@@ -511,6 +513,28 @@ __global__ void __launch_bounds__(RW_THREADS) k_rows_sf(const int4* __restrict__
 // One block per (pair, replica): the split sums of the pair's four rows, weighted, in shared memory, then
 // four lanes per (part, height) add the harmonics nz = lane, lane + 4, ... and combine by a fixed butterfly.
 constexpr int RL_THREADS = 128;
+// V[t][cc] = scale(cc) times the sum over the splits of the pair's row t; rows with sin 0 = 0 are not formed, and zero
+template <typename T, typename F>
+__device__ __forceinline__ void sum_pair_rows(int4 pr, const T* __restrict__ src, int cw, int ncc, int splits, int64_t sstride,
+                                              T* __restrict__ V, F scale) {
+    for (int e = threadIdx.x; e < 4 * ncc; e += RL_THREADS) {
+        const int t = e / ncc, cc = e - t * ncc;
+        T v = 0;
+        if (!((t & 1) && pr.x == 0) && !((t & 2) && pr.y == 0)) {
+            const T* q = src + (int64_t)t * cw + cc;
+            int s = 0;
+            for (; s + 8 <= splits; s += 8) {   // eight loads in flight, added in split order
+                T x[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) x[u] = q[(s + u) * sstride];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) v += x[u];
+            }
+            for (; s < splits; ++s) v += q[s * sstride];
+        }
+        V[e] = v * scale(cc);
+    }
+}
 template <typename T>
 __global__ void __launch_bounds__(RL_THREADS) k_rows_layers(const int4* __restrict__ pairs, int np, int cw, int NZ,
                                                             const T* __restrict__ part, int splits, int m,
@@ -524,26 +548,8 @@ __global__ void __launch_bounds__(RL_THREADS) k_rows_layers(const int4* __restri
     const int4 pr = pairs[p];
     const int ncc = 2 * (pr.z + 1);
     T* V = (T*)rl_smem;   // [4][ncc]
-    const int64_t sstride = (int64_t)m * 4 * np * cw;
-    const T* src = part + ((int64_t)r * np + p) * 4 * cw;
-    for (int e = threadIdx.x; e < 4 * ncc; e += RL_THREADS) {
-        const int t = e / ncc, cc = e - t * ncc;
-        T v = 0;
-        // rows with sin 0 = 0 are not formed
-        if (!((t & 1) && pr.x == 0) && !((t & 2) && pr.y == 0)) {
-            const T* q = src + (int64_t)t * cw + cc;
-            int s = 0;
-            for (; s + 8 <= splits; s += 8) {   // eight loads in flight, added in split order
-                T x[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) x[u] = q[(s + u) * sstride];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) v += x[u];
-            }
-            for (; s < splits; ++s) v += q[s * sstride];
-        }
-        V[e] = v * W[(int64_t)p * (NZ + 1) + (cc >> 1)];
-    }
+    sum_pair_rows(pr, part + ((int64_t)r * np + p) * 4 * cw, cw, ncc, splits, (int64_t)m * 4 * np * cw, V,
+                  [&](int cc) { return W[(int64_t)p * (NZ + 1) + (cc >> 1)]; });
     __syncthreads();
     const T f = qmax ? (T)(1.f / (TC_ZSCALE * pow2_below(qmax[r], 14))) : (T)1;   // a power of two
     const int l4 = threadIdx.x & 3;
@@ -629,37 +635,45 @@ __global__ void __launch_bounds__(ROW_TILE) k_rows_sites(const int4* __restrict_
         if (k < nrep) partial[((int64_t)(rb + k) * nchunk + ch) * n + i] = acc[k];
 }
 
-// wrho[r][col][nz + NZ] = w rho of the signed columns, for the site stages that take every site by itself
+// wrho[r][col][nz + NZ] = w rho of the signed columns, for the site stages that take every site by itself.  One block
+// per (pair, replica): the split sums of the pair's four rows in shared memory, as in k_rows_layers, then the one or
+// two columns that they make up, RC_HARM harmonics at a time.  With a thread per (column, harmonic) adding the splits of
+// its eight values one after the other, b of one replica over 2,048 and 4,320 sites of distinct heights took 74.1 and
+// 77.3 us, 61.9 and 65.8 now; FP32 on the CUDA cores 118.8 and 117.5, now 103.7 and 101.5.
+constexpr int RC_HARM = 256;
 template <typename T>
-__global__ void k_rows_to_cols(const int2* __restrict__ cols, const int* __restrict__ colext, int ncols,
-                               const int4* __restrict__ pairs, const int* __restrict__ colpair, int np, int cw, int NZ,
-                               const T* __restrict__ part, int splits, int m, const T* __restrict__ w,
-                               const float* __restrict__ qmax, c2<T>* __restrict__ wrho) {
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int nzw = 2 * NZ + 1;
-    if (t >= (int64_t)m * ncols * nzw) return;
-    const int z = (int)(t % nzw), col = (int)((t / nzw) % ncols), r = (int)(t / ((int64_t)nzw * ncols));
-    const int nz = z - NZ, az = nz < 0 ? -nz : nz;
-    c2<T> v = cmake<T>(0, 0);
-    const T wt = w[(int64_t)col * nzw + z];
-    if (az <= colext[col] && wt != (T)0) {
-        const int p = colpair[col];
-        const int4 pr = pairs[p];
-        T a[4][2] = {};
-        for (int tt = 0; tt < 4; ++tt) {
-            if (((tt & 1) && pr.x == 0) || ((tt & 2) && pr.y == 0)) continue;
-            for (int s = 0; s < splits; ++s) {
-                const T* q = part + (((int64_t)s * m + r) * np + p) * 4 * cw + (int64_t)tt * cw + 2 * az;
-                a[tt][0] += q[0];
-                a[tt][1] += q[1];
+__global__ void __launch_bounds__(RL_THREADS) k_rows_to_cols(const int2* __restrict__ paircols, const int* __restrict__ colext,
+                                                             int ncols, const int4* __restrict__ pairs, int np, int cw, int NZ,
+                                                             const T* __restrict__ part, int splits, int m,
+                                                             const T* __restrict__ w, const float* __restrict__ qmax,
+                                                             c2<T>* __restrict__ wrho) {
+    grid_wait();
+    extern __shared__ __align__(16) unsigned char rl_smem[];
+    const int p = blockIdx.x, r = blockIdx.y, nzw = 2 * NZ + 1;
+    const int4 pr = pairs[p];
+    const T f = qmax ? (T)(1.f / (TC_ZSCALE * pow2_below(qmax[r], 14))) : (T)1;   // a power of two
+    const int2 pc = paircols[p];
+    T* V = (T*)rl_smem;   // [4][ncc]
+    for (int a0 = 0; a0 <= NZ; a0 += RC_HARM) {   // RC_HARM harmonics at a time
+        const int nh = min(RC_HARM, NZ + 1 - a0), ncc = 2 * max(0, min(nh, pr.z + 1 - a0));
+        __syncthreads();
+        sum_pair_rows(pr, part + ((int64_t)r * np + p) * 4 * cw + 2 * a0, cw, ncc, splits, (int64_t)m * 4 * np * cw, V,
+                      [](int) { return (T)1; });
+        __syncthreads();
+        for (int e = threadIdx.x; e < 4 * nh; e += RL_THREADS) {
+            const int q = e / nh, az = a0 + e % nh, nz = q & 1 ? -az : az, col = q < 2 ? pc.x : pc.y;
+            if (col < 0 || (q & 1 && az == 0)) continue;
+            c2<T> v = cmake<T>(0, 0);
+            const T wt = w[(int64_t)col * nzw + nz + NZ];
+            if (az <= colext[col] && wt != (T)0) {
+                const T* a = V + 2 * (az - a0);
+                const T sy = q < 2 ? (T)1 : (T)-1, sz = q & 1 ? (T)-1 : (T)1, fw = wt * f;
+                v.x = fw * ((a[0] - sy * a[3 * ncc]) - sz * (a[ncc + 1] + sy * a[2 * ncc + 1]));
+                v.y = fw * (sz * (a[1] - sy * a[3 * ncc + 1]) + (a[ncc] + sy * a[2 * ncc]));
             }
+            wrho[((int64_t)r * ncols + col) * nzw + nz + NZ] = v;
         }
-        const T sy = cols[col].y < 0 ? (T)-1 : (T)1, sz = nz < 0 ? (T)-1 : (T)1;
-        const T f = wt * (qmax ? (T)(1.f / (TC_ZSCALE * pow2_below(qmax[r], 14))) : (T)1);
-        v.x = f * ((a[0][0] - sy * a[3][0]) - sz * (a[1][1] + sy * a[2][1]));
-        v.y = f * (sz * (a[0][1] - sy * a[3][1]) + (a[1][0] + sy * a[2][0]));
     }
-    wrho[t] = v;
 }
 
 // ----------------------------------------------------------------------------- host side
@@ -803,10 +817,10 @@ template <typename T>
 cpm_status rows_to_cols(cpm_ctx* c, cudaStream_t st, int cw, int splits, int m, const T* part, const float* qmax, c2<T>* wrho) {
     const RowTable& t = c->rows;
     const KTable& k = c->kt;
-    const int64_t tot = (int64_t)m * k.ncols * k.nzw;
     const T* w = std::is_same<T, float>::value ? (const T*)k.w32 : (const T*)k.w;
-    k_rows_to_cols<T><<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(k.cols, k.colext, k.ncols, t.pairs, t.colpair,
-                                                                     t.np, cw, k.NZ, part, splits, m, w, qmax, wrho);
+    const size_t sm = sizeof(T) * 4 * 2 * std::min(k.NZ + 1, RC_HARM);
+    CPM_CUDA(c, launch_after(k_rows_to_cols<T>, dim3(t.np, m), dim3(RL_THREADS), sm, st, t.paircols, k.colext, k.ncols, t.pairs,
+                             t.np, cw, k.NZ, part, splits, m, w, qmax, wrho));
     CPM_LAUNCH(c, "k_rows_to_cols");
     return CPM_OK;
 }
