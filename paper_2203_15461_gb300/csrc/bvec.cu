@@ -1236,8 +1236,13 @@ cpm_status bvec_run(cpm_ctx* c, int m, int64_t ne, const double* xyz, const doub
     if (recip) {
         prof_begin(c, CPM_K_PHASES);
         if (p.tc) {
+            if (!c->rows.layered) {
+                // the scale of the site stage: from the charges alone, beside the phases
+                if (fork) CPM_CUDA(c, cudaStreamWaitEvent(s2, c->fev[0], 0));
+                CPM_TRY(tc_recip_scales(c, s2, m, ne, Q, qsum));
+                if (fork) CPM_CUDA(c, cudaEventRecord(c->fev[2], s2));
+            }
             CPM_TRY(launch_charge_slots(c, s1, m, ne, p.td.nep, xyz, Q, (float2*)EX, qmax, qlast));
-            if (!c->rows.layered) CPM_TRY(tc_recip_scales(c, s1, m, ne, Q, qsum));
         } else if (p.r64.use) {
             CPM_TRY(launch_qexp(c, s1, m, ne, Q, qlast));
             CPM_TRY(launch_charge_fixed(c, s1, m, ne, p.r64.nep, xyz, Q, qlast, (longlong2*)EX, (longlong2*)EY,
@@ -1305,6 +1310,7 @@ cpm_status bvec_run(cpm_ctx* c, int m, int64_t ne, const double* xyz, const doub
         if (c->rows.layered) {
             CPM_TRY(rows_sites<T>(c, s1, m, (const T*)(scr + p.off_T), part));
         } else if (p.tc) {
+            if (fork) CPM_CUDA(c, cudaStreamWaitEvent(s1, c->fev[2], 0));
             CPM_TRY(tc_recip_sites(c, s1, p.td, m, (const float2*)wr, qsum, scr + p.off_w16, (float*)part));
         } else if (std::is_same<T, float>::value) {
             dim3 gs((unsigned)((n + T2_BS - 1) / T2_BS), p.ctiles, m);

@@ -322,7 +322,13 @@ __global__ void __launch_bounds__(1024) k_qsum_abs(const double* __restrict__ Q,
     __shared__ float ss[32];
     const int r = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float sum = 0.f;
-    for (int64_t j = threadIdx.x; j < ne; j += 1024) sum += fabsf((float)Q[(int64_t)r * ne + j]);
+    for (int64_t j0 = threadIdx.x; j0 < ne; j0 += 8 * 1024) {   // eight loads in flight
+        float q[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) q[k] = j0 + 1024 * k < ne ? (float)Q[(int64_t)r * ne + j0 + 1024 * k] : 0.f;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) sum += fabsf(q[k]);
+    }
     for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
     if (lane == 0) ss[warp] = sum;
     __syncthreads();
