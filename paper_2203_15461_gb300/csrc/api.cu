@@ -1,5 +1,6 @@
 // C ABI of the CPM library: argument checks, device-memory ownership, call ordering and the
 // host-buffer entry point.  All arithmetic runs in the kernels of the other translation units.
+#include <climits>
 #include <cstdarg>
 #include <cstring>
 
@@ -454,7 +455,7 @@ static cpm_status assemble_impl(cpm_ctx* c, int64_t n, const double* xyz, const 
     CPM_TRY(build_col0_sites(c));
     if (c->p.kspace != CPM_KSPACE_P3M) {
         CPM_TRY(build_rows(c));
-        if (c->rows.tcitems && !c->rows.layered) CPM_TRY(tc_recip_prepare(c));
+        if (c->rows.tcitems && !rows_by_height(c, INT_MAX)) CPM_TRY(tc_recip_prepare(c));   // some call takes its site stage
     }
     if (c->p.kspace == CPM_KSPACE_P3M) CPM_TRY(p3m_prepare(c));
     const size_t nn = (size_t)n * n;

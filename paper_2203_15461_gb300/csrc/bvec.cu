@@ -1092,6 +1092,7 @@ struct BvecPlan {
     CellGrid cg;
     int nctiles, ctiles;
     int cw, splits;                     // stored functions per row and charge ranges of the structure factor
+    bool layers;                        // potentials of the sites by way of their heights
     bool rows;                          // reciprocal sums in the product basis: on the CUDA cores (rd, recip_rows.cu)
     RowDims rd;                         // or the tensor cores (tc, td, tc_recip.cu)
     TcRecipDims td;
@@ -1126,7 +1127,8 @@ static BvecPlan<T> plan_bvec(const cpm_ctx* c, int m, int64_t ne) {
         p.cw = p.rd.cw;
         p.splits = p.r64.use ? 1 : p.rd.splits;
     }
-    if (p.rows && c->rows.layered) p.nctiles = c->rows.nchunk;
+    p.layers = p.rows && rows_by_height(c, m);
+    if (p.layers) p.nctiles = c->rows.nchunk;
     const int64_t ptot = (int64_t)m * ne;
     // points with electrolyte phase tables (none with P3M)
     const int64_t pph = p.p3m ? 0 : p.r64.use ? (int64_t)m * p.r64.nep : ptot;
@@ -1143,9 +1145,9 @@ static BvecPlan<T> plan_bvec(const cpm_ctx* c, int m, int64_t ne) {
     p.off_rp = p.off_wr = p.off_T = p.off_w16 = o;
     if (p.rows) {
         p.off_rp = o; o += al(sizeof(T) * (size_t)p.splits * m * 4 * c->rows.np * p.cw);
-        p.off_wr = o; o += c->rows.layered ? 0 : al(sizeof(c2<T>) * grid * m);
-        p.off_T = o; o += c->rows.layered ? al(sizeof(T) * rows_T_elems<T>(c, m)) : 0;
-        p.off_w16 = o; o += p.tc && !c->rows.layered ? al(tc_recip_w16_bytes(p.td)) : 0;
+        p.off_wr = o; o += p.layers ? 0 : al(sizeof(c2<T>) * grid * m);
+        p.off_T = o; o += p.layers ? al(sizeof(T) * rows_T_elems<T>(c, m)) : 0;
+        p.off_w16 = o; o += p.tc && !p.layers ? al(tc_recip_w16_bytes(p.td)) : 0;
     }
     p.off_part = o; o += al(sizeof(T) * (size_t)m * p.nctiles * c->n);
     p.off_real = o; o += al(sizeof(double) * (size_t)m * c->n);
@@ -1216,7 +1218,7 @@ cpm_status bvec_run(cpm_ctx* c, int m, int64_t ne, const double* xyz, const doub
     int* qlast = (int*)(qmax + m);
     float* qsum = (float*)(qlast + m);
     const int nc = m * p.cg.ncells;
-    c->launches += 5 + (ptot > 0 ? 2 : 0) + ((k.nk > 0 && ptot > 0 && !p.p3m) ? 4 + (p.r64.use ? 2 : 0) + (c->rows.layered || !p.tc ? 0 : 2) : 0);
+    c->launches += 5 + (ptot > 0 ? 2 : 0) + ((k.nk > 0 && ptot > 0 && !p.p3m) ? 4 + (p.r64.use ? 2 : 0) + (p.layers || !p.tc ? 0 : 2) : 0);
 
     // Three chains: the origin stream bins the charges (per-replica totals) and runs the cell list and
     // the real-space sum; side stream 1 takes the phase tables and the reciprocal sums; side stream 2 sums the
@@ -1236,7 +1238,7 @@ cpm_status bvec_run(cpm_ctx* c, int m, int64_t ne, const double* xyz, const doub
     if (recip) {
         prof_begin(c, CPM_K_PHASES);
         if (p.tc) {
-            if (!c->rows.layered) {
+            if (!p.layers) {
                 // the scale of the site stage: from the charges alone, beside the phases
                 if (fork) CPM_CUDA(c, cudaStreamWaitEvent(s2, c->fev[0], 0));
                 CPM_TRY(tc_recip_scales(c, s2, m, ne, Q, qsum));
@@ -1303,11 +1305,11 @@ cpm_status bvec_run(cpm_ctx* c, int m, int64_t ne, const double* xyz, const doub
         }
         const Phases<T>& sp = site_tables<T>(c);
         prof_begin(c, CPM_K_SFRED);
-        if (c->rows.layered) CPM_TRY(rows_layers<T>(c, s1, p.cw, p.splits, m, rp, qs, (T*)(scr + p.off_T)));
+        if (p.layers) CPM_TRY(rows_layers<T>(c, s1, p.cw, p.splits, m, rp, qs, (T*)(scr + p.off_T)));
         else CPM_TRY(rows_to_cols<T>(c, s1, p.cw, p.splits, m, rp, qs, wr));
         prof_end(c, CPM_K_SFRED);
         prof_begin(c, CPM_K_SITE);
-        if (c->rows.layered) {
+        if (p.layers) {
             CPM_TRY(rows_sites<T>(c, s1, m, (const T*)(scr + p.off_T), part));
         } else if (p.tc) {
             if (fork) CPM_CUDA(c, cudaStreamWaitEvent(s1, c->fev[2], 0));

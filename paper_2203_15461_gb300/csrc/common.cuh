@@ -162,7 +162,7 @@ struct KTable {
 // The k set in the real product basis (recip_rows.cu): pairs (nx, ny) with nx, ny >= 0 in the order of
 // |k_perp|, four rows (cos / sin of x times cos / sin of y) each.
 constexpr int ROW_TILE = 128;          // sites per block of the height-wise site stage
-constexpr int LAYER_MIN_SITES = 8;     // sites per distinct height from which that stage is taken
+constexpr int LAYER_MIN_SITES = 8;     // sites per distinct height from which the tables by height are made
 constexpr int ROW_TC_PAIRS = 64;       // pairs, charges per step and staged x and y harmonics of a CTA of the
 constexpr int ROW_TC_STEP = 64;        // tensor-core structure factor (tc_recip.cu)
 constexpr int ROW_TC_SLOTS = 50;
@@ -173,7 +173,7 @@ struct RowTable {
     int np = 0, nrows = 0, nslots = 0;   // pairs, rows that are not identically zero, (nx, ny) slots
     int nchunk = 0, ntiles = 0;          // nx ranges and site tiles of the site stage
     int chunkmax = 0;                    // most slots of one range
-    bool layered = false;                // the sites share few heights
+    bool layered = false;                // the tables by height are there
     int4* pairs = nullptr;               // [np] (nx, ny, largest nz, slot)
     int* list = nullptr;                 // [nrows] 4 pair + part
     int2* paircols = nullptr;            // [np] the signed columns (nx, ny) and (nx, -ny) of each pair (-1: none)
@@ -501,6 +501,8 @@ cpm_status launch_charge_slots(cpm_ctx* c, cudaStream_t st, int m, int64_t ne, i
 // largest exponent), and y times 2^62, z times 2^55
 cpm_status launch_charge_fixed(cpm_ctx* c, cudaStream_t st, int m, int64_t ne, int64_t nep, const double* xyz,
                                const double* Q, const int* qexp, longlong2* X, longlong2* Y, longlong2* Z);
+// the site stage of m replicas: by height (rows_layers, rows_sites), or every site by itself (rows_to_cols and on)
+bool rows_by_height(const cpm_ctx* c, int m);
 // qmax (tensor-core stage 1): part is scaled by 2^14 pow2_below(max |Q|, 14)
 template <typename T>
 cpm_status rows_layers(cpm_ctx* c, cudaStream_t st, int cw, int splits, int m, const T* part, const float* qmax, T* Tbuf);

@@ -13,8 +13,7 @@
 // over both signs took four.  Electrodes are stacks of lattice planes, so few distinct heights u carry all
 // sites: stage 2 sums the harmonics once per height instead of once per site, and stage 3 is left with
 // one term per (site, pair, part) instead of one per (site, k).  Electrodes whose sites hardly share
-// heights (more than one height per LAYER_MIN_SITES sites) take the general site stage of bvec.cu or
-// tc_recip.cu, whose operand w rho over signed columns k_rows_to_cols forms from R.
+// heights (rows_by_height) take the general site stage of bvec.cu or tc_recip.cu, whose operand w rho over signed columns k_rows_to_cols forms from R.
 #include <vector>
 
 #include "common.cuh"
@@ -767,6 +766,22 @@ cpm_status rows_sf(cpm_ctx* c, cudaStream_t st, const RowDims& d, int m, int64_t
 }
 template cpm_status rows_sf<double>(cpm_ctx*, cudaStream_t, const RowDims&, int, int64_t, const double2*, const double2*, const double2*, double*);
 template cpm_status rows_sf<float>(cpm_ctx*, cudaStream_t, const RowDims&, int, int64_t, const float2*, const float2*, const float2*, float*);
+
+// Which site stage, both sides measured (b alone, us, by height / every site by itself; plates with their sites moved onto
+// so many heights):
+//   tensor cores (their general stage costs little per replica, more per site):
+//     2,048 sites, 1 replica: 64 heights 46 / 61, 128 54 / 57, 256 79 / 60;  8 replicas: 32 82 / 90, 64 96 / 92, 128 128 / 90
+//     4,320 sites, 1 replica: 64 54 / 71, 130 60 / 66, 270 87 / 71;  8 replicas: 32 102 / 108, 64 115 / 116, 130 141 / 110
+//     16,384 sites, 1 replica: 256 133 / 209, 512 206 / 211;  8 replicas: 128 418 / 526, 256 531 / 524, 512 764 / 521
+//   FP32 on the CUDA cores, one replica: 2,048 sites, 256 heights 90 / 103; 4,320: 270 118 / 128, 540 171 / 128; 8,192:
+//     512 199 / 242; four: 4,320, 540 274 / 313
+//   FP64: 4,320 sites, 540 heights 1,038 / 1,720
+bool rows_by_height(const cpm_ctx* c, int m) {
+    const int64_t nu = c->nzu, n = c->n;
+    if (!c->rows.layered) return false;
+    if (c->rows.tcitems) return nu <= std::max<int64_t>(std::max(48, 128 / m), n / (m == 1 ? 32 : 64));
+    return c->p.k_prec == CPM_PREC_FP64 || m > 1 || nu <= std::max<int64_t>(256, n / 16);
+}
 
 template <typename T>
 cpm_status rows_layers(cpm_ctx* c, cudaStream_t st, int cw, int splits, int m, const T* part, const float* qmax, T* Tbuf) {
