@@ -1218,7 +1218,7 @@ cpm_status bvec_run(cpm_ctx* c, int m, int64_t ne, const double* xyz, const doub
     int* qlast = (int*)(qmax + m);
     float* qsum = (float*)(qlast + m);
     const int nc = m * p.cg.ncells;
-    c->launches += 5 + (ptot > 0 ? 2 : 0) + ((k.nk > 0 && ptot > 0 && !p.p3m) ? 4 + (p.r64.use ? 2 : 0) + (p.layers || !p.tc ? 0 : 2) : 0);
+    c->launches += (c->g.bc != CPM_BC_EW2D ? 5 : 4) + (ptot > 0 ? 2 : 0) + ((k.nk > 0 && ptot > 0 && !p.p3m) ? 4 + (p.r64.use ? 2 : 0) + (p.layers || !p.tc ? 0 : 2) : 0);
 
     // Three chains: the origin stream bins the charges (per-replica totals) and runs the cell list and
     // the real-space sum; side stream 1 takes the phase tables and the reciprocal sums; side stream 2 sums the
@@ -1227,12 +1227,15 @@ cpm_status bvec_run(cpm_ctx* c, int m, int64_t ne, const double* xyz, const doub
     const bool recip = k.nk > 0 && ptot > 0 && !p.p3m;
     const bool fork = !c->prof_on;
     cudaStream_t s0 = st, s1 = st, s2 = st;
-    CPM_CUDA(c, cudaMemsetAsync(cnt, 0, p.off_start - p.off_cnt, st));   // counts, cursors, nonzero counts, charge scales
     if (fork) {
         CPM_TRY(ensure_aux(c));
         s1 = c->aux[0];
         s2 = c->aux[1];
-        CPM_CUDA(c, cudaEventRecord(c->fev[0], s0));
+        if (!recip) CPM_CUDA(c, cudaEventRecord(c->fev[0], s0));   // the mesh and the 2D sum need nothing of what follows
+    }
+    CPM_CUDA(c, cudaMemsetAsync(cnt, 0, p.off_start - p.off_cnt, st));   // counts, cursors, nonzero counts, charge scales
+    if (fork) {
+        if (recip) CPM_CUDA(c, cudaEventRecord(c->fev[0], s0));
         CPM_CUDA(c, cudaStreamWaitEvent(s1, c->fev[0], 0));
     }
     if (recip) {
@@ -1284,8 +1287,12 @@ cpm_status bvec_run(cpm_ctx* c, int m, int64_t ne, const double* xyz, const doub
         const unsigned nbx = (unsigned)std::max<int64_t>(1, (ne + ST_THREADS - 1) / ST_THREADS);
         k_bin<T><<<dim3(nbx, m), ST_THREADS, 0, st>>>(xyz, Q, ne, c->g, p.cg, inv_h, key, cnt, wpos, nzc);
         CPM_LAUNCH(c, "k_bin");
-        k_totals<<<dim3(nbx, m), ST_THREADS, 0, s2>>>(xyz, Q, ne, (double*)(scr + p.off_spart), c->tickets, stats);
-        CPM_LAUNCH(c, "k_totals");
+        // the 2D sum has neither background nor dipole term: beside its FP64 evaluation of the mean potential the
+        // totals, of no use to it, took 5 to 12 us of b of 512 sites and four replicas (164 to 172 us, 158 now)
+        if (c->g.bc != CPM_BC_EW2D) {
+            k_totals<<<dim3(nbx, m), ST_THREADS, 0, s2>>>(xyz, Q, ne, (double*)(scr + p.off_spart), c->tickets, stats);
+            CPM_LAUNCH(c, "k_totals");
+        }
     }
     prof_end(c, CPM_K_CELLS);
     if (recip) {
