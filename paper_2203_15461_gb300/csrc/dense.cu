@@ -187,7 +187,7 @@ __global__ void __launch_bounds__(PF_T) k_potrf(double* Ab, int64_t lda, int kb,
         }
     };
     if (root || rroot) pivot(0, L[0][0]);
-    for (int j = 0; j < NB; ++j) {
+    for (int j = 0; j < kb; ++j) {   // a last block of fewer rows ends there
         __syncthreads();
         if (bad) break;   // set before the barrier; nobody writes it until the next one
         const double piv = s_piv[j & 1], inv = s_inv[j & 1];
@@ -209,7 +209,7 @@ __global__ void __launch_bounds__(PF_T) k_potrf(double* Ab, int64_t lda, int kb,
                     else if (c < i || i > j + 1) L[i][c] = fma(-lij, L[c][j], L[i][c]);   // the next pivot: below
                 }
             }
-        } else if ((root || rroot) && j + 1 < NB) {
+        } else if ((root || rroot) && j + 1 < kb) {
             pivot(j + 1, fma(-L[j + 1][j], L[j + 1][j], L[j + 1][j + 1]));
         }
     }
