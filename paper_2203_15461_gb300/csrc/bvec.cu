@@ -1304,12 +1304,7 @@ cpm_status bvec_run(cpm_ctx* c, int m, int64_t ne, const double* xyz, const doub
                               (longlong2*)(scr + p.off_ipart), (double*)rp));
         else CPM_TRY(rows_sf<T>(c, s1, p.rd, m, ne, EX, EY, EZ, rp));
         prof_end(c, CPM_K_SF);
-        if (fork && p.r64.use) {
-            // its CTAs need a whole SM each: behind the real-space sum, which fills every SM with small blocks for longer,
-            // the rest of this chain would start only then (EDL capacitor: 228 against 208 us)
-            CPM_CUDA(c, cudaEventRecord(c->fev[2], s1));
-            CPM_CUDA(c, cudaStreamWaitEvent(s0, c->fev[2], 0));
-        }
+        if (fork && p.r64.use) CPM_CUDA(c, cudaEventRecord(c->fev[2], s1));
         const Phases<T>& sp = site_tables<T>(c);
         prof_begin(c, CPM_K_SFRED);
         if (p.layers) CPM_TRY(rows_layers<T>(c, s1, p.cw, p.splits, m, rp, qs, (T*)(scr + p.off_T)));
@@ -1361,6 +1356,11 @@ cpm_status bvec_run(cpm_ctx* c, int m, int64_t ne, const double* xyz, const doub
         CPM_LAUNCH(c, "k_cellsort");
     }
     prof_end(c, CPM_K_CELLS);
+    // the CTAs of the integer products need a whole SM each: behind the real-space sum, which fills every SM with small
+    // blocks for longer, the rest of their chain would start only then (EDL capacitor: 228 against 208 us).  Only that
+    // sum waits for them; the cell list runs beside (one FP64 step of
+    // the capacitor 214.6 us with the wait in front of the cell list, 206.3 now)
+    if (fork && recip && p.r64.use) CPM_CUDA(c, cudaStreamWaitEvent(s0, c->fev[2], 0));
     prof_begin(c, CPM_K_REAL);
     if (std::is_same<T, float>::value && c->rpoly.deg) {
         CPM_TRY(real_poly_run(c, st, m, p.cg, start, (const float4*)sorted, real));
