@@ -1068,6 +1068,8 @@ __global__ void k_combine(const T* partial, int nctiles, const double* real, con
     }
     for (; k < nctiles; ++k) tiles.add(pp[(int64_t)k * n]);
     double s = tiles.value();
+    if constexpr (std::is_same<T, float>::value)
+        if (!isfinite(s)) s = sum_fp64(pp, n, nctiles);
     s += rl;
     if (b0) s += bz;
     if (pm) s += pm[t];   // P3M: the mesh potential in place of the Ewald tiles

@@ -86,14 +86,15 @@ struct PartSumF2 {
     }
     __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
 };
-struct PartSumF {   // single FP32 partials, the same two-sum
+struct PartSumF {   // single FP32 partials, the same two-sum; not finite where a sum leaves FP32's range: sum_fp64
     PartSumF2 s;
     __device__ __forceinline__ void add(float x) { s.add(make_float2(x, 0.f)); }
     __device__ __forceinline__ double value() const { return s.value(); }
 };
 
 // sum of terms of type T without loss against FP64: FP32 terms in three FP32 words by two exact two-sums (13
-// instructions of the FP32 pipe; a conversion and an addition in FP64 hold the SM for 32 clocks)
+// instructions of the FP32 pipe; a conversion and an addition in FP64 hold the SM for 32 clocks).  The value is not
+// finite where a sum leaves FP32's range, or a term is no finite number: sum_fp64
 template <typename T> struct TermSum;
 template <> struct TermSum<double> {
     double v = 0.0;
@@ -114,6 +115,14 @@ template <> struct TermSum<float> {
     }
     __device__ __forceinline__ double value() const { return (double)a + ((double)b + (double)c); }
 };
+
+// the same terms again, in FP64
+__device__ __forceinline__ double sum_fp64(const float* __restrict__ p, int64_t stride, int cnt) {
+    double s = 0.0;
+#pragma unroll 1
+    for (int k = 0; k < cnt; ++k) s += (double)p[k * stride];
+    return s;
+}
 
 // ----------------------------------------------------------------------------- device status word
 // Kernels never trap: they set one of these bits and return.  The host reads the

@@ -327,11 +327,14 @@ __global__ void __launch_bounds__(NB_T, 2) k_gemv_reduce(const P* __restrict__ p
             for (int k = 0; k < LD; ++k)
                 if (sp + k < splits) v.add(x[k]);
         }
+        double vs = v.value();
+        if constexpr (std::is_same<P, float>::value)
+            if (!isfinite(vs)) vs = sum_fp64(pi, stride, splits);
         double sv = 0.0;
         for (int g = 0; g < ng; ++g) sv += SG[i * ng + g] * psi[(int64_t)r * ng + g];
         for (int g = 0; g < ngrp; ++g) sv -= SZ[i * ngrp + g] * gmean[(int64_t)r * ngrp + g];
         // the centred products give sum_j S_ij (b_j - b_i): add b_i sum_j S_ij back where rows do not sum to zero
-        const double qi = sv - (srow ? v.value() + b[(int64_t)r * n + i] * srow[i] : v.value());
+        const double qi = sv - (srow ? vs + b[(int64_t)r * n + i] * srow[i] : vs);
         if (i == lo + threadIdx.x) q0 = qi;
         else qr[i] = qi;                        // read back by this thread alone
         a += qi;
