@@ -515,7 +515,7 @@ cpm_status cpm_bvec(cpm_ctx* c, int32_t m, int64_t n_e, const double* xyz, const
     if (!c->assembled) return set_err(c, CPM_E_STATE, "cpm_bvec before cpm_assemble");
     if (m < 1 || n_e < 0 || !b_out || (n_e > 0 && (!xyz || !Q)))
         return set_err(c, CPM_E_ARG, "cpm_bvec: need m >= 1, n_e >= 0 and non-null buffers");
-    if ((int64_t)m * n_e > (int64_t)1 << 30) return set_err(c, CPM_E_ARG, "cpm_bvec: m * n_e too large");
+    if ((int64_t)m * n_e > MAX_POINTS) return set_err(c, CPM_E_ARG, "cpm_bvec: m * n_e too large");
     return bvec(c, m, n_e, xyz, Q, b_out);
 }
 

@@ -17,6 +17,8 @@ namespace cpm {
 // Coulomb constant e / (4 pi eps0 Angstrom) in volts.
 constexpr double KE = 14.399645;
 constexpr double PI = 3.141592653589793;
+// charges of one call, over all replicas, at most
+constexpr int64_t MAX_POINTS = (int64_t)1 << 30;
 
 // ----------------------------------------------------------------------------- complex helpers
 template <typename T> struct C2;

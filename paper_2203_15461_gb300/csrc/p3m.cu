@@ -35,6 +35,8 @@
 //   29 -> 14 us; 16,384 sites x 16 replicas, 64 planes, 141 -> 43 us.
 // Arithmetic in T = double (k_prec = FP64) or float (the single-precision paths); the influence
 // function is computed in FP64 and stored in T.
+#include <limits>
+
 #include "common.cuh"
 
 namespace cpm {
@@ -207,26 +209,33 @@ template <typename T> struct P3mWords { static constexpr int n = std::is_same<T,
 constexpr int P3M_NT = 512;          // threads and charges per chunk of the assignment
 constexpr int P3M_CARRY = 1024;
 
+// Entries of a replica's lists: up to `most` per charge, which for the charges that one call may have is more than an int
+// holds (200 million charges at the corners of bricks).
+typedef unsigned long long p3m_pos;
+constexpr int P3M_MOST = 12;   // stencils of seven points over bricks of 32 x 32 x 4 (and no wider ones): 2 x 2 x 3
+static_assert((uint64_t)MAX_POINTS * P3M_MOST <= (uint64_t)std::numeric_limits<p3m_pos>::max(), "positions in the lists");
+
 // start[r][split][brick]: exclusive sums of the nb counts of a replica, one block each
 constexpr int P3M_SCAN = 256;
-__global__ void __launch_bounds__(P3M_SCAN) k_p3m_scan(const int* __restrict__ count, int nb, int* __restrict__ start) {
+__global__ void __launch_bounds__(P3M_SCAN) k_p3m_scan(const int* __restrict__ count, int nb, p3m_pos* __restrict__ start) {
     grid_wait();
     grid_go();
-    __shared__ int sw[P3M_SCAN / 32];
+    __shared__ p3m_pos sw[P3M_SCAN / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t r0 = (int64_t)blockIdx.x * nb;
-    int carry = 0;
+    p3m_pos carry = 0;
     for (int i0 = 0; i0 < nb; i0 += P3M_SCAN) {
-        const int i = i0 + threadIdx.x, c = i < nb ? count[r0 + i] : 0;
-        int v = c;
+        const int i = i0 + threadIdx.x;
+        const p3m_pos c = i < nb ? count[r0 + i] : 0;
+        p3m_pos v = c;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            const int u = __shfl_up_sync(0xffffffffu, v, o);
+            const p3m_pos u = __shfl_up_sync(0xffffffffu, v, o);
             if (lane >= o) v += u;
         }
         if (lane == 31) sw[warp] = v;
         __syncthreads();
-        int before = carry, all = 0;
+        p3m_pos before = carry, all = 0;
 #pragma unroll
         for (int w = 0; w < P3M_SCAN / 32; ++w) {
             before += w < warp ? sw[w] : 0;
@@ -240,14 +249,14 @@ __global__ void __launch_bounds__(P3M_SCAN) k_p3m_scan(const int* __restrict__ c
 
 // list[r ne most + start + ..]: the charges of every brick and split (`per` charges each); the starts become ends
 __global__ void __launch_bounds__(256) k_p3m_fill(const int* __restrict__ key, int64_t ptot, int64_t ne, int P, P3mBricks br,
-                                                int nsplit, int64_t per, int most, int* __restrict__ start, int* __restrict__ list) {
+                                                int nsplit, int64_t per, int most, p3m_pos* __restrict__ start, int* __restrict__ list) {
     grid_wait();
     const int64_t t = (int64_t)blockIdx.x * 256 + threadIdx.x;
     if (t >= ptot) return;
     const int64_t r = t / ne, j = t - r * ne, row = r * nsplit + j / per;
     int* mine = list + r * ne * most;
     br.each(key[t], P, [&](int brick) {
-        mine[atomicAdd(&start[row * br.n() + brick], 1)] = (int)j;
+        mine[atomicAdd(&start[row * br.n() + brick], (p3m_pos)1)] = (int)j;
     });
 }
 
@@ -255,7 +264,7 @@ template <typename T, int P>
 __global__ void __launch_bounds__(P3M_NT) k_p3m_spread(const int* __restrict__ key,
                                                        const typename P3mV4<T>::t* __restrict__ fq, int64_t ne, int m,
                                                        int Kx, int Ky, int Kz, int BX, int BY,
-                                                       const int* __restrict__ count, const int* __restrict__ start,
+                                                       const int* __restrict__ count, const p3m_pos* __restrict__ start,
                                                        const int* __restrict__ list, int most,
                                                        c2<T>* __restrict__ part, int* __restrict__ flag) {
     grid_wait();
@@ -680,7 +689,7 @@ size_t p3m_scratch_bytes(const cpm_ctx* c, int m, int64_t ne) {
     const int64_t ptot = (int64_t)m * ne;
     const P3mSpread sp = p3m_spread_plan(c, m, ne);
     return p3m_al(sizeof(int) * ptot) + p3m_al(sizeof(typename P3mV4<T>::t) * ptot) +
-           3 * p3m_al(sizeof(int) * (size_t)sp.nsplit * m * sp.nbricks) +   // marks, counts, starts
+           2 * p3m_al(sizeof(int) * (size_t)sp.nsplit * m * sp.nbricks) + p3m_al(sizeof(p3m_pos) * (size_t)sp.nsplit * m * sp.nbricks) +   // marks, counts, starts
            p3m_al(sizeof(int) * (size_t)ptot * sp.br.most(c->p.p3m_order)) + p3m_al(sizeof(c2<T>) * (size_t)sp.nsplit * ((m + 1) / 2) * mesh_pts(c));
 }
 template size_t p3m_scratch_bytes<float>(const cpm_ctx*, int, int64_t);
@@ -793,7 +802,7 @@ template <typename T> static const c2<T>* p3m_twiddles(const cpm_ctx* c) {
 
 template <typename T, int P>
 static cpm_status launch_p3m_pp(cudaStream_t st, cpm_ctx* c, int m, int64_t ne, const int* key,
-                          const typename P3mV4<T>::t* fq, int* flag, const int* count, const int* start, const int* list, int most,
+                          const typename P3mV4<T>::t* fq, int* flag, const int* count, const p3m_pos* start, const int* list, int most,
                           c2<T>* mesh, double* pm) {
     const int Kx = c->p.p3m_mesh[0], Ky = c->p.p3m_mesh[1], Kz = c->p.p3m_mesh[2];
     const P3mSpread sp = p3m_spread_plan(c, m, ne);
@@ -840,8 +849,8 @@ cpm_status p3m_run(cpm_ctx* c, cudaStream_t st, int m, int64_t ne, const double*
     const P3mSpread sp = p3m_spread_plan(c, m, ne);
     const size_t lists = p3m_al(sizeof(int) * (size_t)sp.nsplit * m * sp.nbricks);
     int* count = (int*)((char*)flag + lists);
-    int* start = (int*)((char*)count + lists);
-    int* list = (int*)((char*)start + lists);
+    p3m_pos* start = (p3m_pos*)((char*)count + lists);
+    int* list = (int*)((char*)start + p3m_al(sizeof(p3m_pos) * (size_t)sp.nsplit * m * sp.nbricks));
     const int most = sp.br.most(c->p.p3m_order);
     c2<T>* mesh = (c2<T>*)((char*)list + p3m_al(sizeof(int) * (size_t)ptot * most));
     const int P = c->p.p3m_order;
