@@ -391,6 +391,8 @@ struct cpm_ctx {
     void* p3m_G64 = nullptr;     // the same in FP64 for the P3M elastance when k_prec is single precision
     void* p3m_tw64 = nullptr;
 
+    signed char wide_reduce[3] = {-1, -1, -1};   // k_gemv_reduce in clusters of sixteen: 1 placeable, 0 not, -1 not asked
+
     int64_t launches = 0;        // kernels launched by cpm_bvec / cpm_update / cpm_step_host
 
     // tracing (cpm_profile)

@@ -378,8 +378,9 @@ __global__ void __launch_bounds__(256) k_sum_splits(const P* __restrict__ part, 
 // eight); beyond, eight while the replicas' blocks are one wave of two per SM, and fewer after that: with eight for
 // every batch, 256 replicas of 4,320 sites took 566 us an update, with one block each 507; of 1,031 sites 113 and 101;
 // 64 of 4,320 on the tensor cores 66 and 56 with four.
-static int reduce_cluster(int64_t n, int m) {
-    int cl = m <= 4 ? NB_CLUSTER : 8;
+// wide: the device places clusters of sixteen
+static int reduce_cluster(int64_t n, int m, bool wide) {
+    int cl = m <= 4 && wide ? NB_CLUSTER : 8;
     while (cl > 1 && (m > 4 && (int64_t)m * cl > 2 * 152)) cl /= 2;
     while (cl > 1 && n < (int64_t)cl * (cl > 8 ? 2 * NB_LEAST : NB_LEAST)) cl /= 2;
     return cl;
@@ -395,20 +396,31 @@ static bool reduce_sums_first(int64_t n, int m, int64_t splits) {
 template <typename P>
 static cpm_status launch_reduce(cpm_ctx* c, const void* part, int splits, int m, const double* psi, double* q, double* qtot,
                                 const double* b, const double* srow, const double* SZ, const double* gmean, int ngrp) {
-    const int cl = reduce_cluster(c->n, m);
-    if (cl > 8) CPM_CUDA(c, cudaFuncSetAttribute(k_gemv_reduce<P>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-    const int64_t slice = (c->n + cl - 1) / cl;
+    // clusters beyond eight blocks are not portable: asked once per context whether the largest blocks can be placed
+    signed char& wide = c->wide_reduce[std::is_same<P, double>::value ? 0 : std::is_same<P, float2>::value ? 1 : 2];
     cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = NB_CLUSTER;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    if (m <= 4 && wide < 0) {
+        int fit = 0;
+        cfg.gridDim = dim3(NB_CLUSTER);
+        cfg.blockDim = dim3(NB_T);
+        cfg.numAttrs = 1;
+        wide = cudaFuncSetAttribute(k_gemv_reduce<P>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+               cudaOccupancyMaxActiveClusters(&fit, k_gemv_reduce<P>, &cfg) == cudaSuccess && fit > 0;
+        cudaGetLastError();   // a refusal is an answer
+    }
+    const int cl = reduce_cluster(c->n, m, wide > 0);
+    const int64_t slice = (c->n + cl - 1) / cl;
     cfg.gridDim = dim3((unsigned)cl, (unsigned)m);
     cfg.blockDim = dim3((unsigned)std::min<int64_t>(NB_T, (slice + 31) / 32 * 32));
     cfg.stream = c->stream;
-    cudaLaunchAttribute at[2];
-    at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = (unsigned)cl;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // as launch_after()
     at[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
     cfg.numAttrs = 2;
     CPM_CUDA(c, cudaLaunchKernelEx(&cfg, k_gemv_reduce<P>, (const P*)part, splits, (const double*)upd_sg(c), (int)upd_ng(c), psi,
                                    c->n, m, q, (const double*)c->u, (int)c->p.symm, qtot, b, srow, SZ, gmean, ngrp));
