@@ -111,7 +111,9 @@ typedef struct {
     int32_t symm;        /* 1: S of Eq. (S) (neutral electrodes); 0: S = A^-1 */
     int32_t s_prec;      /* cpm_precision of the S (v - b) product */
     int32_t k_prec;      /* cpm_precision of the b-vector sums (real and reciprocal space) */
-    size_t hbm_budget;   /* bytes of device memory this context may allocate; 0 = no limit */
+    size_t hbm_budget;   /* bytes of device memory this context may allocate; 0 = no limit.  A call whose
+                            scratch does not fit takes slower plans that need less before it refuses, and
+                            the context keeps them until its next geometry */
     int32_t chol;        /* cpm_chol of cpm_invert */
     int32_t kspace;      /* cpm_kspace of the reciprocal part of b (0: Ewald) */
     int32_t p3m_order;   /* P3M assignment order p, 2..7 (kspace = CPM_KSPACE_P3M) */

@@ -165,6 +165,7 @@ static void free_geometry(cpm_ctx* c) {
     c->n = 0;
     c->assembled = c->inverted = false;
     c->has_A = false;
+    c->lean = 0;
 }
 
 static uint64_t fnv1a(uint64_t h, const void* data, size_t bytes) {

@@ -1104,6 +1104,7 @@ struct BvecPlan {
         off_ewT, off_pm, off_p3m, total;
     int c0chunks;
     bool p3m;                           // reciprocal part of b by P3M (p3m.cu)
+    int p3m_m;                          // replicas at a time
     bool tc, real64;
     size_t off_sorted32, off_ipart, off_qmax, off_spart;
 };
@@ -1179,7 +1180,9 @@ static BvecPlan<T> plan_bvec(const cpm_ctx* c, int m, int64_t ne) {
     p.off_pm = p.off_p3m = o;
     if (p.p3m) {
         p.off_pm = o; o += al(sizeof(double) * (size_t)m * c->n);
-        p.off_p3m = o; o += al(p3m_scratch_bytes<T>(c, m, ne));
+        // within a tight budget a few replicas at a time (whole pairs, which share a mesh, while they fit)
+        p.p3m_m = c->lean == 0 ? m : c->lean == 1 ? std::min(m, (m + 7) / 8 * 2) : 1;
+        p.off_p3m = o; o += al(p3m_scratch_bytes<T>(c, p.p3m_m, ne));
     }
     p.total = o;
     return p;
@@ -1337,7 +1340,9 @@ cpm_status bvec_run(cpm_ctx* c, int m, int64_t ne, const double* xyz, const doub
     if (p.p3m && ptot > 0) {
         pm = (double*)(scr + p.off_pm);
         prof_begin(c, CPM_K_P3M);
-        CPM_TRY(p3m_run<T>(c, s1, m, ne, xyz, Q, scr + p.off_p3m, pm));
+        for (int r = 0; r < m; r += p.p3m_m)
+            CPM_TRY(p3m_run<T>(c, s1, std::min(p.p3m_m, m - r), ne, xyz + 3 * (int64_t)r * ne, Q + (int64_t)r * ne,
+                               scr + p.off_p3m, pm + (int64_t)r * n));
         prof_end(c, CPM_K_P3M);
     }
     double* ew = nullptr;
@@ -1433,19 +1438,18 @@ cpm_status ensure_aux(cpm_ctx* c) {
 }
 
 cpm_status reserve_bvec(cpm_ctx* c, int m, int64_t ne) {
-    const bool f32 = c->p.k_prec != CPM_PREC_FP64;
     CPM_TRY(ensure_aux(c));
     CPM_TRY(ensure_tickets(c, 2 * m));   // k_totals takes [0, m), k_col0 [m, 2m)
-    return ensure_scratch(c, f32 ? bvec_scratch_bytes<float>(c, m, ne) : bvec_scratch_bytes<double>(c, m, ne));
+    return reserve_within_budget(c, [&] {
+        return ensure_scratch(c, c->p.k_prec != CPM_PREC_FP64 ? bvec_scratch_bytes<float>(c, m, ne) : bvec_scratch_bytes<double>(c, m, ne));
+    });
 }
 
 cpm_status bvec(cpm_ctx* c, int m, int64_t ne, const double* xyz, const double* Q, double* b_out, float2* bhl) {
-    const bool f32 = c->p.k_prec != CPM_PREC_FP64;
-    const size_t need = f32 ? bvec_scratch_bytes<float>(c, m, ne) : bvec_scratch_bytes<double>(c, m, ne);
-    CPM_TRY(ensure_scratch(c, need));
-    CPM_TRY(ensure_tickets(c, 2 * m));   // k_totals takes [0, m), k_col0 [m, 2m)
+    CPM_TRY(reserve_bvec(c, m, ne));
     char* scr = (char*)c->scratch;
-    return f32 ? bvec_run<float>(c, m, ne, xyz, Q, b_out, bhl, scr) : bvec_run<double>(c, m, ne, xyz, Q, b_out, bhl, scr);
+    return c->p.k_prec != CPM_PREC_FP64 ? bvec_run<float>(c, m, ne, xyz, Q, b_out, bhl, scr)
+                                        : bvec_run<double>(c, m, ne, xyz, Q, b_out, bhl, scr);
 }
 
 }  // namespace cpm

@@ -341,6 +341,8 @@ struct cpm_ctx {
     const double* sg_over = nullptr;   // when set, the update reads these responses and columns
     int ng_over = 0;
 
+    int lean = 0;                // 1, 2: plans of fewer partial sums, for a budget without room for the fast ones
+
     // per-step scratch, grown on demand
     int cap_m = 0;
     int64_t cap_ne = 0;
@@ -474,6 +476,15 @@ size_t phase_elems(const KTable& k, int64_t P);
 // api.cu
 cpm_status ensure_scratch(cpm_ctx* c, size_t bytes);
 cpm_status ensure_tickets(cpm_ctx* c, int m);
+// reserve(), which plans by c->lean and allocates, again with leaner plans while the budget refuses it
+template <typename F> cpm_status reserve_within_budget(cpm_ctx* c, F reserve) {
+    for (;;) {
+        const cpm_status s = reserve();
+        if (s != CPM_E_BUDGET || c->lean >= 2) return s;
+        ++c->lean;
+        c->err.clear();
+    }
+}
 
 // Last-block reduction: every block of a replica stores its partial, then takes a ticket; the
 // block that draws the last ticket sums the partials in block order (a fixed order, so the result

@@ -679,6 +679,7 @@ static P3mSpread p3m_spread_plan(const cpm_ctx* c, int m, int64_t ne) {
     const int64_t nchunks = std::max<int64_t>(1, (ne + P3M_NT - 1) / P3M_NT);
     int64_t ns = std::max<int64_t>(1, (32 * 152 + ctas - 1) / ctas);
     ns = std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(ns, 8), nchunks / 3));
+    if (c->lean) ns = c->lean > 1 ? 1 : (ns + 3) / 4;
     sp.cps = (int)((nchunks + ns - 1) / ns);
     sp.nsplit = (int)((nchunks + sp.cps - 1) / sp.cps);
     return sp;

@@ -692,7 +692,7 @@ template <typename T> RowDims row_dims(const cpm_ctx* c, int m, int64_t ne) {
     // about six blocks per SM, so that the last ones to finish leave little of the GPU idle; no range
     // shorter than one K step
     const int64_t maxs = std::max<int64_t>(1, (ne + RW_BK - 1) / RW_BK);
-    const int64_t want = (6 * 152 + work * m - 1) / std::max<int64_t>(1, work * m);
+    const int64_t want = c->lean > 1 ? 1 : ((6 * 152 + work * m - 1) / std::max<int64_t>(1, work * m)) >> (2 * c->lean);
     d.splits = (int)std::max<int64_t>(1, std::min<int64_t>(want, std::min<int64_t>(maxs, 64)));
     d.chunk = std::max<int64_t>(1, ((ne + d.splits - 1) / d.splits + RW_BK - 1) / RW_BK) * RW_BK;
     d.splits = (int)std::max<int64_t>(1, (ne + d.chunk - 1) / d.chunk);

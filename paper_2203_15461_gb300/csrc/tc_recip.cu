@@ -600,6 +600,7 @@ TcRecipDims tc_recip_dims(const cpm_ctx* c, int m, int64_t ne) {
     for (int s = (int)((steps + RF_RANGE - 1) / RF_RANGE); s <= steps && s <= (int)((steps + RF_RANGE - 1) / RF_RANGE) + 64; ++s) {
         const int64_t spc = (steps + s - 1) / s, used = (steps + spc - 1) / spc;
         if (used != s) continue;
+        if (c->lean && best < 1e300) break;
         const double t = (double)((base * s + 151) / 152) * (double)(spc + 3);
         if (t < 0.97 * best) {
             best = t;

@@ -297,6 +297,7 @@ Rows64Dims rows64_dims(const cpm_ctx* c, int m, int64_t ne) {
     for (int s = least; s <= d.steps && s < least + 64; ++s) {
         const int spc = (d.steps + s - 1) / s;
         if ((d.steps + spc - 1) / spc != s) continue;
+        if (c->lean && best < 1e300) break;
         const double tt = (double)((base * s + 151) / 152) * (spc + 6);
         if (tt < 0.97 * best) {
             best = tt;
@@ -306,7 +307,7 @@ Rows64Dims rows64_dims(const cpm_ctx* c, int m, int64_t ne) {
     }
     // 2 FP64 multiply-adds per (charge, k) at 304 per clock against about 15 us of fixed cost here: 2e7 is 35 us
     // (its partial sums, 16 bytes each, are kept below 128 MiB: beyond that the CUDA cores take the call)
-    d.use = t.items64 > 0 && 2.0 * (double)c->kt.nk * (double)ne * m >= 2e7 &&
+    d.use = c->lean < 2 && t.items64 > 0 && 2.0 * (double)c->kt.nk * (double)ne * m >= 2e7 &&
             sizeof(longlong2) * (size_t)d.splits * m * 4 * t.np * d.cw <= ((size_t)128 << 20);
     return d;
 }

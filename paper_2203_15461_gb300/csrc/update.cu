@@ -454,9 +454,9 @@ static int64_t gemv_colblocks(const cpm_ctx* c) {
 // 25 split counts at each of 42 sizes).  About one wave of blocks whatever their remainder, the rule before: 2,050 sites
 // x 8 87.5 us an update, 77.5 now, x 64 621 and 509; 8,192 x 16 2,124 and 1,781, x 64 8,286 and 6,950; 16,384 x 1 567
 // and 493.  The fewest splits within 1 % (their partial sums are memory).
-static void gemv64_plan(int64_t n, int64_t blocks, int64_t* splits, int64_t* jchunk) {
+static void gemv64_plan(int64_t n, int64_t blocks, int lean, int64_t* splits, int64_t* jchunk) {
     const double busy[5] = {0.0, 0.5, 0.9, 0.95, 1.0};
-    const int64_t most = std::min<int64_t>(64, (n + G6_U - 1) / G6_U);
+    const int64_t most = std::min<int64_t>(lean > 1 ? 1 : 64 >> (2 * lean), (n + G6_U - 1) / G6_U);
     double cost[65], best = 1e300;
     for (int64_t s = 1; s <= most; ++s) {
         const int64_t j = ((n + s - 1) / s + G6_U - 1) / G6_U * G6_U, nb = blocks * ((n + j - 1) / j), k = (nb + 151) / 152;
@@ -469,7 +469,7 @@ static void gemv64_plan(int64_t n, int64_t blocks, int64_t* splits, int64_t* jch
     *splits = (n + *jchunk - 1) / *jchunk;
 }
 
-static cpm_status reserve_update_plan(cpm_ctx* c, int m, int64_t* splits_out, int64_t* jchunk_out) {
+static cpm_status reserve_update_lean(cpm_ctx* c, int m, int64_t* splits_out, int64_t* jchunk_out) {
     const int64_t n = c->n;
     const int64_t colblocks = gemv_colblocks(c);
     const int mr = gemv_fp64(c) ? gemv64_mr(m) : GT_MR;
@@ -479,7 +479,7 @@ static cpm_status reserve_update_plan(cpm_ctx* c, int m, int64_t* splits_out, in
     splits = std::max<int64_t>(1, std::min<int64_t>(splits, (n + GT_JT - 1) / GT_JT));
     int64_t jchunk = (((n + splits - 1) / splits + GT_JT - 1) / GT_JT) * GT_JT;
     splits = (n + jchunk - 1) / jchunk;
-    if (gemv_fp64(c)) gemv64_plan(n, colblocks * rchunks, &splits, &jchunk);
+    if (gemv_fp64(c)) gemv64_plan(n, colblocks * rchunks, c->lean, &splits, &jchunk);
     if (gemv_tma_supported(c)) {
         int64_t cb;
         gemv_tma_plan(n, m, &cb, &splits, &jchunk);
@@ -497,6 +497,10 @@ static cpm_status reserve_update_plan(cpm_ctx* c, int m, int64_t* splits_out, in
     *splits_out = splits;
     *jchunk_out = jchunk;
     return CPM_OK;
+}
+
+static cpm_status reserve_update_plan(cpm_ctx* c, int m, int64_t* splits, int64_t* jchunk) {
+    return reserve_within_budget(c, [&] { return reserve_update_lean(c, m, splits, jchunk); });
 }
 
 cpm_status reserve_update(cpm_ctx* c, int m) {
