@@ -1303,11 +1303,16 @@ cpm_status bvec_run(cpm_ctx* c, int m, int64_t ne, const double* xyz, const doub
     if (recip) {
         const float* qs = p.tc ? qmax : nullptr;
         prof_begin(c, CPM_K_SF);
-        if (p.tc) CPM_TRY(tc_recip_sf(c, s1, p.td, m, (const float2*)EX, qmax, qlast, (float*)rp));
-        else if (p.r64.use)
+        if (p.tc) {
+            // the scale is there long before the site stage: waited for here, the kernels behind follow one another directly
+            if (fork && !p.layers) CPM_CUDA(c, cudaStreamWaitEvent(s1, c->fev[2], 0));
+            CPM_TRY(tc_recip_sf(c, s1, p.td, m, (const float2*)EX, qmax, qlast, (float*)rp, p.layers));
+        } else if (p.r64.use) {
             CPM_TRY(rows64_sf(c, s1, p.r64, m, (const longlong2*)EX, (const longlong2*)EY, (const longlong2*)EZ, qlast,
                               (longlong2*)(scr + p.off_ipart), (double*)rp));
-        else CPM_TRY(rows_sf<T>(c, s1, p.rd, m, ne, EX, EY, EZ, rp));
+        } else {
+            CPM_TRY(rows_sf<T>(c, s1, p.rd, m, ne, EX, EY, EZ, rp));
+        }
         prof_end(c, CPM_K_SF);
         if (fork && p.r64.use) CPM_CUDA(c, cudaEventRecord(c->fev[2], s1));
         const Phases<T>& sp = site_tables<T>(c);
@@ -1319,7 +1324,6 @@ cpm_status bvec_run(cpm_ctx* c, int m, int64_t ne, const double* xyz, const doub
         if (p.layers) {
             CPM_TRY(rows_sites<T>(c, s1, m, (const T*)(scr + p.off_T), part));
         } else if (p.tc) {
-            if (fork) CPM_CUDA(c, cudaStreamWaitEvent(s1, c->fev[2], 0));
             CPM_TRY(tc_recip_sites(c, s1, p.td, m, (const float2*)wr, qsum, scr + p.off_w16, (float*)part));
         } else if (std::is_same<T, float>::value) {
             dim3 gs((unsigned)((n + T2_BS - 1) / T2_BS), p.ctiles, m);

@@ -622,7 +622,7 @@ cpm_status tc_recip_prepare(cpm_ctx* c);
 cpm_status tc_recip_scales(cpm_ctx* c, cudaStream_t st, int m, int64_t ne, const double* Q, float* qsum);
 // tab: the charge phases of launch_charge_slots; part as rows_sf, times 2^14 pow2_below(max |Q|, 14)
 cpm_status tc_recip_sf(cpm_ctx* c, cudaStream_t st, const TcRecipDims& d, int m, const float2* tab, const float* qmax,
-                       const int* qlast, float* part);
+                       const int* qlast, float* part, bool chained);
 // the site stage of electrodes whose sites hardly share heights, from w rho of the signed columns
 cpm_status tc_recip_sites(cpm_ctx* c, cudaStream_t st, const TcRecipDims& d, int m, const float2* wrho,
                           const float* qsum, void* w16, float* site_partial);

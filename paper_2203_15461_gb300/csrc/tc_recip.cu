@@ -348,6 +348,7 @@ __global__ void __launch_bounds__(1024) k_qsum_abs(const double* __restrict__ Q,
 __global__ void __launch_bounds__(1024)
     k_tc_wsplit(const float2* __restrict__ wrho, int m, int nzw, int ncols, const float* __restrict__ qsum, float wmax,
                 int CT, int mr, int ncb, int NB, int KZ, uint32_t* __restrict__ w16, int64_t plane_words) {
+    grid_wait();
     __shared__ float2 tile[32][33];
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int zb = blockIdx.x * 32, cb0 = blockIdx.y * 32, rp = blockIdx.z;
@@ -434,6 +435,7 @@ __global__ void __launch_bounds__(RS_THREADS, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    grid_wait();   // what is above touches nothing that another kernel writes
     const uint32_t stage_bytes = 2 * RS_A + 2 * NB * 128;
 
     if (warp == RS_TMA_WARP && lane == 0) {
@@ -657,13 +659,18 @@ cpm_status tc_recip_scales(cpm_ctx* c, cudaStream_t st, int m, int64_t ne, const
 }
 
 cpm_status tc_recip_sf(cpm_ctx* c, cudaStream_t st, const TcRecipDims& d, int m, const float2* tab, const float* qmax,
-                       const int* qlast, float* part) {
+                       const int* qlast, float* part, bool chained) {
     const KTable& k = c->kt;
     const RowTable& t = c->rows;
     CPM_CUDA(c, cudaFuncSetAttribute(k_tc_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, RF_SMEM));
-    CPM_CUDA(c, launch_after(k_tc_rows, dim3((unsigned)(t.tcitems * (int64_t)m * d.splits)), dim3(RF_THREADS), RF_SMEM, st, 
-        t.tcitem, t.tcrange, t.pairs, tab, (int64_t)m * d.nep, d.nep, k.NX, k.NY, k.NZ, qmax, qlast, t.tcitems, d.splits,
-        d.spc, m, t.np, d.cw, part, c->status, RT_WAIT_NS));
+    const dim3 grid((unsigned)(t.tcitems * (int64_t)m * d.splits));
+    auto launch = [&](auto... a) {   // chained: the kernel in front of this one in the stream is all it waits for
+        if (chained) return launch_after(k_tc_rows, grid, dim3(RF_THREADS), RF_SMEM, st, a...);
+        k_tc_rows<<<grid, RF_THREADS, RF_SMEM, st>>>(a...);
+        return cudaSuccess;
+    };
+    CPM_CUDA(c, launch(t.tcitem, t.tcrange, t.pairs, tab, (int64_t)m * d.nep, d.nep, k.NX, k.NY, k.NZ, qmax, qlast, t.tcitems,
+                       d.splits, d.spc, m, t.np, d.cw, part, c->status, RT_WAIT_NS));
     CPM_LAUNCH(c, "k_tc_rows");
     return CPM_OK;
 }
@@ -675,8 +682,8 @@ cpm_status tc_recip_sites(cpm_ctx* c, cudaStream_t st, const TcRecipDims& d, int
     if (!c->tcz || !c->tcxy) return set_err(c, CPM_E_STATE, "tensor-core reciprocal operands not prepared");
     const int64_t plane_words = (int64_t)d.ngroups * d.NB * (d.KZ / 2);
     dim3 gw((unsigned)((d.KZ / 2 + 31) / 32), (unsigned)((d.ncb * d.CT + 31) / 32), (unsigned)(d.nrb * d.mr));
-    k_tc_wsplit<<<gw, 1024, 0, st>>>(wrho, m, k.nzw, k.ncols, qsum, c->tc_wmax, d.CT, d.mr, d.ncb, d.NB, d.KZ,
-                                     (uint32_t*)w16, plane_words);
+    CPM_CUDA(c, launch_after(k_tc_wsplit, gw, dim3(1024), 0, st, wrho, m, k.nzw, k.ncols, qsum, c->tc_wmax, d.CT, d.mr, d.ncb,
+                             d.NB, d.KZ, (uint32_t*)w16, plane_words));
     CPM_LAUNCH(c, "k_tc_wsplit");
     SiteMaps maps;
     const uint16_t* za = (const uint16_t*)c->tcz;
@@ -689,9 +696,9 @@ cpm_status tc_recip_sites(cpm_ctx* c, cudaStream_t st, const TcRecipDims& d, int
     }
     CPM_CUDA(c, cudaFuncSetAttribute(k_tc_site, cudaFuncAttributeMaxDynamicSharedMemorySize, RS_SMEM));
     const int ntx = (int)(d.npad / RS_BM), ntiles = ntx * d.ngroups;
-    k_tc_site<<<(unsigned)std::min(ntiles, 152), RS_THREADS, RS_SMEM, st>>>(
+    CPM_CUDA(c, launch_after(k_tc_site, dim3((unsigned)std::min(ntiles, 152)), dim3(RS_THREADS), RS_SMEM, st,
         maps, k.colext, k.ncols, k.NZ, d.mr, d.ncb, d.NB, m, ntx, ntiles, c->tcxy, n, qsum, c->tc_wmax, site_partial,
-        c->status, RT_WAIT_NS);
+        c->status, RT_WAIT_NS));
     CPM_LAUNCH(c, "k_tc_site");
     return CPM_OK;
 }
