@@ -11,7 +11,9 @@ mixed path (FP32 b and S, FP64 neutrality and totals; by default the two recipro
 contractions of b run on the tensor cores as two-term fp16 products, ``--k-prec fp32``
 keeps them on the CUDA cores); the plain FP64 path is timed beside it.  Inputs are
 resident in HBM; L2 is flushed (a 256 MB write, then a 256 MB read of a second buffer)
-before every timed step and only the step itself is inside the CUDA events.  Extra fields:
+before every timed step and only the step itself is inside the CUDA events.  The one line on stdout holds the contract's
+keys and the main figures (``summary``: a reader that keeps only the end of a run's output still
+has all of it); everything measured goes to stderr as one JSON line after ``details:``, among it
 256 replicas of the 216-site capacitor per step, a Poisson serving stream, and the
 single-precision S product alone at 16,384 sites (S32 = 1.07 GB) against the HBM peak.
 """
@@ -792,6 +794,32 @@ def rel_l2(a, b):
     return float(np.linalg.norm(np.asarray(a) - np.asarray(b)) / np.linalg.norm(np.asarray(b)))
 
 
+SUMMARY_BYTES = 1400
+
+
+def summary(line: dict) -> dict:
+    """The contract's keys and the main figures of everything measured, within SUMMARY_BYTES of JSON."""
+    def short(v):
+        return float(f"{v:.6g}") if isinstance(v, float) else v
+
+    def pick(d, keys):
+        return {k: short(d[k]) for k in keys if k in d}
+
+    out = pick(line, ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+                      "vs_baseline", "dtype", "data"))
+    out["config"] = pick(line["config"], ("workload", "n_sites", "n_charges", "n_kvectors", "replicas_per_step", "k_prec",
+                                          "parallelism"))
+    out["config"]["l2"] = "flushed before every timed step"
+    out["e2e"] = pick(line["e2e"], ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step"))
+    out["gpu_launches"] = line["gpu_launches"]
+    out["clocks"] = pick(line["clocks"], ("sm_mhz", "sm_max_mhz", "reasons"))
+    out.update(pick(line, ("fp64_value", "speedup_vs_fp64", "rel_err_mixed_vs_fp64", "max_abs_qtot")))
+    out["roofline"] = pick(line.get("roofline", {}), ("kernel", "bound", "achieved", "unit", "frac", "ms_per_launch"))
+    if "cpu_baseline" in line:
+        out["cpu_baseline"] = pick(line["cpu_baseline"], ("value", "unit", "cores", "kind"))
+    return out
+
+
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
@@ -929,7 +957,7 @@ def main():
                              "tensor_complex_mac": FLOP_CMAC}
     # DRAM bytes (read + write) per launch from the committed ncu capture of these kernels on this
     # workload (cold caches); a stored figure, not measured by this run
-    traffic_ncu = {"sf": 58.60e6, "site": 15.56e6, "gemv": 75.07e6, "real": 1.42e6}
+    traffic_ncu = {"gemv": 75.07e6, "real": 1.42e6}
     roof["traffic"] = traffic_ncu.get(top)
     roof["traffic_source"] = ("stored: ncu dram__bytes_read.sum + dram__bytes_write.sum of one launch, "
                               "profiles/launches_edl_capacitor_4320.md")
@@ -1017,7 +1045,8 @@ def main():
     if world > 1:
         dist.barrier()
         dist.destroy_process_group()
-    print(json.dumps(line), flush=True)
+    print("details: " + json.dumps(line), file=sys.stderr, flush=True)
+    print(json.dumps(summary(line)), flush=True)
     return 0
 
 
