@@ -132,7 +132,6 @@ __global__ void __launch_bounds__(ST_THREADS) k_totals(const double* __restrict_
 // Per-replica exclusive scan of cell counts into global start offsets (replica r starts after the
 // nonzero charges of the replicas before it, so the cells of all replicas are contiguous):
 // one block per replica; each thread takes CS_PER consecutive cells of a tile of CS_THREADS x CS_PER.
-// The block is small enough to run beside a structure-factor CTA on its SM.
 constexpr int CS_THREADS = 256, CS_PER = 8;
 __global__ void __launch_bounds__(CS_THREADS) k_cellscan(const int* count, int* start, int ncells, int64_t ne, int m,
                                                          const int* nzc) {
@@ -1225,9 +1224,9 @@ cpm_status bvec_run(cpm_ctx* c, int m, int64_t ne, const double* xyz, const doub
     const int nc = m * p.cg.ncells;
     c->launches += (c->g.bc != CPM_BC_EW2D ? 5 : 4) + (ptot > 0 ? 2 : 0) + ((k.nk > 0 && ptot > 0 && !p.p3m) ? 4 + (p.r64.use ? 2 : 0) + (p.layers || !p.tc ? 0 : 2) : 0);
 
-    // Three chains: the origin stream bins the charges (per-replica totals) and runs the cell list and
-    // the real-space sum; side stream 1 takes the phase tables and the reciprocal sums; side stream 2 sums the
-    // k_perp = 0 column.  k_combine joins them.  With per-kernel profiling on, everything runs on the
+    // Three chains: the origin stream bins the charges and runs the cell list and the real-space sum; side stream 1 takes
+    // the phase tables and the reciprocal sums; side stream 2 the charge scale of the general site stage, the k_perp = 0
+    // column and the per-replica totals.  k_combine joins them.  With per-kernel profiling on, everything runs on the
     // origin stream in the same order.
     const bool recip = k.nk > 0 && ptot > 0 && !p.p3m;
     const bool fork = !c->prof_on;

@@ -173,7 +173,11 @@ struct KTable {
 // The k set in the real product basis (recip_rows.cu): pairs (nx, ny) with nx, ny >= 0 in the order of
 // |k_perp|, four rows (cos / sin of x times cos / sin of y) each.
 constexpr int ROW_TILE = 128;          // sites per block of the height-wise site stage
-constexpr int LAYER_MIN_SITES = 8;     // sites per distinct height from which the tables by height are made
+// Sites per distinct height from which the tables by height are made.  The elastance of 2,048 sites takes 402 ms site by
+// site, by pairs of heights 654 with four sites per height, 168 with eight, 46 with sixteen; FP64 b 1,360 us site by site, by
+// height 1,000, 539 and 293; P3M's interpolation is as fast either way at eight (512 sites x 8: 73 and 72 us a pass) and
+// faster beyond (72.7 and 70.0 at sixteen).  The single-precision site stage has a line of its own (rows_by_height).
+constexpr int LAYER_MIN_SITES = 8;
 constexpr int ROW_TC_PAIRS = 64;       // pairs, charges per step and staged x and y harmonics of a CTA of the
 constexpr int ROW_TC_STEP = 64;        // tensor-core structure factor (tc_recip.cu)
 constexpr int ROW_TC_SLOTS = 50;

@@ -16,7 +16,7 @@ namespace cpm {
 // thread is not load-bound once the next K step is fetched while the current one is multiplied; what
 // matters is that every SM has a tile: 64 x 64 x 64 takes 68 us on one.  64 x 64 tiles are taken from DG_MANY of
 // them on (four per SM), 32 x 32 below.
-constexpr int DG_BM = 64, DG_BK = 16, DG_T = 256, DG_MANY = 4 * 152;
+constexpr int DG_LARGE = 64, DG_SMALL = 32, DG_BK = 16, DG_T = 256, DG_MANY = 4 * 152;
 
 // one tile at (r0, c0), K range [kbeg, kend), kbeg a multiple of DG_BK
 template <bool TA, bool TB, int BM, int BN>
@@ -130,12 +130,12 @@ __global__ void __launch_bounds__(DG_T) k_trinv_level(double* W, double* T, int6
 template <bool TA, bool TB>
 static void dgemm_tiles(cudaStream_t s, int M, int N, int K, double alpha, const double* A, int64_t lda, const double* B,
                         int64_t ldb, double beta, double* C, int64_t ldc, int lower, int tri, const unsigned* status) {
-    const int64_t tm = (M + 63) / 64, tn = (N + 63) / 64, tiles = lower ? tm * (tm + 1) / 2 : tm * tn;
+    const int64_t tm = (M + DG_LARGE - 1) / DG_LARGE, tn = (N + DG_LARGE - 1) / DG_LARGE, tiles = lower ? tm * (tm + 1) / 2 : tm * tn;
     if (tiles >= DG_MANY)
-        k_dgemm<TA, TB, 64, 64><<<dim3((unsigned)tn, (unsigned)tm), DG_T, 0, s>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc,
+        k_dgemm<TA, TB, DG_LARGE, DG_LARGE><<<dim3((unsigned)tn, (unsigned)tm), DG_T, 0, s>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc,
                                                                                  lower, tri, status);
     else
-        k_dgemm<TA, TB, 32, 32><<<dim3((N + 31) / 32, (M + 31) / 32), DG_T, 0, s>>>(M, N, K, alpha, A, lda, B, ldb, beta, C,
+        k_dgemm<TA, TB, DG_SMALL, DG_SMALL><<<dim3((N + DG_SMALL - 1) / DG_SMALL, (M + DG_SMALL - 1) / DG_SMALL), DG_T, 0, s>>>(M, N, K, alpha, A, lda, B, ldb, beta, C,
                                                                                    ldc, lower, tri, status);
 }
 
@@ -359,12 +359,11 @@ cpm_status invert_and_project(cpm_ctx* c) {
     for (int64_t s = NB; s < n; s *= 2) {
         const int64_t pairs = (n - s + 2 * s - 1) / (2 * s);
         for (int step = 1; step <= 2; ++step) {
-            if ((s / 64) * (s / 64) * pairs >= DG_MANY)
-                k_trinv_level<64><<<dim3((unsigned)(s / 64), (unsigned)(s / 64), (unsigned)pairs), DG_T, 0, st>>>(
-                    W, c->S, n, (int)s, step, c->status);
+            const unsigned large = (unsigned)(s / DG_LARGE), small = (unsigned)(s / DG_SMALL);
+            if ((int64_t)large * large * pairs >= DG_MANY)
+                k_trinv_level<DG_LARGE><<<dim3(large, large, (unsigned)pairs), DG_T, 0, st>>>(W, c->S, n, (int)s, step, c->status);
             else
-                k_trinv_level<32><<<dim3((unsigned)(s / 32), (unsigned)(s / 32), (unsigned)pairs), DG_T, 0, st>>>(
-                    W, c->S, n, (int)s, step, c->status);
+                k_trinv_level<DG_SMALL><<<dim3(small, small, (unsigned)pairs), DG_T, 0, st>>>(W, c->S, n, (int)s, step, c->status);
         }
         CPM_LAUNCH(c, "k_trinv_level");
     }

@@ -770,11 +770,12 @@ template cpm_status rows_sf<float>(cpm_ctx*, cudaStream_t, const RowDims&, int, 
 // Which site stage, both sides measured (b alone, us, by height / every site by itself; plates with their sites moved onto
 // so many heights):
 //   tensor cores (their general stage costs little per replica, more per site):
-//     2,048 sites, 1 replica: 64 heights 46 / 61, 128 54 / 57, 256 79 / 60;  8 replicas: 32 82 / 90, 64 96 / 92, 128 128 / 90
-//     4,320 sites, 1 replica: 64 54 / 71, 130 60 / 66, 270 87 / 71;  8 replicas: 32 102 / 108, 64 115 / 116, 130 141 / 110
-//     16,384 sites, 1 replica: 256 133 / 209, 512 206 / 211;  8 replicas: 128 418 / 526, 256 531 / 524, 512 764 / 521
-//   FP32 on the CUDA cores, one replica: 2,048 sites, 256 heights 90 / 103; 4,320: 270 118 / 128, 540 171 / 128; 8,192:
-//     512 199 / 242; four: 4,320, 540 274 / 313
+//     512 sites, 1 replica: 51 heights 39 / 43, 64 40 / 44;  8 replicas: 32 44 / 47, 51 47 / 46, 64 51 / 47
+//     2,048 sites, 1 replica: 64 47 / 58, 97 51 / 57, 128 55 / 54, 204 65 / 58;  8 replicas: 32 81 / 86, 48 89 / 87, 64 96 / 86
+//     4,320 sites, 1 replica: 130 60 / 70, 196 68 / 71, 270 87 / 68;  8 replicas: 48 108 / 112, 64 115 / 115, 96 131 / 111
+//     16,384 sites, 1 replica: 364 147 / 210, 512 207 / 212;  8 replicas: 192 476 / 517, 256 531 / 519, 364 580 / 519
+//   FP32 on the CUDA cores, one replica: 2,048 sites, 256 heights 90 / 103; 4,320: 270 116 / 128, 360 134 / 128, 540 167 /
+//     128; 8,192: 512 200 / 244; four: 4,320, 540 275 / 311
 //   FP64: 4,320 sites, 540 heights 1,038 / 1,720
 bool rows_by_height(const cpm_ctx* c, int m) {
     const int64_t nu = c->nzu, n = c->n;

@@ -10,8 +10,11 @@
 // and a sum of at most 8 x 480 of them below 2^24, so the FP32 accumulation in tensor memory is exact, whatever
 // its order.  The sums S_w are combined as 64-bit integers, over the charge ranges too, and become FP64 once:
 //   R = sum_w S_w 2^(-12 - 7 w).
-// What is left out, i + j >= 8, is below 2^-56 per product where an FP64 multiplication rounds at 2^-54 |P h|; the
-// fixed-point operands are as accurate (2^-56) as the FP64 phases they come from.
+// What is left out, i + j >= 8, is at most 7 x 2^-56 per product P h, about 2^-53.2 (the seven digit products of order 8;
+// random operands 2^-56.2 in the mean square, 2^-53.9 at most), and the fixed-point operands are rounded at 2^-56: errors
+// in units of the replica's largest |Q|, where an FP64 multiply-add rounds relative to its own product and to the sum
+// so far.  A charge of 10^-6 of the largest keeps 35 bits; next to what the sums over all charges hold, b
+// is as far from 80-bit values as with the FP64 pipe (3e-13 on the EDL capacitor).
 //
 // One CTA: 32 pairs (128 rows) x 32 harmonics (64 functions) x one range of charges in steps of 32.  512 builders form
 // the digits: the products Q f_x f_y as the high half of a 64 x 64-bit integer product, two charges at a time

@@ -277,7 +277,7 @@ template <> struct PartSum<float> { using type = PartSumF; };   // partials of t
 // back.  Whole steps, before and now: 4,320 sites x 8 replicas 158.3 and 155.4 us, the product alone x 64 80.0 and
 // 74.5, 512 sites x 4 54.0 and 51.2, 256 small replicas 184 and 178.  Bounded by the latency of the loads and of
 // two cluster barriers, and FP64 at sixteen clocks a warp and SM: one warp adds a block's values (the product x 64
-// 67.9 with a tree per warp, 65.5 now).  48 registers let two blocks of 640 threads share an SM (with 64, one: the
+// 67.9 with a tree per warp, 65.5 without).  48 registers let two blocks of 640 threads share an SM (with 64, one: the
 // product took 89 us).
 constexpr int NB_CLUSTER = 16;  // blocks per replica, at most; more than eight where the replicas are few
 constexpr int NB_T = 640;      // threads per block, at most
