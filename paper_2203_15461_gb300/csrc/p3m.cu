@@ -35,7 +35,7 @@
 //   29 -> 14 us; 16,384 sites x 16 replicas, 64 planes, 141 -> 43 us.
 // Arithmetic in T = double (k_prec = FP64) or float (the single-precision paths); the influence
 // function is computed in FP64 and stored in T.
-#include <limits>
+#include <climits>
 
 #include "common.cuh"
 
@@ -209,33 +209,32 @@ template <typename T> struct P3mWords { static constexpr int n = std::is_same<T,
 constexpr int P3M_NT = 512;          // threads and charges per chunk of the assignment
 constexpr int P3M_CARRY = 1024;
 
-// Entries of a replica's lists: up to `most` per charge, which for the charges that one call may have is more than an int
-// holds (200 million charges at the corners of bricks).
-typedef unsigned long long p3m_pos;
+// Every (replica, split) has a list of its own, at most `most` entries for each of its `per` charges, so that positions in
+// it are ints: the plan takes enough splits for that.
 constexpr int P3M_MOST = 12;   // stencils of seven points over bricks of 32 x 32 x 4 (and no wider ones): 2 x 2 x 3
-static_assert((uint64_t)MAX_POINTS * P3M_MOST <= (uint64_t)std::numeric_limits<p3m_pos>::max(), "positions in the lists");
+static int64_t p3m_split_most(int most) { return (int64_t)INT_MAX / most / P3M_NT; }   // chunks of charges per split
+static_assert(MAX_POINTS / P3M_NT / ((int64_t)INT_MAX / P3M_MOST / P3M_NT) + 1 <= 8, "splits of the largest call");
 
-// start[r][split][brick]: exclusive sums of the nb counts of a replica, one block each
+// start[r][split][brick]: exclusive sums of the nb counts of a (replica, split), one block each
 constexpr int P3M_SCAN = 256;
-__global__ void __launch_bounds__(P3M_SCAN) k_p3m_scan(const int* __restrict__ count, int nb, p3m_pos* __restrict__ start) {
+__global__ void __launch_bounds__(P3M_SCAN) k_p3m_scan(const int* __restrict__ count, int nb, int* __restrict__ start) {
     grid_wait();
     grid_go();
-    __shared__ p3m_pos sw[P3M_SCAN / 32];
+    __shared__ int sw[P3M_SCAN / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t r0 = (int64_t)blockIdx.x * nb;
-    p3m_pos carry = 0;
+    int carry = 0;
     for (int i0 = 0; i0 < nb; i0 += P3M_SCAN) {
-        const int i = i0 + threadIdx.x;
-        const p3m_pos c = i < nb ? count[r0 + i] : 0;
-        p3m_pos v = c;
+        const int i = i0 + threadIdx.x, c = i < nb ? count[r0 + i] : 0;
+        int v = c;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            const p3m_pos u = __shfl_up_sync(0xffffffffu, v, o);
+            const int u = __shfl_up_sync(0xffffffffu, v, o);
             if (lane >= o) v += u;
         }
         if (lane == 31) sw[warp] = v;
         __syncthreads();
-        p3m_pos before = carry, all = 0;
+        int before = carry, all = 0;
 #pragma unroll
         for (int w = 0; w < P3M_SCAN / 32; ++w) {
             before += w < warp ? sw[w] : 0;
@@ -247,16 +246,16 @@ __global__ void __launch_bounds__(P3M_SCAN) k_p3m_scan(const int* __restrict__ c
     }
 }
 
-// list[r ne most + start + ..]: the charges of every brick and split (`per` charges each); the starts become ends
+// list[(r nsplit + split) per most + start + ..]: the charges of every brick; the starts become ends
 __global__ void __launch_bounds__(256) k_p3m_fill(const int* __restrict__ key, int64_t ptot, int64_t ne, int P, P3mBricks br,
-                                                int nsplit, int64_t per, int most, p3m_pos* __restrict__ start, int* __restrict__ list) {
+                                                int nsplit, int64_t per, int most, int* __restrict__ start, int* __restrict__ list) {
     grid_wait();
     const int64_t t = (int64_t)blockIdx.x * 256 + threadIdx.x;
     if (t >= ptot) return;
     const int64_t r = t / ne, j = t - r * ne, row = r * nsplit + j / per;
-    int* mine = list + r * ne * most;
+    int* mine = list + row * per * most;
     br.each(key[t], P, [&](int brick) {
-        mine[atomicAdd(&start[row * br.n() + brick], (p3m_pos)1)] = (int)j;
+        mine[atomicAdd(&start[row * br.n() + brick], 1)] = (int)j;
     });
 }
 
@@ -264,8 +263,8 @@ template <typename T, int P>
 __global__ void __launch_bounds__(P3M_NT) k_p3m_spread(const int* __restrict__ key,
                                                        const typename P3mV4<T>::t* __restrict__ fq, int64_t ne, int m,
                                                        int Kx, int Ky, int Kz, int BX, int BY,
-                                                       const int* __restrict__ count, const p3m_pos* __restrict__ start,
-                                                       const int* __restrict__ list, int most,
+                                                       const int* __restrict__ count, const int* __restrict__ start,
+                                                       const int* __restrict__ list, int64_t per, int most,
                                                        c2<T>* __restrict__ part, int* __restrict__ flag) {
     grid_wait();
     constexpr int NW = P3mWords<T>::n, BZ = P3M_BZ;
@@ -283,7 +282,7 @@ __global__ void __launch_bounds__(P3M_NT) k_p3m_spread(const int* __restrict__ k
     const int total = count[at];
     if (threadIdx.x == 0) flag[((int64_t)blockIdx.z * m + rep) * gridDim.x + bi] = total > 0;
     if (total == 0) return;   // uniform
-    const int* mine = list + base * most + start[at] - total;   // start holds the end
+    const int* mine = list + ((int64_t)rep * gridDim.z + blockIdx.z) * per * most + start[at] - total;   // start holds the end
     auto carry = [&]() {   // every point's words belong to one thread here
         __syncthreads();
         for (int i = threadIdx.x; i < NB; i += P3M_NT) {
@@ -667,7 +666,11 @@ static int64_t mesh_pts(const cpm_ctx* c) {
 // electrolyte, about a third, even out (16,384 sites x 16 replicas: 1,309 us a step without a split, 1,121 with three,
 // 1,109 with five, 1,130 with eight), no split with less than three chunks of charges (4,320 x 8: 190 us with six splits
 // of two, 182.5 with four of three: every split is a partial mesh to be written and added), at most 8.
-struct P3mSpread { int BX, BY, nbricks, nsplit, cps; P3mBricks br; };
+struct P3mSpread {
+    int BX, BY, nbricks, nsplit, cps;
+    P3mBricks br;
+    int64_t per() const { return (int64_t)cps * P3M_NT; }   // charges per split
+};
 static P3mSpread p3m_spread_plan(const cpm_ctx* c, int m, int64_t ne) {
     P3mSpread sp;
     const int Kx = c->p.p3m_mesh[0], Ky = c->p.p3m_mesh[1], Kz = c->p.p3m_mesh[2];
@@ -680,7 +683,7 @@ static P3mSpread p3m_spread_plan(const cpm_ctx* c, int m, int64_t ne) {
     int64_t ns = std::max<int64_t>(1, (32 * 152 + ctas - 1) / ctas);
     ns = std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(ns, 8), nchunks / 3));
     if (c->lean) ns = c->lean > 1 ? 1 : (ns + 3) / 4;
-    sp.cps = (int)((nchunks + ns - 1) / ns);
+    sp.cps = (int)std::min((nchunks + ns - 1) / ns, p3m_split_most(sp.br.most(c->p.p3m_order)));
     sp.nsplit = (int)((nchunks + sp.cps - 1) / sp.cps);
     return sp;
 }
@@ -690,8 +693,8 @@ size_t p3m_scratch_bytes(const cpm_ctx* c, int m, int64_t ne) {
     const int64_t ptot = (int64_t)m * ne;
     const P3mSpread sp = p3m_spread_plan(c, m, ne);
     return p3m_al(sizeof(int) * ptot) + p3m_al(sizeof(typename P3mV4<T>::t) * ptot) +
-           2 * p3m_al(sizeof(int) * (size_t)sp.nsplit * m * sp.nbricks) + p3m_al(sizeof(p3m_pos) * (size_t)sp.nsplit * m * sp.nbricks) +   // marks, counts, starts
-           p3m_al(sizeof(int) * (size_t)ptot * sp.br.most(c->p.p3m_order)) + p3m_al(sizeof(c2<T>) * (size_t)sp.nsplit * ((m + 1) / 2) * mesh_pts(c));
+           3 * p3m_al(sizeof(int) * (size_t)sp.nsplit * m * sp.nbricks) +   // marks, counts, starts
+           p3m_al(sizeof(int) * (size_t)m * sp.nsplit * std::min(sp.per(), ne) * sp.br.most(c->p.p3m_order)) + p3m_al(sizeof(c2<T>) * (size_t)sp.nsplit * ((m + 1) / 2) * mesh_pts(c));
 }
 template size_t p3m_scratch_bytes<float>(const cpm_ctx*, int, int64_t);
 template size_t p3m_scratch_bytes<double>(const cpm_ctx*, int, int64_t);
@@ -803,7 +806,7 @@ template <typename T> static const c2<T>* p3m_twiddles(const cpm_ctx* c) {
 
 template <typename T, int P>
 static cpm_status launch_p3m_pp(cudaStream_t st, cpm_ctx* c, int m, int64_t ne, const int* key,
-                          const typename P3mV4<T>::t* fq, int* flag, const int* count, const p3m_pos* start, const int* list, int most,
+                          const typename P3mV4<T>::t* fq, int* flag, const int* count, const int* start, const int* list, int64_t per, int most,
                           c2<T>* mesh, double* pm) {
     const int Kx = c->p.p3m_mesh[0], Ky = c->p.p3m_mesh[1], Kz = c->p.p3m_mesh[2];
     const P3mSpread sp = p3m_spread_plan(c, m, ne);
@@ -812,7 +815,7 @@ static cpm_status launch_p3m_pp(cudaStream_t st, cpm_ctx* c, int m, int64_t ne, 
                        sizeof(T) * P3M_NT * (3 * P + 1) + sizeof(int) * P3M_NT;
     CPM_CUDA(c, cudaFuncSetAttribute(k_p3m_spread<T, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssm));
     CPM_CUDA(c, launch_after(k_p3m_spread<T, P>, dim3(sp.nbricks, m, sp.nsplit), dim3(P3M_NT), ssm, st, key, fq, ne, m, Kx, Ky, Kz, sp.BX, sp.BY,
-                                                                            count, start, list, most, mesh, flag));
+                                                                            count, start, list, per, most, mesh, flag));
     const int64_t sstride = (int64_t)npairs * Kx * Ky * Kz;
     const c2<T>* tw = p3m_twiddles<T>(c);
     const size_t psm = sizeof(c2<T>) * ((size_t)Kx * Ky + Kx / 2 + Ky / 2);
@@ -850,28 +853,28 @@ cpm_status p3m_run(cpm_ctx* c, cudaStream_t st, int m, int64_t ne, const double*
     const P3mSpread sp = p3m_spread_plan(c, m, ne);
     const size_t lists = p3m_al(sizeof(int) * (size_t)sp.nsplit * m * sp.nbricks);
     int* count = (int*)((char*)flag + lists);
-    p3m_pos* start = (p3m_pos*)((char*)count + lists);
-    int* list = (int*)((char*)start + p3m_al(sizeof(p3m_pos) * (size_t)sp.nsplit * m * sp.nbricks));
+    int* start = (int*)((char*)count + lists);
+    int* list = (int*)((char*)start + lists);
     const int most = sp.br.most(c->p.p3m_order);
-    c2<T>* mesh = (c2<T>*)((char*)list + p3m_al(sizeof(int) * (size_t)ptot * most));
+    const int64_t per = std::min(sp.per(), ne);
+    c2<T>* mesh = (c2<T>*)((char*)list + p3m_al(sizeof(int) * (size_t)m * sp.nsplit * per * most));
     const int P = c->p.p3m_order;
     const int Kx = c->p.p3m_mesh[0], Ky = c->p.p3m_mesh[1], Kz = c->p.p3m_mesh[2];
-    const int64_t per = (int64_t)sp.cps * P3M_NT;
     CPM_CUDA(c, cudaMemsetAsync(count, 0, lists, st));
     k_p3m_prep<T><<<(unsigned)((ptot + 255) / 256), 256, 0, st>>>(xyz, Q, ptot, c->g, Kx, Ky, Kz, P, key, fq, ne, sp.br,
                                                                   sp.nsplit, per, count);
     CPM_LAUNCH(c, "k_p3m_prep");
-    CPM_CUDA(c, launch_after(k_p3m_scan, dim3((unsigned)m), dim3(P3M_SCAN), 0, st, count, sp.nsplit * sp.nbricks, start));
+    CPM_CUDA(c, launch_after(k_p3m_scan, dim3((unsigned)(m * sp.nsplit)), dim3(P3M_SCAN), 0, st, count, sp.nbricks, start));
     CPM_CUDA(c, launch_after(k_p3m_fill, dim3((unsigned)((ptot + 255) / 256)), dim3(256), 0, st, key, ptot, ne, P, sp.br, sp.nsplit,
                              per, most, start, list));
     c->launches += 8;
     switch (P) {
-        case 2: return launch_p3m_pp<T, 2>(st, c, m, ne, key, fq, flag, count, start, list, most, mesh, pm);
-        case 3: return launch_p3m_pp<T, 3>(st, c, m, ne, key, fq, flag, count, start, list, most, mesh, pm);
-        case 4: return launch_p3m_pp<T, 4>(st, c, m, ne, key, fq, flag, count, start, list, most, mesh, pm);
-        case 5: return launch_p3m_pp<T, 5>(st, c, m, ne, key, fq, flag, count, start, list, most, mesh, pm);
-        case 6: return launch_p3m_pp<T, 6>(st, c, m, ne, key, fq, flag, count, start, list, most, mesh, pm);
-        default: return launch_p3m_pp<T, 7>(st, c, m, ne, key, fq, flag, count, start, list, most, mesh, pm);
+        case 2: return launch_p3m_pp<T, 2>(st, c, m, ne, key, fq, flag, count, start, list, per, most, mesh, pm);
+        case 3: return launch_p3m_pp<T, 3>(st, c, m, ne, key, fq, flag, count, start, list, per, most, mesh, pm);
+        case 4: return launch_p3m_pp<T, 4>(st, c, m, ne, key, fq, flag, count, start, list, per, most, mesh, pm);
+        case 5: return launch_p3m_pp<T, 5>(st, c, m, ne, key, fq, flag, count, start, list, per, most, mesh, pm);
+        case 6: return launch_p3m_pp<T, 6>(st, c, m, ne, key, fq, flag, count, start, list, per, most, mesh, pm);
+        default: return launch_p3m_pp<T, 7>(st, c, m, ne, key, fq, flag, count, start, list, per, most, mesh, pm);
     }
 }
 // ----------------------------------------------------------------------------- the P3M elastance
