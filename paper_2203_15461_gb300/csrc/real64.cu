@@ -47,7 +47,12 @@ cpm_status build_real64(cpm_ctx* c, const std::vector<double>& etas) {
     const int nint = 1 + oct * R6_SUB;
     if (oct > 60) return CPM_OK;
     std::vector<double> tab((size_t)etas.size() * nint * R6_ROW);
-    const int N = R6_DEG + 1;
+    constexpr int N = R6_DEG + 1;
+    double node[N], cosine[N][N];   // Chebyshev nodes, cos(j acos(node i)): 0.3 ms of a set-up when formed per interval
+    for (int i = 0; i < N; ++i) {
+        node[i] = std::cos(PI * (i + 0.5) / N);
+        for (int j = 0; j < N; ++j) cosine[j][i] = std::cos(PI * j * (i + 0.5) / N);
+    }
     for (size_t t = 0; t < etas.size(); ++t)
         for (int k = 0; k < nint; ++k) {
             double lo = 0.0, hi = std::ldexp(1.0, e0);
@@ -58,10 +63,10 @@ cpm_status build_real64(cpm_ctx* c, const std::vector<double>& etas) {
             }
             const double mid = 0.5 * (lo + hi), half = 0.5 * (hi - lo);
             double gk[N], ch[N], mono[N] = {}, t0[N] = {}, t1[N] = {}, tn[N] = {};
-            for (int i = 0; i < N; ++i) gk[i] = pair_f(std::sqrt(mid + half * std::cos(PI * (i + 0.5) / N)), c->g.alpha, etas[t]);
+            for (int i = 0; i < N; ++i) gk[i] = pair_f(std::sqrt(mid + half * node[i]), c->g.alpha, etas[t]);
             for (int j = 0; j < N; ++j) {
                 double s = 0.0;
-                for (int i = 0; i < N; ++i) s += gk[i] * std::cos(PI * j * (i + 0.5) / N);
+                for (int i = 0; i < N; ++i) s += gk[i] * cosine[j][i];
                 ch[j] = (j == 0 ? 1.0 : 2.0) * s / N;
             }
             t0[0] = 1.0;
