@@ -185,6 +185,7 @@ constexpr int ROW64_PAIRS = 32, ROW64_HARM = 32, ROW64_STEP = 32;   // the same 
                                                                     // harmonics per CTA
 constexpr int ROW64_EMAX = 2044;       // largest biased exponent of a charge that it can scale (|Q| < 2^1022)
 struct RowTable {
+    char* blob = nullptr;                // the allocation that holds all of the tables below
     int np = 0, nrows = 0, nslots = 0;   // pairs, rows that are not identically zero, (nx, ny) slots
     int nchunk = 0, ntiles = 0;          // nx ranges and site tiles of the site stage
     int chunkmax = 0;                    // most slots of one range

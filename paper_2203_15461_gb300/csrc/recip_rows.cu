@@ -14,6 +14,7 @@
 // sites: stage 2 sums the harmonics once per height instead of once per site, and stage 3 is left with
 // one term per (site, pair, part) instead of one per (site, k).  Electrodes whose sites hardly share
 // heights (rows_by_height) take the general site stage of bvec.cu or tc_recip.cu, whose operand w rho over signed columns k_rows_to_cols forms from R.
+#include <cstring>
 #include <vector>
 
 #include "common.cuh"
@@ -63,21 +64,43 @@ __global__ void k_layer_phases(const double* __restrict__ zu, int nzu, double iz
     ZU[t] = row_phase<T>(row_frac(zu[t % nzu], iz), t / nzu);
 }
 
+constexpr int FX_TAB = 1024;   // entries of each of the two tables of the fixed-point phases
 static cpm_status charge_fixed_table(cpm_ctx* c);
+
+// The tables of a geometry in one allocation, those formed on the host copied at once: with an allocation, a copy and a
+// free each, some fifteen of them, a preparation took 50 to 100 us more (216 sites: FP64 936 us, now 859; FP32 822 and 773;
+// F16X2 828 and 771).
+class RowBlob {
+    struct Part { void** ptr; size_t at; };
+    std::vector<Part> parts;
+    std::vector<char> host;
+    size_t total = 0;
+    static size_t al(size_t b) { return (b + 255) & ~(size_t)255; }
+
+public:
+    template <typename V> void put(V** d, const std::vector<V>& h) {   // before the first room()
+        parts.push_back({(void**)d, total});
+        host.resize(al(total + sizeof(V) * std::max<size_t>(1, h.size())));
+        if (!h.empty()) memcpy(&host[total], h.data(), sizeof(V) * h.size());
+        total = host.size();
+    }
+    template <typename V> void room(V** d, size_t count) {
+        parts.push_back({(void**)d, total});
+        total = al(total + sizeof(V) * std::max<size_t>(1, count));
+    }
+    // the copy is done when the stream is: the blob lives until then
+    cpm_status place(cpm_ctx* c, char** base) {
+        CPM_TRY(dev_alloc(c, (void**)base, total));
+        for (const Part& p : parts) *p.ptr = *base + p.at;
+        CPM_CUDA(c, cudaMemcpyAsync(*base, host.data(), host.size(), cudaMemcpyHostToDevice, c->stream));
+        return CPM_OK;
+    }
+};
 
 void free_rows(cpm_ctx* c) {
     RowTable& t = c->rows;
-    for (void* p : {(void*)t.pairs, (void*)t.list, (void*)t.W, (void*)t.W32, (void*)t.nxoff, (void*)t.chunkb,
-                    (void*)t.zu64, (void*)t.zu32, (void*)t.lperm, (void*)t.ltiles, (void*)t.paircols, (void*)t.tcitem, (void*)t.atiles, (void*)t.item64, (void*)t.fxtab,
-                    (void*)t.tcrange})
-        dev_free(c, p);
+    dev_free(c, t.blob);
     t = RowTable{};
-}
-
-template <typename V> static cpm_status upload(cpm_ctx* c, V** d, const std::vector<V>& h) {
-    CPM_TRY(dev_alloc(c, (void**)d, sizeof(V) * std::max<size_t>(1, h.size())));
-    if (!h.empty()) CPM_CUDA(c, cudaMemcpyAsync(*d, h.data(), sizeof(V) * h.size(), cudaMemcpyHostToDevice, c->stream));
-    return CPM_OK;
 }
 
 // After build_ktable and the site heights (zuniq, zmap): the pairs in the order of |k_perp| with their
@@ -88,6 +111,7 @@ cpm_status build_rows(cpm_ctx* c) {
     const KTable& k = c->kt;
     if (k.nk == 0) return CPM_OK;
     const int64_t n = c->n;
+    RowBlob blob;
     std::vector<int2> cols(k.ncols);
     std::vector<int> ext(k.ncols), zm(n);
     CPM_CUDA(c, cudaMemcpyAsync(cols.data(), k.cols, sizeof(int2) * k.ncols, cudaMemcpyDeviceToHost, c->stream));
@@ -137,8 +161,8 @@ cpm_status build_rows(cpm_ctx* c) {
             if (!ok && (ok = plan_items(*o))) order = *o;
         if (ok) {
             t.tcitems = (int)titem.size();
-            CPM_TRY(upload(c, &t.tcitem, titem));
-            CPM_TRY(upload(c, &t.tcrange, trange));
+            blob.put(&t.tcitem, titem);
+            blob.put(&t.tcrange, trange);
         }
     }
     for (int q : order) {
@@ -163,9 +187,7 @@ cpm_status build_rows(cpm_ctx* c) {
                 i64.push_back(make_int4((int)f, (int)(e - f), z, std::min(ROW64_HARM, mx + 1 - z)));
         }
         t.items64 = (int)i64.size();
-        CPM_TRY(upload(c, &t.item64, i64));
-        CPM_TRY(charge_fixed_table(c));
-        CPM_CUDA(c, cudaStreamSynchronize(c->stream));
+        blob.put(&t.item64, i64);
     }
     t.np = (int)pairs.size();
     t.nrows = (int)list.size();
@@ -204,32 +226,35 @@ cpm_status build_rows(cpm_ctx* c) {
         t.ntiles = (int)tiles.size();
         for (int u = 0; u < c->nzu; ++u)
             for (int f = cnt[u]; f < cnt[u + 1]; f += 64) t.hatiles.push_back(make_int4(u, f, std::min(64, cnt[u + 1] - f), 0));
-        CPM_TRY(upload(c, &t.atiles, t.hatiles));
-        CPM_TRY(upload(c, &t.lperm, perm));
-        CPM_TRY(upload(c, &t.ltiles, tiles));
-        CPM_CUDA(c, cudaStreamSynchronize(c->stream));
+        blob.put(&t.atiles, t.hatiles);
+        blob.put(&t.lperm, perm);
+        blob.put(&t.ltiles, tiles);
     }
     int* dcol = nullptr;
-    CPM_TRY(upload(c, &t.pairs, pairs));
-    CPM_TRY(upload(c, &t.list, list));
-    CPM_TRY(upload(c, &t.nxoff, off));
-    CPM_TRY(upload(c, &t.paircols, pcols));
-    CPM_TRY(upload(c, &t.chunkb, cb));
-    CPM_TRY(upload(c, &dcol, col));
+    blob.put(&t.pairs, pairs);
+    blob.put(&t.list, list);
+    blob.put(&t.nxoff, off);
+    blob.put(&t.paircols, pcols);
+    blob.put(&t.chunkb, cb);
+    blob.put(&dcol, col);
     const size_t nw = (size_t)t.np * (k.NZ + 1), nu = (size_t)c->nzu * (k.NZ + 1);
-    CPM_TRY(dev_alloc(c, (void**)&t.W, sizeof(double) * nw));
-    CPM_TRY(dev_alloc(c, (void**)&t.W32, sizeof(float) * nw));
+    blob.room(&t.W, nw);
+    blob.room(&t.W32, nw);
+    if (t.layered) {
+        blob.room(&t.zu64, nu);
+        blob.room(&t.zu32, nu);
+    }
+    if (c->p.k_prec == CPM_PREC_FP64) blob.room(&t.fxtab, 2 * FX_TAB);
+    CPM_TRY(blob.place(c, &t.blob));
+    if (c->p.k_prec == CPM_PREC_FP64) CPM_TRY(charge_fixed_table(c));
     k_pair_weights<<<(unsigned)((nw + 255) / 256), 256, 0, c->stream>>>(t.pairs, dcol, t.np, k.NZ, k.w, k.w32, t.W, t.W32);
     CPM_LAUNCH(c, "k_pair_weights");
     if (t.layered) {
-        CPM_TRY(dev_alloc(c, (void**)&t.zu64, sizeof(double2) * nu));
-        CPM_TRY(dev_alloc(c, (void**)&t.zu32, sizeof(float2) * nu));
         k_layer_phases<double><<<(unsigned)((nu + 255) / 256), 256, 0, c->stream>>>(c->zuniq, c->nzu, c->g.inv[2], k.NZ, t.zu64);
         k_layer_phases<float><<<(unsigned)((nu + 255) / 256), 256, 0, c->stream>>>(c->zuniq, c->nzu, c->g.inv[2], k.NZ, t.zu32);
         CPM_LAUNCH(c, "k_layer_phases");
     }
     CPM_CUDA(c, cudaStreamSynchronize(c->stream));
-    dev_free(c, dcol);
     return CPM_OK;
 }
 
@@ -318,7 +343,6 @@ __global__ void __launch_bounds__(8 * CP_PTS) k_charge_phases(const double* __re
 // product of two phases is some 40 instructions of a pipe with thirty times the rate.  A phase is evaluated as T1[top
 // ten bits] T2[next ten] (1 - d^2 / 2, d - d^3 / 6) with the angle d < 2 pi 2^-20 of the other 44 bits: the terms
 // left out are below 2^-72, T1 is FP64's own cosine and sine, and T2's are kept as 1 - cos, exact to 2^-62.
-constexpr int FX_TAB = 1024;
 __global__ void k_fixed_tab(longlong2* __restrict__ tab) {   // grid 2 x FX_TAB: T1 | T2
     const int t = threadIdx.x;
     double s, c;
@@ -399,9 +423,6 @@ __global__ void __launch_bounds__(8 * CP_PTS) k_charge_fixed(const double* __res
     }
 }
 static cpm_status charge_fixed_table(cpm_ctx* c) {
-    dev_free(c, c->rows.fxtab);
-    c->rows.fxtab = nullptr;
-    CPM_TRY(dev_alloc(c, (void**)&c->rows.fxtab, sizeof(longlong2) * 2 * FX_TAB));
     k_fixed_tab<<<2, FX_TAB, 0, c->stream>>>(c->rows.fxtab);
     CPM_LAUNCH(c, "k_fixed_tab");
     return CPM_OK;
