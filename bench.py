@@ -957,7 +957,7 @@ def main():
                              "tensor_complex_mac": FLOP_CMAC}
     # DRAM bytes (read + write) per launch from the committed ncu capture of these kernels on this
     # workload (cold caches); a stored figure, not measured by this run
-    traffic_ncu = {"gemv": 75.07e6, "real": 1.42e6}
+    traffic_ncu = {"sf": 15.20e6, "site": 0.99e6, "gemv": 75.02e6, "real": 1.41e6}
     roof["traffic"] = traffic_ncu.get(top)
     roof["traffic_source"] = ("stored: ncu dram__bytes_read.sum + dram__bytes_write.sum of one launch, "
                               "profiles/launches_edl_capacitor_4320.md")
